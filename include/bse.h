@@ -221,10 +221,12 @@ int bse_dipoles(bse_ctx* ctx, bse_interp* interp, int npol, const double* pol_di
 int bse_apply_h(bse_ctx* ctx, bse_interp* interp, int nvec, const void* x, void* y);
 
 /* Same result as bse_apply_h, but allocates no device memory: the per-call
- * scratch comes from one static device array of 32 MiB inside the library
+ * Q, R, operands and partials come from one static device array of 32 MiB inside the library
  * (held by a device from the time the library's device module is loaded on
  * it, at the latest the first bse_ctx_create on that device, until the
- * process exits), not from the handle.  The paper has no counterpart; this
+ * process exits); what set-up allocated for the handle's own intermediate
+ * vectors is used as bse_apply_h uses it, so calls on one handle must not
+ * overlap.  The paper has no counterpart; this
  * exists for callers that must not call cudaMalloc once their work has
  * started, such as a host framework that owns all device memory through its
  * own pool, or a loop where cudaMalloc's implicit device synchronisation is

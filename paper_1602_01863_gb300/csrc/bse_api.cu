@@ -1,4 +1,5 @@
 // extern "C" entry points of the library (see include/bse.h for the contract).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <atomic>
@@ -27,6 +28,20 @@ int upload(bse_ctx* ctx, P** dst, const double* src, size_t ndouble, const char*
     return BSE_OK;
 }
 
+// Hermitian to rounding: [count][nb][nb] complex, against the largest entry.
+bool hermitian(const double* g, int count, int nb) {
+    double big = 0.0, off = 0.0;
+    for (int m = 0; m < count; ++m)
+        for (int i = 0; i < nb; ++i)
+            for (int j = 0; j < nb; ++j) {
+                const double* a = g + 2 * (((size_t)m * nb + i) * nb + j);
+                const double* b = g + 2 * (((size_t)m * nb + j) * nb + i);
+                big = std::max(big, std::max(std::fabs(a[0]), std::fabs(a[1])));
+                off = std::max(off, std::max(std::fabs(a[0] - b[0]), std::fabs(a[1] + b[1])));
+            }
+    return off <= 1e-15 * big;
+}
+
 void free_coarse(bse_coarse* c) {
     if (!c) return;
     cudaFree(c->d_offsets); cudaFree(c->d_gen_v); cudaFree(c->d_gen_c); cudaFree(c->d_mu);
@@ -42,7 +57,9 @@ void free_interp(bse_interp* s) {
                     s->d_vec[1], s->d_vec[2], s->d_part_dot, s->d_part_nrm, s->d_a, s->d_aim, s->d_b, s->d_stop,
                     s->d_basis, s->d_cgs_part, s->d_cgs_h, s->d_pairs, s->d_clist, s->d_cstart,
                     s->d_lker, s->d_lgrid, s->d_tw_fwd, s->d_tc_rows, s->d_tc_slots,
-                    s->d_tc_kinfo, s->d_tc_simg, s->d_tc_aimg, s->d_xscale, s->d_xscale_gen, s->d_H2};
+                    s->d_tc_kinfo, s->d_tc_simg, s->d_tc_aimg, s->d_xscale, s->d_xscale_gen, s->d_H2,
+                    s->d_cUv, s->d_cUc, s->d_cUvc, s->d_cUcc, s->d_cshare, s->d_cctr, s->d_chead, s->d_cphi, s->d_cV,
+                    s->d_cw};
     for (void* p : ptrs) cudaFree(p);
     bse_tc_release(s);
     delete s;
@@ -144,6 +161,7 @@ int bse_build_coarse(bse_ctx* ctx, const bse_model* m, int n_coarse, int kc_prec
     c->eps_inf = m->eps_inf; c->kappa = m->kappa; c->e_k = m->e_k; c->e_gap = m->e_gap;
     c->band_width = m->band_width; c->h0 = m->h0; c->direct_shells = m->direct_shells;
     c->h_const = m->h_const ? 1 : 0; c->exchange_on = m->exchange_on ? 1 : 0;
+    c->unitary = hermitian(m->gen_v, 6, nv) && hermitian(m->gen_c, 6, nc) ? 1 : 0;
     c->alpha = -(m->e_k / c->nkc) * 4.0 * 3.14159265358979323846 / m->eps_inf;
     int rc;
     if ((rc = upload(ctx, &c->d_offsets, m->offsets, nv * nc, "offsets")) != BSE_OK ||

@@ -1517,6 +1517,7 @@ inline bool staged_bands(const bse_interp* s) {
 // Number of <psi, w> block partials one H application leaves in the dot buffer.
 inline int dot_blocks(const bse_interp* s) {
     if (s->scheme == BSE_SCHEME_M2) return m2_blocks(s->N);
+    if (!s->learned && s->common) return bse_common_dot_blocks(s);
     if (!s->learned && staged_bands(s)) return std::min(s->co->nkc, kProlongMaxCtas);
     return vec_blocks(s->N);
 }
@@ -1684,6 +1685,53 @@ inline bool near_tc_active(const bse_interp* s) {
     return s->scheme == BSE_SCHEME_M3 && s->nf_tc && !s->nf_force_cuda_cores;
 }
 
+// H application in the common basis (bse_common.cu).  The near stencil and the
+// K_c apply read only what restrict wrote and run side by side, the apply on
+// the lane's auxiliary stream; profiled runs keep the kernels one after another.
+template <typename T>
+int apply_h_common(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi, void* W, bool prof) {
+    using V = typename Cx<T>::V;
+    const bse_coarse* c = s->co;
+    cudaStream_t st = ctx->stream;
+    const int ln = ctx->lane;
+    const bool m3 = s->scheme == BSE_SCHEME_M3, beside = m3 && !prof && ctx->aux[ln];
+    int rc;
+    {
+        Timer tm(ctx, prof, KC_RESTRICT);
+        if ((rc = bse_common_restrict(ctx, s, nchains, psi, s->d_Q, s->d_Bop, st)) != BSE_OK) return rc;
+    }
+    cudaStream_t kst = beside ? ctx->aux[ln] : st;
+    if (beside) {
+        BSE_CUDA_TRY(ctx, cudaEventRecord(ctx->aux_fork[ln], st));
+        BSE_CUDA_TRY(ctx, cudaStreamWaitEvent(kst, ctx->aux_fork[ln], 0));
+    }
+    {
+        Timer tm(ctx, prof, KC_KCAPPLY);
+        if (c->kc_prec == BSE_PREC_BF16) {
+            if ((rc = bse_tc_apply(ctx, s, nchains, kst, false, 0)) != BSE_OK) return rc;
+        } else {
+            k_kc_apply_simt<T><<<(c->Nc + 7) / 8, 256, 0, kst>>>((const V*)c->d_kc, (const V*)s->d_Q, c->Nc, nchains, (V*)s->d_R);
+        }
+    }
+    if (m3) {
+        Timer tm(ctx, prof, KC_NEAR);
+        if ((rc = bse_common_near(ctx, s, nchains, st)) != BSE_OK) return rc;
+    }
+    if (beside) {
+        BSE_CUDA_TRY(ctx, cudaEventRecord(ctx->aux_join[ln], kst));
+        BSE_CUDA_TRY(ctx, cudaStreamWaitEvent(st, ctx->aux_join[ln], 0));
+    }
+    {
+        Timer tm(ctx, prof, KC_PROLONG);
+        if ((rc = bse_common_prolong(ctx, s, nchains, s->d_R, psi, W, s->d_part_dot, st)) != BSE_OK) return rc;
+    }
+    if (s->learned) {
+        Timer tm(ctx, prof, KC_NEAR);
+        if ((rc = bse_apply_learned(ctx, s, nchains, psi, W, s->d_part_dot)) != BSE_OK) return rc;
+    }
+    return BSE_OK;
+}
+
 // unit: every psi has 2-norm 1 (the Lanczos vectors), so the FP16 piece scale
 // set up for unit vectors applies; otherwise it is computed from the norms.
 template <typename T>
@@ -1702,6 +1750,7 @@ int apply_h_typed(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi_v, v
         return BSE_OK;
     }
     const bool m3 = s->scheme == BSE_SCHEME_M3;
+    if (s->common) return apply_h_common<T>(ctx, s, nchains, psi_v, w_v, prof);
     const bool xh = near_tc_active(s);
     void* X = m3 ? s->d_X : nullptr;
     const float* xscale = unit ? s->d_xscale : s->d_xscale_gen;
@@ -2299,6 +2348,19 @@ int apply_scratch_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const vo
         return BSE_OK;
     }
     const bool m3 = s->scheme == BSE_SCHEME_M3;
+    if (s->common) {
+        int rc;
+        if (c->kc_prec == BSE_PREC_BF16) {
+            BSE_CUDA_TRY(ctx, cudaMemsetAsync(sc.bop, 0, sizeof(__nv_bfloat16) * 16 * (size_t)c->ldk, st));
+            if ((rc = bse_common_restrict(ctx, s, nchains, psi, nullptr, sc.bop, st)) != BSE_OK) return rc;
+            if ((rc = bse_tc_apply_scratch(ctx, s, nchains, sc.bop, sc.part, sc.R)) != BSE_OK) return rc;
+        } else {
+            if ((rc = bse_common_restrict(ctx, s, nchains, psi, sc.Q, nullptr, st)) != BSE_OK) return rc;
+            k_kc_apply_simt<T><<<(c->Nc + 7) / 8, 256, 0, st>>>((const V*)c->d_kc, (const V*)sc.Q, c->Nc, nchains, (V*)sc.R);
+        }
+        if (m3 && (rc = bse_common_near(ctx, s, nchains, st)) != BSE_OK) return rc;
+        return bse_common_prolong(ctx, s, nchains, sc.R, psi, W, sc.dot, st);
+    }
     const bool xh = near_tc_active(s);
     void* X = m3 ? sc.X : nullptr;
     if (xh) k_chain_xscale<<<nchains, 256, 0, st>>>((const float2*)psi, s->N, s->dbound, s->d_xscale_gen);

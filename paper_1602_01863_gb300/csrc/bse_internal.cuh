@@ -152,7 +152,13 @@ struct bse_coarse {
     double2 *d_Uv = nullptr, *d_Uc = nullptr;     // coarse band gauge
     void* d_kc = nullptr;                         // K_c storage
     __nv_bfloat16 *d_kr = nullptr, *d_ki = nullptr; // BF16 planes (inside d_kc)
+    int unitary = 0;                              // the gauge generators are Hermitian: U(k) is unitary
 };
+
+// Layout of the common-basis vectors phi: [group][x][y][L + 2 R][32] reals, group
+// g holding the columns 32 g .. 32 g + 31 of the (chain, transition, re|im)
+// components of a dense point; z starts R points before 0 (periodic halo).
+struct CommonPhi { int R, Lp; };
 
 struct NearEntry { int co; int js_src; int l_src; int near_idx; };   // co packed 3 x 4 bits (+8 bias)
 
@@ -168,6 +174,18 @@ struct bse_interp {
     void* d_Dv = nullptr;            // V [nk][8][nv*nv]
     void* d_Dc = nullptr;            // V [nk][8][nc*nc]
     double2* d_P = nullptr;          // [3][N]
+    // common-basis path (bse_common.cu): the dense tables come from the model and
+    // its gauge is unitary, so overlaps and Method-3 heads factor through U(k)
+    int common = 0;
+    void *d_cUv = nullptr, *d_cUc = nullptr;     // V [nk][nv*nv], [nk][nc*nc] dense gauge
+    void *d_cUvc = nullptr, *d_cUcc = nullptr;   // V [nkc][nv*nv], [nkc][nc*nc] coarse gauge
+    void* d_cshare = nullptr;        // V [4][nkc][8][t] the cells' shares of their corners
+    int* d_cctr = nullptr;           // [4][nkc] shares written (zero between launches)
+    int cphi_R = 0, near_R2 = 0;     // near offsets: |delta|^2 <= near_R2, components within cphi_R
+    double* d_chead = nullptr;       // [nkc] h_head over coarse differences (set-up only)
+    void* d_cphi = nullptr;          // T, layout CommonPhi
+    void* d_cV = nullptr;            // V [4][N] near stencil result
+    void* d_cw = nullptr;            // T near stencil weights
     // M3 tables
     int n_near = 0, smin = 0, ns1 = 0, nslot = 0, rmin = 0, nr1 = 0, nrel = 0;
     NearEntry* d_list = nullptr;
@@ -309,6 +327,14 @@ int bse_apply_learned(bse_ctx* ctx, const bse_interp* s, int nchains, const void
 int bse_near_tc_prepare(bse_ctx* ctx, bse_interp* s, const std::vector<std::vector<NearEntry>>& per_slot);
 int bse_near_tc_launch(bse_ctx* ctx, const bse_interp* s, int nchains, const void* Xh, const float* xscale, void* U,
                        bool prio = false, int prio_value = 0);
+// common-basis path (bse_common.cu)
+int bse_common_prepare(bse_ctx* ctx, bse_interp* s, const double2* Uvd, const double2* Ucd);
+int bse_common_dot_blocks(const bse_interp* s);
+int bse_common_restrict(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, void* Q, __nv_bfloat16* bop,
+                        cudaStream_t st);
+int bse_common_near(bse_ctx* ctx, const bse_interp* s, int nchains, cudaStream_t st);
+int bse_common_prolong(bse_ctx* ctx, const bse_interp* s, int nchains, const void* R, const void* psi, void* W,
+                       double2* dot, cudaStream_t st);
 float bse_near_tc_xscale(const bse_interp* s, double norm);
 size_t bse_tc_part_bytes(const bse_interp* s);
 int bse_tc_apply_scratch(bse_ctx* ctx, const bse_interp* s, int nchains, __nv_bfloat16* bop, float* part, void* R);

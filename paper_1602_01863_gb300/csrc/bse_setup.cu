@@ -604,6 +604,35 @@ int build_m2(bse_ctx* ctx, bse_interp* s) {
     return BSE_OK;
 }
 
+// Method 3's near offsets |delta|^2 <= R2 (three ints each into `offs`, when
+// given) and the boxes of coarse points they reach.
+int near_geometry(bse_ctx* ctx, bse_interp* s, std::vector<int>* offs) {
+    const int nd = s->nd, R2 = (int)std::floor(s->width * s->width * nd * nd + 1e-9);
+    const int rad = (int)std::floor(std::sqrt((double)R2) + 1e-12);
+    s->near_R2 = R2;
+    s->cphi_R = rad;
+    s->n_near = 0;
+    for (int a = -rad; a <= rad; ++a)
+        for (int b = -rad; b <= rad; ++b)
+            for (int cc = -rad; cc <= rad; ++cc)
+                if (a * a + b * b + cc * cc <= R2) {
+                    ++s->n_near;
+                    if (offs) { offs->push_back(a); offs->push_back(b); offs->push_back(cc); }
+                }
+    s->smin = floordiv(-rad, nd);
+    const int smax = floordiv(nd - 1 + rad, nd) + 1;
+    s->ns1 = smax - s->smin + 1;
+    s->nslot = s->ns1 * s->ns1 * s->ns1;
+    s->rmin = s->smin - 1;
+    s->nr1 = smax - s->rmin + 1;
+    s->nrel = s->nr1 * s->nr1 * s->nr1;
+    if (s->ns1 > 15 || s->smin < -8 || smax > 7) {
+        ctx->err = "M3 width too large for the near-field tables";
+        return BSE_ERR_UNSUPPORTED;
+    }
+    return BSE_OK;
+}
+
 template <typename T>
 int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dense) {
     using V = typename Cx<T>::V;
@@ -625,12 +654,25 @@ int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dens
                                                         (V*)s->d_Dv, (V*)s->d_Dc, s->d_P);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(d_Uvd);
-    cudaFree(d_Ucd);
     if (e != cudaSuccess) {
+        cudaFree(d_Uvd);
+        cudaFree(d_Ucd);
         ctx->err = std::string("dense set-up kernels: ") + cudaGetErrorString(e);
         return BSE_ERR_CUDA;
     }
+    // Overlaps that are products through one unitary gauge: the common-basis path
+    // (Method 2 stores its H instead).
+    s->common = s->scheme != BSE_SCHEME_M2 && c->unitary && !(dense && (dense->Dv || dense->Dc));
+    int crc = BSE_OK;
+    if (s->common && s->scheme == BSE_SCHEME_M3) {
+        crc = near_geometry(ctx, s, nullptr);
+        if (crc == BSE_OK) crc = bse_alloc(ctx, (void**)&s->d_chead, sizeof(double) * c->nkc, "coarse head table");
+        if (crc == BSE_OK) k_shape_table<<<blocks_for(c->nkc, 128), 128, 0, st>>>(n, c->kappa, 27, 0, 0.0, 1, s->d_chead);
+    }
+    if (s->common && crc == BSE_OK) crc = bse_common_prepare(ctx, s, d_Uvd, d_Ucd);
+    cudaFree(d_Uvd);
+    cudaFree(d_Ucd);
+    if (crc != BSE_OK) return crc;
     s->dbound = std::sqrt((double)nv) * std::sqrt((double)nc);
     if (dense) TRY(apply_dense_inputs<T>(ctx, s, dense));
     // scratch
@@ -644,29 +686,12 @@ int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dens
     if (s->scheme == BSE_SCHEME_M2) {
         if constexpr (std::is_same<T, double>::value) TRY(build_m2(ctx, s));
     }
-    if (s->scheme == BSE_SCHEME_M3) {
+    if (s->scheme == BSE_SCHEME_M3 && !s->common) {
         TRY(bse_alloc(ctx, &s->d_X, sizeof(V) * nvec * nk * 8 * t, "restricted pieces X"));
         TRY(bse_alloc(ctx, &s->d_U, sizeof(V) * nvec * nk * 8 * t, "near-field pieces"));
-        // near offsets and contribution lists (integer bookkeeping on the host)
-        const int R2 = (int)std::floor(s->width * s->width * nd * nd + 1e-9);
-        const int rad = (int)std::floor(std::sqrt((double)R2) + 1e-12);
+        // contribution lists (integer bookkeeping on the host)
         std::vector<int> offs;
-        for (int a = -rad; a <= rad; ++a)
-            for (int b = -rad; b <= rad; ++b)
-                for (int cc = -rad; cc <= rad; ++cc)
-                    if (a * a + b * b + cc * cc <= R2) { offs.push_back(a); offs.push_back(b); offs.push_back(cc); }
-        s->n_near = (int)offs.size() / 3;
-        s->smin = floordiv(-rad, nd);
-        const int smax = floordiv(nd - 1 + rad, nd) + 1;
-        s->ns1 = smax - s->smin + 1;
-        s->nslot = s->ns1 * s->ns1 * s->ns1;
-        s->rmin = s->smin - 1;
-        s->nr1 = smax - s->rmin + 1;
-        s->nrel = s->nr1 * s->nr1 * s->nr1;
-        if (s->ns1 > 15 || s->smin < -8 || smax > 7) {
-            ctx->err = "M3 width too large for the near-field tables";
-            return BSE_ERR_UNSUPPORTED;
-        }
+        TRY(near_geometry(ctx, s, &offs));
         const int Ndiv = s->Ndiv;
         std::vector<std::vector<NearEntry>> per_slot((size_t)Ndiv * s->nslot);
         for (int js = 0; js < Ndiv; ++js) {
