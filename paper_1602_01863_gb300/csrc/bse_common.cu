@@ -50,6 +50,11 @@ __device__ __forceinline__ void cfmac(V& acc, V a, V b) {
     acc.y = fma(a.y, b.x, fma(-a.x, b.y, acc.y));
 }
 
+// i / len for small i (len <= 64 entries, i < 2^13: the quotient is at least 1/128
+// away from the next integer), with the reciprocal of len: integer divisions by
+// run-time lengths were most of these kernels' instructions.
+__device__ __forceinline__ int quot(int i, float inv) { return (int)(((float)i + 0.5f) * inv); }
+
 // One row (fixed valence index) of a point's block, in place:
 // TO: y[m] = sum_c x[c] Uc[m][c];  else y[c] = sum_m x[m] conj(Uc[m][c]).
 template <bool TO, int NB, typename V>
@@ -94,8 +99,9 @@ __device__ __forceinline__ void rot_col(V* x, int st, const V* U) {
 template <bool TO, typename V>
 __device__ __forceinline__ void rotate_blocks(V* x, int tp, const V* Uv, int rvp, const V* Uc, int rcp, int np, int nv,
                                               int nc) {
+    const float inv_v = 1.f / (float)nv, inv_c = 1.f / (float)nc;
     for (int i = threadIdx.x; i < np * nv; i += blockDim.x) {
-        const int p = i / nv, v = i - p * nv;
+        const int p = quot(i, inv_v), v = i - p * nv;
         V* r = x + p * tp + v * nc;
         const V* U = Uc + p * rcp;
         switch (nc) {
@@ -111,7 +117,7 @@ __device__ __forceinline__ void rotate_blocks(V* x, int tp, const V* Uv, int rvp
     }
     __syncthreads();
     for (int i = threadIdx.x; i < np * nc; i += blockDim.x) {
-        const int p = i / nc, c = i - p * nc;
+        const int p = quot(i, inv_c), c = i - p * nc;
         V* r = x + p * tp + c;
         const V* U = Uv + p * rvp;
         switch (nv) {
@@ -131,10 +137,19 @@ __device__ __forceinline__ void rotate_blocks(V* x, int tp, const V* Uv, int rvp
 // Rows of `len` entries from global src (row r at src + r * len) into shared dst (row pitch `pitch`).
 template <typename V>
 __device__ __forceinline__ void load_rows(V* dst, int pitch, const V* __restrict__ src, int rows, int len) {
+    const float inv = 1.f / (float)len;
     for (int i = threadIdx.x; i < rows * len; i += blockDim.x) {
-        const int r = i / len;
+        const int r = quot(i, inv);
         dst[r * pitch + (i - r * len)] = src[i];
     }
+}
+
+// Weight of corner l at sub-cell position (j1, j2, j3) (interp_weight).
+template <typename T>
+__device__ __forceinline__ T corner_weight(int j1, int j2, int j3, int l, int nd, int nb1) {
+    const int l1 = (l >> 2) & 1, l2 = (l >> 1) & 1, l3 = l & 1;
+    if (nb1) return ((2 * j1 > nd) == l1 && (2 * j2 > nd) == l2 && (2 * j3 > nd) == l3) ? (T)1 : (T)0;
+    return (T)((l1 ? j1 : nd - j1) * (l2 ? j2 : nd - j2) * (l3 ? j3 : nd - j3)) / (T)(nd * nd * nd);
 }
 
 // ------------------------------------------------------- rotate and restrict
@@ -164,6 +179,9 @@ __global__ void __launch_bounds__(256) k_common_restrict(
     V* sUc = sUv + KP * rvp;                            // [KP][rcp]
     V* red = sUc + KP * rcp;                            // [256]
     T* wt = reinterpret_cast<T*>(red + 256);            // [KP][8]
+    int2* pnt = reinterpret_cast<int2*>(wt + KP * 8);   // [KP] the point's place in phi and its halo copy's distance
+    const int L = n * nd, t2 = 2 * t;
+    const float inv_t = 1.f / (float)t, inv_nd = 1.f / (float)nd;
     // corner sums: item (l, e); with few items several threads share one over the points
     const int items = 8 * t, nsp = max(1, 256 / items);
     V acc[2] = {czero<V>(), czero<V>()};
@@ -173,28 +191,33 @@ __global__ void __launch_bounds__(256) k_common_restrict(
         load_rows(X, tp, psi + ((size_t)ch * nkc * Ndiv + kd0) * t, np, t);
         load_rows(sUv, rvp, Uvd + kd0 * rv, np, rv);
         load_rows(sUc, rcp, Ucd + kd0 * rc, np, rc);
-        for (int i = tid; i < np * 8; i += 256) wt[i] = interp_weight_as<T>(k0 + (i >> 3), i & 7, nd, nb1);
+        for (int i = tid; i < np * 8; i += 256) {
+            const int js = k0 + (i >> 3), a = quot(js, inv_nd), j3 = js - a * nd, j1 = quot(a, inv_nd), j2 = a - j1 * nd;
+            wt[i] = corner_weight<T>(j1, j2, j3, i & 7, nd, nb1);
+            if ((i & 7) == 0) {
+                const int x = ci.a * nd + j1, y = ci.b * nd + j2, z = ci.c * nd + j3;
+                pnt[i >> 3] = make_int2((x * L + y) * lay.Lp + z + lay.R, z < lay.R ? L : (z >= L - lay.R ? -L : 0));
+            }
+        }
         __syncthreads();
         rotate_blocks<true>(X, tp, sUv, rvp, sUc, rcp, np, nv, nc);
         if (phi) {
-            // 2 t components of a point lie side by side in the columns of its groups
-            const int t2 = 2 * t, L = n * nd;
+            // the 2 t components of a point lie side by side in the columns of its groups
+            const size_t gs = (size_t)L * L * lay.Lp * 32;
+            const float inv_t2 = 1.f / (float)t2;
             for (int i = tid; i < np * t2; i += 256) {
-                const int r = i / t2, q = i - r * t2, js = k0 + r;
+                const int r = quot(i, inv_t2), q = i - r * t2, col = ch * t2 + q;
+                const int2 pt = pnt[r];
                 const T v = reinterpret_cast<const T*>(X + r * tp)[q];
-                const Int3 j = unflat3(js, nd);
-                const int x = ci.a * nd + j.a, y = ci.b * nd + j.b, z = ci.c * nd + j.c;
-                const int col = ch * t2 + q;
-                T* row = phi + (((size_t)(col >> 5) * L + x) * L + y) * lay.Lp * 32 + (col & 31);
-                row[(size_t)(z + lay.R) * 32] = v;
-                if (z >= L - lay.R) row[(size_t)(z + lay.R - L) * 32] = v;      // periodic halo copies
-                if (z < lay.R) row[(size_t)(z + lay.R + L) * 32] = v;
+                T* at = phi + (size_t)(col >> 5) * gs + (size_t)pt.x * 32 + (col & 31);
+                *at = v;
+                if (pt.y) at[(ptrdiff_t)pt.y * 32] = v;
             }
         }
         for (int a = 0; a < 2; ++a) {
             const int i = nsp > 1 ? tid % items : tid + 256 * a, sp = nsp > 1 ? tid / items : 0;
             if (i >= items || sp >= nsp || (nsp > 1 && a)) continue;
-            const int l = i / t, e = i - l * t;
+            const int l = quot(i, inv_t), e = i - l * t;
             V s = acc[a];
             for (int r = sp; r < np; r += nsp) {
                 const T f = wt[r * 8 + l];
@@ -291,6 +314,7 @@ __global__ void __launch_bounds__(256) k_common_prolong(
     V* cUc = cUv + 8 * rvp;                             // [8][rcp]
     T* wt = reinterpret_cast<T*>(cUc + 8 * rcp);        // [KP][8]
     const T inv = (T)1 / (T)Ndiv;
+    const float inv_t = 1.f / (float)t, inv_nd = 1.f / (float)nd;
     double2 dot = make_double2(0.0, 0.0);
     for (int cell = blockIdx.x; cell < nkc; cell += gridDim.x) {
         const Int3 ci = unflat3(cell, n);
@@ -309,10 +333,13 @@ __global__ void __launch_bounds__(256) k_common_prolong(
             const size_t kd0 = (size_t)cell * Ndiv + k0, g0 = kd0 * t, o0 = (size_t)ch * nkc * Ndiv * t + g0;
             load_rows(sUv, rvp, Uvd + kd0 * rv, np, rv);
             load_rows(sUc, rcp, Ucd + kd0 * rc, np, rc);
-            for (int i = tid; i < np * 8; i += 256) wt[i] = interp_weight_as<T>(k0 + (i >> 3), i & 7, nd, nb1) * inv;
+            for (int i = tid; i < np * 8; i += 256) {
+                const int js = k0 + (i >> 3), a = quot(js, inv_nd), j1 = quot(a, inv_nd);
+                wt[i] = corner_weight<T>(j1, a - j1 * nd, js - a * nd, i & 7, nd, nb1) * inv;
+            }
             __syncthreads();
             for (int i = tid; i < np * t; i += 256) {
-                const int r = i / t, e = i - r * t;
+                const int r = quot(i, inv_t), e = i - r * t;
                 V s = Vn ? Vn[o0 + i] : czero<V>();
 #pragma unroll
                 for (int l = 0; l < 8; ++l) {
@@ -327,7 +354,7 @@ __global__ void __launch_bounds__(256) k_common_prolong(
             rotate_blocks<false>(X, tp, sUv, rvp, sUc, rcp, np, nv, nc);
             T dre = (T)0, dim = (T)0;                   // this thread's few products, then FP64
             for (int i = tid; i < np * t; i += 256) {
-                const int r = i / t, e = i - r * t;
+                const int r = quot(i, inv_t), e = i - r * t;
                 const V s = X[r * tp + e], p = psi[o0 + i];
                 const T de = dE[g0 + i];
                 V w;
@@ -361,197 +388,226 @@ __global__ void __launch_bounds__(256) k_common_prolong(
 //
 // Per target and column (one real component of one chain) one multiply-add per
 // near offset is needed: 808 M for coarse 8^3, n_div 4, w 1, 3 chains of 16
-// transitions, so the FP32 (FP64) pipes bound it, and the split serves to keep
-// shared memory below them.  A block takes one column group (32 columns, one
-// per lane) of 1 x CY x CZ cells.  It walks the source planes x' of their
-// dilated box, double-buffered in shared memory by cp.async (every row of a
-// plane is contiguous in phi, z halo included).  A warp owns the sub-cell
-// rows (j1, TY values of j2, TZ values of j3) of all the block's cells: their
-// weights are the same in every cell, so one broadcast vector load of TZ
-// weights serves CY CZ multiply-adds per weight, and one load of a source
-// column TY TZ of them.  A warp stages its weight rows itself (one row per
-// source row, loaded a row ahead into registers).
+// transitions.  A warp takes one column group (a column per lane) and TY rows
+// (j1, j2 .. j2 + TY - 1) of CZ cells that follow each other along z: their
+// targets are CZ TZ consecutive points, so one load of a source column serves up
+// to TY (2 r + 1) multiply-adds, and since W is the same in every cell one
+// broadcast vector load of TZ weights serves CZ multiply-adds each.  It walks
+// the source rows (delta_1, row u) of its ball in set-up's list; the reach r of
+// each target row along z is a case of a switch, so only offsets inside the ball
+// cost arithmetic and the source row sits in registers.  Sources come straight
+// from phi (the warps of a block share their cells, hence rows, through L1);
+// the weights of the next row are copied to the warp's buffer meanwhile.
+// RM: the largest r that the unrolled body covers (R <= RM); RM = 0 loops over z.
 struct NearStencil {
-    int n, nd, L, Lp, R, R2, nzb, tasks, ntz;   // ntz: z blocks a cell has; tasks: warps per (cell, z block)
-    int cols, t2;                               // 2 t nchains columns in use; 2 t
-    long long N2;                               // 2 N: reals per chain of V
+    int n, L, Lp, R, nd, njb, nzb, nsteps, wrow;   // njb: blocks of TY rows j2; nzb: blocks of TZ targets j3
+    int cols, t2, ntz, warps;                      // columns in use, 2 t, z tiles (of cz cells, the last ones smaller), all warps
+    int cz;
+    long long N2;                                  // 2 N: reals per chain of V
 };
 
-template <typename T, int TY, int TZ, int CY, int CZ, bool STAGED>
-__device__ __forceinline__ void near_body(const T* __restrict__ phi, const T* __restrict__ Wt, T* __restrict__ Vn,
-                                          const NearStencil& s, int cx, int cy0, int cz0, int g, int task, bool active,
-                                          T* planes, T* wbuf) {
-    constexpr int TZP = TZ == 3 ? 4 : TZ;
-    constexpr int I = CY * CZ;
-    const int lane = threadIdx.x & 31, nthr = blockDim.x;
-    const int nd = s.nd, R = s.R, D = 2 * R + 1;
-    const int NY = CY * nd + 2 * R, NZ = CZ * nd + 2 * R, plane = NY * NZ * 32;
-    const int nzs = TZ + 2 * R;
-    // task -> (z block, j1, rows j2 .. j2 + TY - 1)
-    const int nty = (nd + TY - 1) / TY;
-    const int zb = task / (nd * nty), j1 = (task / nty) % nd, j2 = (task % nty) * TY;
-    const int tzn = min(TZ, nd - zb * TZ);                        // targets of this z block
-    T acc[I][TY][TZ];
-#pragma unroll
-    for (int i = 0; i < I; ++i)
-#pragma unroll
-        for (int y = 0; y < TY; ++y)
-#pragma unroll
-            for (int z = 0; z < TZ; ++z) acc[i][y][z] = (T)0;
-    auto fetch = [&](int px, T* dst) {
-        constexpr int PER = 16 / sizeof(T), CH = 32 / PER;        // 16-byte chunks of a point's columns
-        const int x = imod(cx * nd - R + px, s.L);
-        const int rowc = NZ * CH, tot = NY * rowc;
-        for (int c = threadIdx.x; c < tot; c += nthr) {
-            const int r = c / rowc, q = c - r * rowc;
-            const int y = imod(cy0 * nd - R + r, s.L);
-            cpa16(dst + (size_t)r * NZ * 32 + q * PER,
-                  phi + ((((size_t)g * s.L + x) * s.L + y) * s.Lp + cz0 * nd) * 32 + q * PER);
+template <typename T, int TZ>
+__device__ __forceinline__ void load_w(T (&w)[TZ], const T* p) {
+    if constexpr (TZ >= 3 && sizeof(T) == 4) {
+        const float4 q = *reinterpret_cast<const float4*>(p);
+        w[0] = q.x; w[1] = q.y; w[2] = q.z;
+        if (TZ == 4) w[TZ - 1] = q.w;
+    } else if constexpr (TZ >= 2) {
+        using V = typename Cx<T>::V;
+        const V q = reinterpret_cast<const V*>(p)[0];
+        w[0] = q.x; w[1] = q.y;
+        if (TZ >= 3) {
+            const V q2 = reinterpret_cast<const V*>(p)[1];
+            w[2] = q2.x;
+            if (TZ == 4) w[TZ - 1] = q2.y;
         }
-    };
-    const int npx = nd + 2 * R;
-    if (STAGED) {
-        fetch(0, planes);
-        cpa_commit();
+    } else {
+        w[0] = p[0];
     }
-    for (int px = 0; px < npx; ++px) {
-        if (STAGED) {
-            if (px + 1 < npx) fetch(px + 1, planes + ((px + 1) & 1) * plane);
+}
+
+// acc += W v for the target rows of one cell run that reach r sources to each side
+template <typename T, int TZ, int CZ, int RM, int r>
+__device__ __forceinline__ void near_apply(T (&acc)[CZ * TZ], const T (&v)[CZ * TZ + 2 * RM], const T* wb) {
+    constexpr int TZP = TZ == 3 ? 4 : TZ;
+#pragma unroll
+    for (int z = -r; z < TZ + r; ++z) {
+        T w[TZ];
+        load_w<T, TZ>(w, wb + z * TZP);
+#pragma unroll
+        for (int tz = 0; tz < TZ; ++tz)
+            if (z - tz <= r && tz - z <= r) {
+#pragma unroll
+                for (int c = 0; c < CZ; ++c) acc[c * TZ + tz] = fma(w[tz], v[c * TZ + z + RM], acc[c * TZ + tz]);
+            }
+    }
+}
+template <typename T, int TZ, int CZ, int RM, int r>
+__device__ __forceinline__ void near_load(T (&v)[CZ * TZ + 2 * RM], const T* __restrict__ row) {
+#pragma unroll
+    for (int z = -r; z < CZ * TZ + r; ++z) v[z + RM] = __ldg(row + z * 32);
+}
+
+template <typename T, int TY, int TZ, int CZ, int RM>
+__device__ __forceinline__ void near_body(const T* __restrict__ phi, const T* __restrict__ Wt,
+                                          const int2* __restrict__ steps, T* __restrict__ Vn, const NearStencil& s, int g,
+                                          int cx, int cy, int cz0, int j1, int j2, int zb, T* wbuf) {
+    constexpr int TZP = TZ == 3 ? 4 : TZ, PER = 16 / sizeof(T);
+    const int lane = threadIdx.x & 31, nd = s.nd, R = s.R, nzs = TZ + 2 * R;
+    const T* wsrc = Wt + (size_t)((zb * nd + j1) * s.njb + j2 / TY) * s.nsteps * s.wrow;
+    const int xb = cx * nd + j1 - R, yb = cy * nd + j2 - R;
+    const T* base = phi + (size_t)g * s.L * s.L * s.Lp * 32 + (size_t)(cz0 * nd + zb * TZ + R) * 32 + lane;
+    T acc[TY][CZ * TZ];
+#pragma unroll
+    for (int y = 0; y < TY; ++y)
+#pragma unroll
+        for (int z = 0; z < CZ * TZ; ++z) acc[y][z] = (T)0;
+    auto fetch = [&](int i) {
+        T* dst = wbuf + (i & 1) * s.wrow;
+        for (int c = lane * PER; c < s.wrow; c += 32 * PER) cpa16(dst + c, wsrc + (size_t)i * s.wrow + c);
+        cpa_commit();
+    };
+    int2 st = steps[0];
+    fetch(0);
+    for (int i = 0; i < s.nsteps; ++i) {
+        int2 nx = st;
+        if (i + 1 < s.nsteps) {
+            nx = steps[i + 1];
+            fetch(i + 1);
+        } else {
             cpa_commit();
-            cpa_wait<1>();
-            __syncthreads();
         }
-        const T* src = STAGED ? planes + (px & 1) * plane
-                              : phi + ((size_t)g * s.L + imod(cx * nd - R + px, s.L)) * s.L * s.Lp * 32;
-        const int d1 = px - j1;                                   // delta_1 + R
-        if (active && d1 >= 0 && d1 < D) {
-            const int rem1 = s.R2 - (d1 - R) * (d1 - R);
-            // rows of sources: u = 0 .. 2R + TY - 1, delta_2 of target row y is u - y - R
-            const T* wrow = Wt + ((((size_t)(zb * nd + j1) * nd + j2) * D + d1) * D) * nzs * TZP;
-            const size_t wty = (size_t)D * D * nzs * TZP;         // next j2
-            for (int u = 0; u < D + TY - 1; ++u) {
-                int rmax = -1;
-#pragma unroll
-                for (int y = 0; y < TY; ++y) {
-                    const int d2 = u - y, rem = rem1 - (d2 - R) * (d2 - R);
-                    if (d2 >= 0 && d2 < D && rem >= 0 && j2 + y < nd) {
-                        const int r = (int)sqrtf((float)rem + 0.5f);
-                        rmax = max(rmax, r);
+        // st: delta_1 + R | u << 8 | r_max << 16, then the reach + 1 of each target row (0: none), a byte each
+        int x = xb + (st.x & 255), y = yb + ((st.x >> 8) & 255);
+        x += x < 0 ? s.L : (x >= s.L ? -s.L : 0);
+        y += y < 0 ? s.L : (y >= s.L ? -s.L : 0);
+        const T* row = base + ((size_t)x * s.L + y) * s.Lp * 32;
+        const int rm = st.x >> 16;
+        const T* wb = wbuf + (i & 1) * s.wrow + R * TZP;
+        if constexpr (RM > 0) {
+            T v[CZ * TZ + 2 * RM];
+            switch (rm) {
+                case 0: near_load<T, TZ, CZ, RM, 0>(v, row); break;
+                case 1: near_load<T, TZ, CZ, RM, 1>(v, row); break;
+                case 2: near_load<T, TZ, CZ, RM, 2>(v, row); break;
+                case 3: near_load<T, TZ, CZ, RM, 3>(v, row); break;
+                case 4: near_load<T, TZ, CZ, RM, 4>(v, row); break;
+                default:
+                    if constexpr (RM >= 6) {
+                        if (rm == 5) near_load<T, TZ, CZ, RM, 5>(v, row);
+                        else near_load<T, TZ, CZ, RM, 6>(v, row);
                     }
-                }
-                if (rmax < 0) continue;
-                const int z0 = R - rmax, z1 = R + rmax + tzn;     // sources z0 .. z1 - 1 of the z block
-                __syncwarp();
+            }
+            cpa_wait<1>();
+            __syncwarp();
 #pragma unroll
-                for (int y = 0; y < TY; ++y) {
-                    const int d2 = u - y;
-                    const bool in = d2 >= 0 && d2 < D && j2 + y < nd;
-                    const T* w = wrow + y * wty + (size_t)d2 * nzs * TZP;
-                    for (int q = lane + z0 * TZP; q < z1 * TZP; q += 32) wbuf[y * nzs * TZP + q] = in ? w[q] : (T)0;
-                }
-                __syncwarp();
-                const T* row[CY];
-#pragma unroll
-                for (int cy = 0; cy < CY; ++cy) {
-                    const int r = cy * nd + j2 + u;
-                    row[cy] = STAGED ? src + ((size_t)r * NZ + zb * TZ) * 32 + lane
-                                     : src + ((size_t)imod(cy0 * nd - R + r, s.L) * s.Lp + cz0 * nd + zb * TZ) * 32 + lane;
-                }
-#pragma unroll 2
-                for (int zi = z0; zi < z1; ++zi) {
-                    T v[I];
-#pragma unroll
-                    for (int cy = 0; cy < CY; ++cy)
-#pragma unroll
-                        for (int cz = 0; cz < CZ; ++cz) v[cy * CZ + cz] = row[cy][(cz * nd + zi) * 32];
-#pragma unroll
-                    for (int y = 0; y < TY; ++y) {
-                        T w[TZ];
-                        const T* wp = wbuf + (y * nzs + zi) * TZP;
-                        if constexpr (TZP == 4 && sizeof(T) == 4) {
-                            const float4 w4 = *reinterpret_cast<const float4*>(wp);
-                            w[0] = w4.x; w[1] = w4.y; w[2] = w4.z;
-                            if (TZ == 4) w[TZ - 1] = w4.w;
-                        } else {
-#pragma unroll
-                            for (int z = 0; z < TZ; ++z) w[z] = wp[z];
+            for (int y2 = 0; y2 < TY; ++y2) {
+                const T* w = wb + y2 * nzs * TZP;
+                switch ((st.y >> (8 * y2)) & 255) {
+                    case 0: break;
+                    case 1: near_apply<T, TZ, CZ, RM, 0>(acc[y2], v, w); break;
+                    case 2: near_apply<T, TZ, CZ, RM, 1>(acc[y2], v, w); break;
+                    case 3: near_apply<T, TZ, CZ, RM, 2>(acc[y2], v, w); break;
+                    case 4: near_apply<T, TZ, CZ, RM, 3>(acc[y2], v, w); break;
+                    case 5: near_apply<T, TZ, CZ, RM, 4>(acc[y2], v, w); break;
+                    default:
+                        if constexpr (RM >= 6) {
+                            if (((st.y >> (8 * y2)) & 255) == 6) near_apply<T, TZ, CZ, RM, 5>(acc[y2], v, w);
+                            else near_apply<T, TZ, CZ, RM, 6>(acc[y2], v, w);
                         }
+                }
+            }
+        } else {
+            cpa_wait<1>();
+            __syncwarp();
+            for (int z = -rm; z < TZ + rm; ++z) {
+                T v[CZ];
 #pragma unroll
-                        for (int z = 0; z < TZ; ++z) {
-                            // FP64 runs at a small fraction of the issue rate: skip what lies outside the ball
-                            if (sizeof(T) == 8 && w[z] == (T)0) continue;
+                for (int c = 0; c < CZ; ++c) v[c] = __ldg(row + (c * TZ + z) * 32);
 #pragma unroll
-                            for (int i = 0; i < I; ++i) acc[i][y][z] = fma(w[z], v[i], acc[i][y][z]);
-                        }
-                    }
+                for (int y2 = 0; y2 < TY; ++y2) {
+                    T w[TZ];
+                    load_w<T, TZ>(w, wb + (y2 * nzs + z) * TZP);
+#pragma unroll
+                    for (int tz = 0; tz < TZ; ++tz)
+#pragma unroll
+                        for (int c = 0; c < CZ; ++c) acc[y2][c * TZ + tz] = fma(w[tz], v[c], acc[y2][c * TZ + tz]);
                 }
             }
         }
-        if (STAGED) __syncthreads();
+        __syncwarp();
+        st = nx;
     }
     const int col = g * 32 + lane;
-    if (!active || col >= s.cols) return;
+    if (col >= s.cols) return;
     const int ch = col / s.t2, q = col - ch * s.t2;
+    T* out = Vn + (size_t)ch * s.N2 + q;
 #pragma unroll
-    for (int cy = 0; cy < CY; ++cy)
+    for (int c = 0; c < CZ; ++c)
 #pragma unroll
-        for (int cz = 0; cz < CZ; ++cz) {
-            const int cell = (cx * s.n + cy0 + cy) * s.n + cz0 + cz;
+        for (int y = 0; y < TY; ++y)
 #pragma unroll
-            for (int y = 0; y < TY; ++y)
-#pragma unroll
-                for (int z = 0; z < TZ; ++z)
-                    if (j2 + y < nd && z < tzn) {
-                        const size_t kd = (size_t)cell * nd * nd * nd + (j1 * nd + j2 + y) * nd + zb * TZ + z;
-                        Vn[(size_t)ch * s.N2 + kd * s.t2 + q] = acc[cy * CZ + cz][y][z];
-                    }
-        }
+            for (int z = 0; z < TZ; ++z)
+                if (j2 + y < nd && zb * TZ + z < nd) {
+                    const size_t kd = ((size_t)((cx * s.n + cy) * s.n + cz0 + c) * nd + j1) * nd * nd + (j2 + y) * nd + zb * TZ + z;
+                    out[kd * s.t2] = acc[y][c * TZ + z];
+                }
 }
 
-// Grid (tiles of cells, column groups, task groups).  Not STAGED: boxes too wide
-// for two source planes in shared memory read phi directly, cell by cell.
-template <typename T, int TY, int TZ, int CY, int CZ, bool STAGED>
+template <typename T, int TY, int TZ, int RM>
 __global__ void __launch_bounds__(256) k_common_near(const T* __restrict__ phi, const T* __restrict__ Wt,
-                                                     T* __restrict__ Vn, const NearStencil s) {
+                                                     const int2* __restrict__ steps, T* __restrict__ Vn, const NearStencil s) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    constexpr int TZP = TZ == 3 ? 4 : TZ;
-    const int warp = threadIdx.x >> 5;
-    const int NY = CY * s.nd + 2 * s.R, NZ = CZ * s.nd + 2 * s.R;
-    T* planes = reinterpret_cast<T*>(smraw);
-    T* wbuf = planes + (STAGED ? 2 * (size_t)NY * NZ * 32 : 0) + (size_t)warp * TY * (TZ + 2 * s.R) * TZP;
-    const int nty = (s.n + CY - 1) / CY, ntz = (s.n + CZ - 1) / CZ;
-    const int cx = blockIdx.x / (nty * ntz), ty = (blockIdx.x / ntz) % nty, tz = blockIdx.x % ntz;
-    const int cy0 = ty * CY, cz0 = tz * CZ, g = blockIdx.y;
-    const int task = blockIdx.z * (blockDim.x >> 5) + warp;
-    const bool act = task < s.tasks;
-    const int tk = act ? task : 0;
-    // tiles cut by the mesh's end run the smaller body
-    const int ny = min(CY, s.n - cy0), nz = min(CZ, s.n - cz0);
-    if (ny == CY && nz == CZ) near_body<T, TY, TZ, CY, CZ, STAGED>(phi, Wt, Vn, s, cx, cy0, cz0, g, tk, act, planes, wbuf);
-    else if (CY == 2 && nz == CZ) near_body<T, TY, TZ, 1, CZ, STAGED>(phi, Wt, Vn, s, cx, cy0, cz0, g, tk, act, planes, wbuf);
-    else if (CZ == 2 && ny == CY) near_body<T, TY, TZ, CY, 1, STAGED>(phi, Wt, Vn, s, cx, cy0, cz0, g, tk, act, planes, wbuf);
-    else near_body<T, TY, TZ, 1, 1, STAGED>(phi, Wt, Vn, s, cx, cy0, cz0, g, tk, act, planes, wbuf);
+    T* wbuf = reinterpret_cast<T*>(smraw) + (size_t)(threadIdx.x >> 5) * 2 * s.wrow;
+    int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (w >= s.warps) return;
+    // warp: (group, cx, cy, z tile, z block, j1, block of j2), the last fastest
+    const int jb = w % s.njb; w /= s.njb;
+    const int j1 = w % s.nd; w /= s.nd;
+    const int zb = w % s.nzb; w /= s.nzb;
+    const int tz = w % s.ntz; w /= s.ntz;
+    const int cy = w % s.n; w /= s.n;
+    const int cx = w % s.n, g = w / s.n;
+    // z tiles: as many of cz cells as fit, then what is left in powers of two
+    const int full = s.n / s.cz;
+    int cz0 = min(tz, full) * s.cz, cz = s.cz;
+    for (int q = full; q <= tz; ++q) {
+        int left = s.n - cz0, p = 1;
+        while (2 * p <= left) p *= 2;
+        cz = p;
+        if (q < tz) cz0 += p;
+    }
+    if (tz < full) cz = s.cz;
+    if constexpr (RM > 0) {
+        if (cz == 4) near_body<T, TY, TZ, 4, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, j1, jb * TY, zb, wbuf);
+        else if (cz == 2) near_body<T, TY, TZ, 2, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, j1, jb * TY, zb, wbuf);
+        else near_body<T, TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, j1, jb * TY, zb, wbuf);
+    } else {
+        near_body<T, TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, j1, jb * TY, zb, wbuf);
+    }
 }
 
 // Weights of the near stencil, FP64, one thread per entry: index
-// [z block][j1][j2][d1][d2][source z][target z], zero outside the ball (and for
-// the padding targets); scale = alpha / N_div.
+// [z block][j1][block of j2][step][row y][source z][target z] (rows of a step padded
+// to `wrow`), zero outside the ball and for padding; scale = alpha / N_div.
 template <typename T>
-__global__ void k_common_weights(const double* __restrict__ hcoarse, int n, int nd, int nb1, int R, int R2, int TZ, int TZP,
-                                 double kappa, double scale, long long total, T* __restrict__ Wt) {
+__global__ void k_common_weights(const double* __restrict__ hcoarse, const int2* __restrict__ steps, int nsteps, int n, int nd,
+                                 int nb1, int R, int R2, int TY, int TZ, int TZP, int njb, int wrow, double kappa, double scale,
+                                 long long total, T* __restrict__ Wt) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total) return;
-    const int D = 2 * R + 1, nzs = TZ + 2 * R;
-    long long q = i;
-    const int tz = (int)(q % TZP); q /= TZP;
-    const int zi = (int)(q % nzs); q /= nzs;
-    const int d2 = (int)(q % D) - R; q /= D;
-    const int d1 = (int)(q % D) - R; q /= D;
-    const int j2 = (int)(q % nd); q /= nd;
+    const int nzs = TZ + 2 * R;
+    const int e = (int)(i % wrow);
+    long long q = i / wrow;
+    const int2 st = steps[q % nsteps]; q /= nsteps;
+    const int jb = (int)(q % njb); q /= njb;
     const int j1 = (int)(q % nd);
-    const int zb = (int)(q / nd), j3 = zb * TZ + tz, d3 = zi - R - tz;
+    const int zb = (int)(q / nd);
+    const int tz = e % TZP, zi = (e / TZP) % nzs, y = e / (TZP * nzs);
+    const int j2 = jb * TY + y, j3 = zb * TZ + tz;
+    const int d1 = (st.x & 255) - R, d2 = ((st.x >> 8) & 255) - y - R, d3 = zi - R - tz;
     T out = (T)0;
-    if (tz < TZ && j3 < nd && d1 * d1 + d2 * d2 + d3 * d3 <= R2) {
+    if (y < TY && j2 < nd && tz < TZ && j3 < nd && d1 * d1 + d2 * d2 + d3 * d3 <= R2) {
         const double L = (double)n * nd, qa = d1 / L, qb = d2 / L, qc = d3 / L;
         const int js = (j1 * nd + j2) * nd + j3;
         const int g1 = j1 + d1, g2 = j2 + d2, g3 = j3 + d3;
@@ -589,57 +645,66 @@ cudaError_t raise_smem(K kernel, size_t bytes) {
     return e;
 }
 
-// Sub-cell targets a thread owns: TZ = n_div up to 4 (then blocks of 4), TY rows.
+// Targets of a warp within a cell: TZ = n_div up to 4 (then blocks of 4), TY rows.
 inline int near_tz(int nd) { return std::min(nd, 4); }
 inline int near_ty(int nd) { return nd <= 3 ? nd : 2; }
 inline int near_tzp(int nd) { return nd == 3 ? 4 : near_tz(nd); }
 
-template <typename T, int TY, int TZ>
-size_t near_smem(const NearStencil& ns, int cy, int cz, int warps, bool staged) {
-    const size_t NY = cy * ns.nd + 2 * ns.R, NZ = cz * ns.nd + 2 * ns.R;
-    return sizeof(T) * ((staged ? 2 * NY * NZ * 32 : 0) + (size_t)warps * TY * (TZ + 2 * ns.R) * (TZ == 3 ? 4 : TZ));
+// Elements of a step's weights, rounded up to 16 bytes.
+template <typename T>
+int near_wrow(int nd, int R) {
+    const int per = 16 / (int)sizeof(T), e = near_ty(nd) * (near_tz(nd) + 2 * R) * near_tzp(nd);
+    return (e + per - 1) / per * per;
 }
 
-template <typename T, int TY, int TZ, int CY, int CZ, bool STAGED>
-int launch_near_c(bse_ctx* ctx, const bse_interp* s, const NearStencil& ns, const T* phi, T* Vn, cudaStream_t st) {
-    const int groups = (ns.cols + 31) / 32, n = s->n, warps = std::min(ns.tasks, 8);
-    const size_t smem = near_smem<T, TY, TZ>(ns, CY, CZ, warps, STAGED);
-    BSE_CUDA_TRY(ctx, raise_smem(k_common_near<T, TY, TZ, CY, CZ, STAGED>, smem));
-    dim3 grid(n * ((n + CY - 1) / CY) * ((n + CZ - 1) / CZ), groups, (ns.tasks + warps - 1) / warps);
-    k_common_near<T, TY, TZ, CY, CZ, STAGED><<<grid, 32 * warps, smem, st>>>(phi, (const T*)s->d_cw, Vn, ns);
+template <typename T, int TY, int TZ, int RM>
+int launch_near_r(bse_ctx* ctx, const bse_interp* s, NearStencil ns, cudaStream_t st) {
+    const int groups = (ns.cols + 31) / 32, n = s->n;
+    auto tiles = [&](int cz) {
+        int c = n / cz;
+        for (int left = n % cz; left; left &= left - 1) ++c;
+        return c;
+    };
+    const long long per_tile = (long long)groups * n * n * ns.nzb * ns.nd * ns.njb;
+    // Cells per warp: as many as leave four warps per SM (a warp alone on its scheduler
+    // waits out its loads); z blocks do not continue into the next cell.
+    ns.cz = 1;
+    if (RM > 0 && ns.nzb == 1)
+        for (int cz : {2, 4})
+            if (n >= cz && per_tile * tiles(cz) >= 4LL * ctx->sm_count) ns.cz = cz;
+    ns.ntz = tiles(ns.cz);
+    const long long warps = per_tile * ns.ntz;
+    if (warps > 0x7fffffffLL) { ctx->err = "near stencil: too many targets"; return BSE_ERR_UNSUPPORTED; }
+    ns.warps = (int)warps;
+    // small grids: fewer warps per block spread over more SMs
+    const int wpb = warps >= 8LL * 2 * ctx->sm_count ? 8 : 2;
+    const size_t smem = sizeof(T) * 2 * (size_t)ns.wrow * wpb;
+    BSE_CUDA_TRY(ctx, raise_smem(k_common_near<T, TY, TZ, RM>, smem));
+    k_common_near<T, TY, TZ, RM><<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, st>>>(
+        (const T*)s->d_cphi, (const T*)s->d_cw, s->d_csteps, (T*)s->d_cV, ns);
     BSE_CUDA_TRY(ctx, cudaGetLastError());
     return BSE_OK;
-}
-
-template <typename T, int TY, int TZ>
-int launch_near_t(bse_ctx* ctx, const bse_interp* s, const NearStencil& ns, const T* phi, T* Vn, cudaStream_t st) {
-    // Cells per block: as many as leave a block per SM, and whose two source planes fit
-    const int groups = (ns.cols + 31) / 32, n = s->n, warps = std::min(ns.tasks, 8), zg = (ns.tasks + warps - 1) / warps;
-    auto good = [&](int cy, int cz) {
-        return n >= 2 && near_smem<T, TY, TZ>(ns, cy, cz, warps, true) <= (size_t)100 * 1024 &&
-               (long long)n * ((n + cy - 1) / cy) * ((n + cz - 1) / cz) * groups * zg >= ctx->sm_count;
-    };
-    if (good(2, 2)) return launch_near_c<T, TY, TZ, 2, 2, true>(ctx, s, ns, phi, Vn, st);
-    if (good(1, 2)) return launch_near_c<T, TY, TZ, 1, 2, true>(ctx, s, ns, phi, Vn, st);
-    if (near_smem<T, TY, TZ>(ns, 1, 1, warps, true) <= (size_t)200 * 1024)
-        return launch_near_c<T, TY, TZ, 1, 1, true>(ctx, s, ns, phi, Vn, st);
-    return launch_near_c<T, TY, TZ, 1, 1, false>(ctx, s, ns, phi, Vn, st);
 }
 
 template <typename T>
 int near_typed(bse_ctx* ctx, const bse_interp* s, int nchains, cudaStream_t st) {
     NearStencil ns{};
-    ns.n = s->n; ns.nd = s->nd; ns.L = s->n * s->nd; ns.R = s->cphi_R; ns.R2 = s->near_R2; ns.Lp = ns.L + 2 * ns.R;
-    ns.nzb = (s->nd + near_tz(s->nd) - 1) / near_tz(s->nd);
-    ns.tasks = ns.nzb * s->nd * ((s->nd + near_ty(s->nd) - 1) / near_ty(s->nd));
+    const int nd = s->nd;
+    ns.n = s->n; ns.nd = nd; ns.L = s->n * nd; ns.R = s->cphi_R; ns.Lp = s->cphi_Lp;
+    ns.nzb = (nd + near_tz(nd) - 1) / near_tz(nd);
+    ns.njb = (nd + near_ty(nd) - 1) / near_ty(nd);
+    ns.nsteps = s->n_csteps;
+    ns.wrow = near_wrow<T>(nd, ns.R);
     ns.t2 = 2 * s->t; ns.cols = ns.t2 * nchains; ns.N2 = 2LL * s->N;
-    const T* phi = (const T*)s->d_cphi;
-    T* Vn = (T*)s->d_cV;
-    switch (s->nd) {
-        case 1: return launch_near_t<T, 1, 1>(ctx, s, ns, phi, Vn, st);
-        case 2: return launch_near_t<T, 2, 2>(ctx, s, ns, phi, Vn, st);
-        case 3: return launch_near_t<T, 3, 3>(ctx, s, ns, phi, Vn, st);
-        default: return launch_near_t<T, 2, 4>(ctx, s, ns, phi, Vn, st);
+    const bool r4 = ns.R <= 4, r6 = ns.R <= 6;
+    switch (nd) {
+        case 1: return r4 ? launch_near_r<T, 1, 1, 4>(ctx, s, ns, st) : launch_near_r<T, 1, 1, 0>(ctx, s, ns, st);
+        case 2: return r4 ? launch_near_r<T, 2, 2, 4>(ctx, s, ns, st) : launch_near_r<T, 2, 2, 0>(ctx, s, ns, st);
+        case 3: return r4 ? launch_near_r<T, 3, 3, 4>(ctx, s, ns, st) : launch_near_r<T, 3, 3, 0>(ctx, s, ns, st);
+        default:
+            return r4   ? launch_near_r<T, 2, 4, 4>(ctx, s, ns, st)
+                   : r6 ? launch_near_r<T, 2, 4, 6>(ctx, s, ns, st)
+                        : launch_near_r<T, 2, 4, 0>(ctx, s, ns, st);
     }
 }
 
@@ -650,9 +715,9 @@ int restrict_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* p
     const bse_coarse* c = s->co;
     const int KP = rot_points(s, sizeof(V));
     const size_t smem = sizeof(V) * ((size_t)KP * (odd(s->t) + odd(s->nv * s->nv) + odd(s->nc * s->nc)) + 256) +
-                        sizeof(T) * 8 * KP;
+                        (sizeof(T) * 8 + sizeof(int2)) * KP;
     const bool m3 = s->scheme == BSE_SCHEME_M3;
-    CommonPhi lay{s->cphi_R, s->n * s->nd + 2 * s->cphi_R};
+    CommonPhi lay{s->cphi_R, s->cphi_Lp};
     const dim3 grid(c->nkc, nchains);
     auto go = [&](auto kernel) -> int {
         BSE_CUDA_TRY(ctx, raise_smem(kernel, smem));
@@ -710,16 +775,38 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s, const double2* Uvd, const double2
         BSE_CUDA_TRY(ctx, cudaStreamSynchronize(st));
         return BSE_OK;
     }
-    const int L = s->n * s->nd, R = s->cphi_R, TZ = near_tz(s->nd), TZP = near_tzp(s->nd), D = 2 * R + 1;
+    const int nd = s->nd, L = s->n * nd, R = s->cphi_R, TY = near_ty(nd), TZ = near_tz(nd), D = 2 * R + 1;
+    // rows of phi: R points of halo on each side, and what a padded target block reads beyond (zeros)
+    s->cphi_Lp = L + 2 * R + (nd > 4 ? 3 : 0);
     const size_t groups = (2 * (size_t)s->t * BSE_MAX_CHAINS + 31) / 32;
-    const size_t nphi = groups * L * L * (size_t)(L + 2 * R) * 32;
+    const size_t nphi = groups * L * L * (size_t)s->cphi_Lp * 32;
     if ((rc_ = bse_alloc(ctx, &s->d_cphi, sizeof(T) * nphi, "common-basis vectors")) != BSE_OK) return rc_;
     BSE_CUDA_TRY(ctx, cudaMemsetAsync(s->d_cphi, 0, sizeof(T) * nphi, st));      // unused columns stay zero
     if ((rc_ = bse_alloc(ctx, &s->d_cV, sizeof(V) * BSE_MAX_CHAINS * (size_t)s->N, "near stencil result")) != BSE_OK) return rc_;
-    const long long nw = (long long)((s->nd + TZ - 1) / TZ) * s->nd * s->nd * D * D * (TZ + 2 * R) * TZP;
+    // source rows of a warp's targets: (delta_1 + R, u), u - y the delta_2 + R of target row y,
+    // with the reach along z of each row (a byte each, plus one; 0: outside the ball) and the largest
+    std::vector<int2> steps;
+    for (int d1 = 0; d1 < D; ++d1)
+        for (int u = 0; u < D + TY - 1; ++u) {
+            int reach = 0, rmax = -1;
+            for (int y = 0; y < TY; ++y) {
+                const int d2 = u - y, rem = s->near_R2 - (d1 - R) * (d1 - R) - (d2 - R) * (d2 - R);
+                if (d2 < 0 || d2 >= D || rem < 0) continue;
+                const int r = (int)std::sqrt((double)rem + 0.5);
+                reach |= (r + 1) << (8 * y);
+                rmax = std::max(rmax, r);
+            }
+            if (rmax >= 0) steps.push_back(make_int2(d1 | (u << 8) | (rmax << 16), reach));
+        }
+    s->n_csteps = (int)steps.size();
+    if ((rc_ = bse_alloc(ctx, (void**)&s->d_csteps, sizeof(int2) * steps.size(), "near stencil rows")) != BSE_OK) return rc_;
+    BSE_CUDA_TRY(ctx, cudaMemcpy(s->d_csteps, steps.data(), sizeof(int2) * steps.size(), cudaMemcpyHostToDevice));
+    const int nzb = (nd + TZ - 1) / TZ, njb = (nd + TY - 1) / TY, wrow = near_wrow<T>(nd, R);
+    const long long nw = (long long)nzb * nd * njb * s->n_csteps * wrow;
     if ((rc_ = bse_alloc(ctx, &s->d_cw, sizeof(T) * (size_t)nw, "near stencil weights")) != BSE_OK) return rc_;
-    k_common_weights<T><<<(unsigned)((nw + 127) / 128), 128, 0, st>>>(s->d_chead, s->n, s->nd, s->nb1, R, s->near_R2, TZ, TZP,
-                                                                      c->kappa, c->alpha / s->Ndiv, nw, (T*)s->d_cw);
+    k_common_weights<T><<<(unsigned)((nw + 127) / 128), 128, 0, st>>>(s->d_chead, s->d_csteps, s->n_csteps, s->n, nd, s->nb1, R,
+                                                                      s->near_R2, TY, TZ, near_tzp(nd), njb, wrow, c->kappa,
+                                                                      c->alpha / s->Ndiv, nw, (T*)s->d_cw);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {

@@ -155,9 +155,9 @@ struct bse_coarse {
     int unitary = 0;                              // the gauge generators are Hermitian: U(k) is unitary
 };
 
-// Layout of the common-basis vectors phi: [group][x][y][L + 2 R][32] reals, group
+// Layout of the common-basis vectors phi: [group][x][y][Lp][32] reals, group
 // g holding the columns 32 g .. 32 g + 31 of the (chain, transition, re|im)
-// components of a dense point; z starts R points before 0 (periodic halo).
+// components of a dense point; z starts R points before 0 (periodic halo; rows of Lp points).
 struct CommonPhi { int R, Lp; };
 
 struct NearEntry { int co; int js_src; int l_src; int near_idx; };   // co packed 3 x 4 bits (+8 bias)
@@ -182,6 +182,9 @@ struct bse_interp {
     void* d_cshare = nullptr;        // V [4][nkc][8][t] the cells' shares of their corners
     int* d_cctr = nullptr;           // [4][nkc] shares written (zero between launches)
     int cphi_R = 0, near_R2 = 0;     // near offsets: |delta|^2 <= near_R2, components within cphi_R
+    int cphi_Lp = 0;
+    int n_csteps = 0;
+    int2* d_csteps = nullptr;        // source rows of the near stencil
     double* d_chead = nullptr;       // [nkc] h_head over coarse differences (set-up only)
     void* d_cphi = nullptr;          // T, layout CommonPhi
     void* d_cV = nullptr;            // V [4][N] near stencil result
