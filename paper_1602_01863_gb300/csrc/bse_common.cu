@@ -754,14 +754,12 @@ __global__ void k_gauge_to(const double2* __restrict__ src, long long n, typenam
 }
 
 template <typename T>
-int prepare_typed(bse_ctx* ctx, bse_interp* s, const double2* Uvd, const double2* Ucd) {
+int prepare_typed(bse_ctx* ctx, bse_interp* s) {
     using V = typename Cx<T>::V;
     const bse_coarse* c = s->co;
     cudaStream_t st = ctx->stream;
     const size_t rv = s->nv * s->nv, rc = s->nc * s->nc;
-    struct { void** dst; const double2* src; size_t n; } tab[4] = {{&s->d_cUv, Uvd, (size_t)s->nk * rv},
-                                                                   {&s->d_cUc, Ucd, (size_t)s->nk * rc},
-                                                                   {&s->d_cUvc, c->d_Uv, (size_t)c->nkc * rv},
+    struct { void** dst; const double2* src; size_t n; } tab[2] = {{&s->d_cUvc, c->d_Uv, (size_t)c->nkc * rv},
                                                                    {&s->d_cUcc, c->d_Uc, (size_t)c->nkc * rc}};
     int rc_;
     for (auto& x : tab) {
@@ -820,8 +818,8 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s, const double2* Uvd, const double2
 
 int bse_common_dot_blocks(const bse_interp* s) { return std::min(s->co->nkc, BSE_MAX_VEC_BLOCKS); }
 
-int bse_common_prepare(bse_ctx* ctx, bse_interp* s, const double2* Uvd, const double2* Ucd) {
-    return s->vec_prec == BSE_PREC_F64 ? prepare_typed<double>(ctx, s, Uvd, Ucd) : prepare_typed<float>(ctx, s, Uvd, Ucd);
+int bse_common_prepare(bse_ctx* ctx, bse_interp* s) {
+    return s->vec_prec == BSE_PREC_F64 ? prepare_typed<double>(ctx, s) : prepare_typed<float>(ctx, s);
 }
 
 int bse_common_restrict(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, void* Q, __nv_bfloat16* bop,

@@ -171,7 +171,7 @@ struct bse_interp {
     void* d_H2 = nullptr;
     // dense tables
     void* d_dE = nullptr;            // T [N]
-    void* d_Dv = nullptr;            // V [nk][8][nv*nv]
+    void* d_Dv = nullptr;            // V [nk][8][nv*nv] (not on the common-basis path)
     void* d_Dc = nullptr;            // V [nk][8][nc*nc]
     double2* d_P = nullptr;          // [3][N]
     // common-basis path (bse_common.cu): the dense tables come from the model and
@@ -331,7 +331,7 @@ int bse_near_tc_prepare(bse_ctx* ctx, bse_interp* s, const std::vector<std::vect
 int bse_near_tc_launch(bse_ctx* ctx, const bse_interp* s, int nchains, const void* Xh, const float* xscale, void* U,
                        bool prio = false, int prio_value = 0);
 // common-basis path (bse_common.cu)
-int bse_common_prepare(bse_ctx* ctx, bse_interp* s, const double2* Uvd, const double2* Ucd);
+int bse_common_prepare(bse_ctx* ctx, bse_interp* s);
 int bse_common_dot_blocks(const bse_interp* s);
 int bse_common_restrict(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, void* Q, __nv_bfloat16* bop,
                         cudaStream_t st);

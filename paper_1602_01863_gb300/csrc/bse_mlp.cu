@@ -409,190 +409,238 @@ int mlp_grads(bse_ctx* ctx, bse_mlp* m, int B, const float* X, const float* Y, d
 // ================================================ pair data from the method
 namespace {
 
-// Band gauge at integer grid point g (L points per axis) from the generators.
-__device__ void gauge_at(const double2* gen, int nb, const int g[3], int L, double2* U) {
-    double2 A[BSE_MAX_BANDS * BSE_MAX_BANDS];
-    for (int i = 0; i < nb * nb; ++i) A[i] = make_double2(0.0, 0.0);
-    for (int a = 0; a < 3; ++a) {
-        double s, c;
-        sincospi(2.0 * g[a] / L, &s, &c);
-        const double2* g0 = gen + (a * 2) * nb * nb;
-        const double2* g1 = gen + (a * 2 + 1) * nb * nb;
-        for (int i = 0; i < nb * nb; ++i) A[i] = cadd(A[i], cadd(cscale(g0[i], s), cscale(g1[i], 1.0 - c)));
-    }
-    dmat_expm_i(A, nb, U);
+// One block per sampled dense pair (k, k'): the t x t blocks of the explicit
+// model kernel (FP64, dense weight e_k / N_k) and of K^{M1} = (1/N_div) F K_c F^H
+// (FP32), written as network features and targets.
+//  * The gauge at both points comes from a half warp per matrix; the form
+//    factors M(k, G) = Uv^H mu(k, G) Uc from mu(k, G) once and one factor at a time.
+//  * F is a Kronecker product of overlaps (Eq. interpwfn), so K_c blocks are
+//    multiplied by d_c and d_v in turn, t (nv + nc) terms per entry row instead of
+//    t^2, the blocks of all corners of k' at once, and F(k, l) is applied to
+//    their sum.
+//  * Overlaps come from the handle's tables or, on the common-basis path, from
+//    the gauge (FP64, rounded to FP32).
+//  * Rows of X leave in order, whole lines at a time.
+// 512 pairs of 4x6 bands on GB300: 9.80 ms with t x t products per corner pair, form
+// factors of 7 nv nc terms per entry and a thread per gauge; 0.61 ms so (FP64 and
+// shared-memory loads share it).
+constexpr int PTHR = 256;
+size_t pairs_smem(int nv, int nc) {
+    const int t = nv * nc, g = nv * nv + nc * nc;
+    const size_t scratch = std::max(sizeof(double2) * (2 * kGaugeMats * g + 2 * 26 * t), sizeof(float2) * (size_t)(9 * t * t));
+    return sizeof(double2) * (2 * (size_t)g + 2 * 26 * t + g) + scratch + sizeof(float2) * ((size_t)t * t + 16 * g);
 }
 
-// One CTA per sampled dense pair (k, k'): the t x t blocks of the explicit
-// model kernel (FP64, dense weight e_k / N_k) and of K^{M1} = (1/N_div) F K_c F^H
-// (FP32 from the handle's tables), written as network features and targets.
 template <typename T>
-__global__ void __launch_bounds__(576) k_pairs(
-    const int* __restrict__ kd1, const int* __restrict__ kd2, int nblocks, const double2* __restrict__ gen_v,
-    const double2* __restrict__ gen_c, const double2* __restrict__ mu, const typename Cx<T>::V* __restrict__ Kc,
-    const typename Cx<T>::V* __restrict__ Dv, const typename Cx<T>::V* __restrict__ Dc, const T* __restrict__ dE,
-    int n, int nd, int nv, int nc, int nb1, double e_k, double inv_eps, double kappa, int shells, int exchange_on,
-    int d_in, float* __restrict__ X, float* __restrict__ Y) {
-    using V = typename Cx<T>::V;
-    const int blk = blockIdx.x;
-    if (blk >= nblocks) return;
-    const int t = nv * nc, Ndiv = nd * nd * nd, L = n * nd, nk = n * n * n * Ndiv, Nc = t * n * n * n;
-    constexpr int PT = 24;                     // t <= 24 (checked by the host)
-    __shared__ double2 Uv[2][BSE_MAX_BANDS * BSE_MAX_BANDS], Uc[2][BSE_MAX_BANDS * BSE_MAX_BANDS];
-    __shared__ double2 M[2][26][PT];
-    __shared__ float2 Fa[PT * PT], Fb[PT * PT], Tm[PT * PT];
-    __shared__ double hq;
-    const int kk[2] = {kd1[blk], kd2[blk]};
-    int g[2][3];
-    for (int s = 0; s < 2; ++s) {
-        const int cell = kk[s] / Ndiv, js = kk[s] % Ndiv;
-        const Int3 ci = unflat3(cell, n), j = unflat3(js, nd);
-        g[s][0] = ci.a * nd + j.a; g[s][1] = ci.b * nd + j.b; g[s][2] = ci.c * nd + j.c;
+__global__ void __launch_bounds__(PTHR) k_pairs(
+    const int* __restrict__ kd1, const int* __restrict__ kd2, const double2* __restrict__ gen_v,
+    const double2* __restrict__ gen_c, const double2* __restrict__ mu, const double2* __restrict__ Uvc,
+    const double2* __restrict__ Ucc, const typename Cx<T>::V* __restrict__ Kc, const typename Cx<T>::V* __restrict__ Dv,
+    const typename Cx<T>::V* __restrict__ Dc, const T* __restrict__ dE, int n, int nd, int nv, int nc, int nb1, double e_k,
+    double inv_eps, double kappa, int shells, int exchange_on, int d_in, float* __restrict__ X, float* __restrict__ Y) {
+    extern __shared__ __align__(16) unsigned char prsm[];
+    const int blk = blockIdx.x, tid = threadIdx.x, warp = tid >> 5;
+    const int t = nv * nc, rv = nv * nv, rc = nc * nc, g = rv + rc, Ndiv = nd * nd * nd, L = n * nd, nk = n * n * n * Ndiv, Nc = t * n * n * n;
+    double2* U = reinterpret_cast<double2*>(prsm);            // [2][Uv | Uc]
+    double2* M = U + 2 * g;                                    // [2][26][t]
+    double2* O = M + 2 * 26 * t;                               // O^v, O^c
+    unsigned char* scratch = reinterpret_cast<unsigned char*>(O + g);
+    double2* gw = reinterpret_cast<double2*>(scratch);         // gauge scratch, then form-factor scratch
+    double2* fw = gw + 2 * kGaugeMats * g;                     // [2][26][t]
+    float2* Kb = reinterpret_cast<float2*>(scratch);           // [8][t][t] blocks of K_c, then [t][t] their sum behind them
+    float2* Ts = Kb + 8 * t * t;
+    const size_t sbytes = max(sizeof(double2) * (2 * kGaugeMats * g + 2 * 26 * t), sizeof(float2) * (size_t)(9 * t * t));
+    float2* K1 = reinterpret_cast<float2*>(scratch + sbytes);  // [t][t] K^{M1} N_div
+    float2* dd = K1 + t * t;                                   // [2][8][Dv | Dc]
+    __shared__ double sn[2][3], cs[2][3], hq;
+    __shared__ int gi[2][3], cell[2], js[2];
+    if (tid < 2) {
+        const int kd = tid ? kd2[blk] : kd1[blk];
+        cell[tid] = kd / Ndiv;
+        js[tid] = kd % Ndiv;
+        const Int3 ci = unflat3(cell[tid], n), j = unflat3(js[tid], nd);
+        gi[tid][0] = ci.a * nd + j.a; gi[tid][1] = ci.b * nd + j.b; gi[tid][2] = ci.c * nd + j.c;
+        for (int a = 0; a < 3; ++a) sincospi(2.0 * gi[tid][a] / L, &sn[tid][a], &cs[tid][a]);
     }
-    if (threadIdx.x < 2) gauge_at(gen_v, nv, g[threadIdx.x], L, Uv[threadIdx.x]);
-    else if (threadIdx.x < 4) gauge_at(gen_c, nc, g[threadIdx.x - 2], L, Uc[threadIdx.x - 2]);
-    else if (threadIdx.x == 4) {
-        // direct-term shape h(k - k') on the dense grid (minimum image, ties averaged)
-        int cand[3][2], ncand[3];
+    __syncthreads();
+    // gauge (warps 0, 1: a point each, a half warp per manifold); h(k - k') (warp 2); mu(k, G) (the rest)
+    if (warp < 2) {
+        const int half = (tid >> 4) & 1;
+        const double2* E = grp_gauge(half ? gen_c : gen_v, half ? nc : nv, sn[warp], cs[warp],
+                                     gw + warp * kGaugeMats * g + (half ? kGaugeMats * rv : 0));
+        double2* out = U + warp * g + (half ? rv : 0);
+        for (int e = grp_lane(); e < (half ? rc : rv); e += kGaugeLanes) out[e] = E[e];
+    } else if (warp == 2) {
+        // direct-term shape on the dense grid (minimum image, half-way differences average their images)
+        int im[3][2], nimg = 1;
         for (int a = 0; a < 3; ++a) {
-            const int r = imod(g[0][a] - g[1][a], L);
-            if (2 * r < L) { cand[a][0] = r; ncand[a] = 1; }
-            else if (2 * r > L) { cand[a][0] = r - L; ncand[a] = 1; }
-            else { cand[a][0] = r; cand[a][1] = r - L; ncand[a] = 2; }
+            const int r = imod(gi[0][a] - gi[1][a], L);
+            im[a][0] = 2 * r > L ? r - L : r;
+            im[a][1] = 2 * r >= L ? r - L : r;
+            if (im[a][0] != im[a][1]) nimg *= 2;
         }
         double acc = 0.0;
-        int cnt = 0;
-        for (int x = 0; x < ncand[0]; ++x)
-            for (int y = 0; y < ncand[1]; ++y)
-                for (int z = 0; z < ncand[2]; ++z) {
-                    const double q[3] = {(double)cand[0][x] / L, (double)cand[1][y] / L, (double)cand[2][z] / L};
-                    double v = 0.0;
-                    for (int ga = -1; ga <= 1; ++ga)
-                        for (int gb = -1; gb <= 1; ++gb)
-                            for (int gc = -1; gc <= 1; ++gc) {
-                                const int g2 = ga * ga + gb * gb + gc * gc;
-                                if (shells == 1 && g2 != 0) continue;
-                                const double qa = q[0] + ga, qb = q[1] + gb, qc = q[2] + gc;
-                                v += exp(-(double)g2) * 4.0 * kPi / (qa * qa + qb * qb + qc * qc + kappa * kappa);
-                            }
-                    acc += v;
-                    ++cnt;
-                }
-        hq = acc / cnt;
+        for (int q = tid & 31; q < 8 * 27; q += 32) {
+            const int s = q / 27, G = q - 27 * s;
+            bool dup = false;
+            for (int a = 0; a < 3; ++a) dup = dup || (((s >> a) & 1) && im[a][0] == im[a][1]);
+            const int ga = G / 9 - 1, gb = (G / 3) % 3 - 1, gc = G % 3 - 1, g2 = ga * ga + gb * gb + gc * gc;
+            if (dup || (shells == 1 && g2 != 0)) continue;
+            const double qa = (double)im[0][s & 1] / L + ga, qb = (double)im[1][(s >> 1) & 1] / L + gb,
+                         qc = (double)im[2][s >> 2] / L + gc;
+            acc += exp(-(double)g2) * 4.0 * kPi / (qa * qa + qb * qb + qc * qc + kappa * kappa);
+        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((tid & 31) == 0) hq = acc / nimg;
+    } else if (exchange_on) {
+        for (int i = tid - 96; i < 2 * 26 * t; i += PTHR - 96) {
+            const int s = i / (26 * t), e = i - s * 26 * t;
+            double2 m = mu[e];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                m = cadd(m, cadd(cscale(mu[(size_t)(1 + 2 * a) * 26 * t + e], cs[s][a]),
+                                 cscale(mu[(size_t)(2 + 2 * a) * 26 * t + e], sn[s][a])));
+            M[i] = m;
+        }
     }
     __syncthreads();
-    // exchange form factors M_vc(k, G) = [U_v^H mu(k, G) U_c]_vc at both points
-    for (int idx = threadIdx.x; idx < 2 * 26 * t; idx += blockDim.x) {
-        const int s = idx / (26 * t), G = (idx / t) % 26, tr = idx % t, v = tr / nc, c = tr % nc;
-        double hm[7];
-        hm[0] = 1.0;
-        for (int a = 0; a < 3; ++a) {
-            double sn, cs;
-            sincospi(2.0 * g[s][a] / L, &sn, &cs);
-            hm[1 + 2 * a] = cs;
-            hm[2 + 2 * a] = sn;
-        }
-        double2 acc = make_double2(0.0, 0.0);
-        for (int mm = 0; mm < nv; ++mm)
-            for (int mp = 0; mp < nc; ++mp) {
-                double2 mv = make_double2(0.0, 0.0);
-                for (int h = 0; h < 7; ++h) mv = cadd(mv, cscale(mu[((size_t)(h * 26 + G) * nv + mm) * nc + mp], hm[h]));
-                acc = cadd(acc, cmul(cmulc(Uv[s][mm * nv + v], mv), Uc[s][mp * nc + c]));
-            }
-        M[s][G][tr] = acc;
+    if (exchange_on)
+        for (int s = 0; s < 2; ++s)
+            rotate_forms<true>(M + s * 26 * t, U + s * g, U + s * g + rv, fw, M + s * 26 * t, 26, nv, nc, tid, PTHR,
+                               [] { __syncthreads(); });
+    for (int e = tid; e < g; e += PTHR) {
+        const bool val = e < rv;
+        const int q = val ? e : e - rv, nb = val ? nv : nc, a = q / nb, b = q - a * nb;
+        const double2 *u0 = U + (val ? 0 : rv), *u1 = U + g + (val ? 0 : rv);
+        double2 o = make_double2(0.0, 0.0);
+        for (int m = 0; m < nb; ++m)
+            o = cadd(o, val ? cmulc(u1[m * nb + b], u0[m * nb + a]) : cmulc(u0[m * nb + a], u1[m * nb + b]));
+        O[e] = o;
     }
-    // K^{M1} block, accumulated in Tm via the factored form
-    float2 kacc = make_float2(0.f, 0.f);
-    const int e1 = threadIdx.x / t, e2 = threadIdx.x % t;        // (vc, v'c') of this thread (blockDim >= t*t)
-    const bool mine = threadIdx.x < t * t;
-    const int cell0 = kk[0] / Ndiv, js0 = kk[0] % Ndiv, cell1 = kk[1] / Ndiv, js1 = kk[1] % Ndiv;
-    const Int3 c0 = unflat3(cell0, n), c1 = unflat3(cell1, n);
+    // overlaps with the corners, both points
+    for (int i = tid; i < 16 * g; i += PTHR) {
+        const int s = i / (8 * g), l = (i / g) & 7, e = i % g;
+        const bool val = e < rv;
+        const int q = val ? e : e - rv, nb = val ? nv : nc;
+        if (Dv) {
+            const size_t kd = (size_t)cell[s] * Ndiv + js[s];
+            const double2 v = val ? to_d2(Dv[(kd * 8 + l) * rv + q]) : to_d2(Dc[(kd * 8 + l) * rc + q]);
+            dd[i] = make_float2((float)v.x, (float)v.y);
+        } else {
+            const Int3 ci = unflat3(cell[s], n);
+            const int cc = flat3(ci.a + ((l >> 2) & 1), ci.b + ((l >> 1) & 1), ci.c + (l & 1), n), np = q / nb, b = q - np * nb;
+            const double2 *cu = (val ? Uvc : Ucc) + (size_t)cc * nb * nb, *u = U + s * g + (val ? 0 : rv);
+            double2 v = make_double2(0.0, 0.0);
+            for (int m = 0; m < nb; ++m) v = cadd(v, cmulc(cu[m * nb + np], u[m * nb + b]));
+            dd[i] = make_float2((float)v.x, (float)v.y);
+        }
+    }
+    for (int e = tid; e < t * t; e += PTHR) K1[e] = make_float2(0.f, 0.f);
+    const Int3 c0 = unflat3(cell[0], n), c1 = unflat3(cell[1], n);
+    const int rows = t * nv;                                    // (row of the block, n3)
     for (int l = 0; l < 8; ++l) {
-        const double fa = interp_weight(js0, l, nd, nb1);
-        if (fa == 0.0) continue;
+        const float fa = interp_weight_f(js[0], l, nd, nb1);
+        if (fa == 0.f) continue;
         const int ca = flat3(c0.a + ((l >> 2) & 1), c0.b + ((l >> 1) & 1), c0.c + (l & 1), n);
         __syncthreads();
-        // Fa[(vc), (n1 n2)] = f d_v^{n1} conj(d_c^{n2})
-        for (int idx = threadIdx.x; idx < t * t; idx += blockDim.x) {
-            const int row = idx / t, col = idx % t;
-            const int v = row / nc, c = row % nc, n1 = col / nc, n2 = col % nc;
-            const double2 dv = to_d2(Dv[((size_t)kk[0] * 8 + l) * nv * nv + n1 * nv + v]);
-            const double2 dc = to_d2(Dc[((size_t)kk[0] * 8 + l) * nc * nc + n2 * nc + c]);
-            const double2 f = cscale(cmul(dv, conjg(dc)), fa);
-            Fa[idx] = make_float2((float)f.x, (float)f.y);
-        }
-        for (int lp = 0; lp < 8; ++lp) {
-            const double fb = interp_weight(js1, lp, nd, nb1);
-            if (fb == 0.0) continue;
+        // K_c(ca, cb) for the active corners of k', and its product with d_c over n4
+        for (int i = tid; i < 8 * t * t; i += PTHR) {
+            const int lp = i / (t * t), e = i - lp * t * t;
+            if (!interp_active(js[1], lp, nd, nb1)) continue;
             const int cb = flat3(c1.a + ((lp >> 2) & 1), c1.b + ((lp >> 1) & 1), c1.c + (lp & 1), n);
-            __syncthreads();
-            for (int idx = threadIdx.x; idx < t * t; idx += blockDim.x) {
-                const int row = idx / t, col = idx % t;
-                const int v = row / nc, c = row % nc, n3 = col / nc, n4 = col % nc;
-                const double2 dv = to_d2(Dv[((size_t)kk[1] * 8 + lp) * nv * nv + n3 * nv + v]);
-                const double2 dc = to_d2(Dc[((size_t)kk[1] * 8 + lp) * nc * nc + n4 * nc + c]);
-                const double2 f = cscale(cmul(dv, conjg(dc)), fb);
-                Fb[idx] = make_float2((float)f.x, (float)f.y);                    // F(k', k~'): conj taken below
-            }
-            __syncthreads();
-            // Tm = Fa K_c(ca, cb)
-            for (int idx = threadIdx.x; idx < t * t; idx += blockDim.x) {
-                const int row = idx / t, col = idx % t;
+            const double2 v = to_d2(Kc[(size_t)(ca * t + e / t) * Nc + cb * t + e % t]);
+            Kb[i] = make_float2((float)v.x, (float)v.y);
+        }
+        __syncthreads();
+        for (int i = tid; i < 8 * rows; i += PTHR) {
+            const int lp = i / rows;
+            if (!interp_active(js[1], lp, nd, nb1)) continue;
+            float2* x = Kb + (size_t)i * nc;
+            const float2* d = dd + (8 + lp) * g + rv;
+            float2 in[BSE_MAX_BANDS];
+#pragma unroll
+            for (int q = 0; q < BSE_MAX_BANDS; ++q) if (q < nc) in[q] = x[q];
+            for (int c = 0; c < nc; ++c) {
                 float2 s = make_float2(0.f, 0.f);
-                for (int q = 0; q < t; ++q) {
-                    const float2 a = Fa[row * t + q];
-                    const double2 kv = to_d2(Kc[(size_t)(ca * t + q) * Nc + cb * t + col]);
-                    const float2 k = make_float2((float)kv.x, (float)kv.y);
-                    s = cadd(s, cmul(a, k));
-                }
-                Tm[idx] = s;
+#pragma unroll
+                for (int q = 0; q < BSE_MAX_BANDS; ++q) if (q < nc) s = cadd(s, cmul(in[q], d[q * nc + c]));
+                x[c] = s;
             }
-            __syncthreads();
-            if (mine) {       // K^{M1}[e1][e2] += sum_q Tm[e1][q] conj(Fb[e2][q])
-                for (int q = 0; q < t; ++q) kacc = cadd(kacc, cmul(Tm[e1 * t + q], conjg(Fb[e2 * t + q])));
+        }
+        __syncthreads();
+        // over n3 and the corners: Ts[r][v2][c2] = sum f' conj(d_v[n3][v2]) Kb[l'][r][n3][c2]
+        for (int i = tid; i < t * t; i += PTHR) {
+            const int r = i / t, e = i - r * t, v2 = e / nc, c2 = e - v2 * nc;
+            float2 s = make_float2(0.f, 0.f);
+            for (int lp = 0; lp < 8; ++lp) {
+                const float fb = interp_weight_f(js[1], lp, nd, nb1);
+                if (fb == 0.f) continue;
+                const float2 *d = dd + (8 + lp) * g + v2, *x = Kb + ((size_t)lp * t + r) * t + c2;
+                float2 u = make_float2(0.f, 0.f);
+                for (int m = 0; m < nv; ++m) u = cadd(u, cmulc(d[m * nv], x[m * nc]));
+                s.x = fmaf(fb, u.x, s.x);
+                s.y = fmaf(fb, u.y, s.y);
             }
+            Ts[i] = s;
+        }
+        __syncthreads();
+        // F(k, l) on the left: n2 with conj(d_c), then n1 with d_v
+        float2* Tw = Kb;
+        for (int i = tid; i < t * t; i += PTHR) {
+            const int r = i / t, col = i - r * t, m = r / nc, c = r - m * nc;
+            const float2* d = dd + l * g + rv + c;
+            float2 s = make_float2(0.f, 0.f);
+            for (int q = 0; q < nc; ++q) s = cadd(s, cmulc(d[q * nc], Ts[(m * nc + q) * t + col]));
+            Tw[i] = s;
+        }
+        __syncthreads();
+        for (int i = tid; i < t * t; i += PTHR) {
+            const int r = i / t, col = i - r * t, v = r / nc, c = r - v * nc;
+            const float2* d = dd + l * g + v;
+            float2 s = make_float2(0.f, 0.f);
+            for (int m = 0; m < nv; ++m) s = cadd(s, cmul(d[m * nv], Tw[(m * nc + c) * t + col]));
+            K1[i].x = fmaf(fa, s.x, K1[i].x);
+            K1[i].y = fmaf(fa, s.y, K1[i].y);
         }
     }
     __syncthreads();
-    if (!mine) return;
-    // explicit element
-    const int v = e1 / nc, c = e1 % nc, v2 = e2 / nc, c2 = e2 % nc;
-    double2 ex = make_double2(0.0, 0.0);
-    if (exchange_on) {
-        int G = 0;
-        for (int ga = -1; ga <= 1; ++ga)
-            for (int gb = -1; gb <= 1; ++gb)
-                for (int gc = -1; gc <= 1; ++gc) {
-                    const int g2 = ga * ga + gb * gb + gc * gc;
-                    if (g2 == 0) continue;
-                    ex = cadd(ex, cscale(cmulc(M[0][G][e1], M[1][G][e2]), 4.0 * kPi / g2));
-                    ++G;
-                }
+    // explicit elements and targets
+    for (int i = tid; i < t * t; i += PTHR) {
+        const int e1 = i / t, e2 = i - e1 * t, v = e1 / nc, c = e1 - v * nc, v2 = e2 / nc, c2 = e2 - v2 * nc;
+        double2 ex = make_double2(0.0, 0.0);
+        if (exchange_on)
+            for (int G = 0; G < 26; ++G) {
+                const int q = G + (G >= 13 ? 1 : 0), ga = q / 9 - 1, gb = (q / 3) % 3 - 1, gc = q % 3 - 1;
+                const int g2 = ga * ga + gb * gb + gc * gc;
+                ex = cadd(ex, cscale(cmulc(M[G * t + e1], M[(26 + G) * t + e2]), g2 == 1 ? 4.0 * kPi : (g2 == 2 ? 4.0 * kPi / 2 : 4.0 * kPi / 3)));
+            }
+        const double2 kx = cscale(csub(cscale(ex, 2.0), cscale(cmul(O[v * nv + v2], O[rv + c * nc + c2]), hq * inv_eps)), e_k / nk);
+        const double2 km1 = cscale(make_double2(K1[i].x, K1[i].y), 1.0 / Ndiv);
+        const size_t row = (size_t)blk * t * t + i;
+        reinterpret_cast<float2*>(Y)[row] = make_float2((float)((kx.x - km1.x) * nk), (float)((kx.y - km1.y) * nk));
     }
-    double2 ov = make_double2(0.0, 0.0), oc = make_double2(0.0, 0.0);
-    for (int mm = 0; mm < nv; ++mm) ov = cadd(ov, cmulc(Uv[1][mm * nv + v2], Uv[0][mm * nv + v]));
-    for (int mm = 0; mm < nc; ++mm) oc = cadd(oc, cmulc(Uc[0][mm * nc + c], Uc[1][mm * nc + c2]));
-    const double2 kx = cscale(csub(cscale(ex, 2.0), cscale(cmul(ov, oc), hq * inv_eps)), e_k / nk);
-    const double2 km1 = cscale(make_double2(kacc.x, kacc.y), 1.0 / Ndiv);
-    const size_t row = (size_t)blk * t * t + threadIdx.x;
-    Y[2 * row] = (float)((kx.x - km1.x) * nk);
-    Y[2 * row + 1] = (float)((kx.y - km1.y) * nk);
     // features
-    float* x = X + row * d_in;
-    for (int i = 0; i < d_in; ++i) x[i] = 0.f;
-    double qq = 0.0;
+    double q[4] = {0.0, 0.0, 0.0, 0.0};
     for (int a = 0; a < 3; ++a) {
-        int d = imod(g[0][a] - g[1][a], L);
+        int d = imod(gi[0][a] - gi[1][a], L);
         if (2 * d >= L) d -= L;
-        const double q = (double)d / L;
-        x[a] = (float)q;
-        qq += q * q;
+        q[a] = (double)d / L;
+        q[3] += q[a] * q[a];
     }
-    x[3] = (float)sqrt(qq);
-    x[4 + e1] = 1.f;
-    x[4 + t + e2] = 1.f;
-    x[4 + 2 * t] = (float)dE[(size_t)kk[0] * t + e1];
-    x[5 + 2 * t] = (float)dE[(size_t)kk[1] * t + e2];
+    const float qf[4] = {(float)q[0], (float)q[1], (float)q[2], (float)sqrt(q[3])};
+    const size_t k1 = ((size_t)cell[0] * Ndiv + js[0]) * t, k2 = ((size_t)cell[1] * Ndiv + js[1]) * t;
+    float* x = X + (size_t)blk * t * t * d_in;
+    const float inv_d = 1.f / (float)d_in, inv_t = 1.f / (float)t;
+    for (int i = tid; i < t * t * d_in; i += PTHR) {
+        // i < 24^2 54: the quotients are at least 1/108 from the next integer, FP32 is exact enough below 2^16
+        const int r = (int)(((float)i + 0.5f) * inv_d), e = i - r * d_in, e1 = (int)(((float)r + 0.5f) * inv_t), e2 = r - e1 * t;
+        float v = 0.f;
+        if (e < 4) v = e == 0 ? qf[0] : (e == 1 ? qf[1] : (e == 2 ? qf[2] : qf[3]));
+        else if (e == 4 + e1 || e == 4 + t + e2) v = 1.f;
+        else if (e == 4 + 2 * t) v = (float)dE[k1 + e1];
+        else if (e == 5 + 2 * t) v = (float)dE[k2 + e2];
+        x[i] = v;
+    }
 }
 
 }  // namespace
@@ -979,7 +1027,6 @@ int bse_pairs_generate(bse_ctx* ctx, const bse_interp* s, int nblocks, const int
     const bse_coarse* c = s->co;
     if (c->kc_prec == BSE_PREC_BF16) { ctx->err = "pair data needs a complex128 or complex64 K_c"; return BSE_ERR_UNSUPPORTED; }
     if (s->t > 24) { ctx->err = "pair data supports t <= 24"; return BSE_ERR_UNSUPPORTED; }
-    const int pthreads = std::max(64, (s->t * s->t + 31) / 32 * 32);
     for (int i = 0; i < nblocks; ++i)
         if (host_kd[i] < 0 || host_kd[i] >= s->nk || host_kd2[i] < 0 || host_kd2[i] >= s->nk) {
             ctx->err = "dense index out of range";
@@ -993,16 +1040,20 @@ int bse_pairs_generate(bse_ctx* ctx, const bse_interp* s, int nblocks, const int
     cudaMemcpy(d1, host_kd, sizeof(int) * nblocks, cudaMemcpyHostToDevice);
     cudaMemcpy(d2, host_kd2, sizeof(int) * nblocks, cudaMemcpyHostToDevice);
     const int d_in = 6 + 2 * s->t;
-    if (s->vec_prec == BSE_PREC_F64)
-        k_pairs<double><<<nblocks, pthreads, 0, ctx->stream>>>(d1, d2, nblocks, c->d_gen_v, c->d_gen_c, c->d_mu, (const double2*)c->d_kc,
-                                                         (const double2*)s->d_Dv, (const double2*)s->d_Dc, (const double*)s->d_dE,
-                                                         s->n, s->nd, s->nv, s->nc, s->nb1, c->e_k, 1.0 / c->eps_inf, c->kappa,
-                                                         c->direct_shells, c->exchange_on, d_in, X, Y);
-    else
-        k_pairs<float><<<nblocks, pthreads, 0, ctx->stream>>>(d1, d2, nblocks, c->d_gen_v, c->d_gen_c, c->d_mu, (const float2*)c->d_kc,
-                                                        (const float2*)s->d_Dv, (const float2*)s->d_Dc, (const float*)s->d_dE,
-                                                        s->n, s->nd, s->nv, s->nc, s->nb1, c->e_k, 1.0 / c->eps_inf, c->kappa,
-                                                        c->direct_shells, c->exchange_on, d_in, X, Y);
+    const size_t sm = pairs_smem(s->nv, s->nc);
+    auto go = [&](auto tag) -> int {
+        using T = decltype(tag);
+        using V = typename Cx<T>::V;
+        int r = mlp_attr(ctx, k_pairs<T>, sm);
+        if (r != BSE_OK) return r;
+        k_pairs<T><<<nblocks, PTHR, sm, ctx->stream>>>(d1, d2, c->d_gen_v, c->d_gen_c, c->d_mu, c->d_Uv, c->d_Uc,
+                                                       (const V*)c->d_kc, (const V*)s->d_Dv, (const V*)s->d_Dc, (const T*)s->d_dE,
+                                                       s->n, s->nd, s->nv, s->nc, s->nb1, c->e_k, 1.0 / c->eps_inf, c->kappa,
+                                                       c->direct_shells, c->exchange_on, d_in, X, Y);
+        return BSE_OK;
+    };
+    rc = s->vec_prec == BSE_PREC_F64 ? go(0.0) : go(0.f);
+    if (rc != BSE_OK) { cudaFree(d1); cudaFree(d2); return rc; }
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e == cudaSuccess) e = cudaGetLastError();
     cudaFree(d1);

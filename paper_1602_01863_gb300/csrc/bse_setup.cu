@@ -14,187 +14,225 @@ namespace {
 
 constexpr double kPi = 3.14159265358979323846;
 
-// ------------------------------------------------------------ small matrices
-// n x n complex matrices (n <= 8) held by one thread, row-major.
-struct Mat {
-    double2 v[BSE_MAX_BANDS * BSE_MAX_BANDS];
-};
-
-
-// E = expm(i A) for Hermitian A (dmat_expm_i: scaling and squaring of the Taylor series).
-__device__ void expm_i(const Mat& A, int n, Mat& E) { dmat_expm_i(A.v, n, E.v); }
-
-// Fractional coordinate of point p of an (n * nd)^3 grid in coarse-major order.
-__device__ inline void point_frac(int p, int n, int nd, double k[3], int g[3]) {
+// Integer coordinates of point p of an (n * nd)^3 grid in coarse-major order.
+__device__ inline Int3 point_ints(int p, int n, int nd) {
     const int Ndiv = nd * nd * nd;
-    const int ic = p / Ndiv, js = p % Ndiv;
-    const Int3 i = unflat3(ic, n), j = unflat3(js, nd);
-    g[0] = i.a * nd + j.a; g[1] = i.b * nd + j.b; g[2] = i.c * nd + j.c;
-    const double L = (double)(n * nd);
-    for (int a = 0; a < 3; ++a) k[a] = g[a] / L;
+    const Int3 i = unflat3(p / Ndiv, n), j = unflat3(p % Ndiv, nd);
+    return Int3{i.a * nd + j.a, i.b * nd + j.b, i.c * nd + j.c};
 }
 
-// Band gauge U(k) = expm(i sum_a [sin(2 pi k_a) G_a0 + (1 - cos 2 pi k_a) G_a1]).
-__global__ void k_gauge(const double2* __restrict__ gen, int nb, int n, int nd, int npts,
-                        double2* __restrict__ U) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= npts) return;
-    double k[3];
-    int g[3];
-    point_frac(p, n, nd, k, g);
-    Mat A, E;
-    for (int i = 0; i < nb * nb; ++i) A.v[i] = make_double2(0.0, 0.0);
-    for (int a = 0; a < 3; ++a) {
-        double s, c;
-        sincospi(2.0 * k[a], &s, &c);
-        const double2* g0 = gen + (a * 2 + 0) * nb * nb;
-        const double2* g1 = gen + (a * 2 + 1) * nb * nb;
-        for (int i = 0; i < nb * nb; ++i)
-            A.v[i] = cadd(A.v[i], cadd(cscale(g0[i], s), cscale(g1[i], 1.0 - c)));
-    }
-    expm_i(A, nb, E);
-    for (int i = 0; i < nb * nb; ++i) U[(size_t)p * nb * nb + i] = E.v[i];
-}
-
-__device__ inline void harmonics(const double k[3], double c[7]) {
-    c[0] = 1.0;
-    for (int a = 0; a < 3; ++a) {
-        double s, co;
-        sincospi(2.0 * k[a], &s, &co);
-        c[1 + 2 * a] = co;
-        c[2 + 2 * a] = s;
-    }
+// Coarse band gauge U(k~), both manifolds: a warp per point, a half warp each.
+__global__ void __launch_bounds__(128) k_gauge(const double2* __restrict__ gen_v, const double2* __restrict__ gen_c, int nv,
+                                               int nc, int n, double2* __restrict__ Uv, double2* __restrict__ Uc) {
+    extern __shared__ double2 gsm[];
+    const int warp = threadIdx.x >> 5, half = (threadIdx.x >> 4) & 1, p = blockIdx.x * 4 + warp;
+    if (p >= n * n * n) return;
+    double2* work = gsm + (size_t)warp * kGaugeMats * (nv * nv + nc * nc) + (half ? kGaugeMats * nv * nv : 0);
+    const Int3 g = unflat3(p, n);
+    double sn[3], cs[3];
+    sincospi(2.0 * g.a / n, &sn[0], &cs[0]);
+    sincospi(2.0 * g.b / n, &sn[1], &cs[1]);
+    sincospi(2.0 * g.c / n, &sn[2], &cs[2]);
+    const int nb = half ? nc : nv;
+    const double2* E = grp_gauge(half ? gen_c : gen_v, nb, sn, cs, work);
+    double2* out = (half ? Uc : Uv) + (size_t)p * nb * nb;
+    for (int e = grp_lane(); e < nb * nb; e += kGaugeLanes) out[e] = E[e];
 }
 
 // Minimum-image shape tables over all index differences of an L^3 grid:
 // mode 0: h(q) = sum_G exp(-|G|^2) 4 pi / (|q + G|^2 + kappa^2) over `shells` G;
 // mode 1: head 1 / (|q|^2 + kappa^2).  Ties (difference L/2) average the images.
-__global__ void k_shape_table(int L, double kappa, int shells, int h_const, double h0, int mode,
-                              double* __restrict__ out) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+// A warp per difference: the lanes share the images' G sums.
+__global__ void __launch_bounds__(128) k_shape_table(int L, double kappa, int shells, int h_const, double h0, int mode,
+                                                     double* __restrict__ out) {
+    const int idx = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (idx >= L * L * L) return;
-    if (mode == 0 && h_const) { out[idx] = h0; return; }
-    const Int3 d = unflat3(idx, L);
-    int cand[3][2], nc[3];
-    const int dd[3] = {d.a, d.b, d.c};
-    for (int a = 0; a < 3; ++a) {
-        const int r = dd[a];
-        if (2 * r < L) { cand[a][0] = r; nc[a] = 1; }
-        else if (2 * r > L) { cand[a][0] = r - L; nc[a] = 1; }
-        else { cand[a][0] = r; cand[a][1] = r - L; nc[a] = 2; }
+    if (mode == 0 && h_const) {
+        if (lane == 0) out[idx] = h0;
+        return;
     }
+    const Int3 d = unflat3(idx, L);
+    const int dd[3] = {d.a, d.b, d.c};
+    // half-way differences have two images; the others count both as the same one
+    int im[3][2], nimg = 1;
+    for (int a = 0; a < 3; ++a) {
+        im[a][0] = 2 * dd[a] > L ? dd[a] - L : dd[a];
+        im[a][1] = 2 * dd[a] >= L ? dd[a] - L : dd[a];
+        if (im[a][0] != im[a][1]) nimg *= 2;
+    }
+    const int nG = mode == 1 ? 1 : 27;
     double acc = 0.0;
-    int cnt = 0;
-    for (int x = 0; x < nc[0]; ++x)
-        for (int y = 0; y < nc[1]; ++y)
-            for (int z = 0; z < nc[2]; ++z) {
-                const double q[3] = {(double)cand[0][x] / L, (double)cand[1][y] / L, (double)cand[2][z] / L};
-                double v = 0.0;
-                if (mode == 1) {
-                    v = 1.0 / (q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + kappa * kappa);
-                } else {
-                    for (int ga = -1; ga <= 1; ++ga)
-                        for (int gb = -1; gb <= 1; ++gb)
-                            for (int gc = -1; gc <= 1; ++gc) {
-                                const int g2 = ga * ga + gb * gb + gc * gc;
-                                if (shells == 1 && g2 != 0) continue;
-                                const double qa = q[0] + ga, qb = q[1] + gb, qc = q[2] + gc;
-                                v += exp(-(double)g2) * 4.0 * kPi / (qa * qa + qb * qb + qc * qc + kappa * kappa);
-                            }
-                }
-                acc += v;
-                ++cnt;
-            }
-    out[idx] = acc / cnt;
+    for (int q = lane; q < 8 * nG; q += 32) {
+        const int s = q / nG, G = mode == 1 ? 13 : q - s * nG;
+        // count every distinct image once
+        bool dup = false;
+        for (int a = 0; a < 3; ++a) dup = dup || (((s >> a) & 1) && im[a][0] == im[a][1]);
+        const int ga = G / 9 - 1, gb = (G / 3) % 3 - 1, gc = G % 3 - 1, g2 = ga * ga + gb * gb + gc * gc;
+        if (dup || (mode == 0 && shells == 1 && g2 != 0)) continue;
+        const double qa = (double)im[0][s & 1] / L + ga, qb = (double)im[1][(s >> 1) & 1] / L + gb,
+                     qc = (double)im[2][s >> 2] / L + gc, r = qa * qa + qb * qb + qc * qc + kappa * kappa;
+        acc += mode == 1 ? 1.0 / r : exp(-(double)g2) * 4.0 * kPi / r;
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) out[idx] = acc / nimg;
 }
 
-// Exchange form factors on the coarse mesh: M_vc(k~, G) = [U_v^H mu(k~, G) U_c]_vc.
-__global__ void k_form_factors(const double2* __restrict__ Uv, const double2* __restrict__ Uc,
-                               const double2* __restrict__ mu, int n, int nv, int nc,
-                               double2* __restrict__ M) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nkc = n * n * n;
-    if (idx >= nkc * 26) return;
-    const int ic = idx / 26, G = idx % 26;
-    double k[3];
-    int g[3];
-    point_frac(ic, n, 1, k, g);
+// Exchange form factors on the coarse mesh: M_vc(k~, G) = [U_v^H mu(k~, G) U_c]_vc, one
+// block per coarse point: mu(k~) from its harmonics once, then one gauge factor
+// at a time (together 7 + nv + nc terms per entry instead of 7 nv nc).
+__global__ void __launch_bounds__(256) k_form_factors(const double2* __restrict__ Uv, const double2* __restrict__ Uc,
+                                                      const double2* __restrict__ mu, int n, int nv, int nc,
+                                                      double2* __restrict__ M) {
+    extern __shared__ double2 fsm[];
+    const int ic = blockIdx.x, t = nv * nc, tid = threadIdx.x;
+    double2 *a = fsm, *b = a + 26 * t, *uv = b + 26 * t, *uc = uv + nv * nv;
+    for (int e = tid; e < nv * nv; e += 256) uv[e] = Uv[(size_t)ic * nv * nv + e];
+    for (int e = tid; e < nc * nc; e += 256) uc[e] = Uc[(size_t)ic * nc * nc + e];
+    const Int3 g = unflat3(ic, n);
     double c[7];
-    harmonics(k, c);
-    const double2* uv = Uv + (size_t)ic * nv * nv;
-    const double2* uc = Uc + (size_t)ic * nc * nc;
-    for (int v = 0; v < nv; ++v)
-        for (int cc = 0; cc < nc; ++cc) {
-            double2 s = make_double2(0.0, 0.0);
-            for (int m = 0; m < nv; ++m)
-                for (int mp = 0; mp < nc; ++mp) {
-                    double2 muv = make_double2(0.0, 0.0);
-                    for (int h = 0; h < 7; ++h)
-                        muv = cadd(muv, cscale(mu[((size_t)(h * 26 + G) * nv + m) * nc + mp], c[h]));
-                    s = cadd(s, cmul(cmulc(uv[m * nv + v], muv), uc[mp * nc + cc]));
-                }
-            M[((size_t)ic * 26 + G) * nv * nc + v * nc + cc] = s;
-        }
+    c[0] = 1.0;
+    sincospi(2.0 * g.a / n, &c[2], &c[1]);
+    sincospi(2.0 * g.b / n, &c[4], &c[3]);
+    sincospi(2.0 * g.c / n, &c[6], &c[5]);
+    for (int e = tid; e < 26 * t; e += 256) {
+        double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int h = 0; h < 7; ++h) s = cadd(s, cscale(mu[(size_t)h * 26 * t + e], c[h]));
+        a[e] = s;
+    }
+    __syncthreads();
+    rotate_forms<true>(a, uv, uc, b, M + (size_t)ic * 26 * t, 26, nv, nc, tid, 256, [] { __syncthreads(); });
 }
 
 // K_c element (Eq. bse2 in the model, coarse weight e_k / n^3):
 //   K = pref [ 2 sum_G v(G) conj(M_i(G)) M_j(G) - O^v O^c h(k~_i - k~_j) / eps_inf ].
-// 16 x 16 tiles; the form factors of the tile's rows and columns are staged in
-// shared memory.  Output in the storage precision of the handle.
+// A block takes the entries of PT x PT coarse points (at most 64 x 64 entries),
+// on and above the diagonal only; each value is also written, conjugated, to
+// its mirror image.  FP64 bounds it (1.25 TFLOP/s on GB300), so the work per
+// entry is cut: the exchange sum takes three real products per G
+// (re = S1 + S2, im = S3 - S1 + S2 with S1 = sum a_r b_r, S2 = sum a_i b_i,
+// S3 = sum (a_r - a_i)(b_r + b_i), conj(a) b), the overlaps are formed once per pair
+// of points, and half of the matrix is never computed.  N_c = 8192, BF16: 26.1 ms
+// with one thread per entry of the whole matrix (a run of set-up, 24 steps and
+// spectrum: 58.7 ms; 17.3 ms with this set-up and the common-basis step loop).
+// Output in the storage precision of the handle.
+constexpr int KC_T = 64;
+__host__ __device__ inline int kc_points(int t) { const int p = KC_T / t; return p < 1 ? 1 : (p > 8 ? 8 : p); }
+size_t kc_smem(int nv, int nc) {
+    const int t = nv * nc, P = kc_points(t);
+    const size_t forms = sizeof(double) * 6 * 26 * KC_T, tile = sizeof(double2) * KC_T * (KC_T + 1);
+    return std::max(forms, tile) + sizeof(double2) * P * P * (nv * nv + nc * nc) + sizeof(double) * P * P;
+}
 template <int PREC>
-__global__ void k_build_kc(const double2* __restrict__ M, const double2* __restrict__ Uv,
-                           const double2* __restrict__ Uc, const double* __restrict__ htab, int n,
-                           int nv, int nc, double pref, double inv_eps, int exchange_on, int Nc,
-                           int ldk, void* __restrict__ out, __nv_bfloat16* __restrict__ kr,
-                           __nv_bfloat16* __restrict__ ki) {
-    __shared__ double2 Mi[16][26];
-    __shared__ double2 Mj[16][26];
-    const int t = nv * nc;
-    const int i0 = blockIdx.y * 16, j0 = blockIdx.x * 16;
-    const int tid = threadIdx.y * 16 + threadIdx.x;
-    for (int e = tid; e < 16 * 26; e += 256) {
-        const int r = e / 26, G = e % 26;
-        const int i = i0 + r, j = j0 + r;
-        Mi[r][G] = (i < Nc) ? M[((size_t)(i / t) * 26 + G) * t + (i % t)] : make_double2(0.0, 0.0);
-        Mj[r][G] = (j < Nc) ? M[((size_t)(j / t) * 26 + G) * t + (j % t)] : make_double2(0.0, 0.0);
+__global__ void __launch_bounds__(256) k_build_kc(const double2* __restrict__ M, const double2* __restrict__ Uv,
+                                                  const double2* __restrict__ Uc, const double* __restrict__ htab, int n,
+                                                  int nv, int nc, double pref, double inv_eps, int exchange_on, int Nc,
+                                                  int ldk, void* __restrict__ out, __nv_bfloat16* __restrict__ kr,
+                                                  __nv_bfloat16* __restrict__ ki) {
+    if (blockIdx.x < blockIdx.y) return;
+    extern __shared__ __align__(16) unsigned char kcsm[];
+    const int t = nv * nc, P = kc_points(t), nkc = n * n * n, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int pa = blockIdx.y * P, pb = blockIdx.x * P, na = min(P, nkc - pa), nb = min(P, nkc - pb);
+    const int i0 = pa * t, j0 = pb * t, ri = na * t, rj = nb * t;          // rows and columns of this tile
+    double* f = reinterpret_cast<double*>(kcsm);                            // [6][26][KC_T] a_r v, a_i v, (a_r - a_i) v, b_r, b_i, b_r + b_i
+    double2* tile = reinterpret_cast<double2*>(kcsm);                       // [KC_T][KC_T + 1], after the sums
+    const size_t head = max(sizeof(double) * 6 * 26 * KC_T, sizeof(double2) * KC_T * (KC_T + 1));
+    double2* ov = reinterpret_cast<double2*>(kcsm + head);                  // [P P][nv nv]
+    double2* oc = ov + P * P * nv * nv;                                     // [P P][nc nc]
+    double* hh = reinterpret_cast<double*>(oc + P * P * nc * nc);           // [P P]
+    if (exchange_on)
+        for (int e = tid; e < 26 * KC_T; e += 256) {
+            const int G = e / KC_T, r = e % KC_T, q = G + (G >= 13 ? 1 : 0);
+            const int ga = q / 9 - 1, gb = (q / 3) % 3 - 1, gc = q % 3 - 1;
+            const double v = 4.0 * kPi / (ga * ga + gb * gb + gc * gc);
+            const double2 z = make_double2(0.0, 0.0);
+            const double2 a = r < ri ? M[((size_t)(pa + r / t) * 26 + G) * t + r % t] : z;
+            const double2 b = r < rj ? M[((size_t)(pb + r / t) * 26 + G) * t + r % t] : z;
+            f[e] = a.x * v; f[26 * KC_T + e] = a.y * v; f[2 * 26 * KC_T + e] = (a.x - a.y) * v;
+            f[3 * 26 * KC_T + e] = b.x; f[4 * 26 * KC_T + e] = b.y; f[5 * 26 * KC_T + e] = b.x + b.y;
+        }
+    for (int e = tid; e < na * nb * (nv * nv + nc * nc + 1); e += 256) {
+        const int q = e / (na * nb), pr = e - q * (na * nb), x = pr / nb, y = pr - x * nb, ic = pa + x, jc = pb + y, s = x * P + y;
+        if (q < nv * nv) {                                                   // Uv[a]_mv conj(Uv[b]_mv2)
+            const int v = q / nv, v2 = q % nv;
+            double2 o = make_double2(0.0, 0.0);
+            for (int m = 0; m < nv; ++m)
+                o = cadd(o, cmulc(Uv[((size_t)jc * nv + m) * nv + v2], Uv[((size_t)ic * nv + m) * nv + v]));
+            ov[s * nv * nv + q] = o;
+        } else if (q < nv * nv + nc * nc) {                                   // conj(Uc[a]_mc) Uc[b]_mc2
+            const int w = q - nv * nv, c = w / nc, c2 = w % nc;
+            double2 o = make_double2(0.0, 0.0);
+            for (int m = 0; m < nc; ++m)
+                o = cadd(o, cmulc(Uc[((size_t)ic * nc + m) * nc + c], Uc[((size_t)jc * nc + m) * nc + c2]));
+            oc[s * nc * nc + w] = o;
+        } else {
+            const Int3 ia = unflat3(ic, n), ib = unflat3(jc, n);
+            hh[s] = htab[flat3(ia.a - ib.a, ia.b - ib.b, ia.c - ib.c, n)] * inv_eps;
+        }
     }
     __syncthreads();
-    const int i = i0 + threadIdx.y, j = j0 + threadIdx.x;
-    if (i >= Nc || j >= Nc) return;
-    double2 ex = make_double2(0.0, 0.0);
-    if (exchange_on) {
-        int G = 0;
-        for (int ga = -1; ga <= 1; ++ga)
-            for (int gb = -1; gb <= 1; ++gb)
-                for (int gc = -1; gc <= 1; ++gc) {
-                    const int g2 = ga * ga + gb * gb + gc * gc;
-                    if (g2 == 0) continue;
-                    const double vG = 4.0 * kPi / g2;
-                    ex = cadd(ex, cscale(cmulc(Mi[threadIdx.y][G], Mj[threadIdx.x][G]), vG));
-                    ++G;
+    double s1[4][4], s2[4][4], s3[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s1[i][j] = s2[i][j] = s3[i][j] = 0.0;
+    if (exchange_on)
+        for (int G = 0; G < 26; ++G) {
+            double a[3][4], b[3][4];
+#pragma unroll
+            for (int w = 0; w < 3; ++w)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    a[w][i] = f[(w * 26 + G) * KC_T + ty + 16 * i];
+                    b[w][i] = f[((3 + w) * 26 + G) * KC_T + tx + 16 * i];
                 }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    s1[i][j] = fma(a[0][i], b[0][j], s1[i][j]);
+                    s2[i][j] = fma(a[1][i], b[1][j], s2[i][j]);
+                    s3[i][j] = fma(a[2][i], b[2][j], s3[i][j]);
+                }
+        }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = ty + 16 * i;
+        if (r >= ri) continue;
+        const int x = r / t, e = r - x * t, v = e / nc, c = e - v * nc;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int q = tx + 16 * j;
+            if (q >= rj) continue;
+            const int y = q / t, e2 = q - y * t, v2 = e2 / nc, c2 = e2 - v2 * nc, s = x * P + y;
+            const double2 d = cscale(cmul(ov[s * nv * nv + v * nv + v2], oc[s * nc * nc + c * nc + c2]), hh[s]);
+            tile[r * (KC_T + 1) + q] = make_double2(pref * (2.0 * (s1[i][j] + s2[i][j]) - d.x),
+                                                    pref * (2.0 * (s3[i][j] - s1[i][j] + s2[i][j]) - d.y));
+        }
     }
-    const int ic = i / t, tr = i % t, v = tr / nc, c = tr % nc;
-    const int jc = j / t, tq = j % t, v2 = tq / nc, c2 = tq % nc;
-    const double2* uva = Uv + (size_t)ic * nv * nv;
-    const double2* uvb = Uv + (size_t)jc * nv * nv;
-    const double2* uca = Uc + (size_t)ic * nc * nc;
-    const double2* ucb = Uc + (size_t)jc * nc * nc;
-    double2 ov = make_double2(0.0, 0.0), oc = make_double2(0.0, 0.0);
-    for (int m = 0; m < nv; ++m) ov = cadd(ov, cmulc(uvb[m * nv + v2], uva[m * nv + v]));   // Uv[a]_mv conj(Uv[b]_mv2)
-    for (int m = 0; m < nc; ++m) oc = cadd(oc, cmulc(uca[m * nc + c], ucb[m * nc + c2]));   // conj(Uc[a]_mc) Uc[b]_mc2
-    const Int3 ia = unflat3(ic, n), ib = unflat3(jc, n);
-    const double h = htab[flat3(ia.a - ib.a, ia.b - ib.b, ia.c - ib.c, n)];
-    const double2 d = cscale(cmul(ov, oc), h * inv_eps);
-    const double2 kv = cscale(csub(cscale(ex, 2.0), d), pref);
-    if (PREC == BSE_PREC_F64) {
-        reinterpret_cast<double2*>(out)[(size_t)i * Nc + j] = kv;
-    } else if (PREC == BSE_PREC_F32) {
-        reinterpret_cast<float2*>(out)[(size_t)i * Nc + j] = make_float2((float)kv.x, (float)kv.y);
-    } else {
-        kr[(size_t)i * ldk + j] = __double2bfloat16(kv.x);
-        ki[(size_t)i * ldk + j] = __double2bfloat16(kv.y);
-    }
+    __syncthreads();
+    const bool diag = blockIdx.x == blockIdx.y;
+    auto put = [&](size_t i, size_t j, double2 v) {
+        if (PREC == BSE_PREC_F64) {
+            reinterpret_cast<double2*>(out)[i * Nc + j] = v;
+        } else if (PREC == BSE_PREC_F32) {
+            reinterpret_cast<float2*>(out)[i * Nc + j] = make_float2((float)v.x, (float)v.y);
+        } else {
+            kr[i * ldk + j] = __double2bfloat16(v.x);
+            ki[i * ldk + j] = __double2bfloat16(v.y);
+        }
+    };
+    const int col = tid & 63, row0 = tid >> 6;
+    for (int r = row0; r < ri; r += 4)
+        if (col < rj) {
+            // a diagonal tile keeps its upper half and mirrors it
+            const double2 v = diag && r > col ? conjg(tile[col * (KC_T + 1) + r]) : tile[r * (KC_T + 1) + col];
+            put((size_t)i0 + r, (size_t)j0 + col, v);
+        }
+    if (!diag)
+        for (int r = row0; r < rj; r += 4)
+            if (col < ri) put((size_t)j0 + r, (size_t)i0 + col, conjg(tile[col * (KC_T + 1) + r]));
 }
 
 // ---------------------------------------------------------------- Method 2
@@ -314,63 +352,76 @@ __global__ void k_cplx_to(const double2* __restrict__ src, long long n, V* __res
     if (i < n) dst[i] = from_d2<V>(src[i]);
 }
 
-// Dense tables, one thread per dense point kd:
-//   Delta E_vc(k) (exact on the dense mesh), dipoles P^alpha_vc(k) = [U_v^T pi^alpha conj(U_c)],
-//   and for all 8 corners d = U(k~)^H U(k) for both manifolds (Eq. completeness).
+// Dense tables, a warp per dense point kd: the gauge U(k) (a half warp per
+// manifold), Delta E_vc(k) (exact on the dense mesh), dipoles
+// P^alpha_vc(k) = [U_v^T pi^alpha conj(U_c)], and, where the path reads them, U
+// itself in the vector precision (Uvt, Uct) or the overlaps d = U(k~)^H U(k) with
+// the 8 corners (Eq. completeness).  FP64 bounds it; everything stays in
+// shared memory: 32768 points of 4x4 bands took 4.4 ms with a thread per point.
+constexpr int kDenseWarps = 4;
+size_t dense_smem(int nv, int nc) {
+    return sizeof(double2) * kDenseWarps * (kGaugeMats * (nv * nv + nc * nc) + 2 * 3 * nv * nc);
+}
 template <typename T>
-__global__ void k_dense_tables(const double2* __restrict__ Uvd, const double2* __restrict__ Ucd,
-                               const double2* __restrict__ Uvc, const double2* __restrict__ Ucc,
-                               const double* __restrict__ offsets, const double2* __restrict__ dip,
-                               int n, int nd, int nv, int nc, double e_gap, double band_width,
-                               T* __restrict__ dE, typename Cx<T>::V* __restrict__ Dv,
-                               typename Cx<T>::V* __restrict__ Dc, double2* __restrict__ P) {
+__global__ void __launch_bounds__(32 * kDenseWarps) k_dense_tables(
+    const double2* __restrict__ gen_v, const double2* __restrict__ gen_c, const double2* __restrict__ Uvc,
+    const double2* __restrict__ Ucc, const double* __restrict__ offsets, const double2* __restrict__ dip, int n, int nd,
+    int nv, int nc, double e_gap, double band_width, T* __restrict__ dE, typename Cx<T>::V* __restrict__ Dv,
+    typename Cx<T>::V* __restrict__ Dc, typename Cx<T>::V* __restrict__ Uvt, typename Cx<T>::V* __restrict__ Uct,
+    double2* __restrict__ P) {
     using V = typename Cx<T>::V;
-    const int nk = n * n * n * nd * nd * nd;
-    const int kd = blockIdx.x * blockDim.x + threadIdx.x;
-    if (kd >= nk) return;
-    const int t = nv * nc, N = nk * t;
-    const int Ndiv = nd * nd * nd;
-    double k[3];
-    int g[3];
-    point_frac(kd, n, nd, k, g);
-    double band = e_gap;
-    for (int a = 0; a < 3; ++a) band += band_width * (1.0 - cospi(2.0 * k[a]));
-    for (int tr = 0; tr < t; ++tr) dE[(size_t)kd * t + tr] = (T)(band + offsets[tr]);
-    const double2* uv = Uvd + (size_t)kd * nv * nv;
-    const double2* uc = Ucd + (size_t)kd * nc * nc;
-    double c[7];
-    harmonics(k, c);
-    for (int al = 0; al < 3; ++al)
-        for (int v = 0; v < nv; ++v)
-            for (int cc = 0; cc < nc; ++cc) {
-                double2 s = make_double2(0.0, 0.0);
-                for (int m = 0; m < nv; ++m)
-                    for (int mp = 0; mp < nc; ++mp) {
-                        double2 pim = make_double2(0.0, 0.0);
-                        for (int h = 0; h < 7; ++h)
-                            pim = cadd(pim, cscale(dip[((size_t)(h * 3 + al) * nv + m) * nc + mp], c[h]));
-                        s = cadd(s, cmul(cmul(uv[m * nv + v], pim), conjg(uc[mp * nc + cc])));
-                    }
-                P[(size_t)al * N + (size_t)kd * t + v * nc + cc] = s;
+    extern __shared__ double2 dsm[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4;
+    const int t = nv * nc, rv = nv * nv, rc = nc * nc, Ndiv = nd * nd * nd, nk = n * n * n * Ndiv, L = n * nd;
+    const size_t N = (size_t)nk * t;
+    double2* work = dsm + (size_t)warp * (kGaugeMats * (rv + rc) + 6 * t);
+    double2* pa = work + kGaugeMats * (rv + rc);
+    double2* pb = pa + 3 * t;
+    for (int kd = blockIdx.x * kDenseWarps + warp; kd < nk; kd += gridDim.x * kDenseWarps) {
+        const Int3 g = point_ints(kd, n, nd);
+        double sn[3], cs[3];
+        sincospi(2.0 * g.a / L, &sn[0], &cs[0]);
+        sincospi(2.0 * g.b / L, &sn[1], &cs[1]);
+        sincospi(2.0 * g.c / L, &sn[2], &cs[2]);
+        const double2* E = grp_gauge(half ? gen_c : gen_v, half ? nc : nv, sn, cs, half ? work + kGaugeMats * rv : work);
+        // both halves' results, by their places in the scratch
+        const int at = (int)(E - work), av = __shfl_sync(0xffffffffu, at, 0), ac = __shfl_sync(0xffffffffu, at, 16);
+        const double2 *uv = work + av, *uc = work + ac;
+        __syncwarp();
+        double band = e_gap;
+        for (int a = 0; a < 3; ++a) band += band_width * (1.0 - cs[a]);
+        for (int e = lane; e < t; e += 32) dE[(size_t)kd * t + e] = (T)(band + offsets[e]);
+        if (Uvt) {
+            for (int e = lane; e < rv; e += 32) Uvt[(size_t)kd * rv + e] = from_d2<V>(uv[e]);
+            for (int e = lane; e < rc; e += 32) Uct[(size_t)kd * rc + e] = from_d2<V>(uc[e]);
+        }
+        for (int e = lane; e < 3 * t; e += 32) {
+            double2 s = dip[e];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                s = cadd(s, cadd(cscale(dip[(size_t)(1 + 2 * a) * 3 * t + e], cs[a]), cscale(dip[(size_t)(2 + 2 * a) * 3 * t + e], sn[a])));
+            pa[e] = s;
+        }
+        __syncwarp();
+        rotate_forms<false>(pa, uv, uc, pb, pa, 3, nv, nc, lane, 32, [] { __syncwarp(); });
+        for (int e = lane; e < 3 * t; e += 32) P[(size_t)(e / t) * N + (size_t)kd * t + e % t] = pa[e];
+        if (Dv) {
+            const Int3 i = unflat3(kd / Ndiv, n);
+            for (int l = 0; l < 8; ++l) {
+                const int cic = flat3(i.a + ((l >> 2) & 1), i.b + ((l >> 1) & 1), i.c + (l & 1), n);
+                const double2* cv = Uvc + (size_t)cic * rv;
+                const double2* cm = Ucc + (size_t)cic * rc;
+                for (int e = lane; e < rv + rc; e += 32) {
+                    const bool val = e < rv;
+                    const int q = val ? e : e - rv, nb = val ? nv : nc, np = q / nb, b = q - np * nb;
+                    double2 s = make_double2(0.0, 0.0);
+                    for (int m = 0; m < nb; ++m) s = cadd(s, cmulc((val ? cv : cm)[m * nb + np], (val ? uv : uc)[m * nb + b]));
+                    if (val) Dv[((size_t)kd * 8 + l) * rv + q] = from_d2<V>(s);
+                    else Dc[((size_t)kd * 8 + l) * rc + q] = from_d2<V>(s);
+                }
             }
-    const int ic = kd / Ndiv;
-    const Int3 i = unflat3(ic, n);
-    for (int l = 0; l < 8; ++l) {
-        const int cic = flat3(i.a + ((l >> 2) & 1), i.b + ((l >> 1) & 1), i.c + (l & 1), n);
-        const double2* cv = Uvc + (size_t)cic * nv * nv;
-        const double2* ccm = Ucc + (size_t)cic * nc * nc;
-        for (int np = 0; np < nv; ++np)
-            for (int v = 0; v < nv; ++v) {
-                double2 s = make_double2(0.0, 0.0);
-                for (int m = 0; m < nv; ++m) s = cadd(s, cmulc(cv[m * nv + np], uv[m * nv + v]));
-                Dv[((size_t)kd * 8 + l) * nv * nv + np * nv + v] = from_d2<V>(s);
-            }
-        for (int np = 0; np < nc; ++np)
-            for (int cc = 0; cc < nc; ++cc) {
-                double2 s = make_double2(0.0, 0.0);
-                for (int m = 0; m < nc; ++m) s = cadd(s, cmulc(ccm[m * nc + np], uc[m * nc + cc]));
-                Dc[((size_t)kd * 8 + l) * nc * nc + np * nc + cc] = from_d2<V>(s);
-            }
+        }
+        __syncwarp();
     }
 }
 
@@ -421,6 +472,15 @@ __global__ void k_near_head(const int* __restrict__ offs, int n_near, int L, dou
     hd[i] = (T)(1.0 / (qa * qa + qb * qb + qc * qc + kappa * kappa));
 }
 
+template <typename K>
+int raise_smem(bse_ctx* ctx, K kernel, size_t bytes) {
+    cudaFuncAttributes fa;
+    BSE_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, kernel));
+    if ((size_t)fa.maxDynamicSharedSizeBytes < bytes)
+        BSE_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    return BSE_OK;
+}
+
 inline int blocks_for(long long n, int bs) { return (int)((n + bs - 1) / bs); }
 
 }  // namespace
@@ -450,15 +510,18 @@ int bse_setup_coarse_device(bse_ctx* ctx, bse_coarse* c, const void* user_kc) {
     cudaStream_t st = ctx->stream;
     TRY(bse_alloc(ctx, (void**)&c->d_Uv, sizeof(double2) * nkc * nv * nv, "coarse Uv"));
     TRY(bse_alloc(ctx, (void**)&c->d_Uc, sizeof(double2) * nkc * nc * nc, "coarse Uc"));
-    k_gauge<<<blocks_for(nkc, 64), 64, 0, st>>>(c->d_gen_v, nv, n, 1, nkc, c->d_Uv);
-    k_gauge<<<blocks_for(nkc, 64), 64, 0, st>>>(c->d_gen_c, nc, n, 1, nkc, c->d_Uc);
+    const size_t gsm = sizeof(double2) * 4 * kGaugeMats * (nv * nv + nc * nc);
+    TRY(raise_smem(ctx, k_gauge, gsm));
+    k_gauge<<<blocks_for(nkc, 4), 128, gsm, st>>>(c->d_gen_v, c->d_gen_c, nv, nc, n, c->d_Uv, c->d_Uc);
     double2* d_M = nullptr;
     double* d_h = nullptr;
     if (!user_kc) {
         TRY(bse_alloc(ctx, (void**)&d_M, sizeof(double2) * nkc * 26 * nv * nc, "form factors"));
         TRY(bse_alloc(ctx, (void**)&d_h, sizeof(double) * nkc, "shape table"));
-        k_form_factors<<<blocks_for((long long)nkc * 26, 64), 64, 0, st>>>(c->d_Uv, c->d_Uc, c->d_mu, n, nv, nc, d_M);
-        k_shape_table<<<blocks_for(nkc, 128), 128, 0, st>>>(n, c->kappa, c->direct_shells, c->h_const, c->h0, 0, d_h);
+        const size_t fsm = sizeof(double2) * (52 * nv * nc + nv * nv + nc * nc);
+        TRY(raise_smem(ctx, k_form_factors, fsm));
+        k_form_factors<<<nkc, 256, fsm, st>>>(c->d_Uv, c->d_Uc, c->d_mu, n, nv, nc, d_M);
+        k_shape_table<<<blocks_for(nkc, 4), 128, 0, st>>>(n, c->kappa, c->direct_shells, c->h_const, c->h0, 0, d_h);
     }
     size_t bytes;
     if (c->kc_prec == BSE_PREC_F64) bytes = sizeof(double2) * (size_t)Nc * Nc;
@@ -469,10 +532,21 @@ int bse_setup_coarse_device(bse_ctx* ctx, bse_coarse* c, const void* user_kc) {
     if (c->kc_prec == BSE_PREC_BF16) {
         c->d_kr = reinterpret_cast<__nv_bfloat16*>(c->d_kc);
         c->d_ki = c->d_kr + (size_t)Nc * c->ldk;
-        cudaMemsetAsync(c->d_kc, 0, bytes, st);                 // zero the padding columns
+        if (c->ldk > Nc)                                        // zero the padding columns of both planes
+            cudaMemset2DAsync(c->d_kr + Nc, sizeof(__nv_bfloat16) * c->ldk, 0, sizeof(__nv_bfloat16) * (c->ldk - Nc),
+                              2 * (size_t)Nc, st);
     }
     const double pref = c->e_k / nkc;
-    dim3 bs(16, 16), gs(blocks_for(Nc, 16), blocks_for(Nc, 16));
+    const int kt = blocks_for(nkc, kc_points(nv * nc));
+    const dim3 gs(kt, kt);
+    const size_t ksm = kc_smem(nv, nc);
+    auto build = [&](auto kernel, void* out, __nv_bfloat16* kr, __nv_bfloat16* ki) -> int {
+        int r = raise_smem(ctx, kernel, ksm);
+        if (r != BSE_OK) return r;
+        kernel<<<gs, 256, ksm, st>>>(d_M, c->d_Uv, c->d_Uc, d_h, n, nv, nc, pref, 1.0 / c->eps_inf, c->exchange_on, Nc, c->ldk,
+                                     out, kr, ki);
+        return BSE_OK;
+    };
     if (user_kc) {
         const long long ne = (long long)Nc * Nc;
         const double2* u = static_cast<const double2*>(user_kc);
@@ -482,15 +556,13 @@ int bse_setup_coarse_device(bse_ctx* ctx, bse_coarse* c, const void* user_kc) {
             k_kc_from_user<BSE_PREC_F32><<<blocks_for(ne, 256), 256, 0, st>>>(u, Nc, c->ldk, c->d_kc, nullptr, nullptr);
         else
             k_kc_from_user<BSE_PREC_BF16><<<blocks_for(ne, 256), 256, 0, st>>>(u, Nc, c->ldk, nullptr, c->d_kr, c->d_ki);
-    } else if (c->kc_prec == BSE_PREC_F64)
-        k_build_kc<BSE_PREC_F64><<<gs, bs, 0, st>>>(d_M, c->d_Uv, c->d_Uc, d_h, n, nv, nc, pref, 1.0 / c->eps_inf,
-                                                   c->exchange_on, Nc, c->ldk, c->d_kc, nullptr, nullptr);
-    else if (c->kc_prec == BSE_PREC_F32)
-        k_build_kc<BSE_PREC_F32><<<gs, bs, 0, st>>>(d_M, c->d_Uv, c->d_Uc, d_h, n, nv, nc, pref, 1.0 / c->eps_inf,
-                                                   c->exchange_on, Nc, c->ldk, c->d_kc, nullptr, nullptr);
-    else
-        k_build_kc<BSE_PREC_BF16><<<gs, bs, 0, st>>>(d_M, c->d_Uv, c->d_Uc, d_h, n, nv, nc, pref, 1.0 / c->eps_inf,
-                                                    c->exchange_on, Nc, c->ldk, nullptr, c->d_kr, c->d_ki);
+    } else if (c->kc_prec == BSE_PREC_F64) {
+        rc = build(k_build_kc<BSE_PREC_F64>, c->d_kc, nullptr, nullptr);
+    } else if (c->kc_prec == BSE_PREC_F32) {
+        rc = build(k_build_kc<BSE_PREC_F32>, c->d_kc, nullptr, nullptr);
+    } else {
+        rc = build(k_build_kc<BSE_PREC_BF16>, nullptr, c->d_kr, c->d_ki);
+    }
     cudaError_t e = cudaGetLastError();
     cudaError_t e2 = cudaStreamSynchronize(st);
     cudaFree(d_M);
@@ -499,7 +571,7 @@ int bse_setup_coarse_device(bse_ctx* ctx, bse_coarse* c, const void* user_kc) {
         ctx->err = std::string("coarse set-up kernels: ") + cudaGetErrorString(e != cudaSuccess ? e : e2);
         return BSE_ERR_CUDA;
     }
-    return BSE_OK;
+    return rc;
 }
 
 namespace {
@@ -582,8 +654,8 @@ int build_m2(bse_ctx* ctx, bse_interp* s) {
     cudaMemsetAsync(F, 0, sizeof(double2) * (size_t)N * Nc, st);
     k_m2_F<<<blocks_for(N, 128), 128, 0, st>>>((const double2*)s->d_Dv, (const double2*)s->d_Dc, s->n, s->nd, s->nv,
                                                s->nc, s->nb1, N, Nc, F);
-    k_shape_table<<<blocks_for(c->nkc, 128), 128, 0, st>>>(s->n, c->kappa, 27, 0, 0.0, 1, hh);
-    k_shape_table<<<blocks_for((long long)L * L * L, 128), 128, 0, st>>>(L, c->kappa, 27, 0, 0.0, 1, hd);
+    k_shape_table<<<blocks_for(c->nkc, 4), 128, 0, st>>>(s->n, c->kappa, 27, 0, 0.0, 1, hh);
+    k_shape_table<<<blocks_for((long long)L * L * L, 4), 128, 0, st>>>(L, c->kappa, 27, 0, 0.0, 1, hd);
     k_m2_heads<<<blocks_for((long long)Nc * Nc, 256), 256, 0, st>>>(c->d_Uv, c->d_Uc, hh, (const double2*)c->d_kc, s->n,
                                                                    s->nv, s->nc, c->alpha, Nc, A, Km);
     const dim3 b16(16, 16);
@@ -639,40 +711,36 @@ int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dens
     const bse_coarse* c = s->co;
     const int n = s->n, nd = s->nd, nk = s->nk, nv = s->nv, nc = s->nc, t = s->t, N = s->N;
     cudaStream_t st = ctx->stream;
+    // Overlaps that are products through one unitary gauge: the common-basis path
+    // (Method 2 stores its H instead) reads U(k); the others the overlaps.
+    s->common = s->scheme != BSE_SCHEME_M2 && c->unitary && !(dense && (dense->Dv || dense->Dc));
     // dense tables
-    double2 *d_Uvd = nullptr, *d_Ucd = nullptr;
-    TRY(bse_alloc(ctx, (void**)&d_Uvd, sizeof(double2) * (size_t)nk * nv * nv, "dense Uv"));
-    TRY(bse_alloc(ctx, (void**)&d_Ucd, sizeof(double2) * (size_t)nk * nc * nc, "dense Uc"));
     TRY(bse_alloc(ctx, &s->d_dE, sizeof(T) * (size_t)N, "dE"));
-    TRY(bse_alloc(ctx, &s->d_Dv, sizeof(V) * (size_t)nk * 8 * nv * nv, "Dv"));
-    TRY(bse_alloc(ctx, &s->d_Dc, sizeof(V) * (size_t)nk * 8 * nc * nc, "Dc"));
     TRY(bse_alloc(ctx, (void**)&s->d_P, sizeof(double2) * 3 * (size_t)N, "dipoles"));
-    k_gauge<<<blocks_for(nk, 64), 64, 0, st>>>(c->d_gen_v, nv, n, nd, nk, d_Uvd);
-    k_gauge<<<blocks_for(nk, 64), 64, 0, st>>>(c->d_gen_c, nc, n, nd, nk, d_Ucd);
-    k_dense_tables<T><<<blocks_for(nk, 64), 64, 0, st>>>(d_Uvd, d_Ucd, c->d_Uv, c->d_Uc, c->d_offsets, c->d_dip, n,
-                                                        nd, nv, nc, c->e_gap, c->band_width, (T*)s->d_dE,
-                                                        (V*)s->d_Dv, (V*)s->d_Dc, s->d_P);
+    if (s->common) {
+        TRY(bse_alloc(ctx, &s->d_cUv, sizeof(V) * (size_t)nk * nv * nv, "dense gauge"));
+        TRY(bse_alloc(ctx, &s->d_cUc, sizeof(V) * (size_t)nk * nc * nc, "dense gauge"));
+    } else {
+        TRY(bse_alloc(ctx, &s->d_Dv, sizeof(V) * (size_t)nk * 8 * nv * nv, "Dv"));
+        TRY(bse_alloc(ctx, &s->d_Dc, sizeof(V) * (size_t)nk * 8 * nc * nc, "Dc"));
+    }
+    const size_t dsm = dense_smem(nv, nc);
+    TRY(raise_smem(ctx, k_dense_tables<T>, dsm));
+    k_dense_tables<T><<<std::min(blocks_for(nk, kDenseWarps), 16 * std::max(ctx->sm_count, 1)), 32 * kDenseWarps, dsm, st>>>(
+        c->d_gen_v, c->d_gen_c, c->d_Uv, c->d_Uc, c->d_offsets, c->d_dip, n, nd, nv, nc, c->e_gap, c->band_width, (T*)s->d_dE,
+        (V*)s->d_Dv, (V*)s->d_Dc, (V*)s->d_cUv, (V*)s->d_cUc, s->d_P);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
-        cudaFree(d_Uvd);
-        cudaFree(d_Ucd);
         ctx->err = std::string("dense set-up kernels: ") + cudaGetErrorString(e);
         return BSE_ERR_CUDA;
     }
-    // Overlaps that are products through one unitary gauge: the common-basis path
-    // (Method 2 stores its H instead).
-    s->common = s->scheme != BSE_SCHEME_M2 && c->unitary && !(dense && (dense->Dv || dense->Dc));
-    int crc = BSE_OK;
     if (s->common && s->scheme == BSE_SCHEME_M3) {
-        crc = near_geometry(ctx, s, nullptr);
-        if (crc == BSE_OK) crc = bse_alloc(ctx, (void**)&s->d_chead, sizeof(double) * c->nkc, "coarse head table");
-        if (crc == BSE_OK) k_shape_table<<<blocks_for(c->nkc, 128), 128, 0, st>>>(n, c->kappa, 27, 0, 0.0, 1, s->d_chead);
+        TRY(near_geometry(ctx, s, nullptr));
+        TRY(bse_alloc(ctx, (void**)&s->d_chead, sizeof(double) * c->nkc, "coarse head table"));
+        k_shape_table<<<blocks_for(c->nkc, 4), 128, 0, st>>>(n, c->kappa, 27, 0, 0.0, 1, s->d_chead);
     }
-    if (s->common && crc == BSE_OK) crc = bse_common_prepare(ctx, s, d_Uvd, d_Ucd);
-    cudaFree(d_Uvd);
-    cudaFree(d_Ucd);
-    if (crc != BSE_OK) return crc;
+    if (s->common) TRY(bse_common_prepare(ctx, s));
     s->dbound = std::sqrt((double)nv) * std::sqrt((double)nc);
     if (dense) TRY(apply_dense_inputs<T>(ctx, s, dense));
     // scratch
@@ -777,7 +845,7 @@ int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dens
         TRY(bse_alloc(ctx, &s->d_Hc, sizeof(V) * (size_t)c->nkc * s->nrel * nc * nc, "Hc"));
         TRY(bse_alloc(ctx, &s->d_hc, sizeof(T) * s->nrel, "hc"));
         k_near_head<T><<<blocks_for(s->n_near, 128), 128, 0, st>>>(d_offs, s->n_near, n * nd, c->kappa, (T*)s->d_hd);
-        k_shape_table<<<blocks_for(c->nkc, 128), 128, 0, st>>>(n, c->kappa, 27, 0, 0.0, 1, d_hh);
+        k_shape_table<<<blocks_for(c->nkc, 4), 128, 0, st>>>(n, c->kappa, 27, 0, 0.0, 1, d_hh);
         k_heads<T><<<blocks_for((long long)c->nkc * s->nrel, 64), 64, 0, st>>>(
             c->d_Uv, c->d_Uc, d_hh, n, nv, nc, s->rmin, s->nr1, c->alpha, (V*)s->d_Hv, (V*)s->d_Hc, (T*)s->d_hc);
         e = cudaGetLastError();
