@@ -518,37 +518,104 @@ __global__ void __launch_bounds__(256) k_prolong_st(
     if (tid < nchains * 64 && (tid & 63) == 0) part[(size_t)(tid >> 6) * BSE_MAX_VEC_BLOCKS + blockIdx.x] = dred[tid];
 }
 
+// acc += a b with fused multiply-adds (four per complex product: FP64 bounds these kernels)
+template <typename V>
+__device__ __forceinline__ void cfma(V& acc, V a, V b) {
+    acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
+    acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
+}
+
+// RW consecutive rows (pitch n) of a dense matrix times the chains' vectors, by one
+// warp, summed over the lanes; kUnroll column steps in flight.  Rows share the
+// loads of the vectors, which come from L2: they are NCH times the matrix's bytes per row.
+template <int RW, int NCH, typename V>
+__device__ __forceinline__ void rows_times(const V* __restrict__ row, const V* __restrict__ x, int n, int lane, V (&acc)[RW][NCH]) {
+    constexpr int kUnroll = RW == 1 ? 4 : 2;
+    auto step = [&](int j, auto count) {
+        constexpr int C = decltype(count)::value;
+        V k[C][RW];
+#pragma unroll
+        for (int u = 0; u < C; ++u)
+#pragma unroll
+            for (int r = 0; r < RW; ++r) k[u][r] = row[(size_t)r * n + j + 32 * u];
+#pragma unroll
+        for (int u = 0; u < C; ++u)
+#pragma unroll
+            for (int ch = 0; ch < NCH; ++ch) {
+                const V v = x[(size_t)ch * n + j + 32 * u];
+#pragma unroll
+                for (int r = 0; r < RW; ++r) cfma(acc[r][ch], k[u][r], v);
+            }
+    };
+    int j = lane;
+    for (; j + 32 * (kUnroll - 1) < n; j += 32 * kUnroll) step(j, std::integral_constant<int, kUnroll>{});
+    for (; j < n; j += 32) step(j, std::integral_constant<int, 1>{});
+#pragma unroll
+    for (int r = 0; r < RW; ++r)
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch)
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                acc[r][ch].x += __shfl_xor_sync(0xffffffffu, acc[r][ch].x, off);
+                acc[r][ch].y += __shfl_xor_sync(0xffffffffu, acc[r][ch].y, off);
+            }
+}
+
 // ------------------------------------------------- K_c apply on CUDA cores
-// R[ch][i] = sum_j K[i][j] Q[ch][j]; one warp per row, fixed-order shuffle
+// R[ch][i] = sum_j K[i][j] Q[ch][j]; one warp per RW rows, fixed-order shuffle
 // reduction.  Used for complex128 and complex64 storage.
-template <typename T>
+template <typename T, int RW, int NCH>
 __global__ void __launch_bounds__(256) k_kc_apply_simt(const typename Cx<T>::V* __restrict__ K,
                                                       const typename Cx<T>::V* __restrict__ Q, int Nc,
-                                                      int nchains, typename Cx<T>::V* __restrict__ R) {
+                                                      typename Cx<T>::V* __restrict__ R) {
     using V = typename Cx<T>::V;
-    const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
+    const int row = (blockIdx.x * 8 + (threadIdx.x >> 5)) * RW, lane = threadIdx.x & 31;
     if (row >= Nc) return;
-    V acc[BSE_MAX_CHAINS];
+    auto go = [&](auto rows) {
+        constexpr int W = decltype(rows)::value;
+        V acc[W][NCH];
 #pragma unroll
-    for (int ch = 0; ch < BSE_MAX_CHAINS; ++ch) acc[ch] = czero<V>();
-    const V* kr = K + (size_t)row * Nc;
-    for (int j = lane; j < Nc; j += 32) {
-        const V k = kr[j];
+        for (int r = 0; r < W; ++r)
 #pragma unroll
-        for (int ch = 0; ch < BSE_MAX_CHAINS; ++ch)
-            if (ch < nchains) acc[ch] = cadd(acc[ch], cmul(k, Q[(size_t)ch * Nc + j]));
-    }
+            for (int ch = 0; ch < NCH; ++ch) acc[r][ch] = czero<V>();
+        rows_times<W, NCH>(K + (size_t)row * Nc, Q, Nc, lane, acc);
+        if (lane == 0)
 #pragma unroll
-    for (int ch = 0; ch < BSE_MAX_CHAINS; ++ch) {
-        if (ch >= nchains) break;
-        V v = acc[ch];
-        for (int off = 16; off > 0; off >>= 1) {
-            v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
-            v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
+            for (int r = 0; r < W; ++r)
+#pragma unroll
+                for (int ch = 0; ch < NCH; ++ch) R[(size_t)ch * Nc + row + r] = acc[r][ch];
+        return;
+    };
+    if (RW == 1 || row + RW <= Nc) go(std::integral_constant<int, RW>{});
+    else
+        for (int r = row; r < Nc; ++r) {                         // the last, partial group row by row
+            V acc[1][NCH];
+#pragma unroll
+            for (int ch = 0; ch < NCH; ++ch) acc[0][ch] = czero<V>();
+            rows_times<1, NCH>(K + (size_t)r * Nc, Q, Nc, lane, acc);
+            if (lane == 0)
+#pragma unroll
+                for (int ch = 0; ch < NCH; ++ch) R[(size_t)ch * Nc + r] = acc[0][ch];
         }
-        if (lane == 0) R[(size_t)ch * Nc + row] = v;
-    }
+}
+
+template <typename T>
+void launch_kc_simt(const bse_ctx* ctx, const bse_coarse* c, const void* Q, int nchains, void* R, cudaStream_t st) {
+    using V = typename Cx<T>::V;
+    const V *k = (const V*)c->d_kc, *q = (const V*)Q;
+    // several rows per warp once that still leaves 16 warps per SM
+    constexpr int RW = sizeof(T) == 4 ? 4 : 2;
+    auto go = [&](auto chains) {
+        constexpr int NCH = decltype(chains)::value;
+        if ((c->Nc + RW - 1) / RW >= 16 * std::max(ctx->sm_count, 1))
+            k_kc_apply_simt<T, RW, NCH><<<(c->Nc + 8 * RW - 1) / (8 * RW), 256, 0, st>>>(k, q, c->Nc, (V*)R);
+        else
+            k_kc_apply_simt<T, 1, NCH><<<(c->Nc + 7) / 8, 256, 0, st>>>(k, q, c->Nc, (V*)R);
+    };
+    if (nchains == 1) go(std::integral_constant<int, 1>{});
+    else if (nchains == 2) go(std::integral_constant<int, 2>{});
+    else if (nchains == 3) go(std::integral_constant<int, 3>{});
+    else go(std::integral_constant<int, 4>{});
 }
 
 // ---------------------------------------------------------------- near field
@@ -1448,43 +1515,31 @@ __global__ void k_cont_frac(const double* __restrict__ a, const double* __restri
 // one warp per row (grid-stride over rows), every chain per row; block
 // partials of <psi, w> for the Lanczos a_i.
 constexpr int kM2Warps = 8;
+template <int NCH>
 __global__ void __launch_bounds__(32 * kM2Warps) k_m2_apply(const double2* __restrict__ H, const double2* __restrict__ psi,
-                                                            int N, int nchains, double2* __restrict__ w,
-                                                            double2* __restrict__ part) {
-    __shared__ double2 red[BSE_MAX_CHAINS][kM2Warps];
+                                                            int N, double2* __restrict__ w, double2* __restrict__ part) {
+    __shared__ double2 red[NCH][kM2Warps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double2 dot[BSE_MAX_CHAINS];
+    double2 dot[NCH];
 #pragma unroll
-    for (int ch = 0; ch < BSE_MAX_CHAINS; ++ch) dot[ch] = make_double2(0.0, 0.0);
+    for (int ch = 0; ch < NCH; ++ch) dot[ch] = make_double2(0.0, 0.0);
     for (int r = blockIdx.x * kM2Warps + warp; r < N; r += gridDim.x * kM2Warps) {
-        double2 acc[BSE_MAX_CHAINS];
+        double2 acc[1][NCH];
 #pragma unroll
-        for (int ch = 0; ch < BSE_MAX_CHAINS; ++ch) acc[ch] = make_double2(0.0, 0.0);
-        const double2* hr = H + (size_t)r * N;
-        for (int j = lane; j < N; j += 32) {
-            const double2 h = hr[j];
+        for (int ch = 0; ch < NCH; ++ch) acc[0][ch] = make_double2(0.0, 0.0);
+        rows_times<1, NCH>(H + (size_t)r * N, psi, N, lane, acc);
+        if (lane == 0)
 #pragma unroll
-            for (int ch = 0; ch < BSE_MAX_CHAINS; ++ch)
-                if (ch < nchains) acc[ch] = cadd(acc[ch], cmul(h, psi[(size_t)ch * N + j]));
-        }
-#pragma unroll
-        for (int ch = 0; ch < BSE_MAX_CHAINS; ++ch) {
-            if (ch >= nchains) break;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                acc[ch].x += __shfl_xor_sync(0xffffffffu, acc[ch].x, o);
-                acc[ch].y += __shfl_xor_sync(0xffffffffu, acc[ch].y, o);
+            for (int ch = 0; ch < NCH; ++ch) {
+                w[(size_t)ch * N + r] = acc[0][ch];
+                dot[ch] = cadd(dot[ch], cmulc(psi[(size_t)ch * N + r], acc[0][ch]));
             }
-            if (lane == 0) {
-                w[(size_t)ch * N + r] = acc[ch];
-                dot[ch] = cadd(dot[ch], cmulc(psi[(size_t)ch * N + r], acc[ch]));
-            }
-        }
     }
     if (lane == 0)
-        for (int ch = 0; ch < nchains; ++ch) red[ch][warp] = dot[ch];
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) red[ch][warp] = dot[ch];
     __syncthreads();
-    if (threadIdx.x < nchains) {
+    if (threadIdx.x < NCH) {
         double2 sum = make_double2(0.0, 0.0);
         for (int k = 0; k < kM2Warps; ++k) sum = cadd(sum, red[threadIdx.x][k]);
         part[(size_t)threadIdx.x * BSE_MAX_VEC_BLOCKS + blockIdx.x] = sum;
@@ -1492,6 +1547,15 @@ __global__ void __launch_bounds__(32 * kM2Warps) k_m2_apply(const double2* __res
 }
 
 inline int m2_blocks(int N) { return std::min((N + kM2Warps - 1) / kM2Warps, BSE_MAX_VEC_BLOCKS); }
+
+void launch_m2(const bse_interp* s, int nchains, const double2* psi, double2* w, double2* dot, cudaStream_t st) {
+    const double2* H = (const double2*)s->d_H2;
+    const int g = m2_blocks(s->N), b = 32 * kM2Warps;
+    if (nchains == 1) k_m2_apply<1><<<g, b, 0, st>>>(H, psi, s->N, w, dot);
+    else if (nchains == 2) k_m2_apply<2><<<g, b, 0, st>>>(H, psi, s->N, w, dot);
+    else if (nchains == 3) k_m2_apply<3><<<g, b, 0, st>>>(H, psi, s->N, w, dot);
+    else k_m2_apply<4><<<g, b, 0, st>>>(H, psi, s->N, w, dot);
+}
 
 inline int vec_blocks(long long N) {
     long long b = (N + BSE_VEC_THREADS - 1) / BSE_VEC_THREADS;
@@ -1537,17 +1601,27 @@ __global__ void __launch_bounds__(256) k_pieces_to_half(const float2* __restrict
     }
 }
 
+// ||psi||^2 per chain, FP64 block partials (grid: blocks, chains).
+__global__ void __launch_bounds__(256) k_chain_norm2(const float2* __restrict__ psi, int N, double* __restrict__ part) {
+    __shared__ double2 sh[256];
+    const int ch = blockIdx.y;
+    double s = 0.0;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < N; i += gridDim.x * 256) {
+        const float2 v = psi[(size_t)ch * N + i];
+        s += (double)v.x * v.x + (double)v.y * v.y;
+    }
+    const double2 r = block_sum2(make_double2(s, 0.0), sh);
+    if (threadIdx.x == 0) part[(size_t)ch * BSE_MAX_VEC_BLOCKS + blockIdx.x] = r.x;
+}
+
 // FP16 piece scale per chain from the input's 2-norm (bse_near_tc_xscale on
 // the device): the largest power of two with scale dbound ||psi|| <= 2^15.
-__global__ void __launch_bounds__(256) k_chain_xscale(const float2* __restrict__ psi, int N, double dbound,
+__global__ void __launch_bounds__(256) k_chain_xscale(const double* __restrict__ part, int nblk, double dbound,
                                                       float* __restrict__ xscale) {
     __shared__ double2 sh[256];
     const int ch = blockIdx.x;
     double s = 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const float2 v = psi[(size_t)ch * N + i];
-        s += (double)v.x * v.x + (double)v.y * v.y;
-    }
+    for (int i = threadIdx.x; i < nblk; i += 256) s += part[(size_t)ch * BSE_MAX_VEC_BLOCKS + i];
     const double2 r = block_sum2(make_double2(s, 0.0), sh);
     if (threadIdx.x == 0) {
         const double b = fmax(dbound * fmax(sqrt(r.x), 1e-300), 1e-300);
@@ -1555,6 +1629,14 @@ __global__ void __launch_bounds__(256) k_chain_xscale(const float2* __restrict__
         frexp(32768.0 / b, &e);
         xscale[ch] = (float)ldexp(1.0, e - 1);
     }
+}
+
+// The scales of nchains inputs into s->d_xscale_gen.  One block per chain read the
+// whole vector (346 us for 221184 entries of 3 chains); two blocks per SM take 4 us.
+void launch_xscale(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi) {
+    const int nb = std::min({(s->N + 255) / 256, 2 * std::max(ctx->sm_count, 1), BSE_MAX_VEC_BLOCKS});
+    k_chain_norm2<<<dim3(nb, nchains), 256, 0, ctx->stream>>>((const float2*)psi, s->N, s->d_part_nrm);
+    k_chain_xscale<<<nchains, 256, 0, ctx->stream>>>(s->d_part_nrm, nb, s->dbound, s->d_xscale_gen);
 }
 
 // Restrict: staged FP32 kernel for 3x3, 4x4 and 4x6 bands (N_div <= 64), generic otherwise.
@@ -1710,7 +1792,7 @@ int apply_h_common(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi, vo
         if (c->kc_prec == BSE_PREC_BF16) {
             if ((rc = bse_tc_apply(ctx, s, nchains, kst, false, 0)) != BSE_OK) return rc;
         } else {
-            k_kc_apply_simt<T><<<(c->Nc + 7) / 8, 256, 0, kst>>>((const V*)c->d_kc, (const V*)s->d_Q, c->Nc, nchains, (V*)s->d_R);
+            launch_kc_simt<T>(ctx, c, s->d_Q, nchains, s->d_R, kst);
         }
     }
     if (m3) {
@@ -1744,8 +1826,7 @@ int apply_h_typed(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi_v, v
     if (s->scheme == BSE_SCHEME_M2) {
         if constexpr (std::is_same<T, double>::value) {
             Timer tm(ctx, prof, KC_KCAPPLY);
-            k_m2_apply<<<m2_blocks(s->N), 32 * kM2Warps, 0, st>>>((const double2*)s->d_H2, psi, s->N, nchains, W,
-                                                                 s->d_part_dot);
+            launch_m2(s, nchains, psi, W, s->d_part_dot, st);
         }
         return BSE_OK;
     }
@@ -1754,8 +1835,7 @@ int apply_h_typed(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi_v, v
     const bool xh = near_tc_active(s);
     void* X = m3 ? s->d_X : nullptr;
     const float* xscale = unit ? s->d_xscale : s->d_xscale_gen;
-    if (xh && !unit)
-        k_chain_xscale<<<nchains, 256, 0, st>>>((const float2*)psi, s->N, s->dbound, s->d_xscale_gen);
+    if (xh && !unit) launch_xscale(ctx, s, nchains, psi);
     {
         Timer tm(ctx, prof, KC_RESTRICT);
         launch_restrict<T>(ctx, s, nchains, psi, s->d_Q, s->d_Bop, X, xh, xscale, s->d_U);
@@ -1782,7 +1862,7 @@ int apply_h_typed(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi_v, v
                 int rc = bse_tc_apply(ctx, s, nchains, st, false, 0);
                 if (rc != BSE_OK) return rc;
             } else {
-                k_kc_apply_simt<T><<<(c->Nc + 7) / 8, 256, 0, st>>>((const V*)c->d_kc, (const V*)s->d_Q, c->Nc, nchains, (V*)s->d_R);
+                launch_kc_simt<T>(ctx, c, s->d_Q, nchains, s->d_R, st);
             }
         }
         if (m3) {
@@ -2344,7 +2424,7 @@ int apply_scratch_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const vo
     V* W = (V*)w_v;
     if (s->scheme == BSE_SCHEME_M2) {
         if constexpr (std::is_same<T, double>::value)
-            k_m2_apply<<<m2_blocks(s->N), 32 * kM2Warps, 0, st>>>((const double2*)s->d_H2, psi, s->N, nchains, W, sc.dot);
+            launch_m2(s, nchains, psi, W, sc.dot, st);
         return BSE_OK;
     }
     const bool m3 = s->scheme == BSE_SCHEME_M3;
@@ -2356,14 +2436,14 @@ int apply_scratch_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const vo
             if ((rc = bse_tc_apply_scratch(ctx, s, nchains, sc.bop, sc.part, sc.R)) != BSE_OK) return rc;
         } else {
             if ((rc = bse_common_restrict(ctx, s, nchains, psi, sc.Q, nullptr, st)) != BSE_OK) return rc;
-            k_kc_apply_simt<T><<<(c->Nc + 7) / 8, 256, 0, st>>>((const V*)c->d_kc, (const V*)sc.Q, c->Nc, nchains, (V*)sc.R);
+            launch_kc_simt<T>(ctx, c, sc.Q, nchains, sc.R, st);
         }
         if (m3 && (rc = bse_common_near(ctx, s, nchains, st)) != BSE_OK) return rc;
         return bse_common_prolong(ctx, s, nchains, sc.R, psi, W, sc.dot, st);
     }
     const bool xh = near_tc_active(s);
     void* X = m3 ? sc.X : nullptr;
-    if (xh) k_chain_xscale<<<nchains, 256, 0, st>>>((const float2*)psi, s->N, s->dbound, s->d_xscale_gen);
+    if (xh) launch_xscale(ctx, s, nchains, psi);
     if (c->kc_prec == BSE_PREC_BF16) {
         BSE_CUDA_TRY(ctx, cudaMemsetAsync(sc.bop, 0, sizeof(__nv_bfloat16) * 16 * (size_t)c->ldk, st));
         launch_restrict<T>(ctx, s, nchains, psi, nullptr, sc.bop, X, xh, s->d_xscale_gen, sc.U);
@@ -2371,7 +2451,7 @@ int apply_scratch_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const vo
         if (rc != BSE_OK) return rc;
     } else {
         launch_restrict<T>(ctx, s, nchains, psi, sc.Q, nullptr, X, xh, s->d_xscale_gen, sc.U);
-        k_kc_apply_simt<T><<<(c->Nc + 7) / 8, 256, 0, st>>>((const V*)c->d_kc, (const V*)sc.Q, c->Nc, nchains, (V*)sc.R);
+        launch_kc_simt<T>(ctx, c, sc.Q, nchains, sc.R, st);
     }
     if (m3) {
         int rc = bse_launch_near_field(ctx, s, nchains, X, s->d_xscale_gen, sc.U);

@@ -442,10 +442,28 @@ __device__ __forceinline__ void near_apply(T (&acc)[CZ * TZ], const T (&v)[CZ * 
             }
     }
 }
-template <typename T, int TZ, int CZ, int RM, int r>
-__device__ __forceinline__ void near_load(T (&v)[CZ * TZ + 2 * RM], const T* __restrict__ row) {
+// One source row that reaches rm: its columns into registers, then every target
+// row by its own reach r <= rm (code + 1; 0: not reached).  A body per rm: a row
+// array shared by several bodies cost a register move per element.
+template <typename T, int TY, int TZ, int CZ, int rm>
+__device__ __forceinline__ void near_row(T (&acc)[TY][CZ * TZ], const T* __restrict__ row, const T* wb, int wy, int reach) {
+    T v[CZ * TZ + 2 * rm];
 #pragma unroll
-    for (int z = -r; z < CZ * TZ + r; ++z) v[z + RM] = __ldg(row + z * 32);
+    for (int z = -rm; z < CZ * TZ + rm; ++z) v[z + rm] = __ldg(row + z * 32);
+    cpa_wait<1>();
+    __syncwarp();
+#pragma unroll
+    for (int y = 0; y < TY; ++y) {
+        const T* w = wb + y * wy;
+        const int r = ((reach >> (8 * y)) & 255) - 1;
+        if (r == rm) near_apply<T, TZ, CZ, rm, rm>(acc[y], v, w);
+        if constexpr (rm >= 1) if (r == 0) near_apply<T, TZ, CZ, rm, 0>(acc[y], v, w);
+        if constexpr (rm >= 2) if (r == 1) near_apply<T, TZ, CZ, rm, 1>(acc[y], v, w);
+        if constexpr (rm >= 3) if (r == 2) near_apply<T, TZ, CZ, rm, 2>(acc[y], v, w);
+        if constexpr (rm >= 4) if (r == 3) near_apply<T, TZ, CZ, rm, 3>(acc[y], v, w);
+        if constexpr (rm >= 5) if (r == 4) near_apply<T, TZ, CZ, rm, 4>(acc[y], v, w);
+        if constexpr (rm >= 6) if (r == 5) near_apply<T, TZ, CZ, rm, 5>(acc[y], v, w);
+    }
 }
 
 template <typename T, int TY, int TZ, int CZ, int RM>
@@ -485,37 +503,17 @@ __device__ __forceinline__ void near_body(const T* __restrict__ phi, const T* __
         const int rm = st.x >> 16;
         const T* wb = wbuf + (i & 1) * s.wrow + R * TZP;
         if constexpr (RM > 0) {
-            T v[CZ * TZ + 2 * RM];
             switch (rm) {
-                case 0: near_load<T, TZ, CZ, RM, 0>(v, row); break;
-                case 1: near_load<T, TZ, CZ, RM, 1>(v, row); break;
-                case 2: near_load<T, TZ, CZ, RM, 2>(v, row); break;
-                case 3: near_load<T, TZ, CZ, RM, 3>(v, row); break;
-                case 4: near_load<T, TZ, CZ, RM, 4>(v, row); break;
+                case 0: near_row<T, TY, TZ, CZ, 0>(acc, row, wb, nzs * TZP, st.y); break;
+                case 1: near_row<T, TY, TZ, CZ, 1>(acc, row, wb, nzs * TZP, st.y); break;
+                case 2: near_row<T, TY, TZ, CZ, 2>(acc, row, wb, nzs * TZP, st.y); break;
+                case 3: near_row<T, TY, TZ, CZ, 3>(acc, row, wb, nzs * TZP, st.y); break;
+                case 4: near_row<T, TY, TZ, CZ, 4>(acc, row, wb, nzs * TZP, st.y); break;
                 default:
                     if constexpr (RM >= 6) {
-                        if (rm == 5) near_load<T, TZ, CZ, RM, 5>(v, row);
-                        else near_load<T, TZ, CZ, RM, 6>(v, row);
+                        if (rm == 5) near_row<T, TY, TZ, CZ, 5>(acc, row, wb, nzs * TZP, st.y);
+                        else near_row<T, TY, TZ, CZ, 6>(acc, row, wb, nzs * TZP, st.y);
                     }
-            }
-            cpa_wait<1>();
-            __syncwarp();
-#pragma unroll
-            for (int y2 = 0; y2 < TY; ++y2) {
-                const T* w = wb + y2 * nzs * TZP;
-                switch ((st.y >> (8 * y2)) & 255) {
-                    case 0: break;
-                    case 1: near_apply<T, TZ, CZ, RM, 0>(acc[y2], v, w); break;
-                    case 2: near_apply<T, TZ, CZ, RM, 1>(acc[y2], v, w); break;
-                    case 3: near_apply<T, TZ, CZ, RM, 2>(acc[y2], v, w); break;
-                    case 4: near_apply<T, TZ, CZ, RM, 3>(acc[y2], v, w); break;
-                    case 5: near_apply<T, TZ, CZ, RM, 4>(acc[y2], v, w); break;
-                    default:
-                        if constexpr (RM >= 6) {
-                            if (((st.y >> (8 * y2)) & 255) == 6) near_apply<T, TZ, CZ, RM, 5>(acc[y2], v, w);
-                            else near_apply<T, TZ, CZ, RM, 6>(acc[y2], v, w);
-                        }
-                }
             }
         } else {
             cpa_wait<1>();
