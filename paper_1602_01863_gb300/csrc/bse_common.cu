@@ -23,6 +23,7 @@
 // generators keep the general kernels of bse_apply.cu and bse_near_tc.cu.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "bse_internal.cuh"
 
@@ -92,15 +93,43 @@ __device__ __forceinline__ void rot_col(V* x, int st, const V* U) {
     }
 }
 
-// Rotation of `np` blocks x [np][tp] (t = nv nc entries each) in shared memory
-// by Uv [np][rvp], Uc [np][rcp]; block-wide, ends with a barrier.  One thread
-// per row, then one per column: 1 shared load per complex multiply-add, rows
-// padded to an odd number of entries so that a warp's rows spread over the banks.
+// Rotation by one warp of `np` blocks x [np][tp] (t = nv nc entries each) in shared
+// memory by Uv [np][rvp], Uc [np][rcp]; ends with __syncwarp.  FP32: a lane per row,
+// then per column, in place: 1 shared load per complex multiply-add, rows padded
+// to an odd number of entries so that they spread over the banks.  FP64 with few
+// rows, where the chain of multiply-adds of a lane counts, not the loads: a lane per
+// entry, through tmp [np][tp].
 template <bool TO, typename V>
-__device__ __forceinline__ void rotate_blocks(V* x, int tp, const V* Uv, int rvp, const V* Uc, int rcp, int np, int nv,
-                                              int nc) {
+__device__ __forceinline__ void rotate_warp(V* x, V* tmp, int tp, const V* Uv, int rvp, const V* Uc, int rcp, int np, int nv,
+                                            int nc) {
+    const int lane = threadIdx.x & 31;
     const float inv_v = 1.f / (float)nv, inv_c = 1.f / (float)nc;
-    for (int i = threadIdx.x; i < np * nv; i += blockDim.x) {
+    if (sizeof(V) == 16 && np * nv <= 16) {
+        const int t = nv * nc;
+        const float inv_t = 1.f / (float)t;
+        for (int i = lane; i < np * t; i += 32) {
+            const int p = quot(i, inv_t), e = i - p * t, r = quot(e, inv_c), j = e - r * nc;
+            const V *in = x + p * tp + r * nc, *U = Uc + p * rcp + (TO ? j * nc : j);
+            V a = czero<V>();
+            for (int q = 0; q < nc; ++q) {
+                if (TO) cfma(a, in[q], U[q]);
+                else cfmac(a, in[q], U[q * nc]);
+            }
+            tmp[p * tp + e] = a;
+        }
+        __syncwarp();
+        for (int i = lane; i < np * t; i += 32) {
+            const int p = quot(i, inv_t), e = i - p * t, r = quot(e, inv_c), j = e - r * nc;
+            const V *in = tmp + p * tp + j, *U = Uv + p * rvp + (TO ? r * nv : r);
+            V a = czero<V>();
+            for (int q = 0; q < nv; ++q) {
+                if (TO) cfmac(a, in[q * nc], U[q]);
+                else cfma(a, in[q * nc], U[q * nv]);
+            }
+            x[p * tp + e] = a;
+        }
+    } else {
+    for (int i = lane; i < np * nv; i += 32) {
         const int p = quot(i, inv_v), v = i - p * nv;
         V* r = x + p * tp + v * nc;
         const V* U = Uc + p * rcp;
@@ -115,8 +144,8 @@ __device__ __forceinline__ void rotate_blocks(V* x, int tp, const V* Uv, int rvp
             default: rot_row<TO, 8>(r, U); break;
         }
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < np * nc; i += blockDim.x) {
+    __syncwarp();
+    for (int i = lane; i < np * nc; i += 32) {
         const int p = quot(i, inv_c), c = i - p * nc;
         V* r = x + p * tp + c;
         const V* U = Uv + p * rvp;
@@ -131,18 +160,41 @@ __device__ __forceinline__ void rotate_blocks(V* x, int tp, const V* Uv, int rvp
             default: rot_col<TO, 8>(r, nc, U); break;
         }
     }
-    __syncthreads();
+    }
+    __syncwarp();
 }
 
-// Rows of `len` entries from global src (row r at src + r * len) into shared dst (row pitch `pitch`).
+// Rows of `len` entries from global src (row r at src + r * len) into shared dst (row pitch `pitch`), by one warp.
 template <typename V>
 __device__ __forceinline__ void load_rows(V* dst, int pitch, const V* __restrict__ src, int rows, int len) {
     const float inv = 1.f / (float)len;
-    for (int i = threadIdx.x; i < rows * len; i += blockDim.x) {
+#pragma unroll 4
+    for (int i = threadIdx.x & 31; i < rows * len; i += 32) {
         const int r = quot(i, inv);
         dst[r * pitch + (i - r * len)] = src[i];
     }
 }
+
+// Shared memory of a warp that rotates up to KP points: entries, gauge, weights, places.
+template <typename T>
+struct WarpStage {
+    using V = typename Cx<T>::V;
+    V *X, *Tm, *Uv, *Uc;
+    T* wt;         // [KP][8]
+    int2* pnt;     // [KP]
+    static __host__ __device__ size_t bytes(int KP, int nv, int nc) {
+        const size_t v = (size_t)(sizeof(T) == 8 ? 2 : 1) * odd(nv * nc) + odd(nv * nv) + odd(nc * nc);
+        return (KP * (v * sizeof(V) + 8 * sizeof(T) + sizeof(int2)) + 15) / 16 * 16;
+    }
+    __device__ WarpStage(unsigned char* p, int KP, int nv, int nc) {
+        X = reinterpret_cast<V*>(p);
+        Tm = X + KP * odd(nv * nc);
+        Uv = sizeof(T) == 8 ? Tm + KP * odd(nv * nc) : Tm;
+        Uc = Uv + KP * odd(nv * nv);
+        wt = reinterpret_cast<T*>(Uc + KP * odd(nc * nc));
+        pnt = reinterpret_cast<int2*>(wt + KP * 8);
+    }
+};
 
 // Weight of corner l at sub-cell position (j1, j2, j3) (interp_weight).
 template <typename T>
@@ -153,126 +205,149 @@ __device__ __forceinline__ T corner_weight(int j1, int j2, int j3, int l, int nd
 }
 
 // ------------------------------------------------------- rotate and restrict
-// Grid (coarse cell, chain).  The cell's points go through in chunks of KP:
-// psi and the gauge matrices are staged in shared memory, rotated, written to
-// the near field's phi (layout of CommonPhi) and summed with the trilinear
-// weights into the cell's share of its eight corners.  The block whose share of
-// a coarse point is the last of eight (a counter per point and chain, reset
-// there) adds the eight in corner order, rotates the sum back and writes Q: the
-// order does not depend on the blocks' order.
-template <typename T, bool OUT_BF16>
-__global__ void __launch_bounds__(256) k_common_restrict(
+// Grid (coarse cell, group of CPB chains), 8 warps.  A warp takes KP points of the
+// cell at a time: the gauge matrices and weights into its own shared memory and,
+// chain by chain, psi, the rotation, phi for the near stencil (layout of
+// CommonPhi), and the points' weighted sums for the cell's eight corners in
+// registers (lane = transition, EPL of them); the warps' sums add up to the cell's
+// share of each corner.  The block whose share of a coarse point is the last of
+// eight (a counter per point, reset there) adds the eight in corner order, rotates
+// the sum back and writes Q, a warp per point: the order does not depend on the
+// blocks' order.  Memory latency and instruction issue bound it (it reads psi and U
+// and writes phi: 33 MB for coarse 8^3, n_div 4, 4x4 bands, 3 chains), so the warps of a
+// block wait for one another only at the sums and the chains share what they can.
+template <typename T, bool OUT_BF16, int EPL>
+__global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) k_common_restrict(
     const typename Cx<T>::V* __restrict__ psi, const typename Cx<T>::V* __restrict__ Uvd,
     const typename Cx<T>::V* __restrict__ Ucd, const typename Cx<T>::V* __restrict__ Uvc,
-    const typename Cx<T>::V* __restrict__ Ucc, int n, int nd, int nv, int nc, int nb1, int KP,
+    const typename Cx<T>::V* __restrict__ Ucc, int n, int nd, int nv, int nc, int nb1, int nch, int CPB, int KP,
     T* __restrict__ phi, CommonPhi lay, typename Cx<T>::V* __restrict__ share, int* __restrict__ ctr,
     typename Cx<T>::V* __restrict__ Q, __nv_bfloat16* __restrict__ Bop, int ldk) {
     using V = typename Cx<T>::V;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int last_sh[8];
     const int t = nv * nc, tp = odd(t), rv = nv * nv, rc = nc * nc, rvp = odd(rv), rcp = odd(rc);
-    const int Ndiv = nd * nd * nd, nkc = n * n * n, nch = gridDim.y;
-    const int ic = blockIdx.x, ch = blockIdx.y, tid = threadIdx.x;
+    const int Ndiv = nd * nd * nd, nkc = n * n * n;
+    const int ic = blockIdx.x, c0 = blockIdx.y * CPB, c1 = min(nch, c0 + CPB), tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const Int3 ci = unflat3(ic, n);
-    V* X = reinterpret_cast<V*>(smraw);                 // [KP][tp]
-    V* sUv = X + KP * tp;                               // [KP][rvp]
-    V* sUc = sUv + KP * rvp;                            // [KP][rcp]
-    V* red = sUc + KP * rcp;                            // [256]
-    T* wt = reinterpret_cast<T*>(red + 256);            // [KP][8]
-    int2* pnt = reinterpret_cast<int2*>(wt + KP * 8);   // [KP] the point's place in phi and its halo copy's distance
-    const int L = n * nd, t2 = 2 * t;
-    const float inv_t = 1.f / (float)t, inv_nd = 1.f / (float)nd;
-    // corner sums: item (l, e); with few items several threads share one over the points
-    const int items = 8 * t, nsp = max(1, 256 / items);
-    V acc[2] = {czero<V>(), czero<V>()};
-    for (int k0 = 0; k0 < Ndiv; k0 += KP) {
-        const int np = min(KP, Ndiv - k0);
-        const size_t kd0 = (size_t)ic * Ndiv + k0;
-        load_rows(X, tp, psi + ((size_t)ch * nkc * Ndiv + kd0) * t, np, t);
-        load_rows(sUv, rvp, Uvd + kd0 * rv, np, rv);
-        load_rows(sUc, rcp, Ucd + kd0 * rc, np, rc);
-        for (int i = tid; i < np * 8; i += 256) {
-            const int js = k0 + (i >> 3), a = quot(js, inv_nd), j3 = js - a * nd, j1 = quot(a, inv_nd), j2 = a - j1 * nd;
-            wt[i] = corner_weight<T>(j1, j2, j3, i & 7, nd, nb1);
-            if ((i & 7) == 0) {
-                const int x = ci.a * nd + j1, y = ci.b * nd + j2, z = ci.c * nd + j3;
-                pnt[i >> 3] = make_int2((x * L + y) * lay.Lp + z + lay.R, z < lay.R ? L : (z >= L - lay.R ? -L : 0));
+    const size_t wbytes = WarpStage<T>::bytes(KP, nv, nc);
+    const WarpStage<T> w(smraw + warp * wbytes, KP, nv, nc);
+    V* red = reinterpret_cast<V*>(smraw + 8 * wbytes);            // [8 warps][2 halves when t <= 16][8][t]
+    const int L = n * nd;
+    const float inv_nd = 1.f / (float)nd, inv_t = 1.f / (float)t;
+    // lane -> transitions e = lane (, lane + 32); with t <= 16 the half warps share the points
+    const int sub = t <= 16 ? lane >> 4 : 0, nsub = t <= 16 ? 2 : 1, e0 = t <= 16 ? lane & 15 : lane;
+    const int items = 8 * t, parts = 8 * nsub;
+    const bool once = Ndiv <= 8 * KP;                              // a warp's points fit at once: their gauge is loaded once
+    for (int ch = c0; ch < c1; ++ch) {
+        V acc[EPL][8];
+#pragma unroll
+        for (int a = 0; a < EPL; ++a) {
+#pragma unroll
+            for (int l = 0; l < 8; ++l) acc[a][l] = czero<V>();
+        }
+        for (int k0 = warp * KP; k0 < Ndiv; k0 += 8 * KP) {
+            const int np = min(KP, Ndiv - k0);
+            const size_t kd0 = (size_t)ic * Ndiv + k0;
+            load_rows(w.X, tp, psi + ((size_t)ch * nkc * Ndiv + kd0) * t, np, t);
+            if (ch == c0 || !once) {
+                load_rows(w.Uv, rvp, Uvd + kd0 * rv, np, rv);
+                load_rows(w.Uc, rcp, Ucd + kd0 * rc, np, rc);
+                for (int i = lane; i < np * 8; i += 32) {
+                    const int js = k0 + (i >> 3), a = quot(js, inv_nd), j3 = js - a * nd, j1 = quot(a, inv_nd), j2 = a - j1 * nd;
+                    w.wt[i] = corner_weight<T>(j1, j2, j3, i & 7, nd, nb1);
+                    if ((i & 7) == 0) {
+                        const int x = ci.a * nd + j1, y = ci.b * nd + j2, z = ci.c * nd + j3;
+                        w.pnt[i >> 3] = make_int2((x * L + y) * lay.Lp + z + lay.R, z < lay.R ? L : (z >= L - lay.R ? -L : 0));
+                    }
+                }
+            }
+            __syncwarp();
+            rotate_warp<true>(w.X, w.Tm, tp, w.Uv, rvp, w.Uc, rcp, np, nv, nc);
+            if (phi) {
+                // the 2 t components of a point lie side by side in the columns of its groups
+                const size_t gs = (size_t)L * L * lay.Lp * 32;
+                for (int i = lane; i < np * t; i += 32) {
+                    const int r = quot(i, inv_t), e = i - r * t, col = 2 * (ch * t + e);
+                    const int2 pt = w.pnt[r];
+                    const V v = w.X[r * tp + e];
+                    V* at = reinterpret_cast<V*>(phi + (size_t)(col >> 5) * gs + (size_t)pt.x * 32 + (col & 31));
+                    *at = v;
+                    if (pt.y) at[(ptrdiff_t)pt.y * 16] = v;      // periodic halo copy
+                }
+            }
+            for (int r = sub; r < np; r += nsub) {
+                T f[8];
+#pragma unroll
+                for (int l = 0; l < 8; ++l) f[l] = w.wt[r * 8 + l];
+#pragma unroll
+                for (int a = 0; a < EPL; ++a) {
+                    const int e = e0 + 32 * a;
+                    if (e >= t) continue;
+                    const V v = w.X[r * tp + e];
+#pragma unroll
+                    for (int l = 0; l < 8; ++l) {
+                        if (sizeof(T) == 8 && f[l] == (T)0) continue;
+                        acc[a][l].x = fma(f[l], v.x, acc[a][l].x);
+                        acc[a][l].y = fma(f[l], v.y, acc[a][l].y);
+                    }
+                }
+            }
+            __syncwarp();
+        }
+        // the cell's shares: [chain][cell][corner][t], the warps' sums in order
+#pragma unroll
+        for (int a = 0; a < EPL; ++a) {
+            const int e = e0 + 32 * a;
+            if (e < t) {
+#pragma unroll
+                for (int l = 0; l < 8; ++l) red[(warp * nsub + sub) * items + l * t + e] = acc[a][l];
             }
         }
         __syncthreads();
-        rotate_blocks<true>(X, tp, sUv, rvp, sUc, rcp, np, nv, nc);
-        if (phi) {
-            // the 2 t components of a point lie side by side in the columns of its groups
-            const size_t gs = (size_t)L * L * lay.Lp * 32;
-            const float inv_t2 = 1.f / (float)t2;
-            for (int i = tid; i < np * t2; i += 256) {
-                const int r = quot(i, inv_t2), q = i - r * t2, col = ch * t2 + q;
-                const int2 pt = pnt[r];
-                const T v = reinterpret_cast<const T*>(X + r * tp)[q];
-                T* at = phi + (size_t)(col >> 5) * gs + (size_t)pt.x * 32 + (col & 31);
-                *at = v;
-                if (pt.y) at[(ptrdiff_t)pt.y * 32] = v;
-            }
+        V* mine = share + ((size_t)ch * nkc + ic) * items;
+        for (int i = tid; i < items; i += 256) {
+            V s = red[i];
+            for (int q = 1; q < parts; ++q) s = cadd(s, red[q * items + i]);
+            mine[i] = s;
         }
-        for (int a = 0; a < 2; ++a) {
-            const int i = nsp > 1 ? tid % items : tid + 256 * a, sp = nsp > 1 ? tid / items : 0;
-            if (i >= items || sp >= nsp || (nsp > 1 && a)) continue;
-            const int l = quot(i, inv_t), e = i - l * t;
-            V s = acc[a];
-            for (int r = sp; r < np; r += nsp) {
-                const T f = wt[r * 8 + l];
-                const V v = X[r * tp + e];
-                s.x = fma(f, v.x, s.x);
-                s.y = fma(f, v.y, s.y);
-            }
-            acc[a] = s;
-        }
-        __syncthreads();
-    }
-    // the cell's shares: [chain][cell][corner][t]
-    V* mine = share + ((size_t)ch * nkc + ic) * items;
-    if (nsp > 1) {
-        red[tid] = acc[0];
-        __syncthreads();
-        if (tid < items) {
-            V s = red[tid];
-            for (int q = 1; q < nsp; ++q) s = cadd(s, red[q * items + tid]);
-            mine[tid] = s;
-        }
-    } else {
-        for (int a = 0; a < 2; ++a)
-            if (tid + 256 * a < items) mine[tid + 256 * a] = acc[a];
+        if (ch + 1 < c1) __syncthreads();
     }
     __threadfence();
     __syncthreads();
     if (tid < 8) {
         const int dst = flat3(ci.a + ((tid >> 2) & 1), ci.b + ((tid >> 1) & 1), ci.c + (tid & 1), n);
-        int* c = ctr + (size_t)ch * nkc + dst;
+        int* c = ctr + (size_t)blockIdx.y * nkc + dst;
         const bool last = atomicAdd(c, 1) == 7;
         if (last) *c = 0;
         last_sh[tid] = last ? dst : -1;
         __threadfence();
     }
     __syncthreads();
-    for (int l = 0; l < 8; ++l) {
-        const int dst = last_sh[l];
-        if (dst < 0) continue;
-        const Int3 d = unflat3(dst, n);
-        for (int e = tid; e < t; e += 256) {
-            V s = czero<V>();
+    const int dst = last_sh[warp];
+    if (dst < 0) return;
+    const Int3 d = unflat3(dst, n);
+    load_rows(w.Uv, rvp, Uvc + (size_t)dst * rv, 1, rv);
+    load_rows(w.Uc, rcp, Ucc + (size_t)dst * rc, 1, rc);
+    // lane q < 8 finds the cell whose corner q this point is
+    const int cq = flat3(d.a - ((lane >> 2) & 1), d.b - ((lane >> 1) & 1), d.c - (lane & 1), n);
+    int cell[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int cell = flat3(d.a - ((q >> 2) & 1), d.b - ((q >> 1) & 1), d.c - (q & 1), n);
-                s = cadd(s, __ldcg(share + ((size_t)ch * nkc + cell) * items + q * t + e));
-            }
-            X[e] = s;
+    for (int q = 0; q < 8; ++q) cell[q] = __shfl_sync(0xffffffffu, cq, q);
+    for (int ch = c0; ch < c1; ++ch) {
+        for (int e = lane; e < t; e += 32) {
+            V p[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) p[q] = __ldcg(share + ((size_t)ch * nkc + cell[q]) * items + q * t + e);
+            V s = p[0];
+#pragma unroll
+            for (int q = 1; q < 8; ++q) s = cadd(s, p[q]);
+            w.X[e] = s;
         }
-        for (int i = tid; i < rv; i += 256) sUv[i] = Uvc[(size_t)dst * rv + i];
-        for (int i = tid; i < rc; i += 256) sUc[i] = Ucc[(size_t)dst * rc + i];
-        __syncthreads();
-        rotate_blocks<false>(X, tp, sUv, rvp, sUc, rcp, 1, nv, nc);
-        for (int e = tid; e < t; e += 256) {
-            const V s = X[e];
+        __syncwarp();
+        rotate_warp<false>(w.X, w.Tm, tp, w.Uv, rvp, w.Uc, rcp, 1, nv, nc);
+        for (int e = lane; e < t; e += 32) {
+            const V s = w.X[e];
             const size_t row = (size_t)dst * t + e;
             if (!OUT_BF16) {
                 Q[(size_t)ch * nkc * t + row] = s;
@@ -286,100 +361,151 @@ __global__ void __launch_bounds__(256) k_common_restrict(
                 Bop[(size_t)(3 * nch + ch) * ldk + row] = __float2bfloat16_rn(im - __bfloat162float(ih));
             }
         }
-        __syncthreads();
+        __syncwarp();
     }
 }
 
 // ------------------------------------------------------- prolong and diagonal
-// Grid (coarse cell, grid-strided; chain): w = dE psi + from_common[(1/N_div) sum_l f R'(k~_l) + V],
-// R' = to_common(R) at the cell's eight corners, V the near stencil (its weights
-// carry alpha / N_div); FP64 block partials of <psi, w>.
-template <typename T>
-__global__ void __launch_bounds__(256) k_common_prolong(
+// Grid (coarse cell, grid-strided; group of CPB chains), 8 warps:
+// w = dE psi + from_common[(1/N_div) sum_l f R'(k~_l) + V], R' = to_common(R) at the
+// cell's eight corners (a warp each, the chains as blocks of one gauge), V the near
+// stencil (its weights carry alpha / N_div); then a warp takes KP points at a time
+// by itself, chain by chain, as in k_common_restrict.  FP64 block partials of <psi, w>.
+template <typename T, int EPL>
+__global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) k_common_prolong(
     const typename Cx<T>::V* __restrict__ R, const typename Cx<T>::V* __restrict__ Vn,
     const typename Cx<T>::V* __restrict__ Uvd, const typename Cx<T>::V* __restrict__ Ucd,
     const typename Cx<T>::V* __restrict__ Uvc, const typename Cx<T>::V* __restrict__ Ucc, const T* __restrict__ dE,
-    const typename Cx<T>::V* __restrict__ psi, int n, int nd, int nv, int nc, int nb1, int KP,
+    const typename Cx<T>::V* __restrict__ psi, int n, int nd, int nv, int nc, int nb1, int nch, int CPB, int KP,
     typename Cx<T>::V* __restrict__ W, double2* __restrict__ part) {
     using V = typename Cx<T>::V;
     extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ double2 dred[8];
+    __shared__ V dsum[BSE_MAX_CHAINS][256];                       // <psi, w> per chain and thread: a few products each
     const int t = nv * nc, tp = odd(t), rv = nv * nv, rc = nc * nc, rvp = odd(rv), rcp = odd(rc);
-    const int Ndiv = nd * nd * nd, nkc = n * n * n, ch = blockIdx.y, tid = threadIdx.x;
-    V* X = reinterpret_cast<V*>(smraw);                 // [KP][tp]
-    V* sUv = X + KP * tp;                               // [KP][rvp]
-    V* sUc = sUv + KP * rvp;                            // [KP][rcp]
-    V* Rc = sUc + KP * rcp;                             // [8][tp]
-    V* cUv = Rc + 8 * tp;                               // [8][rvp]
-    V* cUc = cUv + 8 * rvp;                             // [8][rcp]
-    T* wt = reinterpret_cast<T*>(cUc + 8 * rcp);        // [KP][8]
+    const int Ndiv = nd * nd * nd, nkc = n * n * n, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int c0 = blockIdx.y * CPB, c1 = min(nch, c0 + CPB), ncb = c1 - c0;
+    V* Rc = reinterpret_cast<V*>(smraw);                          // [8][CPB][tp], then [8][CPB][tp] scratch (FP64)
+    const size_t rbytes = (sizeof(V) * (sizeof(T) == 8 ? 2 : 1) * 8 * CPB * tp + 15) / 16 * 16;
+    const WarpStage<T> w(smraw + rbytes + warp * WarpStage<T>::bytes(KP, nv, nc), KP, nv, nc);
     const T inv = (T)1 / (T)Ndiv;
     const float inv_t = 1.f / (float)t, inv_nd = 1.f / (float)nd;
-    double2 dot = make_double2(0.0, 0.0);
+    const int sub = t <= 16 ? lane >> 4 : 0, nsub = t <= 16 ? 2 : 1, e0 = t <= 16 ? lane & 15 : lane;
+    const bool once = Ndiv <= 8 * KP;
+    double2 dot = make_double2(0.0, 0.0);                         // warp c < ncb: chain c's sum over the block, in FP64
     for (int cell = blockIdx.x; cell < nkc; cell += gridDim.x) {
         const Int3 ci = unflat3(cell, n);
-        __syncthreads();
-        for (int i = tid; i < 8 * (t + rv + rc); i += 256) {
-            const int l = i & 7, q = i >> 3;
-            const size_t cc = flat3(ci.a + ((l >> 2) & 1), ci.b + ((l >> 1) & 1), ci.c + (l & 1), n);
-            if (q < t) Rc[l * tp + q] = R[((size_t)ch * nkc + cc) * t + q];
-            else if (q < t + rv) cUv[l * rvp + (q - t)] = Uvc[cc * rv + (q - t)];
-            else cUc[l * rcp + (q - t - rv)] = Ucc[cc * rc + (q - t - rv)];
+        if (cell != (int)blockIdx.x) __syncthreads();              // the previous cell's corners are no longer read
+        {
+            const size_t cc = flat3(ci.a + ((warp >> 2) & 1), ci.b + ((warp >> 1) & 1), ci.c + (warp & 1), n);
+            V* mine = Rc + (size_t)warp * CPB * tp;
+            for (int c = 0; c < ncb; ++c) load_rows(mine + c * tp, tp, R + ((size_t)(c0 + c) * nkc + cc) * t, 1, t);
+            load_rows(w.Uv, rvp, Uvc + cc * rv, 1, rv);
+            load_rows(w.Uc, rcp, Ucc + cc * rc, 1, rc);
+            __syncwarp();
+            rotate_warp<true>(mine, mine + 8 * CPB * tp, tp, w.Uv, 0, w.Uc, 0, ncb, nv, nc);
         }
         __syncthreads();
-        rotate_blocks<true>(Rc, tp, cUv, rvp, cUc, rcp, 8, nv, nc);
-        for (int k0 = 0; k0 < Ndiv; k0 += KP) {
-            const int np = min(KP, Ndiv - k0);
-            const size_t kd0 = (size_t)cell * Ndiv + k0, g0 = kd0 * t, o0 = (size_t)ch * nkc * Ndiv * t + g0;
-            load_rows(sUv, rvp, Uvd + kd0 * rv, np, rv);
-            load_rows(sUc, rcp, Ucd + kd0 * rc, np, rc);
-            for (int i = tid; i < np * 8; i += 256) {
-                const int js = k0 + (i >> 3), a = quot(js, inv_nd), j1 = quot(a, inv_nd);
-                wt[i] = corner_weight<T>(j1, a - j1 * nd, js - a * nd, i & 7, nd, nb1) * inv;
-            }
-            __syncthreads();
-            for (int i = tid; i < np * t; i += 256) {
-                const int r = quot(i, inv_t), e = i - r * t;
-                V s = Vn ? Vn[o0 + i] : czero<V>();
+        for (int c = 0; c < ncb; ++c) {
+            const int ch = c0 + c;
+            V dsm = czero<V>(), rr[EPL][8];
 #pragma unroll
-                for (int l = 0; l < 8; ++l) {
-                    const T f = wt[r * 8 + l];
-                    const V v = Rc[l * tp + e];
-                    s.x = fma(f, v.x, s.x);
-                    s.y = fma(f, v.y, s.y);
+            for (int a = 0; a < EPL; ++a) {
+#pragma unroll
+                for (int l = 0; l < 8; ++l) rr[a][l] = e0 + 32 * a < t ? Rc[(l * CPB + c) * tp + e0 + 32 * a] : czero<V>();
+            }
+            for (int k0 = warp * KP; k0 < Ndiv; k0 += 8 * KP) {
+                const int np = min(KP, Ndiv - k0);
+                const size_t kd0 = (size_t)cell * Ndiv + k0, g0 = kd0 * t, o0 = (size_t)ch * nkc * Ndiv * t + g0;
+                if (c == 0 || !once) {
+                    load_rows(w.Uv, rvp, Uvd + kd0 * rv, np, rv);
+                    load_rows(w.Uc, rcp, Ucd + kd0 * rc, np, rc);
+                    for (int i = lane; i < np * 8; i += 32) {
+                        const int js = k0 + (i >> 3), a = quot(js, inv_nd), j1 = quot(a, inv_nd);
+                        w.wt[i] = corner_weight<T>(j1, a - j1 * nd, js - a * nd, i & 7, nd, nb1) * inv;
+                    }
+                    __syncwarp();
                 }
-                X[r * tp + e] = s;
-            }
-            __syncthreads();
-            rotate_blocks<false>(X, tp, sUv, rvp, sUc, rcp, np, nv, nc);
-            T dre = (T)0, dim = (T)0;                   // this thread's few products, then FP64
-            for (int i = tid; i < np * t; i += 256) {
-                const int r = quot(i, inv_t), e = i - r * t;
-                const V s = X[r * tp + e], p = psi[o0 + i];
-                const T de = dE[g0 + i];
-                V w;
-                w.x = fma(p.x, de, s.x);
-                w.y = fma(p.y, de, s.y);
-                W[o0 + i] = w;
-                dre = fma(p.x, w.x, fma(p.y, w.y, dre));
-                dim = fma(p.x, w.y, fma(-p.y, w.x, dim));
-            }
-            dot.x += (double)dre;
-            dot.y += (double)dim;
-            __syncthreads();
-        }
-    }
+                // four points' loads in flight at a time; psi and dE of the first of them already here
+                for (int r0 = sub; r0 < np; r0 += 4 * nsub) {
+                    V s[EPL][4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        dot.x += __shfl_down_sync(0xffffffffu, dot.x, o);
-        dot.y += __shfl_down_sync(0xffffffffu, dot.y, o);
+                    for (int a = 0; a < EPL; ++a) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int r = r0 + u * nsub, e = e0 + 32 * a;
+                            s[a][u] = Vn && r < np && e < t ? Vn[o0 + r * t + e] : czero<V>();
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int r = r0 + u * nsub;
+                        if (r >= np) break;
+                        T f[8];
+#pragma unroll
+                        for (int l = 0; l < 8; ++l) f[l] = w.wt[r * 8 + l];
+#pragma unroll
+                        for (int a = 0; a < EPL; ++a) {
+                            const int e = e0 + 32 * a;
+                            if (e >= t) continue;
+                            V q = s[a][u];
+#pragma unroll
+                            for (int l = 0; l < 8; ++l) {
+                                q.x = fma(f[l], rr[a][l].x, q.x);
+                                q.y = fma(f[l], rr[a][l].y, q.y);
+                            }
+                            w.X[r * tp + e] = q;
+                        }
+                    }
+                }
+                V p4[4];
+                T d4[4];
+                auto fetch = [&](int i0) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int i = i0 + 32 * u;
+                        p4[u] = i < np * t ? psi[o0 + i] : czero<V>();
+                        d4[u] = i < np * t ? dE[g0 + i] : (T)0;
+                    }
+                };
+                fetch(lane);
+                __syncwarp();
+                rotate_warp<false>(w.X, w.Tm, tp, w.Uv, rvp, w.Uc, rcp, np, nv, nc);
+                for (int i0 = lane; i0 < np * t; i0 += 128) {
+                    if (i0 != lane) fetch(i0);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int i = i0 + 32 * u;
+                        if (i >= np * t) break;
+                        const int r = quot(i, inv_t), e = i - r * t;
+                        const V s = w.X[r * tp + e], p = p4[u];
+                        V o;
+                        o.x = fma(p.x, d4[u], s.x);
+                        o.y = fma(p.y, d4[u], s.y);
+                        W[o0 + i] = o;
+                        dsm.x = fma(p.x, o.x, fma(p.y, o.y, dsm.x));
+                        dsm.y = fma(p.x, o.y, fma(-p.y, o.x, dsm.y));
+                    }
+                }
+                __syncwarp();
+            }
+            dsum[c][tid] = dsm;
+        }
+        __syncthreads();
+        if (warp < ncb)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const V v = dsum[warp][lane + 32 * q];
+                dot.x += (double)v.x;
+                dot.y += (double)v.y;
+            }
     }
-    if ((tid & 31) == 0) dred[tid >> 5] = dot;
-    __syncthreads();
-    if (tid == 0) {
-        double2 s = dred[0];
-        for (int w = 1; w < 8; ++w) s = cadd(s, dred[w]);
-        part[(size_t)ch * BSE_MAX_VEC_BLOCKS + blockIdx.x] = s;
+    if (warp < ncb) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            dot.x += __shfl_down_sync(0xffffffffu, dot.x, o);
+            dot.y += __shfl_down_sync(0xffffffffu, dot.y, o);
+        }
+        if (lane == 0) part[(size_t)(c0 + warp) * BSE_MAX_VEC_BLOCKS + blockIdx.x] = dot;
     }
 }
 
@@ -388,17 +514,20 @@ __global__ void __launch_bounds__(256) k_common_prolong(
 //
 // Per target and column (one real component of one chain) one multiply-add per
 // near offset is needed: 808 M for coarse 8^3, n_div 4, w 1, 3 chains of 16
-// transitions.  A warp takes one column group (a column per lane) and TY rows
-// (j1, j2 .. j2 + TY - 1) of CZ cells that follow each other along z: their
-// targets are CZ TZ consecutive points, so one load of a source column serves up
-// to TY (2 r + 1) multiply-adds, and since W is the same in every cell one
-// broadcast vector load of TZ weights serves CZ multiply-adds each.  It walks
-// the source rows (delta_1, row u) of its ball in set-up's list; the reach r of
-// each target row along z is a case of a switch, so only offsets inside the ball
-// cost arithmetic and the source row sits in registers.  Sources come straight
-// from phi (the warps of a block share their cells, hence rows, through L1);
-// the weights of the next row are copied to the warp's buffer meanwhile.
-// RM: the largest r that the unrolled body covers (R <= RM); RM = 0 loops over z.
+// transitions.  A warp takes one column group and TY rows (j1, j2 .. j2 + TY - 1) of
+// cells that follow each other along z: a source is loaded once for up to
+// TY (2 r + 1) multiply-adds, and since W is the same in every cell one broadcast
+// load of weights serves every cell of the run.  FP64: a column per lane.  FP32: a
+// complex column per lane, its two halves one packed multiply-add (with single
+// ones the issue slots bound the kernel: 60 M instructions for 25 M), and the half
+// warps take the two halves of the run.
+// It walks the source rows (delta_1, row u) of its ball in set-up's list; the
+// reach r of each target row along z selects an unrolled body, so only offsets
+// inside the ball cost arithmetic and the source row sits in registers.
+// Sources come straight from phi (the warps of a block share their cells, hence
+// rows, through L1); the weights of the next row are copied to the warp's buffer
+// meanwhile.  RM: the largest r that the unrolled body covers (R <= RM); RM = 0
+// loops over the offsets.
 struct NearStencil {
     int n, L, Lp, R, nd, njb, nzb, nsteps, wrow;   // njb: blocks of TY rows j2; nzb: blocks of TZ targets j3
     int cols, t2, ntz, warps;                      // columns in use, 2 t, z tiles (of cz cells, the last ones smaller), all warps
@@ -406,80 +535,102 @@ struct NearStencil {
     long long N2;                                  // 2 N: reals per chain of V
 };
 
-template <typename T, int TZ>
-__device__ __forceinline__ void load_w(T (&w)[TZ], const T* p) {
-    if constexpr (TZ >= 3 && sizeof(T) == 4) {
-        const float4 q = *reinterpret_cast<const float4*>(p);
-        w[0] = q.x; w[1] = q.y; w[2] = q.z;
-        if (TZ == 4) w[TZ - 1] = q.w;
-    } else if constexpr (TZ >= 2) {
-        using V = typename Cx<T>::V;
-        const V q = reinterpret_cast<const V*>(p)[0];
-        w[0] = q.x; w[1] = q.y;
-        if (TZ >= 3) {
-            const V q2 = reinterpret_cast<const V*>(p)[1];
-            w[2] = q2.x;
-            if (TZ == 4) w[TZ - 1] = q2.y;
-        }
+// What a lane holds of a source and of a sum: FP64 one component; FP32 the two of a
+// complex column in a register pair.
+template <typename T> struct NearElem;
+template <> struct NearElem<double> { using E = double; };
+template <> struct NearElem<float> { using E = unsigned long long; };
+
+// Weights of one offset in the table: TZ values, for FP32 each twice (a packed
+// multiply-add's operand), padded to what the vector loads below read.
+template <typename T, int TZ> constexpr int near_tzp() {
+    return sizeof(T) == 4 ? (TZ == 3 ? 8 : 2 * TZ) : (TZ == 3 ? 4 : TZ);
+}
+
+__device__ __forceinline__ double near_fma(double w, double v, double a) { return fma(w, v, a); }
+__device__ __forceinline__ unsigned long long near_fma(unsigned long long w, unsigned long long v, unsigned long long a) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(w), "l"(v), "l"(a));
+    return d;
+}
+__device__ __forceinline__ double near_load(const double* p) { return __ldg(p); }
+__device__ __forceinline__ unsigned long long near_load(const float* p) {
+    return __ldg(reinterpret_cast<const unsigned long long*>(p));
+}
+template <int TZ>
+__device__ __forceinline__ void near_weights(double (&w)[TZ], const double* p) {
+#pragma unroll
+    for (int q = 0; q < TZ; ++q) w[q] = p[q];
+}
+template <int TZ>
+__device__ __forceinline__ void near_weights(unsigned long long (&w)[TZ], const float* p) {
+    if constexpr (TZ == 1) {
+        w[0] = *reinterpret_cast<const unsigned long long*>(p);
     } else {
-        w[0] = p[0];
+#pragma unroll
+        for (int q = 0; q < (TZ + 1) / 2; ++q) {
+            const ulonglong2 f = reinterpret_cast<const ulonglong2*>(p)[q];
+            w[2 * q] = f.x;
+            if (2 * q + 1 < TZ) w[2 * q + 1] = f.y;
+        }
     }
 }
 
-// acc += W v for the target rows of one cell run that reach r sources to each side
-template <typename T, int TZ, int CZ, int RM, int r>
-__device__ __forceinline__ void near_apply(T (&acc)[CZ * TZ], const T (&v)[CZ * TZ + 2 * RM], const T* wb) {
-    constexpr int TZP = TZ == 3 ? 4 : TZ;
+// A row of targets' sums over the offsets -r .. r of a source row that is held from
+// -rm on: a[i] += w[i mod TZ] v[i + offset].
+template <typename T, int TZ, int NT, int rm, int r, typename E>
+__device__ __forceinline__ void near_reach(E (&a)[NT], const E (&v)[NT + 2 * rm], const T* wb) {
 #pragma unroll
-    for (int z = -r; z < TZ + r; ++z) {
-        T w[TZ];
-        load_w<T, TZ>(w, wb + z * TZP);
+    for (int d = -r; d <= r; ++d) {
+        E w[TZ];
+        near_weights(w, wb + d * near_tzp<T, TZ>());
 #pragma unroll
-        for (int tz = 0; tz < TZ; ++tz)
-            if (z - tz <= r && tz - z <= r) {
-#pragma unroll
-                for (int c = 0; c < CZ; ++c) acc[c * TZ + tz] = fma(w[tz], v[c * TZ + z + RM], acc[c * TZ + tz]);
-            }
+        for (int i = 0; i < NT; ++i) a[i] = near_fma(w[i % TZ], v[i + d + rm], a[i]);
     }
 }
 // One source row that reaches rm: its columns into registers, then every target
-// row by its own reach r <= rm (code + 1; 0: not reached).  A body per rm: a row
-// array shared by several bodies cost a register move per element.
-template <typename T, int TY, int TZ, int CZ, int rm>
-__device__ __forceinline__ void near_row(T (&acc)[TY][CZ * TZ], const T* __restrict__ row, const T* wb, int wy, int reach) {
-    T v[CZ * TZ + 2 * rm];
+// row by its own reach r <= rm (code r + 1; 0: not reached).
+template <typename T, int TY, int TZ, int NT, int rm, typename E>
+__device__ __forceinline__ void near_row(E (&acc)[TY][NT], const T* __restrict__ row, const T* wb, int wy, int reach) {
+    E v[NT + 2 * rm];
 #pragma unroll
-    for (int z = -rm; z < CZ * TZ + rm; ++z) v[z + rm] = __ldg(row + z * 32);
+    for (int z = -rm; z < NT + rm; ++z) v[z + rm] = near_load(row + z * 32);
     cpa_wait<1>();
     __syncwarp();
 #pragma unroll
     for (int y = 0; y < TY; ++y) {
         const T* w = wb + y * wy;
         const int r = ((reach >> (8 * y)) & 255) - 1;
-        if (r == rm) near_apply<T, TZ, CZ, rm, rm>(acc[y], v, w);
-        if constexpr (rm >= 1) if (r == 0) near_apply<T, TZ, CZ, rm, 0>(acc[y], v, w);
-        if constexpr (rm >= 2) if (r == 1) near_apply<T, TZ, CZ, rm, 1>(acc[y], v, w);
-        if constexpr (rm >= 3) if (r == 2) near_apply<T, TZ, CZ, rm, 2>(acc[y], v, w);
-        if constexpr (rm >= 4) if (r == 3) near_apply<T, TZ, CZ, rm, 3>(acc[y], v, w);
-        if constexpr (rm >= 5) if (r == 4) near_apply<T, TZ, CZ, rm, 4>(acc[y], v, w);
-        if constexpr (rm >= 6) if (r == 5) near_apply<T, TZ, CZ, rm, 5>(acc[y], v, w);
+        if (r == rm) near_reach<T, TZ, NT, rm, rm>(acc[y], v, w);
+        if constexpr (rm >= 1) { if (r == 0) near_reach<T, TZ, NT, rm, 0>(acc[y], v, w); }
+        if constexpr (rm >= 2) { if (r == 1) near_reach<T, TZ, NT, rm, 1>(acc[y], v, w); }
+        if constexpr (rm >= 3) { if (r == 2) near_reach<T, TZ, NT, rm, 2>(acc[y], v, w); }
+        if constexpr (rm >= 4) { if (r == 3) near_reach<T, TZ, NT, rm, 3>(acc[y], v, w); }
+        if constexpr (rm >= 5) { if (r == 4) near_reach<T, TZ, NT, rm, 4>(acc[y], v, w); }
+        if constexpr (rm >= 6) { if (r == 5) near_reach<T, TZ, NT, rm, 5>(acc[y], v, w); }
     }
 }
 
+// CZ cells per lane: the run's cells, for FP32 half of them per half warp (one
+// cell: the upper half computes it too and writes nothing).
 template <typename T, int TY, int TZ, int CZ, int RM>
 __device__ __forceinline__ void near_body(const T* __restrict__ phi, const T* __restrict__ Wt,
                                           const int2* __restrict__ steps, T* __restrict__ Vn, const NearStencil& s, int g,
-                                          int cx, int cy, int cz0, int j1, int j2, int zb, T* wbuf) {
-    constexpr int TZP = TZ == 3 ? 4 : TZ, PER = 16 / sizeof(T);
-    const int lane = threadIdx.x & 31, nd = s.nd, R = s.R, nzs = TZ + 2 * R;
+                                          int cx, int cy, int cz0, bool split, int j1, int j2, int zb, T* wbuf) {
+    using E = typename NearElem<T>::E;
+    constexpr int TZP = near_tzp<T, TZ>(), PER = 16 / sizeof(T), NT = CZ * TZ, LC = sizeof(T) == 4 ? 2 : 1;
+    const int lane = threadIdx.x & 31, nd = s.nd, R = s.R, wy = (2 * R + 1) * TZP;
+    const int run = LC == 2 ? lane >> 4 : 0, col0 = LC == 2 ? 2 * (lane & 15) : lane;
+    if (split) cz0 += run * CZ;
     const T* wsrc = Wt + (size_t)((zb * nd + j1) * s.njb + j2 / TY) * s.nsteps * s.wrow;
     const int xb = cx * nd + j1 - R, yb = cy * nd + j2 - R;
-    const T* base = phi + (size_t)g * s.L * s.L * s.Lp * 32 + (size_t)(cz0 * nd + zb * TZ + R) * 32 + lane;
-    T acc[TY][CZ * TZ];
+    const T* base = phi + (size_t)g * s.L * s.L * s.Lp * 32 + (size_t)(cz0 * nd + zb * TZ + R) * 32 + col0;
+    E acc[TY][NT];
 #pragma unroll
-    for (int y = 0; y < TY; ++y)
+    for (int y = 0; y < TY; ++y) {
 #pragma unroll
-        for (int z = 0; z < CZ * TZ; ++z) acc[y][z] = (T)0;
+        for (int i = 0; i < NT; ++i) acc[y][i] = (E)0;                // also the pair (0.f, 0.f)
+    }
     auto fetch = [&](int i) {
         T* dst = wbuf + (i & 1) * s.wrow;
         for (int c = lane * PER; c < s.wrow; c += 32 * PER) cpa16(dst + c, wsrc + (size_t)i * s.wrow + c);
@@ -504,56 +655,56 @@ __device__ __forceinline__ void near_body(const T* __restrict__ phi, const T* __
         const T* wb = wbuf + (i & 1) * s.wrow + R * TZP;
         if constexpr (RM > 0) {
             switch (rm) {
-                case 0: near_row<T, TY, TZ, CZ, 0>(acc, row, wb, nzs * TZP, st.y); break;
-                case 1: near_row<T, TY, TZ, CZ, 1>(acc, row, wb, nzs * TZP, st.y); break;
-                case 2: near_row<T, TY, TZ, CZ, 2>(acc, row, wb, nzs * TZP, st.y); break;
-                case 3: near_row<T, TY, TZ, CZ, 3>(acc, row, wb, nzs * TZP, st.y); break;
-                case 4: near_row<T, TY, TZ, CZ, 4>(acc, row, wb, nzs * TZP, st.y); break;
+                case 0: near_row<T, TY, TZ, NT, 0>(acc, row, wb, wy, st.y); break;
+                case 1: near_row<T, TY, TZ, NT, 1>(acc, row, wb, wy, st.y); break;
+                case 2: near_row<T, TY, TZ, NT, 2>(acc, row, wb, wy, st.y); break;
+                case 3: near_row<T, TY, TZ, NT, 3>(acc, row, wb, wy, st.y); break;
+                case 4: near_row<T, TY, TZ, NT, 4>(acc, row, wb, wy, st.y); break;
                 default:
                     if constexpr (RM >= 6) {
-                        if (rm == 5) near_row<T, TY, TZ, CZ, 5>(acc, row, wb, nzs * TZP, st.y);
-                        else near_row<T, TY, TZ, CZ, 6>(acc, row, wb, nzs * TZP, st.y);
+                        if (rm == 5) near_row<T, TY, TZ, NT, 5>(acc, row, wb, wy, st.y);
+                        else near_row<T, TY, TZ, NT, 6>(acc, row, wb, wy, st.y);
                     }
             }
         } else {
             cpa_wait<1>();
             __syncwarp();
-            for (int z = -rm; z < TZ + rm; ++z) {
-                T v[CZ];
+            for (int d = -rm; d <= rm; ++d) {
+                E v[NT];
 #pragma unroll
-                for (int c = 0; c < CZ; ++c) v[c] = __ldg(row + (c * TZ + z) * 32);
+                for (int z = 0; z < NT; ++z) v[z] = near_load(row + (z + d) * 32);
 #pragma unroll
-                for (int y2 = 0; y2 < TY; ++y2) {
-                    T w[TZ];
-                    load_w<T, TZ>(w, wb + (y2 * nzs + z) * TZP);
+                for (int q = 0; q < TY; ++q) {
+                    E w[TZ];
+                    near_weights(w, wb + q * wy + d * TZP);
 #pragma unroll
-                    for (int tz = 0; tz < TZ; ++tz)
-#pragma unroll
-                        for (int c = 0; c < CZ; ++c) acc[y2][c * TZ + tz] = fma(w[tz], v[c], acc[y2][c * TZ + tz]);
+                    for (int z = 0; z < NT; ++z) acc[q][z] = near_fma(w[z % TZ], v[z], acc[q][z]);
                 }
             }
         }
         __syncwarp();
         st = nx;
     }
-    const int col = g * 32 + lane;
-    if (col >= s.cols) return;
+    const int col = g * 32 + col0;
+    if (col >= s.cols || (run && !split)) return;
     const int ch = col / s.t2, q = col - ch * s.t2;
     T* out = Vn + (size_t)ch * s.N2 + q;
 #pragma unroll
-    for (int c = 0; c < CZ; ++c)
+    for (int c = 0; c < CZ; ++c) {
 #pragma unroll
-        for (int y = 0; y < TY; ++y)
+        for (int y = 0; y < TY; ++y) {
 #pragma unroll
             for (int z = 0; z < TZ; ++z)
                 if (j2 + y < nd && zb * TZ + z < nd) {
                     const size_t kd = ((size_t)((cx * s.n + cy) * s.n + cz0 + c) * nd + j1) * nd * nd + (j2 + y) * nd + zb * TZ + z;
-                    out[kd * s.t2] = acc[y][c * TZ + z];
+                    *reinterpret_cast<E*>(out + kd * s.t2) = acc[y][c * TZ + z];
                 }
+        }
+    }
 }
 
 template <typename T, int TY, int TZ, int RM>
-__global__ void __launch_bounds__(256) k_common_near(const T* __restrict__ phi, const T* __restrict__ Wt,
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 3) k_common_near(const T* __restrict__ phi, const T* __restrict__ Wt,
                                                      const int2* __restrict__ steps, T* __restrict__ Vn, const NearStencil s) {
     extern __shared__ __align__(16) unsigned char smraw[];
     T* wbuf = reinterpret_cast<T*>(smraw) + (size_t)(threadIdx.x >> 5) * 2 * s.wrow;
@@ -576,34 +727,35 @@ __global__ void __launch_bounds__(256) k_common_near(const T* __restrict__ phi, 
         if (q < tz) cz0 += p;
     }
     if (tz < full) cz = s.cz;
+    constexpr int H = sizeof(T) == 4 ? 2 : 1;            // cells per lane: half of the run's in FP32
     if constexpr (RM > 0) {
-        if (cz == 4) near_body<T, TY, TZ, 4, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, j1, jb * TY, zb, wbuf);
-        else if (cz == 2) near_body<T, TY, TZ, 2, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, j1, jb * TY, zb, wbuf);
-        else near_body<T, TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, j1, jb * TY, zb, wbuf);
+        if (cz == 4) near_body<T, TY, TZ, 4 / H, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, H == 2, j1, jb * TY, zb, wbuf);
+        else if (cz == 2) near_body<T, TY, TZ, 2 / H, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, H == 2, j1, jb * TY, zb, wbuf);
+        else near_body<T, TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, false, j1, jb * TY, zb, wbuf);
     } else {
-        near_body<T, TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, j1, jb * TY, zb, wbuf);
+        near_body<T, TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, false, j1, jb * TY, zb, wbuf);
     }
 }
 
 // Weights of the near stencil, FP64, one thread per entry: index
-// [z block][j1][block of j2][step][row y][source z][target z] (rows of a step padded
-// to `wrow`), zero outside the ball and for padding; scale = alpha / N_div.
+// [z block][j1][block of j2][step][row y][delta_3 + R][target z] (near_tzp entries per
+// offset, for FP32 every value twice; steps padded to `wrow`), zero outside the ball and for padding; scale = alpha / N_div.
 template <typename T>
 __global__ void k_common_weights(const double* __restrict__ hcoarse, const int2* __restrict__ steps, int nsteps, int n, int nd,
                                  int nb1, int R, int R2, int TY, int TZ, int TZP, int njb, int wrow, double kappa, double scale,
                                  long long total, T* __restrict__ Wt) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total) return;
-    const int nzs = TZ + 2 * R;
+    const int D = 2 * R + 1;
     const int e = (int)(i % wrow);
     long long q = i / wrow;
     const int2 st = steps[q % nsteps]; q /= nsteps;
     const int jb = (int)(q % njb); q /= njb;
     const int j1 = (int)(q % nd);
     const int zb = (int)(q / nd);
-    const int tz = e % TZP, zi = (e / TZP) % nzs, y = e / (TZP * nzs);
+    const int tz = (e % TZP) / (sizeof(T) == 4 ? 2 : 1), y = e / (TZP * D);
     const int j2 = jb * TY + y, j3 = zb * TZ + tz;
-    const int d1 = (st.x & 255) - R, d2 = ((st.x >> 8) & 255) - y - R, d3 = zi - R - tz;
+    const int d1 = (st.x & 255) - R, d2 = ((st.x >> 8) & 255) - y - R, d3 = (e / TZP) % D - R;
     T out = (T)0;
     if (y < TY && j2 < nd && tz < TZ && j3 < nd && d1 * d1 + d2 * d2 + d3 * d3 <= R2) {
         const double L = (double)n * nd, qa = d1 / L, qb = d2 / L, qc = d3 / L;
@@ -628,14 +780,21 @@ __global__ void k_common_weights(const double* __restrict__ hcoarse, const int2*
     Wt[i] = out;
 }
 
-int rot_points(const bse_interp* s, size_t vsz) {
-    const size_t per = vsz * (odd(s->t) + odd(s->nv * s->nv) + odd(s->nc * s->nc));
-    return (int)std::max<size_t>(1, std::min<size_t>(std::min(s->Ndiv, 64), 32768 / per));
+// Points a warp rotates at a time: the cell's points over 8 warps, at most 8 (a row per
+// lane for 4 valence bands), and 10 KB of shared memory.
+template <typename T>
+int rot_points(const bse_interp* s) {
+    int kp = std::min((s->Ndiv + 7) / 8, 8);
+    while (kp > 1 && WarpStage<T>::bytes(kp, s->nv, s->nc) > 10240) --kp;
+    return kp;
+}
+// Chains per block: all of them once the cells alone fill the SMs.
+int rot_chains(const bse_ctx* ctx, const bse_interp* s, int nchains) {
+    return s->co->nkc >= 2 * std::max(ctx->sm_count, 1) ? nchains : 1;
 }
 
 template <typename K>
 cudaError_t raise_smem(K kernel, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
     if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < bytes)
@@ -646,12 +805,20 @@ cudaError_t raise_smem(K kernel, size_t bytes) {
 // Targets of a warp within a cell: TZ = n_div up to 4 (then blocks of 4), TY rows.
 inline int near_tz(int nd) { return std::min(nd, 4); }
 inline int near_ty(int nd) { return nd <= 3 ? nd : 2; }
-inline int near_tzp(int nd) { return nd == 3 ? 4 : near_tz(nd); }
+template <typename T>
+int near_tzp_of(int nd) {
+    switch (near_tz(nd)) {
+        case 1: return near_tzp<T, 1>();
+        case 2: return near_tzp<T, 2>();
+        case 3: return near_tzp<T, 3>();
+        default: return near_tzp<T, 4>();
+    }
+}
 
 // Elements of a step's weights, rounded up to 16 bytes.
 template <typename T>
 int near_wrow(int nd, int R) {
-    const int per = 16 / (int)sizeof(T), e = near_ty(nd) * (near_tz(nd) + 2 * R) * near_tzp(nd);
+    const int per = 16 / (int)sizeof(T), e = near_ty(nd) * (2 * R + 1) * near_tzp_of<T>(nd);
     return (e + per - 1) / per * per;
 }
 
@@ -675,7 +842,7 @@ int launch_near_r(bse_ctx* ctx, const bse_interp* s, NearStencil ns, cudaStream_
     if (warps > 0x7fffffffLL) { ctx->err = "near stencil: too many targets"; return BSE_ERR_UNSUPPORTED; }
     ns.warps = (int)warps;
     // small grids: fewer warps per block spread over more SMs
-    const int wpb = warps >= 8LL * 2 * ctx->sm_count ? 8 : 2;
+    const int wpb = warps >= 8LL * ctx->sm_count ? 4 : 2;
     const size_t smem = sizeof(T) * 2 * (size_t)ns.wrow * wpb;
     BSE_CUDA_TRY(ctx, raise_smem(k_common_near<T, TY, TZ, RM>, smem));
     k_common_near<T, TY, TZ, RM><<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, st>>>(
@@ -711,38 +878,41 @@ int restrict_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* p
                    cudaStream_t st) {
     using V = typename Cx<T>::V;
     const bse_coarse* c = s->co;
-    const int KP = rot_points(s, sizeof(V));
-    const size_t smem = sizeof(V) * ((size_t)KP * (odd(s->t) + odd(s->nv * s->nv) + odd(s->nc * s->nc)) + 256) +
-                        (sizeof(T) * 8 + sizeof(int2)) * KP;
+    const int KP = rot_points<T>(s), CPB = rot_chains(ctx, s, nchains);
+    const size_t smem = 8 * WarpStage<T>::bytes(KP, s->nv, s->nc) + sizeof(V) * 8 * (s->t <= 16 ? 2 : 1) * 8 * s->t;
     const bool m3 = s->scheme == BSE_SCHEME_M3;
     CommonPhi lay{s->cphi_R, s->cphi_Lp};
-    const dim3 grid(c->nkc, nchains);
+    const dim3 grid(c->nkc, (nchains + CPB - 1) / CPB);
     auto go = [&](auto kernel) -> int {
         BSE_CUDA_TRY(ctx, raise_smem(kernel, smem));
         kernel<<<grid, 256, smem, st>>>((const V*)psi, (const V*)s->d_cUv, (const V*)s->d_cUc, (const V*)s->d_cUvc,
-                                        (const V*)s->d_cUcc, s->n, s->nd, s->nv, s->nc, s->nb1, KP,
+                                        (const V*)s->d_cUcc, s->n, s->nd, s->nv, s->nc, s->nb1, nchains, CPB, KP,
                                         m3 ? (T*)s->d_cphi : nullptr, lay, (V*)s->d_cshare, s->d_cctr, (V*)Q, bop, c->ldk);
         BSE_CUDA_TRY(ctx, cudaGetLastError());
         return BSE_OK;
     };
-    return c->kc_prec == BSE_PREC_BF16 ? go(k_common_restrict<T, true>) : go(k_common_restrict<T, false>);
+    if (c->kc_prec == BSE_PREC_BF16) return s->t <= 32 ? go(k_common_restrict<T, true, 1>) : go(k_common_restrict<T, true, 2>);
+    return s->t <= 32 ? go(k_common_restrict<T, false, 1>) : go(k_common_restrict<T, false, 2>);
 }
 
 template <typename T>
 int prolong_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* R, const void* psi, void* W, double2* dot,
                   cudaStream_t st) {
     using V = typename Cx<T>::V;
-    const int KP = rot_points(s, sizeof(V));
-    const size_t smem = sizeof(V) * (size_t)(KP + 8) * (odd(s->t) + odd(s->nv * s->nv) + odd(s->nc * s->nc)) +
-                        sizeof(T) * 8 * KP;
-    BSE_CUDA_TRY(ctx, raise_smem(k_common_prolong<T>, smem));
-    const dim3 grid(bse_common_dot_blocks(s), nchains);
-    k_common_prolong<T><<<grid, 256, smem, st>>>((const V*)R, s->scheme == BSE_SCHEME_M3 ? (const V*)s->d_cV : nullptr,
-                                                 (const V*)s->d_cUv, (const V*)s->d_cUc, (const V*)s->d_cUvc,
-                                                 (const V*)s->d_cUcc, (const T*)s->d_dE, (const V*)psi, s->n, s->nd,
-                                                 s->nv, s->nc, s->nb1, KP, (V*)W, dot);
-    BSE_CUDA_TRY(ctx, cudaGetLastError());
-    return BSE_OK;
+    const int KP = rot_points<T>(s), CPB = rot_chains(ctx, s, nchains);
+    const size_t smem = (sizeof(V) * (sizeof(T) == 8 ? 2 : 1) * 8 * CPB * odd(s->t) + 15) / 16 * 16 +
+                        8 * WarpStage<T>::bytes(KP, s->nv, s->nc);
+    const dim3 grid(bse_common_dot_blocks(s), (nchains + CPB - 1) / CPB);
+    auto go = [&](auto kernel) -> int {
+        BSE_CUDA_TRY(ctx, raise_smem(kernel, smem));
+        kernel<<<grid, 256, smem, st>>>((const V*)R, s->scheme == BSE_SCHEME_M3 ? (const V*)s->d_cV : nullptr,
+                                        (const V*)s->d_cUv, (const V*)s->d_cUc, (const V*)s->d_cUvc, (const V*)s->d_cUcc,
+                                        (const T*)s->d_dE, (const V*)psi, s->n, s->nd, s->nv, s->nc, s->nb1, nchains, CPB, KP,
+                                        (V*)W, dot);
+        BSE_CUDA_TRY(ctx, cudaGetLastError());
+        return BSE_OK;
+    };
+    return s->t <= 32 ? go(k_common_prolong<T, 1>) : go(k_common_prolong<T, 2>);
 }
 
 template <typename T>
@@ -801,7 +971,7 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s) {
     const long long nw = (long long)nzb * nd * njb * s->n_csteps * wrow;
     if ((rc_ = bse_alloc(ctx, &s->d_cw, sizeof(T) * (size_t)nw, "near stencil weights")) != BSE_OK) return rc_;
     k_common_weights<T><<<(unsigned)((nw + 127) / 128), 128, 0, st>>>(s->d_chead, s->d_csteps, s->n_csteps, s->n, nd, s->nb1, R,
-                                                                      s->near_R2, TY, TZ, near_tzp(nd), njb, wrow, c->kappa,
+                                                                      s->near_R2, TY, TZ, near_tzp_of<T>(nd), njb, wrow, c->kappa,
                                                                       c->alpha / s->Ndiv, nw, (T*)s->d_cw);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
