@@ -175,6 +175,19 @@ __device__ __forceinline__ void load_rows(V* dst, int pitch, const V* __restrict
     }
 }
 
+// A lane's share of rows of t entries: entry e (and, for t > 32, e + 32) of rows sub,
+// sub + nsub, ...: no division inside the loops, whole lines of rows side by side.
+struct LaneMap {
+    int e, sub, nsub;          // lanes left over take no row (sub beyond every row count)
+    __device__ explicit LaneMap(int t) {
+        const int lane = threadIdx.x & 31;
+        nsub = t <= 32 ? 32 / t : 1;
+        sub = t <= 32 ? lane / t : 0;
+        e = lane - sub * t;
+        if (sub >= nsub) sub = 1 << 20;
+    }
+};
+
 // Shared memory of a warp that rotates up to KP points: entries, gauge, weights, places.
 template <typename T>
 struct WarpStage {
@@ -232,12 +245,11 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
     const Int3 ci = unflat3(ic, n);
     const size_t wbytes = WarpStage<T>::bytes(KP, nv, nc);
     const WarpStage<T> w(smraw + warp * wbytes, KP, nv, nc);
-    V* red = reinterpret_cast<V*>(smraw + 8 * wbytes);            // [8 warps][2 halves when t <= 16][8][t]
+    V* red = reinterpret_cast<V*>(smraw + 8 * wbytes);            // [8 warps][nsub][8][t]
     const int L = n * nd;
-    const float inv_nd = 1.f / (float)nd, inv_t = 1.f / (float)t;
-    // lane -> transitions e = lane (, lane + 32); with t <= 16 the half warps share the points
-    const int sub = t <= 16 ? lane >> 4 : 0, nsub = t <= 16 ? 2 : 1, e0 = t <= 16 ? lane & 15 : lane;
-    const int items = 8 * t, parts = 8 * nsub;
+    const float inv_nd = 1.f / (float)nd;
+    const LaneMap m(t);
+    const int items = 8 * t, parts = 8 * m.nsub;
     const bool once = Ndiv <= 8 * KP;                              // a warp's points fit at once: their gauge is loaded once
     for (int ch = c0; ch < c1; ++ch) {
         V acc[EPL][8];
@@ -249,7 +261,15 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
         for (int k0 = warp * KP; k0 < Ndiv; k0 += 8 * KP) {
             const int np = min(KP, Ndiv - k0);
             const size_t kd0 = (size_t)ic * Ndiv + k0;
-            load_rows(w.X, tp, psi + ((size_t)ch * nkc * Ndiv + kd0) * t, np, t);
+            const V* src = psi + ((size_t)ch * nkc * Ndiv + kd0) * t;
+#pragma unroll 4
+            for (int r = m.sub; r < np; r += m.nsub) {
+#pragma unroll
+                for (int a = 0; a < EPL; ++a) {
+                    const int e = m.e + 32 * a;
+                    if (EPL == 1 || e < t) w.X[r * tp + e] = src[r * t + e];
+                }
+            }
             if (ch == c0 || !once) {
                 load_rows(w.Uv, rvp, Uvd + kd0 * rv, np, rv);
                 load_rows(w.Uc, rcp, Ucd + kd0 * rc, np, rc);
@@ -267,23 +287,28 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
             if (phi) {
                 // the 2 t components of a point lie side by side in the columns of its groups
                 const size_t gs = (size_t)L * L * lay.Lp * 32;
-                for (int i = lane; i < np * t; i += 32) {
-                    const int r = quot(i, inv_t), e = i - r * t, col = 2 * (ch * t + e);
-                    const int2 pt = w.pnt[r];
-                    const V v = w.X[r * tp + e];
-                    V* at = reinterpret_cast<V*>(phi + (size_t)(col >> 5) * gs + (size_t)pt.x * 32 + (col & 31));
-                    *at = v;
-                    if (pt.y) at[(ptrdiff_t)pt.y * 16] = v;      // periodic halo copy
+#pragma unroll
+                for (int a = 0; a < EPL; ++a) {
+                    const int e = m.e + 32 * a, col = 2 * (ch * t + e);
+                    if (EPL == 2 && e >= t) continue;
+                    T* at0 = phi + (size_t)(col >> 5) * gs + (col & 31);
+                    for (int r = m.sub; r < np; r += m.nsub) {
+                        const int2 pt = w.pnt[r];
+                        const V v = w.X[r * tp + e];
+                        V* at = reinterpret_cast<V*>(at0 + (size_t)pt.x * 32);
+                        *at = v;
+                        if (pt.y) at[(ptrdiff_t)pt.y * 16] = v;  // periodic halo copy
+                    }
                 }
             }
-            for (int r = sub; r < np; r += nsub) {
+            for (int r = m.sub; r < np; r += m.nsub) {
                 T f[8];
 #pragma unroll
                 for (int l = 0; l < 8; ++l) f[l] = w.wt[r * 8 + l];
 #pragma unroll
                 for (int a = 0; a < EPL; ++a) {
-                    const int e = e0 + 32 * a;
-                    if (e >= t) continue;
+                    const int e = m.e + 32 * a;
+                    if (EPL == 2 && e >= t) continue;
                     const V v = w.X[r * tp + e];
 #pragma unroll
                     for (int l = 0; l < 8; ++l) {
@@ -296,12 +321,13 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
             __syncwarp();
         }
         // the cell's shares: [chain][cell][corner][t], the warps' sums in order
+        if (m.sub < m.nsub) {
 #pragma unroll
-        for (int a = 0; a < EPL; ++a) {
-            const int e = e0 + 32 * a;
-            if (e < t) {
+            for (int a = 0; a < EPL; ++a) {
+                const int e = m.e + 32 * a;
+                if (EPL == 2 && e >= t) continue;
 #pragma unroll
-                for (int l = 0; l < 8; ++l) red[(warp * nsub + sub) * items + l * t + e] = acc[a][l];
+                for (int l = 0; l < 8; ++l) red[(warp * m.nsub + m.sub) * items + l * t + e] = acc[a][l];
             }
         }
         __syncthreads();
@@ -388,8 +414,8 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
     const size_t rbytes = (sizeof(V) * (sizeof(T) == 8 ? 2 : 1) * 8 * CPB * tp + 15) / 16 * 16;
     const WarpStage<T> w(smraw + rbytes + warp * WarpStage<T>::bytes(KP, nv, nc), KP, nv, nc);
     const T inv = (T)1 / (T)Ndiv;
-    const float inv_t = 1.f / (float)t, inv_nd = 1.f / (float)nd;
-    const int sub = t <= 16 ? lane >> 4 : 0, nsub = t <= 16 ? 2 : 1, e0 = t <= 16 ? lane & 15 : lane;
+    const float inv_nd = 1.f / (float)nd;
+    const LaneMap m(t);
     const bool once = Ndiv <= 8 * KP;
     double2 dot = make_double2(0.0, 0.0);                         // warp c < ncb: chain c's sum over the block, in FP64
     for (int cell = blockIdx.x; cell < nkc; cell += gridDim.x) {
@@ -411,7 +437,7 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
 #pragma unroll
             for (int a = 0; a < EPL; ++a) {
 #pragma unroll
-                for (int l = 0; l < 8; ++l) rr[a][l] = e0 + 32 * a < t ? Rc[(l * CPB + c) * tp + e0 + 32 * a] : czero<V>();
+                for (int l = 0; l < 8; ++l) rr[a][l] = m.e + 32 * a < t ? Rc[(l * CPB + c) * tp + m.e + 32 * a] : czero<V>();
             }
             for (int k0 = warp * KP; k0 < Ndiv; k0 += 8 * KP) {
                 const int np = min(KP, Ndiv - k0);
@@ -425,28 +451,28 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
                     }
                     __syncwarp();
                 }
-                // four points' loads in flight at a time; psi and dE of the first of them already here
-                for (int r0 = sub; r0 < np; r0 += 4 * nsub) {
+                // four points' loads in flight at a time; psi and dE of the first four before the rotation
+                for (int r0 = m.sub; r0 < np; r0 += 4 * m.nsub) {
                     V s[EPL][4];
 #pragma unroll
                     for (int a = 0; a < EPL; ++a) {
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            const int r = r0 + u * nsub, e = e0 + 32 * a;
+                            const int r = r0 + u * m.nsub, e = m.e + 32 * a;
                             s[a][u] = Vn && r < np && e < t ? Vn[o0 + r * t + e] : czero<V>();
                         }
                     }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        const int r = r0 + u * nsub;
+                        const int r = r0 + u * m.nsub;
                         if (r >= np) break;
                         T f[8];
 #pragma unroll
                         for (int l = 0; l < 8; ++l) f[l] = w.wt[r * 8 + l];
 #pragma unroll
                         for (int a = 0; a < EPL; ++a) {
-                            const int e = e0 + 32 * a;
-                            if (e >= t) continue;
+                            const int e = m.e + 32 * a;
+                            if (EPL == 2 && e >= t) continue;
                             V q = s[a][u];
 #pragma unroll
                             for (int l = 0; l < 8; ++l) {
@@ -457,33 +483,41 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
                         }
                     }
                 }
-                V p4[4];
-                T d4[4];
-                auto fetch = [&](int i0) {
+                V p4[EPL][4];
+                T d4[EPL][4];
+                auto fetch = [&](int r0) {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int i = i0 + 32 * u;
-                        p4[u] = i < np * t ? psi[o0 + i] : czero<V>();
-                        d4[u] = i < np * t ? dE[g0 + i] : (T)0;
+                    for (int a = 0; a < EPL; ++a) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int r = r0 + u * m.nsub, e = m.e + 32 * a;
+                            const bool in = r < np && e < t;
+                            p4[a][u] = in ? psi[o0 + r * t + e] : czero<V>();
+                            d4[a][u] = in ? dE[g0 + r * t + e] : (T)0;
+                        }
                     }
                 };
-                fetch(lane);
+                fetch(m.sub);
                 __syncwarp();
                 rotate_warp<false>(w.X, w.Tm, tp, w.Uv, rvp, w.Uc, rcp, np, nv, nc);
-                for (int i0 = lane; i0 < np * t; i0 += 128) {
-                    if (i0 != lane) fetch(i0);
+                for (int r0 = m.sub; r0 < np; r0 += 4 * m.nsub) {
+                    if (r0 != m.sub) fetch(r0);
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        const int i = i0 + 32 * u;
-                        if (i >= np * t) break;
-                        const int r = quot(i, inv_t), e = i - r * t;
-                        const V s = w.X[r * tp + e], p = p4[u];
-                        V o;
-                        o.x = fma(p.x, d4[u], s.x);
-                        o.y = fma(p.y, d4[u], s.y);
-                        W[o0 + i] = o;
-                        dsm.x = fma(p.x, o.x, fma(p.y, o.y, dsm.x));
-                        dsm.y = fma(p.x, o.y, fma(-p.y, o.x, dsm.y));
+                        const int r = r0 + u * m.nsub;
+                        if (r >= np) break;
+#pragma unroll
+                        for (int a = 0; a < EPL; ++a) {
+                            const int e = m.e + 32 * a;
+                            if (EPL == 2 && e >= t) continue;
+                            const V s = w.X[r * tp + e], p = p4[a][u];
+                            V o;
+                            o.x = fma(p.x, d4[a][u], s.x);
+                            o.y = fma(p.y, d4[a][u], s.y);
+                            W[o0 + r * t + e] = o;
+                            dsm.x = fma(p.x, o.x, fma(p.y, o.y, dsm.x));
+                            dsm.y = fma(p.x, o.y, fma(-p.y, o.x, dsm.y));
+                        }
                     }
                 }
                 __syncwarp();
@@ -529,7 +563,8 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
 // meanwhile.  RM: the largest r that the unrolled body covers (R <= RM); RM = 0
 // loops over the offsets.
 struct NearStencil {
-    int n, L, Lp, R, nd, njb, nzb, nsteps, wrow;   // njb: blocks of TY rows j2; nzb: blocks of TZ targets j3
+    int n, L, Lp, R, nd, njb, nzb;                 // njb: blocks of TY rows j2; nzb: blocks of TZ targets j3
+    int nsteps, wrow, wbytes;                      // source rows, weights of one, shared memory of a warp
     int cols, t2, ntz, warps;                      // columns in use, 2 t, z tiles (of cz cells, the last ones smaller), all warps
     int cz;
     long long N2;                                  // 2 N: reals per chain of V
@@ -589,7 +624,9 @@ __device__ __forceinline__ void near_reach(E (&a)[NT], const E (&v)[NT + 2 * rm]
     }
 }
 // One source row that reaches rm: its columns into registers, then every target
-// row by its own reach r <= rm (code r + 1; 0: not reached).
+// row.  FP64 takes each row's own reach r <= rm (code r + 1; 0: not reached); FP32
+// takes rm for every row that is reached (zero weights beyond its own: an eighth
+// more multiply-adds, but no selection among bodies).
 template <typename T, int TY, int TZ, int NT, int rm, typename E>
 __device__ __forceinline__ void near_row(E (&acc)[TY][NT], const T* __restrict__ row, const T* wb, int wy, int reach) {
     E v[NT + 2 * rm];
@@ -600,6 +637,10 @@ __device__ __forceinline__ void near_row(E (&acc)[TY][NT], const T* __restrict__
 #pragma unroll
     for (int y = 0; y < TY; ++y) {
         const T* w = wb + y * wy;
+        if constexpr (sizeof(T) == 4) {
+            if (reach & (255 << (8 * y))) near_reach<T, TZ, NT, rm, rm>(acc[y], v, w);
+            continue;
+        }
         const int r = ((reach >> (8 * y)) & 255) - 1;
         if (r == rm) near_reach<T, TZ, NT, rm, rm>(acc[y], v, w);
         if constexpr (rm >= 1) { if (r == 0) near_reach<T, TZ, NT, rm, 0>(acc[y], v, w); }
@@ -622,8 +663,20 @@ __device__ __forceinline__ void near_body(const T* __restrict__ phi, const T* __
     const int lane = threadIdx.x & 31, nd = s.nd, R = s.R, wy = (2 * R + 1) * TZP;
     const int run = LC == 2 ? lane >> 4 : 0, col0 = LC == 2 ? 2 * (lane & 15) : lane;
     if (split) cz0 += run * CZ;
-    const T* wsrc = Wt + (size_t)((zb * nd + j1) * s.njb + j2 / TY) * s.nsteps * s.wrow;
-    const int xb = cx * nd + j1 - R, yb = cy * nd + j2 - R;
+    // rows' places, wrapped around the zone, once per warp: [2 R + 1] planes, [2 R + TY] rows
+    int* xo = reinterpret_cast<int*>(wbuf + 2 * s.wrow);
+    int* yo = xo + 2 * R + 1;
+    for (int i = lane; i <= 2 * R; i += 32) {
+        int x = cx * nd + j1 - R + i;
+        x += x < 0 ? s.L : (x >= s.L ? -s.L : 0);
+        xo[i] = x * s.L * s.Lp;
+    }
+    for (int i = lane; i < 2 * R + TY; i += 32) {
+        int y = cy * nd + j2 - R + i;
+        y += y < 0 ? s.L : (y >= s.L ? -s.L : 0);
+        yo[i] = y * s.Lp;
+    }
+    const T* wsrc = Wt + (size_t)((zb * nd + j1) * s.njb + j2 / TY) * s.nsteps * s.wrow + lane * PER;
     const T* base = phi + (size_t)g * s.L * s.L * s.Lp * 32 + (size_t)(cz0 * nd + zb * TZ + R) * 32 + col0;
     E acc[TY][NT];
 #pragma unroll
@@ -631,28 +684,31 @@ __device__ __forceinline__ void near_body(const T* __restrict__ phi, const T* __
 #pragma unroll
         for (int i = 0; i < NT; ++i) acc[y][i] = (E)0;                // also the pair (0.f, 0.f)
     }
-    auto fetch = [&](int i) {
-        T* dst = wbuf + (i & 1) * s.wrow;
-        for (int c = lane * PER; c < s.wrow; c += 32 * PER) cpa16(dst + c, wsrc + (size_t)i * s.wrow + c);
+    T* wdst = wbuf + lane * PER;
+    auto fetch = [&](int half) {
+        T* dst = wdst + half;
+        if (lane * PER < s.wrow) cpa16(dst, wsrc);
+        if (s.wrow > 32 * PER)
+            for (int c = 32 * PER; c + lane * PER < s.wrow; c += 32 * PER) cpa16(dst + c, wsrc + c);
+        wsrc += s.wrow;
         cpa_commit();
     };
     int2 st = steps[0];
+    int cur = 0;                                                      // 0 or wrow: the buffer of this step's weights
     fetch(0);
+    __syncwarp();
     for (int i = 0; i < s.nsteps; ++i) {
         int2 nx = st;
         if (i + 1 < s.nsteps) {
             nx = steps[i + 1];
-            fetch(i + 1);
+            fetch(s.wrow - cur);
         } else {
             cpa_commit();
         }
         // st: delta_1 + R | u << 8 | r_max << 16, then the reach + 1 of each target row (0: none), a byte each
-        int x = xb + (st.x & 255), y = yb + ((st.x >> 8) & 255);
-        x += x < 0 ? s.L : (x >= s.L ? -s.L : 0);
-        y += y < 0 ? s.L : (y >= s.L ? -s.L : 0);
-        const T* row = base + ((size_t)x * s.L + y) * s.Lp * 32;
+        const T* row = base + (size_t)(unsigned)(xo[st.x & 255] + yo[(st.x >> 8) & 255]) * 32;
         const int rm = st.x >> 16;
-        const T* wb = wbuf + (i & 1) * s.wrow + R * TZP;
+        const T* wb = wbuf + cur + R * TZP;
         if constexpr (RM > 0) {
             switch (rm) {
                 case 0: near_row<T, TY, TZ, NT, 0>(acc, row, wb, wy, st.y); break;
@@ -684,6 +740,7 @@ __device__ __forceinline__ void near_body(const T* __restrict__ phi, const T* __
         }
         __syncwarp();
         st = nx;
+        cur = s.wrow - cur;
     }
     const int col = g * 32 + col0;
     if (col >= s.cols || (run && !split)) return;
@@ -707,7 +764,7 @@ template <typename T, int TY, int TZ, int RM>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 3) k_common_near(const T* __restrict__ phi, const T* __restrict__ Wt,
                                                      const int2* __restrict__ steps, T* __restrict__ Vn, const NearStencil s) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    T* wbuf = reinterpret_cast<T*>(smraw) + (size_t)(threadIdx.x >> 5) * 2 * s.wrow;
+    T* wbuf = reinterpret_cast<T*>(smraw + (size_t)(threadIdx.x >> 5) * s.wbytes);
     int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (w >= s.warps) return;
     // warp: (group, cx, cy, z tile, z block, j1, block of j2), the last fastest
@@ -843,7 +900,8 @@ int launch_near_r(bse_ctx* ctx, const bse_interp* s, NearStencil ns, cudaStream_
     ns.warps = (int)warps;
     // small grids: fewer warps per block spread over more SMs
     const int wpb = warps >= 8LL * ctx->sm_count ? 4 : 2;
-    const size_t smem = sizeof(T) * 2 * (size_t)ns.wrow * wpb;
+    ns.wbytes = (int)((sizeof(T) * 2 * (size_t)ns.wrow + sizeof(int) * (4 * ns.R + 1 + TY) + 15) / 16 * 16);
+    const size_t smem = (size_t)ns.wbytes * wpb;
     BSE_CUDA_TRY(ctx, raise_smem(k_common_near<T, TY, TZ, RM>, smem));
     k_common_near<T, TY, TZ, RM><<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, st>>>(
         (const T*)s->d_cphi, (const T*)s->d_cw, s->d_csteps, (T*)s->d_cV, ns);
@@ -879,7 +937,7 @@ int restrict_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* p
     using V = typename Cx<T>::V;
     const bse_coarse* c = s->co;
     const int KP = rot_points<T>(s), CPB = rot_chains(ctx, s, nchains);
-    const size_t smem = 8 * WarpStage<T>::bytes(KP, s->nv, s->nc) + sizeof(V) * 8 * (s->t <= 16 ? 2 : 1) * 8 * s->t;
+    const size_t smem = 8 * WarpStage<T>::bytes(KP, s->nv, s->nc) + sizeof(V) * 8 * (s->t <= 32 ? 32 / s->t : 1) * 8 * s->t;
     const bool m3 = s->scheme == BSE_SCHEME_M3;
     CommonPhi lay{s->cphi_R, s->cphi_Lp};
     const dim3 grid(c->nkc, (nchains + CPB - 1) / CPB);
