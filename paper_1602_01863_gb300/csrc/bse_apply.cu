@@ -1581,6 +1581,7 @@ inline bool staged_bands(const bse_interp* s) {
 // Number of <psi, w> block partials one H application leaves in the dot buffer.
 inline int dot_blocks(const bse_interp* s) {
     if (s->scheme == BSE_SCHEME_M2) return m2_blocks(s->N);
+    if (s->learned && s->learned_fused) return bse_lconv_dot_blocks(s);
     if (!s->learned && s->common) return bse_common_dot_blocks(s);
     if (!s->learned && staged_bands(s)) return std::min(s->co->nkc, kProlongMaxCtas);
     return vec_blocks(s->N);

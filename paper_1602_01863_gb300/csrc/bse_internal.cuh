@@ -244,7 +244,8 @@ struct bse_interp {
     double2* d_cgs_h = nullptr;      // [4][m + 1]
     // learned near-diagonal residual (M1 + periodic convolution with the stencil)
     int learned = 0, learned_radius = 0;
-    float2* d_lker = nullptr;        // DFT of the stencil [t][t][L^3]
+    int learned_fused = 0;           // the three-kernel convolution serves this handle (bse_lconv.cu)
+    float2* d_lker = nullptr;        // DFT of the stencil [t][t][L^3], or [L^2][L][t][t] (bse_lconv.cu)
     float2* d_lgrid = nullptr;       // 2 x [4][t][L^3] work grids
     float2* d_tw_fwd = nullptr;      // [2 L] twiddles (forward, inverse)
     float2* d_tw_inv = nullptr;
@@ -327,6 +328,11 @@ struct ApplyScratch {
 };
 int bse_launch_near_field(bse_ctx* ctx, const bse_interp* s, int nchains, const void* X, const float* xscale, void* U);
 int bse_apply_learned(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, void* w, double2* dot);
+// learned correction in three kernels (bse_lconv.cu)
+bool bse_lconv_usable(const bse_ctx* ctx, const bse_interp* s);
+int bse_lconv_dot_blocks(const bse_interp* s);
+int bse_lconv_kernel(bse_ctx* ctx, const bse_interp* s, const float2* ker, float2* out);
+int bse_lconv_apply(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, void* w, double2* dot);
 int bse_near_tc_prepare(bse_ctx* ctx, bse_interp* s, const std::vector<std::vector<NearEntry>>& per_slot);
 int bse_near_tc_launch(bse_ctx* ctx, const bse_interp* s, int nchains, const void* Xh, const float* xscale, void* U,
                        bool prio = false, int prio_value = 0);

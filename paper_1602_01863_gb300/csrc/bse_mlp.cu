@@ -687,8 +687,9 @@ __global__ void k_dE_avg(const T* __restrict__ dE, int nk, int t, float* __restr
 
 // T(delta) = (out(delta) + conj(out(-delta))^T) / (2 N_k), scattered onto the
 // periodic grid kernel ker[e1][e2][x][y][z].
+// swap: channel e2 t + e1 (bse_lconv.cu) instead of e1 t + e2.
 __global__ void k_stencil_scatter(const float* __restrict__ out, const int* __restrict__ offs, const int* __restrict__ neg,
-                                  int noff, int L, int t, float inv_nk, float2* __restrict__ ker) {
+                                  int noff, int L, int t, float inv_nk, int swap, float2* __restrict__ ker) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)noff * t * t) return;
     const int o = (int)(i / (t * t)), e1 = (int)((i / t) % t), e2 = (int)(i % t);
@@ -696,7 +697,8 @@ __global__ void k_stencil_scatter(const float* __restrict__ out, const int* __re
     const float re = 0.5f * (out[2 * i] + out[2 * j]) * inv_nk;
     const float im = 0.5f * (out[2 * i + 1] - out[2 * j + 1]) * inv_nk;
     const int x = imod(offs[3 * o], L), y = imod(offs[3 * o + 1], L), z = imod(offs[3 * o + 2], L);
-    ker[(((size_t)e1 * t + e2) * L + x) * L * L + (size_t)y * L + z] = make_float2(re, im);
+    const size_t chan = swap ? (size_t)e2 * t + e1 : (size_t)e1 * t + e2;
+    ker[(chan * L + x) * L * L + (size_t)y * L + z] = make_float2(re, im);
 }
 
 // One axis of a separable DFT on [chan][L][L][L]: out_j = sum_n in_n w^{j n},
@@ -915,6 +917,7 @@ int dft3(bse_ctx* ctx, float2* a, float2* tmp, int L, long long nchan, const flo
 // Learned term for nchains vectors: w += T * psi (periodic convolution via
 // separable DFTs), with the <psi, w> partials recomputed.
 int bse_apply_learned(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, void* w, double2* dot) {
+    if (s->learned_fused) return bse_lconv_apply(ctx, s, nchains, psi, w, dot);
     const int L = s->n * s->nd, t = s->t;
     const long long L3 = (long long)L * L * L;
     const long long nchan = (long long)nchains * t;
@@ -1126,16 +1129,19 @@ int bse_interp_set_learned(bse_ctx* ctx, bse_interp* s, bse_mlp* m, int radius) 
         if ((rc = mlp_forward(ctx, m, nb, d_X + r0 * m->d_in, d_out + 2 * r0)) != BSE_OK) { cleanup(); return rc; }
     }
     // Hermitian stencil on the periodic grid, then its DFT (one channel per band pair)
-    cudaMemsetAsync(s->d_lker, 0, sizeof(float2) * (size_t)t * t * L3, ctx->stream);
+    const bool fused = bse_lconv_usable(ctx, s);
+    float2* mesh = fused ? d_ktmp : s->d_lker;
+    cudaMemsetAsync(mesh, 0, sizeof(float2) * (size_t)t * t * L3, ctx->stream);
     k_stencil_scatter<<<(int)((rows + 255) / 256), 256, 0, ctx->stream>>>(d_out, d_offs, d_neg, noff, L, t, 1.f / s->nk,
-                                                                        s->d_lker);
-    rc = dft3(ctx, s->d_lker, d_ktmp, L, (long long)t * t, s->d_tw_fwd);
+                                                                        fused ? 1 : 0, mesh);
+    rc = fused ? bse_lconv_kernel(ctx, s, d_ktmp, s->d_lker) : dft3(ctx, s->d_lker, d_ktmp, L, (long long)t * t, s->d_tw_fwd);
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e == cudaSuccess) e = cudaGetLastError();
     cleanup();
     if (rc != BSE_OK) return rc;
     if (e != cudaSuccess) { ctx->err = std::string("learned stencil: ") + cudaGetErrorString(e); return BSE_ERR_CUDA; }
     s->learned = 1;
+    s->learned_fused = fused ? 1 : 0;
     s->learned_radius = radius;
     return BSE_OK;
 }
