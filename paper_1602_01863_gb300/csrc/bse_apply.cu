@@ -1146,60 +1146,99 @@ __global__ void __launch_bounds__(BSE_VEC_THREADS) k_lanczos_axpy(
     }
 }
 
-// Classical Gram-Schmidt pass, part 1: partials of h_j = <V_j, w>, j = 0..nb-1.
+__device__ __forceinline__ double warp_sum_d(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Classical Gram-Schmidt pass, part 1: h_j = <V_j, w>, j = 0..nb-1, of every chain
+// (grid: blocks per vector, vectors, chains).  With several blocks per vector
+// the last of them (a counter per vector and chain, reset there) sums their
+// partials in order.
 template <typename T>
-__global__ void __launch_bounds__(BSE_VEC_THREADS) k_cgs_dots(const typename Cx<T>::V* __restrict__ basis,
-                                                             const typename Cx<T>::V* __restrict__ W, int nb,
-                                                             int mb, int N, int ch, int nblk,
-                                                             double2* __restrict__ part) {
-    __shared__ double2 sh[BSE_VEC_THREADS];
-    const int j = blockIdx.y;
-    const auto* vj = basis + ((size_t)ch * mb + j) * N;
+__global__ void __launch_bounds__(256) k_cgs_dots(const typename Cx<T>::V* __restrict__ basis, const typename Cx<T>::V* __restrict__ W,
+                                                  int mb, int N, double2* __restrict__ part, int* __restrict__ ctr,
+                                                  double2* __restrict__ h) {
+    __shared__ double2 sh[8];
+    __shared__ int last;
+    const int j = blockIdx.y, ch = blockIdx.z, tid = threadIdx.x, lane = tid & 31;
+    const size_t slot = (size_t)ch * mb + j;
+    const auto* vj = basis + slot * N;
     const auto* w = W + (size_t)ch * N;
     double2 s = make_double2(0.0, 0.0);
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < N; g += gridDim.x * blockDim.x) {
+#pragma unroll 4
+    for (int g = blockIdx.x * 256 + tid; g < N; g += gridDim.x * 256) {
         const double2 a = to_d2(vj[g]), b = to_d2(w[g]);
-        s.x += a.x * b.x + a.y * b.y;
-        s.y += a.x * b.y - a.y * b.x;
+        s.x = fma(a.x, b.x, fma(a.y, b.y, s.x));
+        s.y = fma(a.x, b.y, fma(-a.y, b.x, s.y));
     }
-    s = block_sum2(s, sh);
-    if (threadIdx.x == 0) part[(size_t)j * nblk + blockIdx.x] = s;
-    (void)nb;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s.x += __shfl_down_sync(0xffffffffu, s.x, o);
+        s.y += __shfl_down_sync(0xffffffffu, s.y, o);
+    }
+    if (lane == 0) sh[tid >> 5] = s;
+    __syncthreads();
+    if (tid != 0) return;
+    for (int q = 1; q < 8; ++q) s = cadd(s, sh[q]);
+    if (gridDim.x > 1) {
+        part[slot * gridDim.x + blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(ctr + slot, 1) == (int)gridDim.x - 1;
+        if (!last) return;
+        ctr[slot] = 0;
+        __threadfence();
+        s = make_double2(0.0, 0.0);
+        for (int q = 0; q < (int)gridDim.x; ++q) s = cadd(s, __ldcg(part + slot * gridDim.x + q));
+    }
+    h[slot] = s;
 }
 
-__global__ void k_cgs_reduce(const double2* __restrict__ part, int nblk, double2* __restrict__ h) {
-    __shared__ double2 sh[256];
-    const int j = blockIdx.x;
-    double2 s = make_double2(0.0, 0.0);
-    for (int i = threadIdx.x; i < nblk; i += blockDim.x) s = cadd(s, part[(size_t)j * nblk + i]);
-    s = block_sum2(s, sh);
-    if (threadIdx.x == 0) h[j] = s;
-}
-
-// Part 2: w <- w - sum_j h_j V_j; block partials of ||w||^2.
+// Part 2: w <- w - sum_j h_j V_j; block partials of ||w||^2 (grid: blocks, chains).  A
+// block takes 32 entries at a time and its eight warps share the vectors, so
+// that a few thousand entries still fill the SMs and no thread waits for more
+// than an eighth of the vectors (N = 4608, 50 vectors: 26 us with a thread per entry).
 template <typename T>
-__global__ void __launch_bounds__(BSE_VEC_THREADS) k_cgs_update(const typename Cx<T>::V* __restrict__ basis,
-                                                               typename Cx<T>::V* __restrict__ W,
-                                                               const double2* __restrict__ h, int nb, int mb,
-                                                               int N, int ch, double* __restrict__ part) {
+__global__ void __launch_bounds__(256) k_cgs_update(const typename Cx<T>::V* __restrict__ basis, typename Cx<T>::V* __restrict__ W,
+                                                    const double2* __restrict__ h, int nb, int mb, int N,
+                                                    double* __restrict__ part) {
     using V = typename Cx<T>::V;
-    __shared__ double2 sh[BSE_VEC_THREADS];
+    __shared__ double2 sh[8][32];
+    const int ch = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const V* base = basis + (size_t)ch * mb * N;
+    const double2* hc = h + (size_t)ch * mb;
     double nrm = 0.0;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < N; g += gridDim.x * blockDim.x) {
-        double2 w = to_d2(W[(size_t)ch * N + g]);
-        for (int j = 0; j < nb; ++j) {
-            const double2 v = to_d2(basis[((size_t)ch * mb + j) * N + g]);
-            const double2 hj = h[j];
-            w.x -= hj.x * v.x - hj.y * v.y;
-            w.y -= hj.x * v.y + hj.y * v.x;
+    for (int g0 = blockIdx.x * 32; g0 < N; g0 += gridDim.x * 32) {
+        const int g = g0 + lane;
+        double2 s = make_double2(0.0, 0.0);
+        if (g < N)
+#pragma unroll 4
+            for (int j = warp; j < nb; j += 8) {
+                const double2 v = to_d2(base[(size_t)j * N + g]), hj = hc[j];
+                s.x = fma(hj.x, v.x, fma(-hj.y, v.y, s.x));
+                s.y = fma(hj.x, v.y, fma(hj.y, v.x, s.y));
+            }
+        sh[warp][lane] = s;
+        __syncthreads();
+        if (warp == 0 && g < N) {
+            for (int q = 1; q < 8; ++q) s = cadd(s, sh[q][lane]);
+            const V wv = from_d2<V>(csub(to_d2(W[(size_t)ch * N + g]), s));
+            W[(size_t)ch * N + g] = wv;
+            const double2 wd = to_d2(wv);
+            nrm += wd.x * wd.x + wd.y * wd.y;
         }
-        const V wv = from_d2<V>(w);
-        W[(size_t)ch * N + g] = wv;
-        const double2 wd = to_d2(wv);
-        nrm += wd.x * wd.x + wd.y * wd.y;
+        __syncthreads();
     }
-    const double2 s = block_sum2(make_double2(nrm, 0.0), sh);
-    if (threadIdx.x == 0) part[(size_t)ch * BSE_MAX_VEC_BLOCKS + blockIdx.x] = s.x;
+    if (warp == 0) {
+        nrm = warp_sum_d(nrm);
+        if (lane == 0) part[(size_t)ch * BSE_MAX_VEC_BLOCKS + blockIdx.x] = nrm;
+    }
+}
+inline int cgs_blocks(int N) { return std::min((N + 31) / 32, BSE_MAX_VEC_BLOCKS); }
+// Blocks per vector of k_cgs_dots: two per SM over all vectors, at least 1024 entries each.
+inline int cgs_dot_blocks(const bse_ctx* ctx, int N, int nvec) {
+    return std::max(1, std::min({2 * std::max(ctx->sm_count, 1) / std::max(nvec, 1), (N + 1023) / 1024, 64}));
 }
 
 // FP32 vectors, two complex entries per float4 (N even).  The vector update is
@@ -1207,12 +1246,6 @@ __global__ void __launch_bounds__(BSE_VEC_THREADS) k_cgs_update(const typename C
 // over its few entries and across threads and blocks in FP64, in a fixed order.
 // GB300 runs FP64 at 1/64 of the FP32 rate, so per-entry FP64 work would bound
 // these kernels.
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // w <- w - a_i psi_i - b_i psi_{i-1}; block partials of ||w||^2 (every chain in one pass).
 __global__ void __launch_bounds__(256) k_lanczos_axpy4(float4* __restrict__ W, const float4* __restrict__ psi,
                                                        const float4* __restrict__ psi_prev, const double* __restrict__ a,
@@ -1986,12 +2019,15 @@ int ensure_state(bse_ctx* ctx, bse_interp* s, int m, bool reorth, int nw) {
     }
     if (reorth && s->basis_m < m + 1) {
         drop_graph(s);
-        cudaFree(s->d_basis); cudaFree(s->d_cgs_part); cudaFree(s->d_cgs_h);
-        s->d_basis = nullptr; s->d_cgs_part = s->d_cgs_h = nullptr;
+        cudaFree(s->d_basis); cudaFree(s->d_cgs_part); cudaFree(s->d_cgs_h); cudaFree(s->d_cgs_ctr);
+        s->d_basis = nullptr; s->d_cgs_part = s->d_cgs_h = nullptr; s->d_cgs_ctr = nullptr;
         s->basis_m = 0;
         if ((rc = bse_alloc(ctx, &s->d_basis, sizeof(V) * BSE_MAX_CHAINS * (size_t)(m + 1) * s->N, "Lanczos basis")) != BSE_OK) return rc;
-        if ((rc = bse_alloc(ctx, (void**)&s->d_cgs_part, sizeof(double2) * (size_t)(m + 1) * BSE_MAX_VEC_BLOCKS, "CGS partials")) != BSE_OK) return rc;
-        if ((rc = bse_alloc(ctx, (void**)&s->d_cgs_h, sizeof(double2) * (size_t)(m + 1), "CGS coefficients")) != BSE_OK) return rc;
+        const size_t nv = BSE_MAX_CHAINS * (size_t)(m + 1);
+        if ((rc = bse_alloc(ctx, (void**)&s->d_cgs_part, sizeof(double2) * nv * 64, "CGS partials")) != BSE_OK) return rc;
+        if ((rc = bse_alloc(ctx, (void**)&s->d_cgs_h, sizeof(double2) * nv, "CGS coefficients")) != BSE_OK) return rc;
+        if ((rc = bse_alloc(ctx, (void**)&s->d_cgs_ctr, sizeof(int) * nv, "CGS counters")) != BSE_OK) return rc;
+        BSE_CUDA_TRY(ctx, cudaMemset(s->d_cgs_ctr, 0, sizeof(int) * nv));
         s->basis_m = m + 1;
     }
     if (nw > s->eps_nw) {
@@ -2056,15 +2092,13 @@ int enqueue_chains(bse_ctx* ctx, bse_interp* s, int nch, int m, bool reorth, boo
         else
             k_lanczos_axpy<T><<<nb, BSE_VEC_THREADS, 0, st>>>(W, B, A, s->d_a, s->d_b, i, m, N, nch, s->d_part_nrm, s->d_stop);
         if (reorth) {
-            for (int ch = 0; ch < nch; ++ch)
-                for (int pass = 0; pass < 2; ++pass) {
-                    dim3 g(nb, i + 1);
-                    k_cgs_dots<T><<<g, BSE_VEC_THREADS, 0, st>>>(basis, W, i + 1, mb, N, ch, nb, s->d_cgs_part);
-                    k_cgs_reduce<<<i + 1, 256, 0, st>>>(s->d_cgs_part, nb, s->d_cgs_h);
-                    k_cgs_update<T><<<nb, BSE_VEC_THREADS, 0, st>>>(basis, W, s->d_cgs_h, i + 1, mb, N, ch, s->d_part_nrm);
-                }
+            for (int pass = 0; pass < 2; ++pass) {
+                k_cgs_dots<T><<<dim3(cgs_dot_blocks(ctx, N, nch * (i + 1)), i + 1, nch), 256, 0, st>>>(
+                    basis, W, mb, N, s->d_cgs_part, s->d_cgs_ctr, s->d_cgs_h);
+                k_cgs_update<T><<<dim3(cgs_blocks(N), nch), 256, 0, st>>>(basis, W, s->d_cgs_h, i + 1, mb, N, s->d_part_nrm);
+            }
         }
-        k_reduce_b<<<nch, 256, 0, st>>>(s->d_part_nrm, nb, i, m, s->d_a, s->d_b, s->d_stop);
+        k_reduce_b<<<nch, 256, 0, st>>>(s->d_part_nrm, reorth ? cgs_blocks(N) : nb, i, m, s->d_a, s->d_b, s->d_stop);
         }
         if (rule && (i + 1) % rule->every == 0) {
             const int nblk = (rule->nw + kConvThreads - 1) / kConvThreads;

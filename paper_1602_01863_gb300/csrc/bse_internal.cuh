@@ -240,8 +240,9 @@ struct bse_interp {
     int m_alloc = 0;
     void* d_basis = nullptr;         // V [4][m + 1][N] when reorthogonalising
     int basis_m = 0;
-    double2* d_cgs_part = nullptr;   // [4][(m+1)][nblk]
+    double2* d_cgs_part = nullptr;   // [4][m + 1][blocks per vector, at most 64]
     double2* d_cgs_h = nullptr;      // [4][m + 1]
+    int* d_cgs_ctr = nullptr;        // [4][m + 1] blocks done (zero between launches)
     // learned near-diagonal residual (M1 + periodic convolution with the stencil)
     int learned = 0, learned_radius = 0;
     int learned_fused = 0;           // the three-kernel convolution serves this handle (bse_lconv.cu)
