@@ -548,233 +548,72 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
 //
 // Per target and column (one real component of one chain) one multiply-add per
 // near offset is needed: 808 M for coarse 8^3, n_div 4, w 1, 3 chains of 16
-// transitions.  A warp takes one column group and TY rows (j1, j2 .. j2 + TY - 1) of
+// transitions.  A warp takes one column group, a column per lane, and TY rows of
 // cells that follow each other along z: a source is loaded once for up to
 // TY (2 r + 1) multiply-adds, and since W is the same in every cell one broadcast
-// load of weights serves every cell of the run.  FP64: a column per lane.  FP32: a
-// complex column per lane, its two halves one packed multiply-add (with single
-// ones the issue slots bound the kernel: 60 M instructions for 25 M), and the half
-// warps take the two halves of the run.
+// load of weights serves every cell of the run.
 // It walks the source rows (delta_1, row u) of its ball in set-up's list; the
-// reach r of each target row along z selects an unrolled body, so only offsets
+// reach r of the row along z selects an unrolled body, so only offsets
 // inside the ball cost arithmetic and the source row sits in registers.
 // Sources come straight from phi (the warps of a block share their cells, hence
 // rows, through L1); the weights of the next row are copied to the warp's buffer
 // meanwhile.  RM: the largest r that the unrolled body covers (R <= RM); RM = 0
 // loops over the offsets.
 struct NearStencil {
-    int n, L, Lp, R, nd, njb, nzb;                 // njb: blocks of TY rows j2; nzb: blocks of TZ targets j3
+    int n, L, Lp, R, nd, njb, nzb;                 // njb: weight blocks along y; nzb: blocks of TZ targets j3
+    int nyb;                                       // FP32: pairs of target rows along the whole zone
     int nsteps, wrow, wbytes;                      // source rows, weights of one, shared memory of a warp
     int cols, t2, ntz, warps;                      // columns in use, 2 t, z tiles (of cz cells, the last ones smaller), all warps
     int cz;
     long long N2;                                  // 2 N: reals per chain of V
 };
 
-// What a lane holds of a source and of a sum: FP64 one component; FP32 the two of a
-// complex column in a register pair.
-template <typename T> struct NearElem;
-template <> struct NearElem<double> { using E = double; };
-template <> struct NearElem<float> { using E = unsigned long long; };
+// Weights of one offset of one FP64 target row in the table: TZ values, padded
+// to what the loads below read.
+template <int TZ> constexpr int near_tzp() { return TZ == 3 ? 4 : TZ; }
 
-// Weights of one offset in the table: TZ values, for FP32 each twice (a packed
-// multiply-add's operand), padded to what the vector loads below read.
-template <typename T, int TZ> constexpr int near_tzp() {
-    return sizeof(T) == 4 ? (TZ == 3 ? 8 : 2 * TZ) : (TZ == 3 ? 4 : TZ);
-}
-
-__device__ __forceinline__ double near_fma(double w, double v, double a) { return fma(w, v, a); }
-__device__ __forceinline__ unsigned long long near_fma(unsigned long long w, unsigned long long v, unsigned long long a) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(w), "l"(v), "l"(a));
-    return d;
-}
-__device__ __forceinline__ double near_load(const double* p) { return __ldg(p); }
-__device__ __forceinline__ unsigned long long near_load(const float* p) {
-    return __ldg(reinterpret_cast<const unsigned long long*>(p));
-}
-template <int TZ>
-__device__ __forceinline__ void near_weights(double (&w)[TZ], const double* p) {
-#pragma unroll
-    for (int q = 0; q < TZ; ++q) w[q] = p[q];
-}
-template <int TZ>
-__device__ __forceinline__ void near_weights(unsigned long long (&w)[TZ], const float* p) {
-    if constexpr (TZ == 1) {
-        w[0] = *reinterpret_cast<const unsigned long long*>(p);
-    } else {
-#pragma unroll
-        for (int q = 0; q < (TZ + 1) / 2; ++q) {
-            const ulonglong2 f = reinterpret_cast<const ulonglong2*>(p)[q];
-            w[2 * q] = f.x;
-            if (2 * q + 1 < TZ) w[2 * q + 1] = f.y;
+// A warp's weights buffer (two rows of the table) and the places of its source rows,
+// wrapped around the zone: [2 R + 1] planes from x0, [2 R + TY] rows from y0.
+template <typename T, int TY>
+struct NearWarp {
+    static constexpr int PER = 16 / sizeof(T);
+    T *wbuf, *wdst;
+    const T* wsrc;
+    int *xo, *yo;
+    __device__ NearWarp(T* buf, const T* Wt, int block, const NearStencil& s, int x0, int y0) {
+        const int lane = threadIdx.x & 31;
+        wbuf = buf;
+        wdst = buf + lane * PER;
+        wsrc = Wt + (size_t)block * s.nsteps * s.wrow + lane * PER;
+        xo = reinterpret_cast<int*>(buf + 2 * s.wrow);
+        yo = xo + 2 * s.R + 1;
+        for (int i = lane; i <= 2 * s.R; i += 32) {
+            int x = x0 - s.R + i;
+            x += x < 0 ? s.L : (x >= s.L ? -s.L : 0);
+            xo[i] = x * s.L * s.Lp;
+        }
+        for (int i = lane; i < 2 * s.R + TY; i += 32) {
+            int y = y0 - s.R + i;
+            y += y < 0 ? s.L : (y >= s.L ? -s.L : 0);
+            yo[i] = y * s.Lp;
         }
     }
-}
-
-// A row of targets' sums over the offsets -r .. r of a source row that is held from
-// -rm on: a[i] += w[i mod TZ] v[i + offset].
-template <typename T, int TZ, int NT, int rm, int r, typename E>
-__device__ __forceinline__ void near_reach(E (&a)[NT], const E (&v)[NT + 2 * rm], const T* wb) {
-#pragma unroll
-    for (int d = -r; d <= r; ++d) {
-        E w[TZ];
-        near_weights(w, wb + d * near_tzp<T, TZ>());
-#pragma unroll
-        for (int i = 0; i < NT; ++i) a[i] = near_fma(w[i % TZ], v[i + d + rm], a[i]);
-    }
-}
-// One source row that reaches rm: its columns into registers, then every target
-// row.  FP64 takes each row's own reach r <= rm (code r + 1; 0: not reached); FP32
-// takes rm for every row that is reached (zero weights beyond its own: an eighth
-// more multiply-adds, but no selection among bodies).
-template <typename T, int TY, int TZ, int NT, int rm, typename E>
-__device__ __forceinline__ void near_row(E (&acc)[TY][NT], const T* __restrict__ row, const T* wb, int wy, int reach) {
-    E v[NT + 2 * rm];
-#pragma unroll
-    for (int z = -rm; z < NT + rm; ++z) v[z + rm] = near_load(row + z * 32);
-    cpa_wait<1>();
-    __syncwarp();
-#pragma unroll
-    for (int y = 0; y < TY; ++y) {
-        const T* w = wb + y * wy;
-        if constexpr (sizeof(T) == 4) {
-            if (reach & (255 << (8 * y))) near_reach<T, TZ, NT, rm, rm>(acc[y], v, w);
-            continue;
-        }
-        const int r = ((reach >> (8 * y)) & 255) - 1;
-        if (r == rm) near_reach<T, TZ, NT, rm, rm>(acc[y], v, w);
-        if constexpr (rm >= 1) { if (r == 0) near_reach<T, TZ, NT, rm, 0>(acc[y], v, w); }
-        if constexpr (rm >= 2) { if (r == 1) near_reach<T, TZ, NT, rm, 1>(acc[y], v, w); }
-        if constexpr (rm >= 3) { if (r == 2) near_reach<T, TZ, NT, rm, 2>(acc[y], v, w); }
-        if constexpr (rm >= 4) { if (r == 3) near_reach<T, TZ, NT, rm, 3>(acc[y], v, w); }
-        if constexpr (rm >= 5) { if (r == 4) near_reach<T, TZ, NT, rm, 4>(acc[y], v, w); }
-        if constexpr (rm >= 6) { if (r == 5) near_reach<T, TZ, NT, rm, 5>(acc[y], v, w); }
-    }
-}
-
-// CZ cells per lane: the run's cells, for FP32 half of them per half warp (one
-// cell: the upper half computes it too and writes nothing).
-template <typename T, int TY, int TZ, int CZ, int RM>
-__device__ __forceinline__ void near_body(const T* __restrict__ phi, const T* __restrict__ Wt,
-                                          const int2* __restrict__ steps, T* __restrict__ Vn, const NearStencil& s, int g,
-                                          int cx, int cy, int cz0, bool split, int j1, int j2, int zb, T* wbuf) {
-    using E = typename NearElem<T>::E;
-    constexpr int TZP = near_tzp<T, TZ>(), PER = 16 / sizeof(T), NT = CZ * TZ, LC = sizeof(T) == 4 ? 2 : 1;
-    const int lane = threadIdx.x & 31, nd = s.nd, R = s.R, wy = (2 * R + 1) * TZP;
-    const int run = LC == 2 ? lane >> 4 : 0, col0 = LC == 2 ? 2 * (lane & 15) : lane;
-    if (split) cz0 += run * CZ;
-    // rows' places, wrapped around the zone, once per warp: [2 R + 1] planes, [2 R + TY] rows
-    int* xo = reinterpret_cast<int*>(wbuf + 2 * s.wrow);
-    int* yo = xo + 2 * R + 1;
-    for (int i = lane; i <= 2 * R; i += 32) {
-        int x = cx * nd + j1 - R + i;
-        x += x < 0 ? s.L : (x >= s.L ? -s.L : 0);
-        xo[i] = x * s.L * s.Lp;
-    }
-    for (int i = lane; i < 2 * R + TY; i += 32) {
-        int y = cy * nd + j2 - R + i;
-        y += y < 0 ? s.L : (y >= s.L ? -s.L : 0);
-        yo[i] = y * s.Lp;
-    }
-    const T* wsrc = Wt + (size_t)((zb * nd + j1) * s.njb + j2 / TY) * s.nsteps * s.wrow + lane * PER;
-    const T* base = phi + (size_t)g * s.L * s.L * s.Lp * 32 + (size_t)(cz0 * nd + zb * TZ + R) * 32 + col0;
-    E acc[TY][NT];
-#pragma unroll
-    for (int y = 0; y < TY; ++y) {
-#pragma unroll
-        for (int i = 0; i < NT; ++i) acc[y][i] = (E)0;                // also the pair (0.f, 0.f)
-    }
-    T* wdst = wbuf + lane * PER;
-    auto fetch = [&](int half) {
+    // the next row of weights, into the buffer's half 0 or wrow
+    __device__ __forceinline__ void fetch(int half, int wrow) {
+        const int lane = threadIdx.x & 31;
         T* dst = wdst + half;
-        if (lane * PER < s.wrow) cpa16(dst, wsrc);
-        if (s.wrow > 32 * PER)
-            for (int c = 32 * PER; c + lane * PER < s.wrow; c += 32 * PER) cpa16(dst + c, wsrc + c);
-        wsrc += s.wrow;
+        if (lane * PER < wrow) cpa16(dst, wsrc);
+        if (wrow > 32 * PER)
+            for (int c = 32 * PER; c + lane * PER < wrow; c += 32 * PER) cpa16(dst + c, wsrc + c);
+        wsrc += wrow;
         cpa_commit();
-    };
-    int2 st = steps[0];
-    int cur = 0;                                                      // 0 or wrow: the buffer of this step's weights
-    fetch(0);
-    __syncwarp();
-    for (int i = 0; i < s.nsteps; ++i) {
-        int2 nx = st;
-        if (i + 1 < s.nsteps) {
-            nx = steps[i + 1];
-            fetch(s.wrow - cur);
-        } else {
-            cpa_commit();
-        }
-        // st: delta_1 + R | u << 8 | r_max << 16, then the reach + 1 of each target row (0: none), a byte each
-        const T* row = base + (size_t)(unsigned)(xo[st.x & 255] + yo[(st.x >> 8) & 255]) * 32;
-        const int rm = st.x >> 16;
-        const T* wb = wbuf + cur + R * TZP;
-        if constexpr (RM > 0) {
-            switch (rm) {
-                case 0: near_row<T, TY, TZ, NT, 0>(acc, row, wb, wy, st.y); break;
-                case 1: near_row<T, TY, TZ, NT, 1>(acc, row, wb, wy, st.y); break;
-                case 2: near_row<T, TY, TZ, NT, 2>(acc, row, wb, wy, st.y); break;
-                case 3: near_row<T, TY, TZ, NT, 3>(acc, row, wb, wy, st.y); break;
-                case 4: near_row<T, TY, TZ, NT, 4>(acc, row, wb, wy, st.y); break;
-                default:
-                    if constexpr (RM >= 6) {
-                        if (rm == 5) near_row<T, TY, TZ, NT, 5>(acc, row, wb, wy, st.y);
-                        else near_row<T, TY, TZ, NT, 6>(acc, row, wb, wy, st.y);
-                    }
-            }
-        } else {
-            cpa_wait<1>();
-            __syncwarp();
-            for (int d = -rm; d <= rm; ++d) {
-                E v[NT];
-#pragma unroll
-                for (int z = 0; z < NT; ++z) v[z] = near_load(row + (z + d) * 32);
-#pragma unroll
-                for (int q = 0; q < TY; ++q) {
-                    E w[TZ];
-                    near_weights(w, wb + q * wy + d * TZP);
-#pragma unroll
-                    for (int z = 0; z < NT; ++z) acc[q][z] = near_fma(w[z % TZ], v[z], acc[q][z]);
-                }
-            }
-        }
-        __syncwarp();
-        st = nx;
-        cur = s.wrow - cur;
     }
-    const int col = g * 32 + col0;
-    if (col >= s.cols || (run && !split)) return;
-    const int ch = col / s.t2, q = col - ch * s.t2;
-    T* out = Vn + (size_t)ch * s.N2 + q;
-#pragma unroll
-    for (int c = 0; c < CZ; ++c) {
-#pragma unroll
-        for (int y = 0; y < TY; ++y) {
-#pragma unroll
-            for (int z = 0; z < TZ; ++z)
-                if (j2 + y < nd && zb * TZ + z < nd) {
-                    const size_t kd = ((size_t)((cx * s.n + cy) * s.n + cz0 + c) * nd + j1) * nd * nd + (j2 + y) * nd + zb * TZ + z;
-                    *reinterpret_cast<E*>(out + kd * s.t2) = acc[y][c * TZ + z];
-                }
-        }
-    }
-}
+    // st: delta_1 + R | u << 8 | r_max << 16, then the reach + 1 of each target row (0: none), a byte each
+    __device__ __forceinline__ size_t at(int2 st) const { return (size_t)(unsigned)(xo[st.x & 255] + yo[(st.x >> 8) & 255]) * 32; }
+};
 
-template <typename T, int TY, int TZ, int RM>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 3) k_common_near(const T* __restrict__ phi, const T* __restrict__ Wt,
-                                                     const int2* __restrict__ steps, T* __restrict__ Vn, const NearStencil s) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    T* wbuf = reinterpret_cast<T*>(smraw + (size_t)(threadIdx.x >> 5) * s.wbytes);
-    int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (w >= s.warps) return;
-    // warp: (group, cx, cy, z tile, z block, j1, block of j2), the last fastest
-    const int jb = w % s.njb; w /= s.njb;
-    const int j1 = w % s.nd; w /= s.nd;
-    const int zb = w % s.nzb; w /= s.nzb;
-    const int tz = w % s.ntz; w /= s.ntz;
-    const int cy = w % s.n; w /= s.n;
-    const int cx = w % s.n, g = w / s.n;
-    // z tiles: as many of cz cells as fit, then what is left in powers of two
+// z tile tz: as many tiles of s.cz cells as fit, then what is left in powers of two.
+__device__ __forceinline__ int2 near_tile(const NearStencil& s, int tz) {
     const int full = s.n / s.cz;
     int cz0 = min(tz, full) * s.cz, cz = s.cz;
     for (int q = full; q <= tz; ++q) {
@@ -783,26 +622,304 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 3) k_common_near(con
         cz = p;
         if (q < tz) cz0 += p;
     }
-    if (tz < full) cz = s.cz;
-    constexpr int H = sizeof(T) == 4 ? 2 : 1;            // cells per lane: half of the run's in FP32
-    if constexpr (RM > 0) {
-        if (cz == 4) near_body<T, TY, TZ, 4 / H, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, H == 2, j1, jb * TY, zb, wbuf);
-        else if (cz == 2) near_body<T, TY, TZ, 2 / H, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, H == 2, j1, jb * TY, zb, wbuf);
-        else near_body<T, TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, false, j1, jb * TY, zb, wbuf);
-    } else {
-        near_body<T, TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, cz0, false, j1, jb * TY, zb, wbuf);
+    return make_int2(cz0, tz < full ? s.cz : cz);
+}
+
+// FP64.  A row of targets' sums over the offsets -r .. r of a source row that is
+// held from -rm on: a[i] += w[i mod TZ] v[i + offset].
+template <int TZ, int NT, int rm, int r>
+__device__ __forceinline__ void near_reach(double (&a)[NT], const double (&v)[NT + 2 * rm], const double* wb) {
+#pragma unroll
+    for (int d = -r; d <= r; ++d) {
+        double w[TZ];
+#pragma unroll
+        for (int q = 0; q < TZ; ++q) w[q] = wb[d * near_tzp<TZ>() + q];
+#pragma unroll
+        for (int i = 0; i < NT; ++i) a[i] = fma(w[i % TZ], v[i + d + rm], a[i]);
+    }
+}
+// One source row that reaches rm: its columns into registers, then every target
+// row with its own reach r <= rm (code r + 1; 0: not reached).
+template <int TY, int TZ, int NT, int rm>
+__device__ __forceinline__ void near_row(double (&acc)[TY][NT], const double* __restrict__ row, const double* wb, int wy, int reach) {
+    double v[NT + 2 * rm];
+#pragma unroll
+    for (int z = -rm; z < NT + rm; ++z) v[z + rm] = __ldg(row + z * 32);
+    cpa_wait<1>();
+    __syncwarp();
+#pragma unroll
+    for (int y = 0; y < TY; ++y) {
+        const double* w = wb + y * wy;
+        const int r = ((reach >> (8 * y)) & 255) - 1;
+        if (r == rm) near_reach<TZ, NT, rm, rm>(acc[y], v, w);
+        if constexpr (rm >= 1) { if (r == 0) near_reach<TZ, NT, rm, 0>(acc[y], v, w); }
+        if constexpr (rm >= 2) { if (r == 1) near_reach<TZ, NT, rm, 1>(acc[y], v, w); }
+        if constexpr (rm >= 3) { if (r == 2) near_reach<TZ, NT, rm, 2>(acc[y], v, w); }
+        if constexpr (rm >= 4) { if (r == 3) near_reach<TZ, NT, rm, 3>(acc[y], v, w); }
+        if constexpr (rm >= 5) { if (r == 4) near_reach<TZ, NT, rm, 4>(acc[y], v, w); }
+        if constexpr (rm >= 6) { if (r == 5) near_reach<TZ, NT, rm, 5>(acc[y], v, w); }
     }
 }
 
-// Weights of the near stencil, FP64, one thread per entry: index
-// [z block][j1][block of j2][step][row y][delta_3 + R][target z] (near_tzp entries per
-// offset, for FP32 every value twice; steps padded to `wrow`), zero outside the ball and for padding; scale = alpha / N_div.
+template <int TY, int TZ, int CZ, int RM>
+__device__ __forceinline__ void near_body(const double* __restrict__ phi, const double* __restrict__ Wt,
+                                          const int2* __restrict__ steps, double* __restrict__ Vn, const NearStencil& s, int g,
+                                          int cx, int cy, int cz0, int j1, int j2, int zb, double* wbuf) {
+    constexpr int TZP = near_tzp<TZ>(), NT = CZ * TZ;
+    const int lane = threadIdx.x & 31, nd = s.nd, R = s.R, wy = (2 * R + 1) * TZP;
+    NearWarp<double, TY> nw(wbuf, Wt, (zb * nd + j1) * s.njb + j2 / TY, s, cx * nd + j1, cy * nd + j2);
+    const double* base = phi + (size_t)g * s.L * s.L * s.Lp * 32 + (size_t)(cz0 * nd + zb * TZ + R) * 32 + lane;
+    double acc[TY][NT];
+#pragma unroll
+    for (int y = 0; y < TY; ++y) {
+#pragma unroll
+        for (int i = 0; i < NT; ++i) acc[y][i] = 0.0;
+    }
+    int2 st = steps[0];
+    int cur = 0;                                                      // 0 or wrow: the buffer of this step's weights
+    nw.fetch(0, s.wrow);
+    __syncwarp();
+    for (int i = 0; i < s.nsteps; ++i) {
+        int2 nx = st;
+        if (i + 1 < s.nsteps) {
+            nx = steps[i + 1];
+            nw.fetch(s.wrow - cur, s.wrow);
+        } else {
+            cpa_commit();
+        }
+        const double* row = base + nw.at(st);
+        const int rm = st.x >> 16;
+        const double* wb = wbuf + cur + R * TZP;
+        if constexpr (RM > 0) {
+            switch (rm) {
+                case 0: near_row<TY, TZ, NT, 0>(acc, row, wb, wy, st.y); break;
+                case 1: near_row<TY, TZ, NT, 1>(acc, row, wb, wy, st.y); break;
+                case 2: near_row<TY, TZ, NT, 2>(acc, row, wb, wy, st.y); break;
+                case 3: near_row<TY, TZ, NT, 3>(acc, row, wb, wy, st.y); break;
+                case 4: near_row<TY, TZ, NT, 4>(acc, row, wb, wy, st.y); break;
+                default:
+                    if constexpr (RM >= 6) {
+                        if (rm == 5) near_row<TY, TZ, NT, 5>(acc, row, wb, wy, st.y);
+                        else near_row<TY, TZ, NT, 6>(acc, row, wb, wy, st.y);
+                    }
+            }
+        } else {
+            cpa_wait<1>();
+            __syncwarp();
+            for (int d = -rm; d <= rm; ++d) {
+                double v[NT];
+#pragma unroll
+                for (int z = 0; z < NT; ++z) v[z] = __ldg(row + (z + d) * 32);
+#pragma unroll
+                for (int q = 0; q < TY; ++q) {
+#pragma unroll
+                    for (int z = 0; z < NT; ++z) acc[q][z] = fma(wb[q * wy + d * TZP + z % TZ], v[z], acc[q][z]);
+                }
+            }
+        }
+        __syncwarp();
+        st = nx;
+        cur = s.wrow - cur;
+    }
+    const int col = g * 32 + lane;
+    if (col >= s.cols) return;
+    const int ch = col / s.t2, q = col - ch * s.t2;
+    double* out = Vn + (size_t)ch * s.N2 + q;
+#pragma unroll
+    for (int c = 0; c < CZ; ++c) {
+#pragma unroll
+        for (int y = 0; y < TY; ++y) {
+#pragma unroll
+            for (int z = 0; z < TZ; ++z)
+                if (j2 + y < nd && zb * TZ + z < nd) {
+                    const size_t kd = ((size_t)((cx * s.n + cy) * s.n + cz0 + c) * nd + j1) * nd * nd + (j2 + y) * nd + zb * TZ + z;
+                    out[kd * s.t2] = acc[y][c * TZ + z];
+                }
+        }
+    }
+}
+
+template <int TY, int TZ, int RM>
+__global__ void __launch_bounds__(128, 3) k_common_near(const double* __restrict__ phi, const double* __restrict__ Wt,
+                                                        const int2* __restrict__ steps, double* __restrict__ Vn, const NearStencil s) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    double* wbuf = reinterpret_cast<double*>(smraw + (size_t)(threadIdx.x >> 5) * s.wbytes);
+    int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (w >= s.warps) return;
+    // warp: (group, cx, cy, z tile, z block, j1, block of j2), the last fastest
+    const int jb = w % s.njb; w /= s.njb;
+    const int j1 = w % s.nd; w /= s.nd;
+    const int zb = w % s.nzb; w /= s.nzb;
+    const int2 tile = near_tile(s, w % s.ntz); w /= s.ntz;
+    const int cy = w % s.n; w /= s.n;
+    const int cx = w % s.n, g = w / s.n;
+    if constexpr (RM > 0) {
+        if (tile.y == 4) near_body<TY, TZ, 4, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf);
+        else if (tile.y == 2) near_body<TY, TZ, 2, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf);
+        else near_body<TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf);
+    } else {
+        near_body<TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf);
+    }
+}
+
+// FP32: the two rows Y, Y + 1 (Y even, along the whole zone: a pair may belong to two
+// cells) are the halves of packed multiply-adds, so the weights of an offset lie as
+// they are used, row pair by row pair, and a broadcast load of them serves twice the
+// multiply-adds that it serves when each weight is stored twice for a packed complex
+// column: shared-memory bandwidth bounds this kernel, not the multiply-adds.  The
+// source is the operand to double, once per load.  Both rows take the larger reach
+// of the two (zero weights beyond their own).
+using F2 = unsigned long long;                                        // a register pair
+__device__ __forceinline__ F2 ffma2(F2 w, F2 v, F2 a) {
+    F2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(w), "l"(v), "l"(a));
+    return d;
+}
+__device__ __forceinline__ F2 twice(float x) {
+    F2 d;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
+    return d;
+}
+// The TZ weight pairs of one offset (16-byte loads where each offset starts on 16 bytes).
+template <int TZ>
+__device__ __forceinline__ void near_pairs(F2 (&w)[TZ], const float* p) {
+    if constexpr (TZ % 2) {
+#pragma unroll
+        for (int q = 0; q < TZ; ++q) w[q] = reinterpret_cast<const F2*>(p)[q];
+    } else {
+#pragma unroll
+        for (int q = 0; q < TZ; q += 2) {
+            const ulonglong2 f = *reinterpret_cast<const ulonglong2*>(p + 2 * q);
+            w[q] = f.x;
+            w[q + 1] = f.y;
+        }
+    }
+}
+template <int TZ, int NT, int rm>
+__device__ __forceinline__ void near_row32(F2 (&acc)[NT], const float* __restrict__ row, const float* wb) {
+    F2 v[NT + 2 * rm];
+#pragma unroll
+    for (int z = -rm; z < NT + rm; ++z) v[z + rm] = twice(__ldg(row + z * 32));
+    cpa_wait<1>();
+    __syncwarp();
+#pragma unroll
+    for (int d = -rm; d <= rm; ++d) {
+        F2 w[TZ];
+        near_pairs<TZ>(w, wb + d * 2 * TZ);
+#pragma unroll
+        for (int i = 0; i < NT; ++i) acc[i] = ffma2(w[i % TZ], v[i + d + rm], acc[i]);
+    }
+}
+
+template <int TZ, int CZ, int RM>
+__device__ __forceinline__ void near_body32(const float* __restrict__ phi, const float* __restrict__ Wt,
+                                            const int2* __restrict__ steps, float* __restrict__ Vn, const NearStencil& s, int g,
+                                            int X, int Y, int cz0, int zb, float* wbuf) {
+    constexpr int NT = CZ * TZ;
+    const int lane = threadIdx.x & 31, nd = s.nd, R = s.R, cx = X / nd, j1 = X - cx * nd, cy = Y / nd, j2 = Y - cy * nd;
+    NearWarp<float, 2> nw(wbuf, Wt, (zb * nd + j1) * s.njb + (nd % 2 ? j2 : j2 / 2), s, X, Y);
+    const float* base = phi + (size_t)g * s.L * s.L * s.Lp * 32 + (size_t)(cz0 * nd + zb * TZ + R) * 32 + lane;
+    F2 acc[NT];
+#pragma unroll
+    for (int i = 0; i < NT; ++i) acc[i] = 0;                          // the pair (0.f, 0.f)
+    int2 st = steps[0];
+    int cur = 0;                                                      // 0 or wrow: the buffer of this step's weights
+    nw.fetch(0, s.wrow);
+    __syncwarp();
+    for (int i = 0; i < s.nsteps; ++i) {
+        int2 nx = st;
+        if (i + 1 < s.nsteps) {
+            nx = steps[i + 1];
+            nw.fetch(s.wrow - cur, s.wrow);
+        } else {
+            cpa_commit();
+        }
+        const float* row = base + nw.at(st);
+        const int rm = st.x >> 16;
+        const float* wb = wbuf + cur + R * 2 * TZ;
+        if constexpr (RM > 0) {
+            switch (rm) {
+                case 0: near_row32<TZ, NT, 0>(acc, row, wb); break;
+                case 1: near_row32<TZ, NT, 1>(acc, row, wb); break;
+                case 2: near_row32<TZ, NT, 2>(acc, row, wb); break;
+                case 3: near_row32<TZ, NT, 3>(acc, row, wb); break;
+                case 4: near_row32<TZ, NT, 4>(acc, row, wb); break;
+                default:
+                    if constexpr (RM >= 6) {
+                        if (rm == 5) near_row32<TZ, NT, 5>(acc, row, wb);
+                        else near_row32<TZ, NT, 6>(acc, row, wb);
+                    }
+            }
+        } else {
+            cpa_wait<1>();
+            __syncwarp();
+            for (int d = -rm; d <= rm; ++d) {
+                F2 w[TZ];
+                near_pairs<TZ>(w, wb + d * 2 * TZ);
+#pragma unroll
+                for (int z = 0; z < NT; ++z) acc[z] = ffma2(w[z % TZ], twice(__ldg(row + (z + d) * 32)), acc[z]);
+            }
+        }
+        __syncwarp();
+        st = nx;
+        cur = s.wrow - cur;
+    }
+    const int col = g * 32 + lane;
+    if (col >= s.cols) return;
+    const int ch = col / s.t2, q = col - ch * s.t2;
+    float* out = Vn + (size_t)ch * s.N2 + q;
+    // the second row: the next one of the cell or the first of the next cell; none beyond the zone
+    const bool two = Y + 1 < s.L, same = j2 + 1 < nd;
+    const size_t k0 = ((size_t)((cx * s.n + cy) * s.n + cz0) * nd + j1) * nd * nd + j2 * nd + zb * TZ;
+    const size_t k1 = same ? k0 + nd : ((size_t)((cx * s.n + cy + 1) * s.n + cz0) * nd + j1) * nd * nd + zb * TZ;
+#pragma unroll
+    for (int c = 0; c < CZ; ++c) {
+#pragma unroll
+        for (int z = 0; z < TZ; ++z)
+            if (zb * TZ + z < nd) {
+                const F2 a = acc[c * TZ + z];
+                const size_t o = (size_t)c * nd * nd * nd + z;
+                out[(k0 + o) * s.t2] = __uint_as_float((unsigned)a);
+                if (two) out[(k1 + o) * s.t2] = __uint_as_float((unsigned)(a >> 32));
+            }
+    }
+}
+
+template <int TZ, int RM>
+__global__ void __launch_bounds__(128, 5) k_common_near32(const float* __restrict__ phi, const float* __restrict__ Wt,
+                                                          const int2* __restrict__ steps, float* __restrict__ Vn,
+                                                          const NearStencil s) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    float* wbuf = reinterpret_cast<float*>(smraw + (size_t)(threadIdx.x >> 5) * s.wbytes);
+    int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (w >= s.warps) return;
+    // warp: (group, z tile, z block, row X, pair of rows Y), the last fastest
+    const int yb = w % s.nyb; w /= s.nyb;
+    const int X = w % s.L; w /= s.L;
+    const int zb = w % s.nzb; w /= s.nzb;
+    const int2 tile = near_tile(s, w % s.ntz);
+    const int g = w / s.ntz;
+    if constexpr (RM > 0) {
+        if (tile.y == 4) near_body32<TZ, 4, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf);
+        else if (tile.y == 2) near_body32<TZ, 2, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf);
+        else near_body32<TZ, 1, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf);
+    } else {
+        near_body32<TZ, 1, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf);
+    }
+}
+
+// Weights of the near stencil, FP64 arithmetic, one thread per entry: index
+// [z block][j1][block of j2][step] and then, for FP64, [row y][delta_3 + R][target z]
+// (near_tzp entries per offset), for FP32 [delta_3 + R][target z][row y] (blocks start at
+// every second row of the zone, taken modulo the cell); steps padded to `wrow`, zero outside the
+// ball and for padding; scale = alpha / N_div.
 template <typename T>
 __global__ void k_common_weights(const double* __restrict__ hcoarse, const int2* __restrict__ steps, int nsteps, int n, int nd,
                                  int nb1, int R, int R2, int TY, int TZ, int TZP, int njb, int wrow, double kappa, double scale,
                                  long long total, T* __restrict__ Wt) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total) return;
+    constexpr bool pairs = sizeof(T) == 4;
     const int D = 2 * R + 1;
     const int e = (int)(i % wrow);
     long long q = i / wrow;
@@ -810,11 +927,11 @@ __global__ void k_common_weights(const double* __restrict__ hcoarse, const int2*
     const int jb = (int)(q % njb); q /= njb;
     const int j1 = (int)(q % nd);
     const int zb = (int)(q / nd);
-    const int tz = (e % TZP) / (sizeof(T) == 4 ? 2 : 1), y = e / (TZP * D);
-    const int j2 = jb * TY + y, j3 = zb * TZ + tz;
-    const int d1 = (st.x & 255) - R, d2 = ((st.x >> 8) & 255) - y - R, d3 = (e / TZP) % D - R;
+    const int tz = pairs ? (e / 2) % TZ : e % TZP, y = pairs ? e % 2 : e / (TZP * D), o3 = pairs ? e / (2 * TZ) : (e / TZP) % D;
+    const int j2 = pairs ? (jb * (nd % 2 ? 1 : 2) + y) % nd : jb * TY + y, j3 = zb * TZ + tz;
+    const int d1 = (st.x & 255) - R, d2 = ((st.x >> 8) & 255) - y - R, d3 = o3 - R;
     T out = (T)0;
-    if (y < TY && j2 < nd && tz < TZ && j3 < nd && d1 * d1 + d2 * d2 + d3 * d3 <= R2) {
+    if (y < TY && j2 < nd && tz < TZ && j3 < nd && o3 < D && d1 * d1 + d2 * d2 + d3 * d3 <= R2) {
         const double L = (double)n * nd, qa = d1 / L, qb = d2 / L, qc = d3 / L;
         const int js = (j1 * nd + j2) * nd + j3;
         const int g1 = j1 + d1, g2 = j2 + d2, g3 = j3 + d3;
@@ -859,35 +976,33 @@ cudaError_t raise_smem(K kernel, size_t bytes) {
     return e;
 }
 
-// Targets of a warp within a cell: TZ = n_div up to 4 (then blocks of 4), TY rows.
+// Targets of a warp within a cell: TZ = n_div up to 4 (then blocks of 4), TY rows
+// (FP32: pairs of rows of the zone).
 inline int near_tz(int nd) { return std::min(nd, 4); }
-inline int near_ty(int nd) { return nd <= 3 ? nd : 2; }
 template <typename T>
-int near_tzp_of(int nd) {
-    switch (near_tz(nd)) {
-        case 1: return near_tzp<T, 1>();
-        case 2: return near_tzp<T, 2>();
-        case 3: return near_tzp<T, 3>();
-        default: return near_tzp<T, 4>();
-    }
-}
+int near_ty(int nd) { return sizeof(T) == 4 ? 2 : (nd <= 3 ? nd : 2); }
+inline int near_tzp_of(int nd) { return near_tz(nd) == 3 ? near_tzp<3>() : near_tz(nd); }
+// Blocks of rows with weights of their own: FP32 pairs start at any row of a cell when n_div is odd.
+template <typename T>
+int near_njb(int nd) { return sizeof(T) == 4 && nd % 2 ? nd : (nd + near_ty<T>(nd) - 1) / near_ty<T>(nd); }
 
 // Elements of a step's weights, rounded up to 16 bytes.
 template <typename T>
 int near_wrow(int nd, int R) {
-    const int per = 16 / (int)sizeof(T), e = near_ty(nd) * (2 * R + 1) * near_tzp_of<T>(nd);
+    const int per = 16 / (int)sizeof(T), e = near_ty<T>(nd) * (2 * R + 1) * (sizeof(T) == 4 ? near_tz(nd) : near_tzp_of(nd));
     return (e + per - 1) / per * per;
 }
 
-template <typename T, int TY, int TZ, int RM>
-int launch_near_r(bse_ctx* ctx, const bse_interp* s, NearStencil ns, cudaStream_t st) {
+template <typename T, typename K>
+int launch_near_k(bse_ctx* ctx, const bse_interp* s, K kernel, int RM, NearStencil ns, cudaStream_t st) {
     const int groups = (ns.cols + 31) / 32, n = s->n;
     auto tiles = [&](int cz) {
         int c = n / cz;
         for (int left = n % cz; left; left &= left - 1) ++c;
         return c;
     };
-    const long long per_tile = (long long)groups * n * n * ns.nzb * ns.nd * ns.njb;
+    const long long per_tile = (long long)groups * ns.nzb *
+                               (sizeof(T) == 4 ? (long long)ns.L * ns.nyb : (long long)n * n * ns.nd * ns.njb);
     // Cells per warp: as many as leave four warps per SM (a warp alone on its scheduler
     // waits out its loads); z blocks do not continue into the next cell.
     ns.cz = 1;
@@ -900,13 +1015,18 @@ int launch_near_r(bse_ctx* ctx, const bse_interp* s, NearStencil ns, cudaStream_
     ns.warps = (int)warps;
     // small grids: fewer warps per block spread over more SMs
     const int wpb = warps >= 8LL * ctx->sm_count ? 4 : 2;
-    ns.wbytes = (int)((sizeof(T) * 2 * (size_t)ns.wrow + sizeof(int) * (4 * ns.R + 1 + TY) + 15) / 16 * 16);
+    ns.wbytes = (int)((sizeof(T) * 2 * (size_t)ns.wrow + sizeof(int) * (4 * ns.R + 1 + near_ty<T>(ns.nd)) + 15) / 16 * 16);
     const size_t smem = (size_t)ns.wbytes * wpb;
-    BSE_CUDA_TRY(ctx, raise_smem(k_common_near<T, TY, TZ, RM>, smem));
-    k_common_near<T, TY, TZ, RM><<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, st>>>(
-        (const T*)s->d_cphi, (const T*)s->d_cw, s->d_csteps, (T*)s->d_cV, ns);
+    BSE_CUDA_TRY(ctx, raise_smem(kernel, smem));
+    kernel<<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, st>>>((const T*)s->d_cphi, (const T*)s->d_cw, s->d_csteps,
+                                                                       (T*)s->d_cV, ns);
     BSE_CUDA_TRY(ctx, cudaGetLastError());
     return BSE_OK;
+}
+template <typename T, int TY, int TZ, int RM>
+int launch_near_r(bse_ctx* ctx, const bse_interp* s, const NearStencil& ns, cudaStream_t st) {
+    if constexpr (sizeof(T) == 4) return launch_near_k<T>(ctx, s, k_common_near32<TZ, RM>, RM, ns, st);
+    else return launch_near_k<T>(ctx, s, k_common_near<TY, TZ, RM>, RM, ns, st);
 }
 
 template <typename T>
@@ -915,7 +1035,8 @@ int near_typed(bse_ctx* ctx, const bse_interp* s, int nchains, cudaStream_t st) 
     const int nd = s->nd;
     ns.n = s->n; ns.nd = nd; ns.L = s->n * nd; ns.R = s->cphi_R; ns.Lp = s->cphi_Lp;
     ns.nzb = (nd + near_tz(nd) - 1) / near_tz(nd);
-    ns.njb = (nd + near_ty(nd) - 1) / near_ty(nd);
+    ns.njb = near_njb<T>(nd);
+    ns.nyb = (ns.L + 1) / 2;
     ns.nsteps = s->n_csteps;
     ns.wrow = near_wrow<T>(nd, ns.R);
     ns.t2 = 2 * s->t; ns.cols = ns.t2 * nchains; ns.N2 = 2LL * s->N;
@@ -999,7 +1120,7 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s) {
         BSE_CUDA_TRY(ctx, cudaStreamSynchronize(st));
         return BSE_OK;
     }
-    const int nd = s->nd, L = s->n * nd, R = s->cphi_R, TY = near_ty(nd), TZ = near_tz(nd), D = 2 * R + 1;
+    const int nd = s->nd, L = s->n * nd, R = s->cphi_R, TY = near_ty<T>(nd), TZ = near_tz(nd), D = 2 * R + 1;
     // rows of phi: R points of halo on each side, and what a padded target block reads beyond (zeros)
     s->cphi_Lp = L + 2 * R + (nd > 4 ? 3 : 0);
     const size_t groups = (2 * (size_t)s->t * BSE_MAX_CHAINS + 31) / 32;
@@ -1025,11 +1146,11 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s) {
     s->n_csteps = (int)steps.size();
     if ((rc_ = bse_alloc(ctx, (void**)&s->d_csteps, sizeof(int2) * steps.size(), "near stencil rows")) != BSE_OK) return rc_;
     BSE_CUDA_TRY(ctx, cudaMemcpy(s->d_csteps, steps.data(), sizeof(int2) * steps.size(), cudaMemcpyHostToDevice));
-    const int nzb = (nd + TZ - 1) / TZ, njb = (nd + TY - 1) / TY, wrow = near_wrow<T>(nd, R);
+    const int nzb = (nd + TZ - 1) / TZ, njb = near_njb<T>(nd), wrow = near_wrow<T>(nd, R);
     const long long nw = (long long)nzb * nd * njb * s->n_csteps * wrow;
     if ((rc_ = bse_alloc(ctx, &s->d_cw, sizeof(T) * (size_t)nw, "near stencil weights")) != BSE_OK) return rc_;
     k_common_weights<T><<<(unsigned)((nw + 127) / 128), 128, 0, st>>>(s->d_chead, s->d_csteps, s->n_csteps, s->n, nd, s->nb1, R,
-                                                                      s->near_R2, TY, TZ, near_tzp_of<T>(nd), njb, wrow, c->kappa,
+                                                                      s->near_R2, TY, TZ, near_tzp_of(nd), njb, wrow, c->kappa,
                                                                       c->alpha / s->Ndiv, nw, (T*)s->d_cw);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
