@@ -1285,9 +1285,9 @@ __global__ void __launch_bounds__(256) k_lanczos_axpy4(float4* __restrict__ W, c
 // reorthogonalisation; 512 threads per block, one block per SM, grid-stride).  GB300 issues FP64
 // at a small fraction of its FP32 rate, so the FP64 work here is per block or
 // per warp, never per element:
-//  * a_i: warp 0 of every block sums the <psi, w> block partials of the H
+//  * a_i: a warp per chain in every block sums the <psi, w> block partials of the H
 //    application in FP64, in the same fixed order in every block (block 0
-//    stores a_i and its imaginary part);
+//    stores a_i and its imaginary part), while the vectors' first loads are on their way;
 //  * the update and ||w||^2 in FP32 per thread and per warp (shuffles), the 8
 //    warp sums of a block in FP64 into its partial;
 //  * the last block to finish (a counter that it resets) sums the block
@@ -1305,33 +1305,49 @@ __global__ void __launch_bounds__(512) k_lanczos_axpy4_ab(float4* __restrict__ W
     __shared__ float ab_sh[NCH][2];
     __shared__ int run_sh[NCH];
     __shared__ int last_sh;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0) {
+    constexpr int U = 4;                                   // entries in flight per thread
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = gridDim.x * blockDim.x;
+    const int g0 = blockIdx.x * blockDim.x + threadIdx.x;
+    float4 w[U], p[U], q[U];
+    auto load = [&](int ch, int g) {
 #pragma unroll
-        for (int ch = 0; ch < NCH; ++ch) {
-            const int run = stop[ch] == 0;                 // uniform over the grid until the last block
-            // the imaginary part (a Hermiticity diagnostic) in block 0 only
-            double2 s = make_double2(0.0, 0.0);
-            if (run) {
-                if (blockIdx.x == 0)
-                    for (int i = lane; i < ndot; i += 32) s = cadd(s, dot[(size_t)ch * BSE_MAX_VEC_BLOCKS + i]);
-                else
-                    for (int i = lane; i < ndot; i += 32) s.x += dot[(size_t)ch * BSE_MAX_VEC_BLOCKS + i].x;
+        for (int u = 0; u < U; ++u)
+            if (g + u * G < N4) {
+                const size_t o = (size_t)ch * N4 + g + u * G;
+                w[u] = W[o]; p[u] = psi[o]; q[u] = psi_prev[o];
             }
+    };
+    load(0, g0);                                           // on their way while a_i is summed
+    if (warp < NCH) {
+        const int ch = warp, run = stop[ch] == 0;          // uniform over the grid until the last block
+        // the imaginary part (a Hermiticity diagnostic) in block 0 only; eight loads in flight
+        double2 s = make_double2(0.0, 0.0);
+        if (run) {
+            const double2* d = dot + (size_t)ch * BSE_MAX_VEC_BLOCKS;
+            for (int i0 = lane; i0 < ndot; i0 += 256) {
+                double2 v[8];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                s.x += __shfl_down_sync(0xffffffffu, s.x, o);
-                if (blockIdx.x == 0) s.y += __shfl_down_sync(0xffffffffu, s.y, o);
-            }
-            if (lane == 0) {
-                run_sh[ch] = run;
-                a_sh[ch] = s.x;
-                ab_sh[ch][0] = (float)s.x;
-                ab_sh[ch][1] = (float)b[ch * (m + 1) + step];
-                if (blockIdx.x == 0 && run) {
-                    a[ch * m + step] = s.x;
-                    aim[ch * m + step] = s.y;
+                for (int u = 0; u < 8; ++u) v[u] = i0 + 32 * u < ndot ? d[i0 + 32 * u] : make_double2(0.0, 0.0);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    s.x += v[u].x;
+                    if (blockIdx.x == 0) s.y += v[u].y;
                 }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s.x += __shfl_down_sync(0xffffffffu, s.x, o);
+            if (blockIdx.x == 0) s.y += __shfl_down_sync(0xffffffffu, s.y, o);
+        }
+        if (lane == 0) {
+            run_sh[ch] = run;
+            a_sh[ch] = s.x;
+            ab_sh[ch][0] = (float)s.x;
+            ab_sh[ch][1] = (float)b[ch * (m + 1) + step];
+            if (blockIdx.x == 0 && run) {
+                a[ch * m + step] = s.x;
+                aim[ch * m + step] = s.y;
             }
         }
     }
@@ -1342,29 +1358,19 @@ __global__ void __launch_bounds__(512) k_lanczos_axpy4_ab(float4* __restrict__ W
         nrm[ch] = 0.f;
         if (!run_sh[ch]) continue;
         const float ai = ab_sh[ch][0], bi = ab_sh[ch][1];
-        const int G = gridDim.x * blockDim.x;
-        // two entries per pass: both loads in flight before either update
-        for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < N4; g += 2 * G) {
-            const bool two = g + G < N4;
-            const size_t o = (size_t)ch * N4 + g, o2 = o + G;
-            const float4 w = W[o], p = psi[o], q = psi_prev[o];
-            float4 w2 = make_float4(0.f, 0.f, 0.f, 0.f), p2 = w2, q2 = w2;
-            if (two) { w2 = W[o2]; p2 = psi[o2]; q2 = psi_prev[o2]; }
-            float4 r;
-            r.x = fmaf(-bi, q.x, fmaf(-ai, p.x, w.x));
-            r.y = fmaf(-bi, q.y, fmaf(-ai, p.y, w.y));
-            r.z = fmaf(-bi, q.z, fmaf(-ai, p.z, w.z));
-            r.w = fmaf(-bi, q.w, fmaf(-ai, p.w, w.w));
-            W[o] = r;
-            nrm[ch] = fmaf(r.x, r.x, fmaf(r.y, r.y, fmaf(r.z, r.z, fmaf(r.w, r.w, nrm[ch]))));
-            if (two) {
-                r.x = fmaf(-bi, q2.x, fmaf(-ai, p2.x, w2.x));
-                r.y = fmaf(-bi, q2.y, fmaf(-ai, p2.y, w2.y));
-                r.z = fmaf(-bi, q2.z, fmaf(-ai, p2.z, w2.z));
-                r.w = fmaf(-bi, q2.w, fmaf(-ai, p2.w, w2.w));
-                W[o2] = r;
-                nrm[ch] = fmaf(r.x, r.x, fmaf(r.y, r.y, fmaf(r.z, r.z, fmaf(r.w, r.w, nrm[ch]))));
-            }
+        for (int g = g0; g < N4; g += U * G) {
+            if (ch > 0 || g != g0) load(ch, g);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (g + u * G < N4) {
+                    float4 r;
+                    r.x = fmaf(-bi, q[u].x, fmaf(-ai, p[u].x, w[u].x));
+                    r.y = fmaf(-bi, q[u].y, fmaf(-ai, p[u].y, w[u].y));
+                    r.z = fmaf(-bi, q[u].z, fmaf(-ai, p[u].z, w[u].z));
+                    r.w = fmaf(-bi, q[u].w, fmaf(-ai, p[u].w, w[u].w));
+                    W[(size_t)ch * N4 + g + u * G] = r;
+                    nrm[ch] = fmaf(r.x, r.x, fmaf(r.y, r.y, fmaf(r.z, r.z, fmaf(r.w, r.w, nrm[ch]))));
+                }
         }
     }
 #pragma unroll
@@ -1384,11 +1390,10 @@ __global__ void __launch_bounds__(512) k_lanczos_axpy4_ab(float4* __restrict__ W
     __syncthreads();
     if (threadIdx.x == 0) last_sh = atomicAdd(ctr, 1) == (int)gridDim.x - 1;
     __syncthreads();
-    if (!last_sh || warp != 0) return;
+    if (!last_sh || warp >= NCH) return;
     __threadfence();
-#pragma unroll
-    for (int ch = 0; ch < NCH; ++ch) {
-        if (!run_sh[ch]) continue;
+    const int ch = warp;
+    if (run_sh[ch]) {
         double s = 0.0, am = lane == 0 ? fabs(a_sh[ch]) : 0.0;
         for (int i = lane; i < (int)gridDim.x; i += 32) s += __ldcg(part + (size_t)ch * BSE_MAX_VEC_BLOCKS + i);
         for (int j = lane; j < step; j += 32) am = fmax(am, fabs(a[ch * m + j]));
@@ -1403,7 +1408,7 @@ __global__ void __launch_bounds__(512) k_lanczos_axpy4_ab(float4* __restrict__ W
             if (!(bn >= 1e-12 * am)) stop[ch] = step + 1;
         }
     }
-    if (lane == 0) *ctr = 0;
+    if (threadIdx.x == 0) *ctr = 0;
 }
 
 // psi_{i+1} = w / b_{i+1} (written over psi_{i-1}), also into the basis when kept.

@@ -230,7 +230,7 @@ __device__ __forceinline__ T corner_weight(int j1, int j2, int j3, int l, int nd
 // and writes phi: 33 MB for coarse 8^3, n_div 4, 4x4 bands, 3 chains), so the warps of a
 // block wait for one another only at the sums and the chains share what they can.
 template <typename T, bool OUT_BF16, int EPL>
-__global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) k_common_restrict(
+__global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 4 : 2)) k_common_restrict(
     const typename Cx<T>::V* __restrict__ psi, const typename Cx<T>::V* __restrict__ Uvd,
     const typename Cx<T>::V* __restrict__ Ucd, const typename Cx<T>::V* __restrict__ Uvc,
     const typename Cx<T>::V* __restrict__ Ucc, int n, int nd, int nv, int nc, int nb1, int nch, int CPB, int KP,
