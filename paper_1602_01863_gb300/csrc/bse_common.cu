@@ -565,8 +565,37 @@ struct NearStencil {
     int nsteps, wrow, wbytes;                      // source rows, weights of one, shared memory of a warp
     int cols, t2, ntz, warps;                      // columns in use, 2 t, z tiles (of cz cells, the last ones smaller), all warps
     int cz;
+    int split;                                     // the source rows of a warp's targets go to the four warps of a block
     long long N2;                                  // 2 N: reals per chain of V
 };
+
+// Small grids (at most one warp per scheduler, so cz = 1) wait out the latency of a
+// source row nsteps times in a row: there the four warps of a block take a quarter of
+// the rows of the same targets each and their sums are added in warp order.
+// Coarse 4^3, n_div 2, 3x3 bands, 1 vector, FP64: 17.1 -> 10.1 us.
+__device__ __forceinline__ int2 near_steps(const NearStencil& s) {
+    if (!s.split) return make_int2(0, s.nsteps);
+    const int part = threadIdx.x >> 5;
+    return make_int2(part * s.nsteps / 4, (part + 1) * s.nsteps / 4);
+}
+// Adds the four warps' sums into warp 0's; false for the others, which are done.
+template <int N, typename E, typename Add>
+__device__ __forceinline__ bool near_gather(E (&acc)[N], unsigned char* red, Add add) {
+    E* r = reinterpret_cast<E*>(red);
+    const int part = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (part) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) r[((part - 1) * N + i) * 32 + lane] = acc[i];
+    }
+    __syncthreads();
+    if (part) return false;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) acc[i] = add(acc[i], r[(q * N + i) * 32 + lane]);
+    }
+    return true;
+}
 
 // Weights of one offset of one FP64 target row in the table: TZ values, padded
 // to what the loads below read.
@@ -580,11 +609,11 @@ struct NearWarp {
     T *wbuf, *wdst;
     const T* wsrc;
     int *xo, *yo;
-    __device__ NearWarp(T* buf, const T* Wt, int block, const NearStencil& s, int x0, int y0) {
+    __device__ NearWarp(T* buf, const T* Wt, int block, int step0, const NearStencil& s, int x0, int y0) {
         const int lane = threadIdx.x & 31;
         wbuf = buf;
         wdst = buf + lane * PER;
-        wsrc = Wt + (size_t)block * s.nsteps * s.wrow + lane * PER;
+        wsrc = Wt + ((size_t)block * s.nsteps + step0) * s.wrow + lane * PER;
         xo = reinterpret_cast<int*>(buf + 2 * s.wrow);
         yo = xo + 2 * s.R + 1;
         for (int i = lane; i <= 2 * s.R; i += 32) {
@@ -664,10 +693,11 @@ __device__ __forceinline__ void near_row(double (&acc)[TY][NT], const double* __
 template <int TY, int TZ, int CZ, int RM>
 __device__ __forceinline__ void near_body(const double* __restrict__ phi, const double* __restrict__ Wt,
                                           const int2* __restrict__ steps, double* __restrict__ Vn, const NearStencil& s, int g,
-                                          int cx, int cy, int cz0, int j1, int j2, int zb, double* wbuf) {
+                                          int cx, int cy, int cz0, int j1, int j2, int zb, double* wbuf, unsigned char* red) {
     constexpr int TZP = near_tzp<TZ>(), NT = CZ * TZ;
     const int lane = threadIdx.x & 31, nd = s.nd, R = s.R, wy = (2 * R + 1) * TZP;
-    NearWarp<double, TY> nw(wbuf, Wt, (zb * nd + j1) * s.njb + j2 / TY, s, cx * nd + j1, cy * nd + j2);
+    const int2 span = CZ == 1 ? near_steps(s) : make_int2(0, s.nsteps);
+    NearWarp<double, TY> nw(wbuf, Wt, (zb * nd + j1) * s.njb + j2 / TY, span.x, s, cx * nd + j1, cy * nd + j2);
     const double* base = phi + (size_t)g * s.L * s.L * s.Lp * 32 + (size_t)(cz0 * nd + zb * TZ + R) * 32 + lane;
     double acc[TY][NT];
 #pragma unroll
@@ -675,13 +705,13 @@ __device__ __forceinline__ void near_body(const double* __restrict__ phi, const 
 #pragma unroll
         for (int i = 0; i < NT; ++i) acc[y][i] = 0.0;
     }
-    int2 st = steps[0];
+    int2 st = steps[span.x];
     int cur = 0;                                                      // 0 or wrow: the buffer of this step's weights
     nw.fetch(0, s.wrow);
     __syncwarp();
-    for (int i = 0; i < s.nsteps; ++i) {
+    for (int i = span.x; i < span.y; ++i) {
         int2 nx = st;
-        if (i + 1 < s.nsteps) {
+        if (i + 1 < span.y) {
             nx = steps[i + 1];
             nw.fetch(s.wrow - cur, s.wrow);
         } else {
@@ -721,6 +751,11 @@ __device__ __forceinline__ void near_body(const double* __restrict__ phi, const 
         st = nx;
         cur = s.wrow - cur;
     }
+    if constexpr (CZ == 1)
+        if (s.split) {
+            double (&flat)[TY * NT] = reinterpret_cast<double (&)[TY * NT]>(acc);
+            if (!near_gather(flat, red, [](double a, double b) { return a + b; })) return;
+        }
     const int col = g * 32 + lane;
     if (col >= s.cols) return;
     const int ch = col / s.t2, q = col - ch * s.t2;
@@ -744,7 +779,8 @@ __global__ void __launch_bounds__(128, 3) k_common_near(const double* __restrict
                                                         const int2* __restrict__ steps, double* __restrict__ Vn, const NearStencil s) {
     extern __shared__ __align__(16) unsigned char smraw[];
     double* wbuf = reinterpret_cast<double*>(smraw + (size_t)(threadIdx.x >> 5) * s.wbytes);
-    int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    unsigned char* red = smraw + (size_t)4 * s.wbytes;
+    int w = s.split ? blockIdx.x : blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (w >= s.warps) return;
     // warp: (group, cx, cy, z tile, z block, j1, block of j2), the last fastest
     const int jb = w % s.njb; w /= s.njb;
@@ -754,11 +790,11 @@ __global__ void __launch_bounds__(128, 3) k_common_near(const double* __restrict
     const int cy = w % s.n; w /= s.n;
     const int cx = w % s.n, g = w / s.n;
     if constexpr (RM > 0) {
-        if (tile.y == 4) near_body<TY, TZ, 4, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf);
-        else if (tile.y == 2) near_body<TY, TZ, 2, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf);
-        else near_body<TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf);
+        if (tile.y == 4) near_body<TY, TZ, 4, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf, red);
+        else if (tile.y == 2) near_body<TY, TZ, 2, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf, red);
+        else near_body<TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf, red);
     } else {
-        near_body<TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf);
+        near_body<TY, TZ, 1, RM>(phi, Wt, steps, Vn, s, g, cx, cy, tile.x, j1, jb * TY, zb, wbuf, red);
     }
 }
 
@@ -814,21 +850,22 @@ __device__ __forceinline__ void near_row32(F2 (&acc)[NT], const float* __restric
 template <int TZ, int CZ, int RM>
 __device__ __forceinline__ void near_body32(const float* __restrict__ phi, const float* __restrict__ Wt,
                                             const int2* __restrict__ steps, float* __restrict__ Vn, const NearStencil& s, int g,
-                                            int X, int Y, int cz0, int zb, float* wbuf) {
+                                            int X, int Y, int cz0, int zb, float* wbuf, unsigned char* red) {
     constexpr int NT = CZ * TZ;
     const int lane = threadIdx.x & 31, nd = s.nd, R = s.R, cx = X / nd, j1 = X - cx * nd, cy = Y / nd, j2 = Y - cy * nd;
-    NearWarp<float, 2> nw(wbuf, Wt, (zb * nd + j1) * s.njb + (nd % 2 ? j2 : j2 / 2), s, X, Y);
+    const int2 span = CZ == 1 ? near_steps(s) : make_int2(0, s.nsteps);
+    NearWarp<float, 2> nw(wbuf, Wt, (zb * nd + j1) * s.njb + (nd % 2 ? j2 : j2 / 2), span.x, s, X, Y);
     const float* base = phi + (size_t)g * s.L * s.L * s.Lp * 32 + (size_t)(cz0 * nd + zb * TZ + R) * 32 + lane;
     F2 acc[NT];
 #pragma unroll
     for (int i = 0; i < NT; ++i) acc[i] = 0;                          // the pair (0.f, 0.f)
-    int2 st = steps[0];
+    int2 st = steps[span.x];
     int cur = 0;                                                      // 0 or wrow: the buffer of this step's weights
     nw.fetch(0, s.wrow);
     __syncwarp();
-    for (int i = 0; i < s.nsteps; ++i) {
+    for (int i = span.x; i < span.y; ++i) {
         int2 nx = st;
-        if (i + 1 < s.nsteps) {
+        if (i + 1 < span.y) {
             nx = steps[i + 1];
             nw.fetch(s.wrow - cur, s.wrow);
         } else {
@@ -864,6 +901,12 @@ __device__ __forceinline__ void near_body32(const float* __restrict__ phi, const
         st = nx;
         cur = s.wrow - cur;
     }
+    if constexpr (CZ == 1)
+        if (s.split && !near_gather(acc, red, [](F2 a, F2 b) {
+                const float2 x = *reinterpret_cast<const float2*>(&a), y = *reinterpret_cast<const float2*>(&b), z = cadd(x, y);
+                return *reinterpret_cast<const F2*>(&z);
+            }))
+            return;
     const int col = g * 32 + lane;
     if (col >= s.cols) return;
     const int ch = col / s.t2, q = col - ch * s.t2;
@@ -891,7 +934,8 @@ __global__ void __launch_bounds__(128, 5) k_common_near32(const float* __restric
                                                           const NearStencil s) {
     extern __shared__ __align__(16) unsigned char smraw[];
     float* wbuf = reinterpret_cast<float*>(smraw + (size_t)(threadIdx.x >> 5) * s.wbytes);
-    int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    unsigned char* red = smraw + (size_t)4 * s.wbytes;
+    int w = s.split ? blockIdx.x : blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (w >= s.warps) return;
     // warp: (group, z tile, z block, row X, pair of rows Y), the last fastest
     const int yb = w % s.nyb; w /= s.nyb;
@@ -900,11 +944,11 @@ __global__ void __launch_bounds__(128, 5) k_common_near32(const float* __restric
     const int2 tile = near_tile(s, w % s.ntz);
     const int g = w / s.ntz;
     if constexpr (RM > 0) {
-        if (tile.y == 4) near_body32<TZ, 4, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf);
-        else if (tile.y == 2) near_body32<TZ, 2, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf);
-        else near_body32<TZ, 1, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf);
+        if (tile.y == 4) near_body32<TZ, 4, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf, red);
+        else if (tile.y == 2) near_body32<TZ, 2, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf, red);
+        else near_body32<TZ, 1, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf, red);
     } else {
-        near_body32<TZ, 1, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf);
+        near_body32<TZ, 1, RM>(phi, Wt, steps, Vn, s, g, X, 2 * yb, tile.x, zb, wbuf, red);
     }
 }
 
@@ -967,8 +1011,11 @@ int rot_chains(const bse_ctx* ctx, const bse_interp* s, int nchains) {
     return s->co->nkc >= 2 * std::max(ctx->sm_count, 1) ? nchains : 1;
 }
 
+// `fixed`: at least the kernel's static shared memory.  Within the 48 KB that every
+// kernel has there is nothing to ask the driver for (2 to 4 us a launch).
 template <typename K>
-cudaError_t raise_smem(K kernel, size_t bytes) {
+cudaError_t raise_smem(K kernel, size_t bytes, size_t fixed) {
+    if (bytes + fixed <= 48 * 1024) return cudaSuccess;
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
     if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < bytes)
@@ -1013,12 +1060,13 @@ int launch_near_k(bse_ctx* ctx, const bse_interp* s, K kernel, int RM, NearStenc
     const long long warps = per_tile * ns.ntz;
     if (warps > 0x7fffffffLL) { ctx->err = "near stencil: too many targets"; return BSE_ERR_UNSUPPORTED; }
     ns.warps = (int)warps;
-    // small grids: fewer warps per block spread over more SMs
-    const int wpb = warps >= 8LL * ctx->sm_count ? 4 : 2;
+    // small grids: fewer warps per block spread over more SMs, or the rows of a warp over a block
     ns.wbytes = (int)((sizeof(T) * 2 * (size_t)ns.wrow + sizeof(int) * (4 * ns.R + 1 + near_ty<T>(ns.nd)) + 15) / 16 * 16);
-    const size_t smem = (size_t)ns.wbytes * wpb;
-    BSE_CUDA_TRY(ctx, raise_smem(kernel, smem));
-    kernel<<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, st>>>((const T*)s->d_cphi, (const T*)s->d_cw, s->d_csteps,
+    ns.split = ns.cz == 1 && warps <= 4LL * ctx->sm_count && ns.nsteps >= 8;
+    const int wpb = ns.split ? 4 : (warps >= 8LL * ctx->sm_count ? 4 : 2);
+    const size_t smem = (size_t)ns.wbytes * wpb + (ns.split ? 3 * 32 * sizeof(double) * near_ty<T>(ns.nd) * near_tz(ns.nd) : 0);
+    BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, 0));
+    kernel<<<(unsigned)(ns.split ? warps : (warps + wpb - 1) / wpb), 32 * wpb, smem, st>>>((const T*)s->d_cphi, (const T*)s->d_cw, s->d_csteps,
                                                                        (T*)s->d_cV, ns);
     BSE_CUDA_TRY(ctx, cudaGetLastError());
     return BSE_OK;
@@ -1063,7 +1111,7 @@ int restrict_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* p
     CommonPhi lay{s->cphi_R, s->cphi_Lp};
     const dim3 grid(c->nkc, (nchains + CPB - 1) / CPB);
     auto go = [&](auto kernel) -> int {
-        BSE_CUDA_TRY(ctx, raise_smem(kernel, smem));
+        BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, 64));
         kernel<<<grid, 256, smem, st>>>((const V*)psi, (const V*)s->d_cUv, (const V*)s->d_cUc, (const V*)s->d_cUvc,
                                         (const V*)s->d_cUcc, s->n, s->nd, s->nv, s->nc, s->nb1, nchains, CPB, KP,
                                         m3 ? (T*)s->d_cphi : nullptr, lay, (V*)s->d_cshare, s->d_cctr, (V*)Q, bop, c->ldk);
@@ -1083,7 +1131,7 @@ int prolong_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* R,
                         8 * WarpStage<T>::bytes(KP, s->nv, s->nc);
     const dim3 grid(bse_common_dot_blocks(s), (nchains + CPB - 1) / CPB);
     auto go = [&](auto kernel) -> int {
-        BSE_CUDA_TRY(ctx, raise_smem(kernel, smem));
+        BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, sizeof(V) * BSE_MAX_CHAINS * 256));
         kernel<<<grid, 256, smem, st>>>((const V*)R, s->scheme == BSE_SCHEME_M3 ? (const V*)s->d_cV : nullptr,
                                         (const V*)s->d_cUv, (const V*)s->d_cUc, (const V*)s->d_cUvc, (const V*)s->d_cUcc,
                                         (const T*)s->d_dE, (const V*)psi, s->n, s->nd, s->nv, s->nc, s->nb1, nchains, CPB, KP,
