@@ -100,7 +100,11 @@ int bse_ctx_create(bse_ctx** out, int device, void* cuda_stream) {
         ctx->own_stream = true;
     }
     cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device);
-    if (bse_alloc(ctx, (void**)&ctx->d_status, sizeof(int), "status word") != BSE_OK) {
+    if (bse_alloc(ctx, (void**)&ctx->d_status, sizeof(int), "status word") != BSE_OK ||
+        cudaHostAlloc((void**)&ctx->h_status, sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(ctx->d_status);
+        if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
         delete ctx;
         return BSE_ERR_OOM;
     }
@@ -112,6 +116,7 @@ int bse_ctx_create(bse_ctx** out, int device, void* cuda_stream) {
     if (bse_noalloc_prepare(ctx) != BSE_OK || bse_prepare_aux(ctx) != BSE_OK) {
         bse_release_ctx_state(ctx);
         cudaFree(ctx->d_status);
+        cudaFreeHost(ctx->h_status);
         if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
         delete ctx;
         return BSE_ERR_CUDA;
@@ -124,6 +129,7 @@ void bse_ctx_destroy(bse_ctx* ctx) {
     if (!ctx) return;
     bse_release_ctx_state(ctx);
     cudaFree(ctx->d_status);
+    cudaFreeHost(ctx->h_status);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
 }

@@ -114,6 +114,7 @@ struct bse_ctx {
     bool own_stream = false;          // created by the context (caller passed NULL)
     std::string err;
     int* d_status = nullptr;          // device status word: bit value 1 / 2 = a bounded wait gave up in the K_c apply / near field
+    int* h_status = nullptr;          // page-locked copy of it
     double kt_ms[KC_COUNT] = {0, 0, 0, 0, 0};
     long long kt_n[KC_COUNT] = {0, 0, 0, 0, 0};
     int sm_count = 0;
