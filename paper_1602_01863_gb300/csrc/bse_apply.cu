@@ -1103,33 +1103,63 @@ __device__ inline double2 block_sum2(double2 v, double2* sh) {
     return r;
 }
 
-// a_i = Re sum(partials), one block per chain; the imaginary part is kept as a
+// The Lanczos coefficients are sums of a few hundred block partials: every block of
+// the kernel that needs one forms it itself, in the same order as the others, and
+// block 0 stores it (a launch of one block per chain for each took 3 to 5 us of a step);
+// each chain has blocks of its own then, so that the sums of the chains run side by side.
+
+// a_i = Re sum(partials) by a block of 256 threads; the imaginary part is kept as a
 // Hermiticity diagnostic.
-__global__ void k_reduce_a(const double2* __restrict__ part, int nblk, int step, int m,
-                           double* __restrict__ a, double* __restrict__ aim, const int* __restrict__ stop) {
-    __shared__ double2 sh[256];
-    const int ch = blockIdx.x;
-    if (stop[ch]) return;
+__device__ __forceinline__ double block_a(const double2* __restrict__ dot, int ndot, int ch, int step, int m,
+                                          double* __restrict__ a, double* __restrict__ aim, double2* sh) {
     double2 s = make_double2(0.0, 0.0);
-    for (int i = threadIdx.x; i < nblk; i += blockDim.x) s = cadd(s, part[(size_t)ch * BSE_MAX_VEC_BLOCKS + i]);
+    for (int i = threadIdx.x; i < ndot; i += blockDim.x) s = cadd(s, dot[(size_t)ch * BSE_MAX_VEC_BLOCKS + i]);
     s = block_sum2(s, sh);
-    if (threadIdx.x == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         a[ch * m + step] = s.x;
         aim[ch * m + step] = s.y;
     }
+    return s.x;
+}
+
+// b_{i+1} = sqrt(sum partials) by a block of 256 threads; breakdown (true) when
+// b_{i+1} < 1e-12 max_j |a_j|.  Block 0 stores both.
+__device__ __forceinline__ bool block_b(const double* __restrict__ part, int nblk, int ch, int step, int m,
+                                        const double* __restrict__ a, double* __restrict__ b, int* __restrict__ stop,
+                                        double2* sh, double& bn) {
+    double s = 0.0, am = 0.0;
+    for (int i = threadIdx.x; i < nblk; i += blockDim.x) s += part[(size_t)ch * BSE_MAX_VEC_BLOCKS + i];
+    for (int j = threadIdx.x; j <= step; j += blockDim.x) am = fmax(am, fabs(a[ch * m + j]));
+    const double2 r = block_sum2(make_double2(s, 0.0), sh);
+    // block maximum of |a_j| (the second component of sh is free)
+    sh[threadIdx.x].y = am;
+    __syncthreads();
+    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+        if (threadIdx.x < o) sh[threadIdx.x].y = fmax(sh[threadIdx.x].y, sh[threadIdx.x + o].y);
+        __syncthreads();
+    }
+    bn = sqrt(r.x);
+    const bool down = !(bn >= 1e-12 * sh[0].y);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        b[ch * (m + 1) + step + 1] = bn;
+        if (down) stop[ch] = step + 1;
+    }
+    __syncthreads();
+    return down;
 }
 
 // w <- w - a_i psi_i - b_i psi_{i-1}; block partials of ||w||^2.
 template <typename T>
 __global__ void __launch_bounds__(BSE_VEC_THREADS) k_lanczos_axpy(
     typename Cx<T>::V* __restrict__ W, const typename Cx<T>::V* __restrict__ psi,
-    const typename Cx<T>::V* __restrict__ psi_prev, const double* __restrict__ a, const double* __restrict__ b,
-    int step, int m, int N, int nchains, double* __restrict__ part, const int* __restrict__ stop) {
+    const typename Cx<T>::V* __restrict__ psi_prev, const double2* __restrict__ dot, int ndot, double* __restrict__ a,
+    double* __restrict__ aim, const double* __restrict__ b, int step, int m, int N, int nchains, double* __restrict__ part,
+    const int* __restrict__ stop) {
     using V = typename Cx<T>::V;
     __shared__ double2 sh[BSE_VEC_THREADS];
-    for (int ch = 0; ch < nchains; ++ch) {
+    for (int ch = blockIdx.y; ch < nchains; ch += gridDim.y) {
         if (stop[ch]) continue;
-        const double ai = a[ch * m + step];
+        const double ai = block_a(dot, ndot, ch, step, m, a, aim, sh);
         const double bi = b[ch * (m + 1) + step];
         double nrm = 0.0;
         for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < N; g += gridDim.x * blockDim.x) {
@@ -1248,15 +1278,17 @@ inline int cgs_dot_blocks(const bse_ctx* ctx, int N, int nvec) {
 // these kernels.
 // w <- w - a_i psi_i - b_i psi_{i-1}; block partials of ||w||^2 (every chain in one pass).
 __global__ void __launch_bounds__(256) k_lanczos_axpy4(float4* __restrict__ W, const float4* __restrict__ psi,
-                                                       const float4* __restrict__ psi_prev, const double* __restrict__ a,
+                                                       const float4* __restrict__ psi_prev, const double2* __restrict__ dot,
+                                                       int ndot, double* __restrict__ a, double* __restrict__ aim,
                                                        const double* __restrict__ b, int step, int m, int N4,
                                                        int nchains, double* __restrict__ part,
                                                        const int* __restrict__ stop) {
+    __shared__ double2 sh[256];
     __shared__ double red[BSE_MAX_CHAINS][8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int ch = 0; ch < nchains; ++ch) {
+    for (int ch = blockIdx.y; ch < nchains; ch += gridDim.y) {
         const bool run = !stop[ch];
-        const float ai = (float)a[ch * m + step], bi = (float)b[ch * (m + 1) + step];
+        const float ai = run ? (float)block_a(dot, ndot, ch, step, m, a, aim, sh) : 0.f, bi = (float)b[ch * (m + 1) + step];
         float nrm = 0.f;
         if (run)
             for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < N4; g += gridDim.x * blockDim.x) {
@@ -1274,7 +1306,7 @@ __global__ void __launch_bounds__(256) k_lanczos_axpy4(float4* __restrict__ W, c
         if (lane == 0) red[ch][warp] = ws;
     }
     __syncthreads();
-    if (threadIdx.x < nchains && !stop[threadIdx.x]) {
+    if (threadIdx.x < nchains && threadIdx.x % gridDim.y == blockIdx.y && !stop[threadIdx.x]) {
         double s = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[threadIdx.x][w];
         part[(size_t)threadIdx.x * BSE_MAX_VEC_BLOCKS + blockIdx.x] = s;
@@ -1293,6 +1325,8 @@ __global__ void __launch_bounds__(256) k_lanczos_axpy4(float4* __restrict__ W, c
 //  * the last block to finish (a counter that it resets) sums the block
 //    partials in FP64 in a fixed order into b_{i+1} and applies the breakdown
 //    test b_{i+1} < 1e-12 max_j |a_j|.
+// N = 524288, 3 chains (50 MB): 28 us with one warp summing a_i chain after chain before the
+// first vector load and half the entries in flight, 15.7 us so.
 template <int NCH>
 __global__ void __launch_bounds__(512) k_lanczos_axpy4_ab(float4* __restrict__ W, const float4* __restrict__ psi,
                                                           const float4* __restrict__ psi_prev,
@@ -1411,18 +1445,31 @@ __global__ void __launch_bounds__(512) k_lanczos_axpy4_ab(float4* __restrict__ W
     if (threadIdx.x == 0) *ctr = 0;
 }
 
-// psi_{i+1} = w / b_{i+1} (written over psi_{i-1}), also into the basis when kept.
+// psi_{i+1} = w / b_{i+1} (written over psi_{i-1}), also into the basis when kept.  b_{i+1}
+// from the nblk partials of ||w||^2 (0: it is there already).  Block 0 may store a breakdown
+// while others start: they skip the chain by the stop word or by the same test.
 __global__ void __launch_bounds__(256) k_lanczos_scale4(const float4* __restrict__ W, float4* __restrict__ out,
-                                                        const double* __restrict__ b, int step, int m, int N4,
+                                                        const double* __restrict__ part, int nblk, const double* __restrict__ a,
+                                                        double* __restrict__ b, int step, int m, int N4,
                                                         int nchains, float4* __restrict__ basis, int mb,
-                                                        const int* __restrict__ stop) {
+                                                        int* __restrict__ stop) {
     // 1 / b_{i+1} once per block (FP64 is slow per element on GB300)
     __shared__ float inv_sh[BSE_MAX_CHAINS];
-    if (threadIdx.x < nchains) inv_sh[threadIdx.x] = (float)(1.0 / b[threadIdx.x * (m + 1) + step + 1]);
+    __shared__ int stop_sh[BSE_MAX_CHAINS];
+    __shared__ double2 sh[256];
+    if (threadIdx.x < nchains) {
+        stop_sh[threadIdx.x] = stop[threadIdx.x];
+        if (!nblk) inv_sh[threadIdx.x] = (float)(1.0 / b[threadIdx.x * (m + 1) + step + 1]);
+    }
     __syncthreads();
-    for (int ch = 0; ch < nchains; ++ch) {
-        if (stop[ch]) continue;
-        const float inv = inv_sh[ch];
+    for (int ch = blockIdx.y; ch < nchains; ch += gridDim.y) {
+        if (stop_sh[ch]) continue;
+        float inv = inv_sh[ch];
+        if (nblk) {
+            double bn;
+            if (block_b(part, nblk, ch, step, m, a, b, stop, sh, bn)) continue;
+            inv = (float)(1.0 / bn);
+        }
         for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < N4; g += gridDim.x * blockDim.x) {
             const float4 w = W[(size_t)ch * N4 + g];
             const float4 v = make_float4(w.x * inv, w.y * inv, w.z * inv, w.w * inv);
@@ -1432,39 +1479,33 @@ __global__ void __launch_bounds__(256) k_lanczos_scale4(const float4* __restrict
     }
 }
 
-// b_{i+1} = sqrt(sum partials); breakdown when b_{i+1} < 1e-12 max_j |a_j|.
-__global__ void k_reduce_b(const double* __restrict__ part, int nblk, int step, int m, const double* __restrict__ a,
-                           double* __restrict__ b, int* __restrict__ stop) {
+// b_{i+1} by itself, for a convergence check before the scale: one launch of a block per chain in turn.
+__global__ void __launch_bounds__(256) k_reduce_b(const double* __restrict__ part, int nblk, int nchains, int step, int m,
+                                                  const double* __restrict__ a, double* __restrict__ b, int* __restrict__ stop) {
     __shared__ double2 sh[256];
-    const int ch = blockIdx.x;
-    if (stop[ch]) return;
-    double s = 0.0, am = 0.0;
-    for (int i = threadIdx.x; i < nblk; i += blockDim.x) s += part[(size_t)ch * BSE_MAX_VEC_BLOCKS + i];
-    for (int j = threadIdx.x; j <= step; j += blockDim.x) am = fmax(am, fabs(a[ch * m + j]));
-    const double2 r = block_sum2(make_double2(s, 0.0), sh);
-    // block maximum of |a_j| (the second component of sh is free)
-    sh[threadIdx.x].y = am;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x].y = fmax(sh[threadIdx.x].y, sh[threadIdx.x + o].y);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const double bn = sqrt(r.x);
-        b[ch * (m + 1) + step + 1] = bn;
-        if (!(bn >= 1e-12 * sh[0].y)) stop[ch] = step + 1;
+    for (int ch = 0; ch < nchains; ++ch) {
+        double bn;
+        if (!stop[ch]) block_b(part, nblk, ch, step, m, a, b, stop, sh, bn);
     }
 }
 
-// psi_{i+1} = w / b_{i+1} (written over psi_{i-1}), also into the basis when kept.
+// The same for any vector length and precision.
 template <typename T>
 __global__ void __launch_bounds__(BSE_VEC_THREADS) k_lanczos_scale(
-    const typename Cx<T>::V* __restrict__ W, typename Cx<T>::V* __restrict__ out, const double* __restrict__ b,
-    int step, int m, int N, int nchains, typename Cx<T>::V* __restrict__ basis, int mb, const int* __restrict__ stop) {
+    const typename Cx<T>::V* __restrict__ W, typename Cx<T>::V* __restrict__ out, const double* __restrict__ part, int nblk,
+    const double* __restrict__ a, double* __restrict__ b, int step, int m, int N, int nchains,
+    typename Cx<T>::V* __restrict__ basis, int mb, int* __restrict__ stop) {
     using V = typename Cx<T>::V;
-    for (int ch = 0; ch < nchains; ++ch) {
-        if (stop[ch]) continue;
-        const double inv = 1.0 / b[ch * (m + 1) + step + 1];
+    __shared__ int stop_sh[BSE_MAX_CHAINS];
+    __shared__ double2 sh[256];
+    if (threadIdx.x < nchains) stop_sh[threadIdx.x] = stop[threadIdx.x];
+    __syncthreads();
+    for (int ch = blockIdx.y; ch < nchains; ch += gridDim.y) {
+        if (stop_sh[ch]) continue;
+        double bn;
+        if (!nblk) bn = b[ch * (m + 1) + step + 1];
+        else if (block_b(part, nblk, ch, step, m, a, b, stop, sh, bn)) continue;
+        const double inv = 1.0 / bn;
         for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < N; g += gridDim.x * blockDim.x) {
             const double2 w = to_d2(W[(size_t)ch * N + g]);
             const V v = from_d2<V>(make_double2(w.x * inv, w.y * inv));
@@ -2066,6 +2107,7 @@ int enqueue_chains(bse_ctx* ctx, bse_interp* s, int nch, int m, bool reorth, boo
     const int mb = s->basis_m;
     // FP32 vectors with an even length: float4 update kernels, one float4 per thread and chain
     const bool vec4 = std::is_same<T, float>::value && (N % 2) == 0;
+    const int nbn = reorth ? cgs_blocks(N) : nb;               // block partials of ||w||^2 (not of the float4 update alone)
     const int nb4 = (int)std::min<long long>(std::max<long long>((N / 2 + 255) / 256, 1), BSE_MAX_VEC_BLOCKS);
     cudaMemsetAsync(s->d_stop, 0, sizeof(int) * BSE_MAX_CHAINS, st);
     // psi_1 = P / ||P|| in B, psi_0 = 0 in A
@@ -2090,12 +2132,12 @@ int enqueue_chains(bse_ctx* ctx, bse_interp* s, int nch, int m, bool reorth, boo
             else BSE_AXPY_AB(4);
 #undef BSE_AXPY_AB
         } else {
-        k_reduce_a<<<nch, 256, 0, st>>>(s->d_part_dot, dot_blocks(s), i, m, s->d_a, s->d_aim, s->d_stop);
         if (vec4)
-            k_lanczos_axpy4<<<nb4, 256, 0, st>>>((float4*)W, (const float4*)B, (const float4*)A, s->d_a, s->d_b, i, m,
-                                                 N / 2, nch, s->d_part_nrm, s->d_stop);
+            k_lanczos_axpy4<<<dim3(nb4, nch), 256, 0, st>>>((float4*)W, (const float4*)B, (const float4*)A, s->d_part_dot, dot_blocks(s),
+                                                 s->d_a, s->d_aim, s->d_b, i, m, N / 2, nch, s->d_part_nrm, s->d_stop);
         else
-            k_lanczos_axpy<T><<<nb, BSE_VEC_THREADS, 0, st>>>(W, B, A, s->d_a, s->d_b, i, m, N, nch, s->d_part_nrm, s->d_stop);
+            k_lanczos_axpy<T><<<dim3(nb, nch), BSE_VEC_THREADS, 0, st>>>(W, B, A, s->d_part_dot, dot_blocks(s), s->d_a, s->d_aim, s->d_b,
+                                                              i, m, N, nch, s->d_part_nrm, s->d_stop);
         if (reorth) {
             for (int pass = 0; pass < 2; ++pass) {
                 k_cgs_dots<T><<<dim3(cgs_dot_blocks(ctx, N, nch * (i + 1)), i + 1, nch), 256, 0, st>>>(
@@ -2103,8 +2145,9 @@ int enqueue_chains(bse_ctx* ctx, bse_interp* s, int nch, int m, bool reorth, boo
                 k_cgs_update<T><<<dim3(cgs_blocks(N), nch), 256, 0, st>>>(basis, W, s->d_cgs_h, i + 1, mb, N, s->d_part_nrm);
             }
         }
-        k_reduce_b<<<nch, 256, 0, st>>>(s->d_part_nrm, reorth ? cgs_blocks(N) : nb, i, m, s->d_a, s->d_b, s->d_stop);
+        if (rule) k_reduce_b<<<1, 256, 0, st>>>(s->d_part_nrm, nbn, nch, i, m, s->d_a, s->d_b, s->d_stop);
         }
+        const int nbs = (vec4 && !reorth) || rule ? 0 : nbn;    // partials left for the scale to sum
         if (rule && (i + 1) % rule->every == 0) {
             const int nblk = (rule->nw + kConvThreads - 1) / kConvThreads;
             k_conv_eval<<<dim3(nblk, nch), kConvThreads, 0, st>>>(s->d_a, s->d_b, i + 1, m, s->d_pn2, rule->pref, rule->eta,
@@ -2114,10 +2157,11 @@ int enqueue_chains(bse_ctx* ctx, bse_interp* s, int nch, int m, bool reorth, boo
                                               s->d_stop);
         }
         if (vec4)
-            k_lanczos_scale4<<<nb4, 256, 0, st>>>((const float4*)W, (float4*)A, s->d_b, i, m, N / 2, nch, (float4*)basis,
-                                                  mb, s->d_stop);
+            k_lanczos_scale4<<<dim3(nb4, nbs ? nch : 1), 256, 0, st>>>((const float4*)W, (float4*)A, s->d_part_nrm, nbs, s->d_a, s->d_b, i, m, N / 2,
+                                                  nch, (float4*)basis, mb, s->d_stop);
         else
-            k_lanczos_scale<T><<<nb, BSE_VEC_THREADS, 0, st>>>(W, A, s->d_b, i, m, N, nch, basis, mb, s->d_stop);
+            k_lanczos_scale<T><<<dim3(nb, nch), BSE_VEC_THREADS, 0, st>>>(W, A, s->d_part_nrm, nbs, s->d_a, s->d_b, i, m, N, nch, basis, mb,
+                                                               s->d_stop);
         std::swap(A, B);
         if (poll && rule && (i + 1) % rule->every == 0) {
             int stop[BSE_MAX_CHAINS] = {0, 0, 0, 0};

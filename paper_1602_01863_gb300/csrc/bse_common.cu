@@ -16,9 +16,9 @@
 // per (corner, corner) pair.  W depends on the sub-cell position and the
 // offset alone; set-up evaluates it once in FP64.
 // Measured on GB300, one H application, against the general kernels: coarse 8^3,
-// n_div 4, 4x4 bands, 3 vectors FP64 98.5 -> 9.45 ms; coarse 4^3, n_div 2, 3x3
-// bands, 1 vector FP64 1105 -> 140 us; coarse 7^3, n_div 3, 3x5 bands, 4 vectors
-// FP32 1.80 -> 0.44 ms.
+// n_div 4, 4x4 bands, 3 vectors FP64 98.5 -> 3.31 ms; coarse 4^3, n_div 2, 3x3
+// bands, 1 vector FP64 1105 -> 60 us; coarse 7^3, n_div 3, 3x5 bands, 4 vectors
+// FP32 1.80 -> 0.19 ms.
 // Caller-supplied overlaps (not a product through one basis) and non-Hermitian
 // generators keep the general kernels of bse_apply.cu and bse_near_tc.cu.
 #include <algorithm>
@@ -229,6 +229,7 @@ __device__ __forceinline__ T corner_weight(int j1, int j2, int j3, int l, int nd
 // blocks' order.  Memory latency and instruction issue bound it (it reads psi and U
 // and writes phi: 33 MB for coarse 8^3, n_div 4, 4x4 bands, 3 chains), so the warps of a
 // block wait for one another only at the sums and the chains share what they can.
+// Four FP32 blocks per SM (64 registers) hold 512 cells at once: 28 us, with three 31 us.
 template <typename T, bool OUT_BF16, int EPL>
 __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 4 : 2)) k_common_restrict(
     const typename Cx<T>::V* __restrict__ psi, const typename Cx<T>::V* __restrict__ Uvd,
@@ -804,7 +805,9 @@ __global__ void __launch_bounds__(128, 3) k_common_near(const double* __restrict
 // multiply-adds that it serves when each weight is stored twice for a packed complex
 // column: shared-memory bandwidth bounds this kernel, not the multiply-adds.  The
 // source is the operand to double, once per load.  Both rows take the larger reach
-// of the two (zero weights beyond their own).
+// of the two (zero weights beyond their own).  Coarse 8^3, n_div 4, 4x4 bands, 3 chains beside
+// the K_c apply: 130 us with weights stored twice, 122 us so, 110 us since the apply leaves it
+// registers (84 us alone); with 80 registers (six blocks per SM, all warps at once) 124 us.
 using F2 = unsigned long long;                                        // a register pair
 __device__ __forceinline__ F2 ffma2(F2 w, F2 v, F2 a) {
     F2 d;
