@@ -32,10 +32,9 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 N_OMEGA = 1000
-# DRAM bytes (read + write) of one near-field launch on this workload from the
-# committed ncu capture (profiles/k_near_tc_single_system.md: 428.7 + 56.5 MB),
-# or None when the kernel changed since the capture.
-NEAR_TRAFFIC = 485.2e6
+# DRAM bytes (read + write) of one near-stencil launch on this workload from an ncu
+# capture of that kernel (profiles/k_common_near32_single_system.md).
+NEAR_TRAFFIC = None
 
 
 def parse():
@@ -136,6 +135,14 @@ def algorithmic(sysd, nchains, kc_bytes_per_entry, vec_bytes):
         "restrict": {"bytes": dbytes + nchains * N * vec_bytes + nchains * Nk * nbar * t * vec_bytes},
         "prolong": {"bytes": dbytes + nchains * (3 * N * vec_bytes + Nk * nbar * t * vec_bytes) + N * vec_bytes / 2},
     }
+
+
+def near_field_offsets(nd, width):
+    """Dense offsets within the near region: |delta|^2 <= floor(width^2 n_div^2)."""
+    import math
+    R2 = math.floor(width * width * nd * nd + 1e-9)
+    r = int(math.floor(math.sqrt(R2) + 1e-12))
+    return sum(1 for a in range(-r, r + 1) for b in range(-r, r + 1) for c in range(-r, r + 1) if a * a + b * b + c * c <= R2)
 
 
 def near_field_work(nd, width, t, nchains, nkc, nb1=False):
@@ -262,20 +269,15 @@ def run_ours(args):
     peaks = json.load(open(peaks_path)) if os.path.exists(peaks_path) else {}
     hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
     peak_src = "measured" if "hbm_gbs" in peaks else "fallback"
-    # FP16 dense tensor peak (the near field's operands): the measured BF16 figure
-    # (FP16 and BF16 run at the same dense rate); sustained, since the kernel is
-    # timed inside a long Haydock run
-    f16_peak = float(peaks.get("bf16_tflops_sustained", 1700.0))
-    nfw = near_field_work(sysm.n_div, 1.0, info["nv"] * info["nc"], p, sysm.nk_coarse)
     if dom == "near_field":
-        achieved = nfw["useful_flops"] / (kt[dom][0] * 1e-3) / 1e12
-        roof = {"bound": "tensor", "kernel": "k_near_tc (M3 near field, tcgen05 FP16 operands, FP32 accumulation)",
-                "achieved": achieved, "peak": f16_peak, "unit": "TFLOP/s", "frac": achieved / f16_peak,
-                "traffic": NEAR_TRAFFIC,
-                "peak_source": f"{peak_src} bf16 sustained (FP16 dense rate = BF16)",
-                "flops": "useful flops of the factored near field per launch "
-                         f"({nfw['useful_flops'] / 1e9:.1f} GFLOP: stage 1 y1, z; head block once on y1 - h_c z)",
-                "issued_tflops": nfw["issued_flops"] / (kt[dom][0] * 1e-3) / 1e12}
+        # the scalar stencil in the common basis: one FP32 multiply-add per target column and near offset
+        flops = 2.0 * near_field_offsets(sysm.n_div, 1.0) * 2 * info["N"] * p
+        achieved = flops / (kt[dom][0] * 1e-3) / 1e12
+        fp32_peak = 2 * 128 * 152 * 2.07e-3                 # nominal: 128 FP32 multiply-adds per SM and clock at 2070 MHz
+        roof = {"bound": "fp32", "kernel": "k_common_near32 (M3 near pairs as a stencil in the common basis, packed FP32)",
+                "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s", "frac": achieved / fp32_peak,
+                "traffic": NEAR_TRAFFIC, "peak_source": "nominal FP32 rate (no measured one)",
+                "flops": f"one multiply-add per real column and near offset ({flops / 1e9:.2f} GFLOP per launch)"}
     else:
         achieved = alg[dom]["bytes"] / (kt[dom][0] * 1e-3) / 1e9
         roof = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
