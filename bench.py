@@ -32,9 +32,10 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 N_OMEGA = 1000
-# DRAM bytes (read + write) of one near-stencil launch on this workload from an ncu
-# capture of that kernel (profiles/k_common_near32_single_system.md).
-NEAR_TRAFFIC = None
+# DRAM bytes (read + write) of one near-stencil launch on this workload from the
+# committed ncu capture (profiles/k_common_single_system.md), or None when the
+# kernel changed since the capture.
+NEAR_TRAFFIC = 15.9e6
 
 
 def parse():
