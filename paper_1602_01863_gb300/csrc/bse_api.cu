@@ -24,7 +24,7 @@ template <typename P>
 int upload(bse_ctx* ctx, P** dst, const double* src, size_t ndouble, const char* what) {
     int rc = bse_alloc(ctx, (void**)dst, sizeof(double) * ndouble, what);
     if (rc != BSE_OK) return rc;
-    BSE_CUDA_TRY(ctx, cudaMemcpy(*dst, src, sizeof(double) * ndouble, cudaMemcpyHostToDevice));
+    BSE_CUDA_TRY(ctx, bse_upload(ctx, *dst, src, sizeof(double) * ndouble));
     return BSE_OK;
 }
 
@@ -108,7 +108,7 @@ int bse_ctx_create(bse_ctx** out, int device, void* cuda_stream) {
         delete ctx;
         return BSE_ERR_OOM;
     }
-    cudaMemset(ctx->d_status, 0, sizeof(int));
+    cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->stream);
     ctx->serial = bse_next_serial();
     // Load the library's device module and look up the no-allocation scratch
     // here, at set-up, so that bse_apply_h_noalloc never triggers the lazy
@@ -187,18 +187,18 @@ int bse_coarse_get_kc(bse_ctx* ctx, const bse_coarse* c, double* host_kc) {
     if (!ctx || !c || !host_kc) return BSE_ERR_ARG;
     const size_t Nc = c->Nc;
     if (c->kc_prec == BSE_PREC_F64) {
-        BSE_CUDA_TRY(ctx, cudaMemcpy(host_kc, c->d_kc, sizeof(double2) * Nc * Nc, cudaMemcpyDeviceToHost));
+        BSE_CUDA_TRY(ctx, bse_download(ctx, host_kc, c->d_kc, sizeof(double2) * Nc * Nc));
         return BSE_OK;
     }
     if (c->kc_prec == BSE_PREC_F32) {
         std::vector<float2> tmp(Nc * Nc);
-        BSE_CUDA_TRY(ctx, cudaMemcpy(tmp.data(), c->d_kc, sizeof(float2) * Nc * Nc, cudaMemcpyDeviceToHost));
+        BSE_CUDA_TRY(ctx, bse_download(ctx, tmp.data(), c->d_kc, sizeof(float2) * Nc * Nc));
         for (size_t i = 0; i < Nc * Nc; ++i) { host_kc[2 * i] = tmp[i].x; host_kc[2 * i + 1] = tmp[i].y; }
         return BSE_OK;
     }
     std::vector<__nv_bfloat16> re(Nc * c->ldk), im(Nc * c->ldk);
-    BSE_CUDA_TRY(ctx, cudaMemcpy(re.data(), c->d_kr, sizeof(__nv_bfloat16) * Nc * c->ldk, cudaMemcpyDeviceToHost));
-    BSE_CUDA_TRY(ctx, cudaMemcpy(im.data(), c->d_ki, sizeof(__nv_bfloat16) * Nc * c->ldk, cudaMemcpyDeviceToHost));
+    BSE_CUDA_TRY(ctx, bse_download(ctx, re.data(), c->d_kr, sizeof(__nv_bfloat16) * Nc * c->ldk));
+    BSE_CUDA_TRY(ctx, bse_download(ctx, im.data(), c->d_ki, sizeof(__nv_bfloat16) * Nc * c->ldk));
     for (size_t i = 0; i < Nc; ++i)
         for (size_t j = 0; j < Nc; ++j) {
             host_kc[2 * (i * Nc + j)] = (double)__bfloat162float(re[i * c->ldk + j]);
@@ -338,7 +338,7 @@ int bse_set_stop_rule(bse_ctx* ctx, double tol, int check_every, double s_eps, d
         int rc = bse_alloc(ctx, (void**)&ctx->d_stop_omega, sizeof(double) * nw, "stop-rule frequencies");
         if (rc != BSE_OK) return rc;
     }
-    BSE_CUDA_TRY(ctx, cudaMemcpy(ctx->d_stop_omega, omega, sizeof(double) * nw, cudaMemcpyHostToDevice));
+    BSE_CUDA_TRY(ctx, bse_upload(ctx, ctx->d_stop_omega, omega, sizeof(double) * nw));
     ctx->stop_nw = nw;
     ctx->stop_tol = tol;
     ctx->stop_every = check_every;

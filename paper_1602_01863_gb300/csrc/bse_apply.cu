@@ -2053,7 +2053,7 @@ int ensure_state(bse_ctx* ctx, bse_interp* s, int m, bool reorth, int nw) {
         if ((rc = bse_alloc(ctx, (void**)&s->d_dirs, sizeof(double) * 3 * BSE_MAX_CHAINS, "directions")) != BSE_OK) return rc;
         if ((rc = bse_alloc(ctx, (void**)&s->d_pn2, sizeof(double) * BSE_MAX_CHAINS, "norms")) != BSE_OK) return rc;
         if ((rc = bse_alloc(ctx, (void**)&s->d_lz_ctr, sizeof(int), "Lanczos counter")) != BSE_OK) return rc;
-        BSE_CUDA_TRY(ctx, cudaMemset(s->d_lz_ctr, 0, sizeof(int)));
+        BSE_CUDA_TRY(ctx, cudaMemsetAsync(s->d_lz_ctr, 0, sizeof(int), ctx->stream));
     }
     if (s->m_alloc < m) {
         drop_graph(s);
@@ -2075,7 +2075,7 @@ int ensure_state(bse_ctx* ctx, bse_interp* s, int m, bool reorth, int nw) {
         if ((rc = bse_alloc(ctx, (void**)&s->d_cgs_part, sizeof(double2) * nv * 64, "CGS partials")) != BSE_OK) return rc;
         if ((rc = bse_alloc(ctx, (void**)&s->d_cgs_h, sizeof(double2) * nv, "CGS coefficients")) != BSE_OK) return rc;
         if ((rc = bse_alloc(ctx, (void**)&s->d_cgs_ctr, sizeof(int) * nv, "CGS counters")) != BSE_OK) return rc;
-        BSE_CUDA_TRY(ctx, cudaMemset(s->d_cgs_ctr, 0, sizeof(int) * nv));
+        BSE_CUDA_TRY(ctx, cudaMemsetAsync(s->d_cgs_ctr, 0, sizeof(int) * nv, ctx->stream));
         s->basis_m = m + 1;
     }
     if (nw > s->eps_nw) {
@@ -2208,14 +2208,14 @@ int finish_run(bse_ctx* ctx, bse_interp* s, int nch, int m, double* a, double* b
 int check_status(bse_ctx* ctx, int status) {
     if (status != 0) {
         ctx->err = bse_timeout_message(status);
-        cudaMemset(ctx->d_status, 0, sizeof(int));
+        cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->stream);
         return BSE_ERR_TIMEOUT;
     }
     return BSE_OK;
 }
 int read_status(bse_ctx* ctx) {
     int status = 0;
-    BSE_CUDA_TRY(ctx, cudaMemcpy(&status, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost));
+    BSE_CUDA_TRY(ctx, bse_download(ctx, &status, ctx->d_status, sizeof(int)));
     return check_status(ctx, status);
 }
 

@@ -1197,7 +1197,7 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s) {
         }
     s->n_csteps = (int)steps.size();
     if ((rc_ = bse_alloc(ctx, (void**)&s->d_csteps, sizeof(int2) * steps.size(), "near stencil rows")) != BSE_OK) return rc_;
-    BSE_CUDA_TRY(ctx, cudaMemcpy(s->d_csteps, steps.data(), sizeof(int2) * steps.size(), cudaMemcpyHostToDevice));
+    BSE_CUDA_TRY(ctx, bse_upload(ctx, s->d_csteps, steps.data(), sizeof(int2) * steps.size()));
     const int nzb = (nd + TZ - 1) / TZ, njb = near_njb<T>(nd), wrow = near_wrow<T>(nd, R);
     const long long nw = (long long)nzb * nd * njb * s->n_csteps * wrow;
     if ((rc_ = bse_alloc(ctx, &s->d_cw, sizeof(T) * (size_t)nw, "near stencil weights")) != BSE_OK) return rc_;

@@ -283,6 +283,20 @@ int bse_noalloc_prepare(bse_ctx* ctx);
 
 int bse_alloc(bse_ctx* ctx, void** p, size_t bytes, const char* what);
 
+// Copies between host and device in order with the context's kernels, finished on
+// return.  cudaMemcpy and cudaMemset run on the legacy default stream, which a
+// non-blocking stream of the caller's (any torch.cuda.Stream) does not wait for.
+inline cudaError_t bse_copy(bse_ctx* ctx, void* dst, const void* src, size_t bytes, cudaMemcpyKind kind) {
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, kind, ctx->stream);
+    return e == cudaSuccess ? cudaStreamSynchronize(ctx->stream) : e;
+}
+inline cudaError_t bse_upload(bse_ctx* ctx, void* dst, const void* src, size_t bytes) {
+    return bse_copy(ctx, dst, src, bytes, cudaMemcpyHostToDevice);
+}
+inline cudaError_t bse_download(bse_ctx* ctx, void* dst, const void* src, size_t bytes) {
+    return bse_copy(ctx, dst, src, bytes, cudaMemcpyDeviceToHost);
+}
+
 // Status word bits raised by bounded device waits: 1 = tensor-core K_c apply,
 // 2 = tensor-core near field.
 inline const char* bse_timeout_message(int status) {

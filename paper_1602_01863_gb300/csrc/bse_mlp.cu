@@ -975,9 +975,9 @@ int bse_mlp_create(bse_ctx* ctx, int d_in, int max_batch, const float* init_para
     A((void**)&m->d_gpart, sizeof(float) * (size_t)m->blocks * np, "gradient shares");
     A((void**)&m->d_part, sizeof(double) * m->blocks, "loss partials");
     if (rc != BSE_OK) { free_mlp(m); return rc; }
-    cudaMemcpy(m->d_p, init_params, sizeof(float) * np, cudaMemcpyHostToDevice);
-    cudaMemset(m->d_m, 0, sizeof(float) * np);
-    cudaMemset(m->d_v, 0, sizeof(float) * np);
+    bse_upload(ctx, m->d_p, init_params, sizeof(float) * np);
+    cudaMemsetAsync(m->d_m, 0, sizeof(float) * np, ctx->stream);
+    cudaMemsetAsync(m->d_v, 0, sizeof(float) * np, ctx->stream);
     k_to_bf16<<<(np + 255) / 256, 256, 0, ctx->stream>>>(m->d_p, np, m->d_w);
     if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) { free_mlp(m); ctx->err = "MLP set-up failed"; return BSE_ERR_CUDA; }
     *out = m;
@@ -988,7 +988,7 @@ void bse_mlp_free(bse_mlp* m) { free_mlp(m); }
 
 int bse_mlp_get_params(bse_ctx* ctx, const bse_mlp* m, float* host) {
     if (!ctx || !m || !host) return BSE_ERR_ARG;
-    BSE_CUDA_TRY(ctx, cudaMemcpy(host, m->d_p, sizeof(float) * m->nparams, cudaMemcpyDeviceToHost));
+    BSE_CUDA_TRY(ctx, bse_download(ctx, host, m->d_p, sizeof(float) * m->nparams));
     return BSE_OK;
 }
 
@@ -1006,7 +1006,7 @@ int bse_mlp_gradients(bse_ctx* ctx, bse_mlp* m, int batch, const float* X, const
     if (batch < 1 || batch > m->max_batch) { ctx->err = "batch outside 1..max_batch"; return BSE_ERR_ARG; }
     int rc = mlp_grads(ctx, m, batch, X, Y, loss);
     if (rc != BSE_OK) return rc;
-    BSE_CUDA_TRY(ctx, cudaMemcpy(grad_host, m->d_g, sizeof(float) * m->nparams, cudaMemcpyDeviceToHost));
+    BSE_CUDA_TRY(ctx, bse_download(ctx, grad_host, m->d_g, sizeof(float) * m->nparams));
     return BSE_OK;
 }
 
@@ -1040,8 +1040,9 @@ int bse_pairs_generate(bse_ctx* ctx, const bse_interp* s, int nblocks, const int
     int rc;
     if ((rc = bse_alloc(ctx, (void**)&d1, sizeof(int) * nblocks, "pair indices")) != BSE_OK) return rc;
     if ((rc = bse_alloc(ctx, (void**)&d2, sizeof(int) * nblocks, "pair indices")) != BSE_OK) { cudaFree(d1); return rc; }
-    cudaMemcpy(d1, host_kd, sizeof(int) * nblocks, cudaMemcpyHostToDevice);
-    cudaMemcpy(d2, host_kd2, sizeof(int) * nblocks, cudaMemcpyHostToDevice);
+    // the caller's arrays outlive the wait below
+    cudaMemcpyAsync(d1, host_kd, sizeof(int) * nblocks, cudaMemcpyHostToDevice, ctx->stream);
+    cudaMemcpyAsync(d2, host_kd2, sizeof(int) * nblocks, cudaMemcpyHostToDevice, ctx->stream);
     const int d_in = 6 + 2 * s->t;
     const size_t sm = pairs_smem(s->nv, s->nc);
     auto go = [&](auto tag) -> int {
@@ -1117,9 +1118,10 @@ int bse_interp_set_learned(bse_ctx* ctx, bse_interp* s, bse_mlp* m, int radius) 
         tw[j] = make_float2((float)std::cos(ang), (float)-std::sin(ang));          // forward: exp(-2 pi i j / L)
         tw[L + j] = make_float2((float)std::cos(ang), (float)std::sin(ang));       // inverse: exp(+2 pi i j / L)
     }
-    cudaMemcpy(s->d_tw_fwd, tw.data(), sizeof(float2) * 2 * L, cudaMemcpyHostToDevice);
-    cudaMemcpy(d_offs, offs.data(), sizeof(int) * offs.size(), cudaMemcpyHostToDevice);
-    cudaMemcpy(d_neg, neg.data(), sizeof(int) * noff, cudaMemcpyHostToDevice);
+    // the vectors outlive the wait below (and cudaFree in `cleanup` waits too)
+    cudaMemcpyAsync(s->d_tw_fwd, tw.data(), sizeof(float2) * 2 * L, cudaMemcpyHostToDevice, ctx->stream);
+    cudaMemcpyAsync(d_offs, offs.data(), sizeof(int) * offs.size(), cudaMemcpyHostToDevice, ctx->stream);
+    cudaMemcpyAsync(d_neg, neg.data(), sizeof(int) * noff, cudaMemcpyHostToDevice, ctx->stream);
     if (s->vec_prec == BSE_PREC_F64) k_dE_avg<double><<<t, 256, 0, ctx->stream>>>((const double*)s->d_dE, s->nk, t, d_avg);
     else k_dE_avg<float><<<t, 256, 0, ctx->stream>>>((const float*)s->d_dE, s->nk, t, d_avg);
     // network inference over every (near offset, vc, v'c'), in chunks of max_batch rows

@@ -584,7 +584,7 @@ int bse_near_tc_prepare(bse_ctx* ctx, bse_interp* s, const std::vector<std::vect
     auto upload = [&](void** dst, const void* src, size_t bytes, const char* what) -> int {
         int rc = bse_alloc(ctx, dst, bytes, what);
         if (rc != BSE_OK) return rc;
-        BSE_CUDA_TRY(ctx, cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice));
+        BSE_CUDA_TRY(ctx, bse_upload(ctx, *dst, src, bytes));
         return BSE_OK;
     };
     int rc;

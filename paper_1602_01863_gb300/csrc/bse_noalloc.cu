@@ -118,9 +118,9 @@ extern "C" int bse_apply_h_noalloc(bse_ctx* ctx, bse_interp* s, int nvec, const 
         return BSE_ERR_CUDA;
     }
     int status = 0;
-    BSE_CUDA_TRY(ctx, cudaMemcpy(&status, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost));
+    BSE_CUDA_TRY(ctx, bse_download(ctx, &status, ctx->d_status, sizeof(int)));
     if (status) {
-        cudaMemset(ctx->d_status, 0, sizeof(int));
+        cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->stream);
         ctx->err = bse_timeout_message(status);
         return BSE_ERR_TIMEOUT;
     }

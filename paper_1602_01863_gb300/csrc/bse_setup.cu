@@ -794,8 +794,8 @@ int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dens
         }
         TRY(bse_alloc(ctx, (void**)&s->d_list, sizeof(NearEntry) * flat.size(), "near list"));
         TRY(bse_alloc(ctx, (void**)&s->d_list_start, sizeof(int) * start.size(), "near list starts"));
-        BSE_CUDA_TRY(ctx, cudaMemcpy(s->d_list, flat.data(), sizeof(NearEntry) * flat.size(), cudaMemcpyHostToDevice));
-        BSE_CUDA_TRY(ctx, cudaMemcpy(s->d_list_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice));
+        BSE_CUDA_TRY(ctx, bse_upload(ctx, s->d_list, flat.data(), sizeof(NearEntry) * flat.size()));
+        BSE_CUDA_TRY(ctx, bse_upload(ctx, s->d_list_start, start.data(), sizeof(int) * start.size()));
         // Cell-batched form: the same contributions, with the source named by its
         // (js', corner) pair index, so one coarse cell's targets share a slot's
         // source rows staged in shared memory.
@@ -830,16 +830,16 @@ int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dens
                 TRY(bse_alloc(ctx, (void**)&s->d_pairs, sizeof(int) * pairs.size(), "near pairs"));
                 TRY(bse_alloc(ctx, (void**)&s->d_clist, sizeof(int) * clist.size(), "cell near list"));
                 TRY(bse_alloc(ctx, (void**)&s->d_cstart, sizeof(int) * cstart.size(), "cell near list starts"));
-                BSE_CUDA_TRY(ctx, cudaMemcpy(s->d_pairs, pairs.data(), sizeof(int) * pairs.size(), cudaMemcpyHostToDevice));
-                BSE_CUDA_TRY(ctx, cudaMemcpy(s->d_clist, clist.data(), sizeof(int) * clist.size(), cudaMemcpyHostToDevice));
-                BSE_CUDA_TRY(ctx, cudaMemcpy(s->d_cstart, cstart.data(), sizeof(int) * cstart.size(), cudaMemcpyHostToDevice));
+                BSE_CUDA_TRY(ctx, bse_upload(ctx, s->d_pairs, pairs.data(), sizeof(int) * pairs.size()));
+                BSE_CUDA_TRY(ctx, bse_upload(ctx, s->d_clist, clist.data(), sizeof(int) * clist.size()));
+                BSE_CUDA_TRY(ctx, bse_upload(ctx, s->d_cstart, cstart.data(), sizeof(int) * cstart.size()));
             }
         }
         int* d_offs = nullptr;
         double* d_hh = nullptr;
         TRY(bse_alloc(ctx, (void**)&d_offs, sizeof(int) * offs.size(), "near offsets"));
         TRY(bse_alloc(ctx, (void**)&d_hh, sizeof(double) * c->nkc, "coarse head table"));
-        BSE_CUDA_TRY(ctx, cudaMemcpy(d_offs, offs.data(), sizeof(int) * offs.size(), cudaMemcpyHostToDevice));
+        BSE_CUDA_TRY(ctx, bse_upload(ctx, d_offs, offs.data(), sizeof(int) * offs.size()));
         TRY(bse_alloc(ctx, &s->d_hd, sizeof(T) * s->n_near, "near head values"));
         TRY(bse_alloc(ctx, &s->d_Hv, sizeof(V) * (size_t)c->nkc * s->nrel * nv * nv, "Hv"));
         TRY(bse_alloc(ctx, &s->d_Hc, sizeof(V) * (size_t)c->nkc * s->nrel * nc * nc, "Hc"));
@@ -864,8 +864,8 @@ int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dens
             const float h4[4] = {xs, xs, xs, xs};
             TRY(bse_alloc(ctx, (void**)&s->d_xscale, sizeof(float) * 4, "piece scales"));
             TRY(bse_alloc(ctx, (void**)&s->d_xscale_gen, sizeof(float) * 4, "piece scales"));
-            BSE_CUDA_TRY(ctx, cudaMemcpy(s->d_xscale, h4, sizeof(h4), cudaMemcpyHostToDevice));
-            BSE_CUDA_TRY(ctx, cudaMemcpy(s->d_xscale_gen, h4, sizeof(h4), cudaMemcpyHostToDevice));
+            BSE_CUDA_TRY(ctx, bse_upload(ctx, s->d_xscale, h4, sizeof(h4)));
+            BSE_CUDA_TRY(ctx, bse_upload(ctx, s->d_xscale_gen, h4, sizeof(h4)));
         }
     }
     if (c->kc_prec == BSE_PREC_BF16) TRY(bse_tc_prepare(ctx, s));

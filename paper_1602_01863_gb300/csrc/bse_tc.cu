@@ -506,7 +506,7 @@ TcChoice tune(bse_ctx* ctx, bse_interp* s, TcState& st) {
     TcChoice best = {5, std::min(16, kb_row)};
     void* d_buf = nullptr;
     if (bse_alloc(ctx, &d_buf, bytes, "autotune partials") != BSE_OK) { cudaGetLastError(); return best; }
-    cudaMemset(d_buf, 0, bytes);
+    cudaMemsetAsync(d_buf, 0, bytes, ctx->stream);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -548,7 +548,7 @@ int bse_tc_prepare(bse_ctx* ctx, bse_interp* s) {
     int rc;
     if ((rc = bse_alloc(ctx, (void**)&s->d_Bop, sizeof(__nv_bfloat16) * BN * (size_t)c->ldk, "split-BF16 operand")) != BSE_OK)
         return rc;
-    BSE_CUDA_TRY(ctx, cudaMemset(s->d_Bop, 0, sizeof(__nv_bfloat16) * BN * (size_t)c->ldk));
+    BSE_CUDA_TRY(ctx, cudaMemsetAsync(s->d_Bop, 0, sizeof(__nv_bfloat16) * BN * (size_t)c->ldk, ctx->stream));
     TcState* st = new TcState();
     if ((rc = make_map(ctx, &st->map_kr, c->d_kr, c->ldk, c->Nc, BM)) != BSE_OK ||
         (rc = make_map(ctx, &st->map_ki, c->d_ki, c->ldk, c->Nc, BM)) != BSE_OK ||
@@ -564,7 +564,8 @@ int bse_tc_prepare(bse_ctx* ctx, bse_interp* s) {
         delete st;
         return rc;
     }
-    BSE_CUDA_TRY(ctx, cudaMemset(s->d_part, 0, p.bytes));
+    BSE_CUDA_TRY(ctx, cudaMemsetAsync(s->d_part, 0, p.bytes, ctx->stream));
+    BSE_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));      // the handle may be used by another context
     s->tc_ctas = p.ctas;
     s->tc_kblocks = p.sc.chunk_kb;
     s->tc_stages = p.stages;
