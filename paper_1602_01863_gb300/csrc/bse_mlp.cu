@@ -617,7 +617,9 @@ __global__ void __launch_bounds__(PTHR) k_pairs(
         const double2 kx = cscale(csub(cscale(ex, 2.0), cscale(cmul(O[v * nv + v2], O[rv + c * nc + c2]), hq * inv_eps)), e_k / nk);
         const double2 km1 = cscale(make_double2(K1[i].x, K1[i].y), 1.0 / Ndiv);
         const size_t row = (size_t)blk * t * t + i;
-        reinterpret_cast<float2*>(Y)[row] = make_float2((float)((kx.x - km1.x) * nk), (float)((kx.y - km1.y) * nk));
+        // one real at a time: the caller's Y need not lie on 8 bytes
+        Y[2 * row] = (float)((kx.x - km1.x) * nk);
+        Y[2 * row + 1] = (float)((kx.y - km1.y) * nk);
     }
     // features
     double q[4] = {0.0, 0.0, 0.0, 0.0};
