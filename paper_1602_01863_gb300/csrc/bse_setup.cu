@@ -108,11 +108,15 @@ __global__ void __launch_bounds__(256) k_form_factors(const double2* __restrict_
 //   K = pref [ 2 sum_G v(G) conj(M_i(G)) M_j(G) - O^v O^c h(k~_i - k~_j) / eps_inf ].
 // A block takes the entries of PT x PT coarse points (at most 64 x 64 entries),
 // on and above the diagonal only; each value is also written, conjugated, to
-// its mirror image.  FP64 bounds it (1.25 TFLOP/s on GB300), so the work per
-// entry is cut: the exchange sum takes three real products per G
-// (re = S1 + S2, im = S3 - S1 + S2 with S1 = sum a_r b_r, S2 = sum a_i b_i,
-// S3 = sum (a_r - a_i)(b_r + b_i), conj(a) b), the overlaps are formed once per pair
-// of points, and half of the matrix is never computed.  N_c = 8192, BF16: 26.1 ms
+// its mirror image; the diagonal is real.  FP64 bounds it (1.25 TFLOP/s on GB300), so
+// the work per entry is cut: the overlaps are formed once per pair of points, half of
+// the matrix is never computed, and where K_c is rounded to FP32 or BF16 the exchange
+// sum takes three real products per G (re = S1 + S2, im = S3 - S1 + S2 with
+// S1 = sum a_r b_r, S2 = sum a_i b_i, S3 = sum (a_r - a_i)(b_r + b_i), conj(a) b) and
+// not four.  Its imaginary part is a difference of larger sums: over random form
+// factors the error of the 64-bit sums is 2.1e-14 against 1.5e-14 of four products
+// (real part 1.2e-14 against 1.5e-14; sums up to 330), far below the rounding of either
+// storage, but not of complex128, which keeps four.  N_c = 8192, BF16: 26.1 ms
 // with one thread per entry of the whole matrix (a run of set-up, 24 steps and
 // spectrum: 58.7 ms; 17.3 ms with this set-up and the common-basis step loop).
 // Output in the storage precision of the handle.
@@ -171,7 +175,8 @@ __global__ void __launch_bounds__(256) k_build_kc(const double2* __restrict__ M,
         }
     }
     __syncthreads();
-    double s1[4][4], s2[4][4], s3[4][4];
+    constexpr bool three = PREC != BSE_PREC_F64;
+    double s1[4][4], s2[4][4], s3[4][4];                                     // S1, S2, S3, or the two parts
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -180,7 +185,7 @@ __global__ void __launch_bounds__(256) k_build_kc(const double2* __restrict__ M,
         for (int G = 0; G < 26; ++G) {
             double a[3][4], b[3][4];
 #pragma unroll
-            for (int w = 0; w < 3; ++w)
+            for (int w = 0; w < (three ? 3 : 2); ++w)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     a[w][i] = f[(w * 26 + G) * KC_T + ty + 16 * i];
@@ -190,9 +195,14 @@ __global__ void __launch_bounds__(256) k_build_kc(const double2* __restrict__ M,
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    s1[i][j] = fma(a[0][i], b[0][j], s1[i][j]);
-                    s2[i][j] = fma(a[1][i], b[1][j], s2[i][j]);
-                    s3[i][j] = fma(a[2][i], b[2][j], s3[i][j]);
+                    if constexpr (three) {
+                        s1[i][j] = fma(a[0][i], b[0][j], s1[i][j]);
+                        s2[i][j] = fma(a[1][i], b[1][j], s2[i][j]);
+                        s3[i][j] = fma(a[2][i], b[2][j], s3[i][j]);
+                    } else {
+                        s1[i][j] = fma(a[0][i], b[0][j], fma(a[1][i], b[1][j], s1[i][j]));
+                        s2[i][j] = fma(a[0][i], b[1][j], fma(-a[1][i], b[0][j], s2[i][j]));
+                    }
                 }
         }
     __syncthreads();
@@ -207,8 +217,8 @@ __global__ void __launch_bounds__(256) k_build_kc(const double2* __restrict__ M,
             if (q >= rj) continue;
             const int y = q / t, e2 = q - y * t, v2 = e2 / nc, c2 = e2 - v2 * nc, s = x * P + y;
             const double2 d = cscale(cmul(ov[s * nv * nv + v * nv + v2], oc[s * nc * nc + c * nc + c2]), hh[s]);
-            tile[r * (KC_T + 1) + q] = make_double2(pref * (2.0 * (s1[i][j] + s2[i][j]) - d.x),
-                                                    pref * (2.0 * (s3[i][j] - s1[i][j] + s2[i][j]) - d.y));
+            const double re = three ? s1[i][j] + s2[i][j] : s1[i][j], im = three ? s3[i][j] - s1[i][j] + s2[i][j] : s2[i][j];
+            tile[r * (KC_T + 1) + q] = make_double2(pref * (2.0 * re - d.x), pref * (2.0 * im - d.y));
         }
     }
     __syncthreads();
@@ -226,8 +236,9 @@ __global__ void __launch_bounds__(256) k_build_kc(const double2* __restrict__ M,
     const int col = tid & 63, row0 = tid >> 6;
     for (int r = row0; r < ri; r += 4)
         if (col < rj) {
-            // a diagonal tile keeps its upper half and mirrors it
-            const double2 v = diag && r > col ? conjg(tile[col * (KC_T + 1) + r]) : tile[r * (KC_T + 1) + col];
+            // a diagonal tile keeps its upper half and mirrors it; its diagonal is real
+            double2 v = diag && r > col ? conjg(tile[col * (KC_T + 1) + r]) : tile[r * (KC_T + 1) + col];
+            if (diag && r == col) v.y = 0.0;
             put((size_t)i0 + r, (size_t)j0 + col, v);
         }
     if (!diag)
