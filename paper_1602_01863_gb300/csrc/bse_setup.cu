@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(256) k_form_factors(const double2* __restrict_
 
 // K_c element (Eq. bse2 in the model, coarse weight e_k / n^3):
 //   K = pref [ 2 sum_G v(G) conj(M_i(G)) M_j(G) - O^v O^c h(k~_i - k~_j) / eps_inf ].
-// A block takes the entries of PT x PT coarse points (at most 64 x 64 entries),
+// A block takes the entries of P x P coarse points (at most 64 x 64 entries),
 // on and above the diagonal only; each value is also written, conjugated, to
 // its mirror image; the diagonal is real.  FP64 bounds it (1.25 TFLOP/s on GB300), so
 // the work per entry is cut: the overlaps are formed once per pair of points, half of
@@ -120,22 +120,30 @@ __global__ void __launch_bounds__(256) k_form_factors(const double2* __restrict_
 // with one thread per entry of the whole matrix (a run of set-up, 24 steps and
 // spectrum: 58.7 ms; 17.3 ms with this set-up and the common-basis step loop).
 // Output in the storage precision of the handle.
+// A tile is filled with as many points as 64 entries hold, so that no multiply-add is
+// spent on padding; only the pairs' overlaps of 1x1 bands have to leave some (54 points
+// of 64).  Coarse 16^3, 1x1 bands, the whole of bse_build_coarse: 5.8 ms with a thread per
+// entry, 74 ms with at most eight points to a tile (64 of 4096 entries used), 2.8 ms so.
 constexpr int KC_T = 64;
-__host__ __device__ inline int kc_points(int t) { const int p = KC_T / t; return p < 1 ? 1 : (p > 8 ? 8 : p); }
-size_t kc_smem(int nv, int nc) {
-    const int t = nv * nc, P = kc_points(t);
+constexpr size_t KC_SMEM = 200 * 1024;
+size_t kc_smem(int nv, int nc, int P) {
     const size_t forms = sizeof(double) * 6 * 26 * KC_T, tile = sizeof(double2) * KC_T * (KC_T + 1);
     return std::max(forms, tile) + sizeof(double2) * P * P * (nv * nv + nc * nc) + sizeof(double) * P * P;
+}
+int kc_points(int nv, int nc) {
+    int P = std::max(1, KC_T / (nv * nc));
+    while (P > 1 && kc_smem(nv, nc, P) > KC_SMEM) --P;
+    return P;
 }
 template <int PREC>
 __global__ void __launch_bounds__(256) k_build_kc(const double2* __restrict__ M, const double2* __restrict__ Uv,
                                                   const double2* __restrict__ Uc, const double* __restrict__ htab, int n,
-                                                  int nv, int nc, double pref, double inv_eps, int exchange_on, int Nc,
-                                                  int ldk, void* __restrict__ out, __nv_bfloat16* __restrict__ kr,
+                                                  int nv, int nc, int P, double pref, double inv_eps, int exchange_on,
+                                                  int Nc, int ldk, void* __restrict__ out, __nv_bfloat16* __restrict__ kr,
                                                   __nv_bfloat16* __restrict__ ki) {
     if (blockIdx.x < blockIdx.y) return;
     extern __shared__ __align__(16) unsigned char kcsm[];
-    const int t = nv * nc, P = kc_points(t), nkc = n * n * n, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int t = nv * nc, nkc = n * n * n, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int pa = blockIdx.y * P, pb = blockIdx.x * P, na = min(P, nkc - pa), nb = min(P, nkc - pb);
     const int i0 = pa * t, j0 = pb * t, ri = na * t, rj = nb * t;          // rows and columns of this tile
     double* f = reinterpret_cast<double*>(kcsm);                            // [6][26][KC_T] a_r v, a_i v, (a_r - a_i) v, b_r, b_i, b_r + b_i
@@ -548,13 +556,13 @@ int bse_setup_coarse_device(bse_ctx* ctx, bse_coarse* c, const void* user_kc) {
                               2 * (size_t)Nc, st);
     }
     const double pref = c->e_k / nkc;
-    const int kt = blocks_for(nkc, kc_points(nv * nc));
+    const int P = kc_points(nv, nc), kt = blocks_for(nkc, P);
     const dim3 gs(kt, kt);
-    const size_t ksm = kc_smem(nv, nc);
+    const size_t ksm = kc_smem(nv, nc, P);
     auto build = [&](auto kernel, void* out, __nv_bfloat16* kr, __nv_bfloat16* ki) -> int {
         int r = raise_smem(ctx, kernel, ksm);
         if (r != BSE_OK) return r;
-        kernel<<<gs, 256, ksm, st>>>(d_M, c->d_Uv, c->d_Uc, d_h, n, nv, nc, pref, 1.0 / c->eps_inf, c->exchange_on, Nc, c->ldk,
+        kernel<<<gs, 256, ksm, st>>>(d_M, c->d_Uv, c->d_Uc, d_h, n, nv, nc, P, pref, 1.0 / c->eps_inf, c->exchange_on, Nc, c->ldk,
                                      out, kr, ki);
         return BSE_OK;
     };
