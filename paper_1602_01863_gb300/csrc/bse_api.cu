@@ -24,7 +24,8 @@ template <typename P>
 int upload(bse_ctx* ctx, P** dst, const double* src, size_t ndouble, const char* what) {
     int rc = bse_alloc(ctx, (void**)dst, sizeof(double) * ndouble, what);
     if (rc != BSE_OK) return rc;
-    BSE_CUDA_TRY(ctx, bse_upload(ctx, *dst, src, sizeof(double) * ndouble));
+    // the caller's array outlives the set-up's wait (and cudaFree after an error waits too)
+    BSE_CUDA_TRY(ctx, cudaMemcpyAsync(*dst, src, sizeof(double) * ndouble, cudaMemcpyHostToDevice, ctx->stream));
     return BSE_OK;
 }
 

@@ -1,20 +1,23 @@
 // Small dense complex matrices (n <= BSE_MAX_BANDS, row-major double2 arrays in
-// shared memory) worked on by 16 lanes, shared by the set-up kernels (band
+// shared memory) worked on by G lanes, shared by the set-up kernels (band
 // gauge) and the pair-data kernel of the learned residual.
 #pragma once
 
 #include "bse_internal.cuh"
 
-constexpr int kGaugeLanes = 16;                     // lanes per matrix
+constexpr int kGaugeLanes = 16;                     // lanes per matrix, unless the bands are few
 constexpr int kGaugeMats = 6;                       // n x n matrices of scratch grp_gauge needs
 
-// The 16 lanes of the calling lane's half warp, as a sync mask, and its place among them.
-__device__ inline unsigned grp_mask() { return 0xffffu << (threadIdx.x & 16); }
-__device__ inline int grp_lane() { return threadIdx.x & 15; }
+// The G (a power of two) lanes that work with the calling lane, as a sync mask, and its place among them.
+template <int G = kGaugeLanes>
+__device__ inline unsigned grp_mask() { return (G == 32 ? 0xffffffffu : (1u << G) - 1u) << (threadIdx.x & 31 & ~(G - 1)); }
+template <int G = kGaugeLanes>
+__device__ inline int grp_lane() { return threadIdx.x & (G - 1); }
 
-// C = A B by 16 lanes, an entry per lane and round.
+// C = A B by G lanes, an entry per lane and round.
+template <int G>
 __device__ inline void grp_mul(const double2* A, const double2* B, double2* C, int n) {
-    for (int e = grp_lane(); e < n * n; e += kGaugeLanes) {
+    for (int e = grp_lane<G>(); e < n * n; e += G) {
         const int i = e / n, j = e - i * n;
         double2 s = make_double2(0.0, 0.0);
         for (int k = 0; k < n; ++k) {
@@ -24,22 +27,23 @@ __device__ inline void grp_mul(const double2* A, const double2* B, double2* C, i
         }
         C[e] = s;
     }
-    __syncwarp(grp_mask());
+    __syncwarp(grp_mask<G>());
 }
 
 // Band gauge U(k) = expm(i sum_a [sin(2 pi k_a) G_a0 + (1 - cos 2 pi k_a) G_a1]) from
-// sn[a] = sin(2 pi k_a), cs[a] = cos(2 pi k_a), by 16 lanes (a half warp); the
+// sn[a] = sin(2 pi k_a), cs[a] = cos(2 pi k_a), by G lanes; the
 // result's address (inside `work`, kGaugeMats n^2 entries of shared memory) is returned.
 // Scaling and squaring of the Taylor polynomial of degree 15 (||X||_F <= 1/2: the
 // remainder is below 1e-18), evaluated in powers of X^4 (Paterson-Stockmeyer): six
 // products and the squarings instead of one product per term, each with an
 // entry per lane: one thread per matrix spent 24 products in local memory.
+template <int G = kGaugeLanes>
 __device__ inline const double2* grp_gauge(const double2* gen, int n, const double* sn, const double* cs, double2* work) {
-    const int nn = n * n, ln = grp_lane();
-    const unsigned mask = grp_mask();
+    const int nn = n * n, ln = grp_lane<G>();
+    const unsigned mask = grp_mask<G>();
     double2 *X = work, *X2 = X + nn, *X3 = X2 + nn, *X4 = X3 + nn, *E = X4 + nn, *T = E + nn;
     double fro = 0.0;
-    for (int e = ln; e < nn; e += kGaugeLanes) {
+    for (int e = ln; e < nn; e += G) {
         double2 a = make_double2(0.0, 0.0);
         for (int ax = 0; ax < 3; ++ax) {
             const double2 g0 = gen[(ax * 2 + 0) * nn + e], g1 = gen[(ax * 2 + 1) * nn + e];
@@ -49,16 +53,16 @@ __device__ inline const double2* grp_gauge(const double2* gen, int n, const doub
         fro += a.x * a.x + a.y * a.y;
         X[e] = make_double2(-a.y, a.x);                       // i A
     }
-    for (int o = 8; o > 0; o >>= 1) fro += __shfl_xor_sync(mask, fro, o);
+    for (int o = G / 2; o > 0; o >>= 1) fro += __shfl_xor_sync(mask, fro, o);
     fro = sqrt(fro);
     int s = 0;
     while (fro > 0.5 && s < 1000) { fro *= 0.5; ++s; }
     const double sc = ldexp(1.0, -s);
-    for (int e = ln; e < nn; e += kGaugeLanes) X[e] = cscale(X[e], sc);
+    for (int e = ln; e < nn; e += G) X[e] = cscale(X[e], sc);
     __syncwarp(mask);
-    grp_mul(X, X, X2, n);
-    grp_mul(X2, X, X3, n);
-    grp_mul(X2, X2, X4, n);
+    grp_mul<G>(X, X, X2, n);
+    grp_mul<G>(X2, X, X3, n);
+    grp_mul<G>(X2, X2, X4, n);
     // E = B_3, then E <- X^4 E + B_j, B_j = sum_{i < 4} X^i / (4 j + i)!
     double inv[16];
     inv[0] = 1.0;
@@ -66,8 +70,8 @@ __device__ inline const double2* grp_gauge(const double2* gen, int n, const doub
     for (int k = 1; k < 16; ++k) inv[k] = inv[k - 1] / k;
 #pragma unroll
     for (int j = 3; j >= 0; --j) {
-        if (j < 3) grp_mul(X4, E, T, n);
-        for (int e = ln; e < nn; e += kGaugeLanes) {
+        if (j < 3) grp_mul<G>(X4, E, T, n);
+        for (int e = ln; e < nn; e += G) {
             double2 v = j < 3 ? T[e] : make_double2(0.0, 0.0);
             v = cadd(v, cadd(cadd(cscale(X3[e], inv[4 * j + 3]), cscale(X2[e], inv[4 * j + 2])), cscale(X[e], inv[4 * j + 1])));
             if (e / n == e % n) v.x += inv[4 * j];
@@ -76,7 +80,7 @@ __device__ inline const double2* grp_gauge(const double2* gen, int n, const doub
         __syncwarp(mask);
     }
     for (int q = 0; q < s; ++q) {
-        grp_mul(E, E, T, n);
+        grp_mul<G>(E, E, T, n);
         double2* x = E;
         E = T;
         T = x;

@@ -371,17 +371,24 @@ __global__ void k_cplx_to(const double2* __restrict__ src, long long n, V* __res
     if (i < n) dst[i] = from_d2<V>(src[i]);
 }
 
-// Dense tables, a warp per dense point kd: the gauge U(k) (a half warp per
+// Dense tables, 2 G lanes per dense point kd: the gauge U(k) (G lanes per
 // manifold), Delta E_vc(k) (exact on the dense mesh), dipoles
 // P^alpha_vc(k) = [U_v^T pi^alpha conj(U_c)], and, where the path reads them, U
 // itself in the vector precision (Uvt, Uct) or the overlaps d = U(k~)^H U(k) with
-// the 8 corners (Eq. completeness).  FP64 bounds it; everything stays in
-// shared memory: 32768 points of 4x4 bands took 4.4 ms with a thread per point.
+// the 8 corners (Eq. completeness).  FP64 bounds it, a warp instruction at a time
+// (16 clocks of an SM, idle lanes or not): sines and cosines come from a table of the L
+// values per axis, and few bands leave a warp to several points: G = 16 lanes from
+// 3 bands on, 4 for 2x2 and 1x2, 1 for 1x1.  Everything stays in shared memory:
+// 32768 points of 4x4 bands took 4.4 ms with a thread per point.  Set-up of a Method-1
+// handle, FP32, with a thread, with a warp per point, and so: 110592 points of 1x1 bands
+// 0.75, 2.1, 0.45 ms; 125000 of 2x2 bands 2.0, 2.7, 0.9 ms; 125000 of 1x3 bands 3.2, 3.7, 2.7 ms.
 constexpr int kDenseWarps = 4;
-size_t dense_smem(int nv, int nc) {
-    return sizeof(double2) * kDenseWarps * (kGaugeMats * (nv * nv + nc * nc) + 2 * 3 * nv * nc);
+int dense_lanes(int nv, int nc) { const int nb = std::max(nv, nc); return nb == 1 ? 1 : (nb == 2 ? 4 : kGaugeLanes); }
+size_t dense_smem(int nv, int nc, int L) {
+    const int points = kDenseWarps * (16 / dense_lanes(nv, nc));
+    return sizeof(double2) * ((size_t)points * (kGaugeMats * (nv * nv + nc * nc) + 2 * 3 * nv * nc) + L);
 }
-template <typename T>
+template <typename T, int G>
 __global__ void __launch_bounds__(32 * kDenseWarps) k_dense_tables(
     const double2* __restrict__ gen_v, const double2* __restrict__ gen_c, const double2* __restrict__ Uvc,
     const double2* __restrict__ Ucc, const double* __restrict__ offsets, const double2* __restrict__ dip, int n, int nd,
@@ -390,47 +397,50 @@ __global__ void __launch_bounds__(32 * kDenseWarps) k_dense_tables(
     double2* __restrict__ P) {
     using V = typename Cx<T>::V;
     extern __shared__ double2 dsm[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4;
+    constexpr int S = 2 * G, PB = 32 * kDenseWarps / S;              // lanes per point, points per block
+    const int sub = threadIdx.x / S, lane = threadIdx.x % S, half = lane / G, first = threadIdx.x & 31 & ~(S - 1);
+    const unsigned mask = grp_mask<S>();
     const int t = nv * nc, rv = nv * nv, rc = nc * nc, Ndiv = nd * nd * nd, nk = n * n * n * Ndiv, L = n * nd;
     const size_t N = (size_t)nk * t;
-    double2* work = dsm + (size_t)warp * (kGaugeMats * (rv + rc) + 6 * t);
+    double2* trig = dsm;                                               // [L] cos, sin of 2 pi x / L
+    double2* work = dsm + L + (size_t)sub * (kGaugeMats * (rv + rc) + 6 * t);
     double2* pa = work + kGaugeMats * (rv + rc);
     double2* pb = pa + 3 * t;
-    for (int kd = blockIdx.x * kDenseWarps + warp; kd < nk; kd += gridDim.x * kDenseWarps) {
+    for (int x = threadIdx.x; x < L; x += 32 * kDenseWarps) sincospi(2.0 * x / L, &trig[x].y, &trig[x].x);
+    __syncthreads();
+    for (int kd = blockIdx.x * PB + sub; kd < nk; kd += gridDim.x * PB) {
         const Int3 g = point_ints(kd, n, nd);
-        double sn[3], cs[3];
-        sincospi(2.0 * g.a / L, &sn[0], &cs[0]);
-        sincospi(2.0 * g.b / L, &sn[1], &cs[1]);
-        sincospi(2.0 * g.c / L, &sn[2], &cs[2]);
-        const double2* E = grp_gauge(half ? gen_c : gen_v, half ? nc : nv, sn, cs, half ? work + kGaugeMats * rv : work);
-        // both halves' results, by their places in the scratch
-        const int at = (int)(E - work), av = __shfl_sync(0xffffffffu, at, 0), ac = __shfl_sync(0xffffffffu, at, 16);
+        const double2 ta = trig[g.a], tb = trig[g.b], tc = trig[g.c];
+        const double sn[3] = {ta.y, tb.y, tc.y}, cs[3] = {ta.x, tb.x, tc.x};
+        const double2* E = grp_gauge<G>(half ? gen_c : gen_v, half ? nc : nv, sn, cs, half ? work + kGaugeMats * rv : work);
+        // both manifolds' results, by their places in the scratch
+        const int at = (int)(E - work), av = __shfl_sync(mask, at, first), ac = __shfl_sync(mask, at, first + G);
         const double2 *uv = work + av, *uc = work + ac;
-        __syncwarp();
+        __syncwarp(mask);
         double band = e_gap;
         for (int a = 0; a < 3; ++a) band += band_width * (1.0 - cs[a]);
-        for (int e = lane; e < t; e += 32) dE[(size_t)kd * t + e] = (T)(band + offsets[e]);
+        for (int e = lane; e < t; e += S) dE[(size_t)kd * t + e] = (T)(band + offsets[e]);
         if (Uvt) {
-            for (int e = lane; e < rv; e += 32) Uvt[(size_t)kd * rv + e] = from_d2<V>(uv[e]);
-            for (int e = lane; e < rc; e += 32) Uct[(size_t)kd * rc + e] = from_d2<V>(uc[e]);
+            for (int e = lane; e < rv; e += S) Uvt[(size_t)kd * rv + e] = from_d2<V>(uv[e]);
+            for (int e = lane; e < rc; e += S) Uct[(size_t)kd * rc + e] = from_d2<V>(uc[e]);
         }
-        for (int e = lane; e < 3 * t; e += 32) {
+        for (int e = lane; e < 3 * t; e += S) {
             double2 s = dip[e];
 #pragma unroll
             for (int a = 0; a < 3; ++a)
                 s = cadd(s, cadd(cscale(dip[(size_t)(1 + 2 * a) * 3 * t + e], cs[a]), cscale(dip[(size_t)(2 + 2 * a) * 3 * t + e], sn[a])));
             pa[e] = s;
         }
-        __syncwarp();
-        rotate_forms<false>(pa, uv, uc, pb, pa, 3, nv, nc, lane, 32, [] { __syncwarp(); });
-        for (int e = lane; e < 3 * t; e += 32) P[(size_t)(e / t) * N + (size_t)kd * t + e % t] = pa[e];
+        __syncwarp(mask);
+        rotate_forms<false>(pa, uv, uc, pb, pa, 3, nv, nc, lane, S, [mask] { __syncwarp(mask); });
+        for (int e = lane; e < 3 * t; e += S) P[(size_t)(e / t) * N + (size_t)kd * t + e % t] = pa[e];
         if (Dv) {
             const Int3 i = unflat3(kd / Ndiv, n);
             for (int l = 0; l < 8; ++l) {
                 const int cic = flat3(i.a + ((l >> 2) & 1), i.b + ((l >> 1) & 1), i.c + (l & 1), n);
                 const double2* cv = Uvc + (size_t)cic * rv;
                 const double2* cm = Ucc + (size_t)cic * rc;
-                for (int e = lane; e < rv + rc; e += 32) {
+                for (int e = lane; e < rv + rc; e += S) {
                     const bool val = e < rv;
                     const int q = val ? e : e - rv, nb = val ? nv : nc, np = q / nb, b = q - np * nb;
                     double2 s = make_double2(0.0, 0.0);
@@ -440,7 +450,7 @@ __global__ void __launch_bounds__(32 * kDenseWarps) k_dense_tables(
                 }
             }
         }
-        __syncwarp();
+        __syncwarp(mask);
     }
 }
 
@@ -491,8 +501,11 @@ __global__ void k_near_head(const int* __restrict__ offs, int n_near, int L, dou
     hd[i] = (T)(1.0 / (qa * qa + qb * qb + qc * qc + kappa * kappa));
 }
 
+// Within the 48 KB that every kernel has there is nothing to ask the driver for (these
+// kernels have no shared memory but the dynamic one).
 template <typename K>
 int raise_smem(bse_ctx* ctx, K kernel, size_t bytes) {
+    if (bytes <= 48 * 1024) return BSE_OK;
     cudaFuncAttributes fa;
     BSE_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, kernel));
     if ((size_t)fa.maxDynamicSharedSizeBytes < bytes)
@@ -743,11 +756,19 @@ int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dens
         TRY(bse_alloc(ctx, &s->d_Dv, sizeof(V) * (size_t)nk * 8 * nv * nv, "Dv"));
         TRY(bse_alloc(ctx, &s->d_Dc, sizeof(V) * (size_t)nk * 8 * nc * nc, "Dc"));
     }
-    const size_t dsm = dense_smem(nv, nc);
-    TRY(raise_smem(ctx, k_dense_tables<T>, dsm));
-    k_dense_tables<T><<<std::min(blocks_for(nk, kDenseWarps), 16 * std::max(ctx->sm_count, 1)), 32 * kDenseWarps, dsm, st>>>(
-        c->d_gen_v, c->d_gen_c, c->d_Uv, c->d_Uc, c->d_offsets, c->d_dip, n, nd, nv, nc, c->e_gap, c->band_width, (T*)s->d_dE,
-        (V*)s->d_Dv, (V*)s->d_Dc, (V*)s->d_cUv, (V*)s->d_cUc, s->d_P);
+    auto tables = [&](auto lanes) -> int {
+        constexpr int G = decltype(lanes)::value;
+        const size_t dsm = dense_smem(nv, nc, n * nd);
+        TRY(raise_smem(ctx, k_dense_tables<T, G>, dsm));
+        const int blocks = std::min(blocks_for(nk, kDenseWarps * (16 / G)), 16 * std::max(ctx->sm_count, 1));
+        k_dense_tables<T, G><<<blocks, 32 * kDenseWarps, dsm, st>>>(
+            c->d_gen_v, c->d_gen_c, c->d_Uv, c->d_Uc, c->d_offsets, c->d_dip, n, nd, nv, nc, c->e_gap, c->band_width,
+            (T*)s->d_dE, (V*)s->d_Dv, (V*)s->d_Dc, (V*)s->d_cUv, (V*)s->d_cUc, s->d_P);
+        return BSE_OK;
+    };
+    const int lanes = dense_lanes(nv, nc);
+    TRY(lanes == 1 ? tables(std::integral_constant<int, 1>{})
+                   : lanes == 4 ? tables(std::integral_constant<int, 4>{}) : tables(std::integral_constant<int, kGaugeLanes>{}));
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
