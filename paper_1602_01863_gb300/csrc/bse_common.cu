@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
     typename Cx<T>::V* __restrict__ W, double2* __restrict__ part) {
     using V = typename Cx<T>::V;
     extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ V dsum[BSE_MAX_CHAINS][256];                       // <psi, w> per chain and thread: a few products each
+    __shared__ DotSum<T> dsum[BSE_MAX_CHAINS][256];               // <psi, w> per chain and thread
     const int t = nv * nc, tp = odd(t), rv = nv * nv, rc = nc * nc, rvp = odd(rv), rcp = odd(rc);
     const int Ndiv = nd * nd * nd, nkc = n * n * n, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int c0 = blockIdx.y * CPB, c1 = min(nch, c0 + CPB), ncb = c1 - c0;
@@ -434,7 +434,8 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
         __syncthreads();
         for (int c = 0; c < ncb; ++c) {
             const int ch = c0 + c;
-            V dsm = czero<V>(), rr[EPL][8];
+            DotSum<T> dsm;
+            V rr[EPL][8];
 #pragma unroll
             for (int a = 0; a < EPL; ++a) {
 #pragma unroll
@@ -516,8 +517,7 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
                             o.x = fma(p.x, d4[a][u], s.x);
                             o.y = fma(p.y, d4[a][u], s.y);
                             W[o0 + r * t + e] = o;
-                            dsm.x = fma(p.x, o.x, fma(p.y, o.y, dsm.x));
-                            dsm.y = fma(p.x, o.y, fma(-p.y, o.x, dsm.y));
+                            dsm.add(p, o);
                         }
                     }
                 }
@@ -526,13 +526,12 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
             dsum[c][tid] = dsm;
         }
         __syncthreads();
-        if (warp < ncb)
+        if (warp < ncb) {
+            DotSum<T> low;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const V v = dsum[warp][lane + 32 * q];
-                dot.x += (double)v.x;
-                dot.y += (double)v.y;
-            }
+            for (int q = 0; q < 8; ++q) dsum[warp][lane + 32 * q].into(dot, low);
+            dot = cadd(dot, low.value());
+        }
     }
     if (warp < ncb) {
 #pragma unroll
@@ -1135,7 +1134,7 @@ int prolong_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* R,
                         8 * WarpStage<T>::bytes(KP, s->nv, s->nc);
     const dim3 grid(bse_common_dot_blocks(s), (nchains + CPB - 1) / CPB);
     auto go = [&](auto kernel) -> int {
-        BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, sizeof(V) * BSE_MAX_CHAINS * 256));
+        BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, sizeof(DotSum<T>) * BSE_MAX_CHAINS * 256));
         kernel<<<grid, 256, smem, st>>>((const V*)R, s->scheme == BSE_SCHEME_M3 ? (const V*)s->d_cV : nullptr,
                                         (const V*)s->d_cUv, (const V*)s->d_cUc, (const V*)s->d_cUvc, (const V*)s->d_cUcc,
                                         (const T*)s->d_dE, (const V*)psi, s->n, s->nd, s->nv, s->nc, s->nb1, nchains, CPB, KP,

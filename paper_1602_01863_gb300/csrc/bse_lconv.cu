@@ -278,8 +278,7 @@ __global__ void __launch_bounds__(LTHR) k_lconv_mix(float2* __restrict__ grid, c
     for (int i = tid; i < L * c; i += LTHR) g[i] = b[i];
 }
 
-// Back along y and z, w += scale * value, and the block's FP64 partial of <psi, w>
-// (FP32 vectors: a thread's few products in FP32).
+// Back along y and z, w += scale * value, and the block's FP64 partial of <psi, w>.
 template <typename T>
 __global__ void __launch_bounds__(LTHR) k_lconv_inv(const float2* __restrict__ grid, const LShape q,
                                                     const float2* __restrict__ tw_g, const typename Cx<T>::V* __restrict__ psi,
@@ -305,7 +304,7 @@ __global__ void __launch_bounds__(LTHR) k_lconv_inv(const float2* __restrict__ g
     lines_inv(s, ne * L, [&](int l) { const int e = quot(l, inv_L); return e * (L - 1) * P + e * (P - L) + l; }, P, L, q.A, q.B, tw);
     lines_inv(s, ne * L, [&](int l) { return l * P; }, 1, L, q.A, q.B, tw);
     const size_t nk = (size_t)L2 * L;
-    T dre = (T)0, dim = (T)0;
+    DotSum<T> dot;
 #pragma unroll 4
     for (int i = tid; i < L2 * EG; i += LTHR) {
         const int e = i & (EG - 1), p = i / EG, y = quot(p, inv_L), z = p - y * L;
@@ -317,10 +316,9 @@ __global__ void __launch_bounds__(LTHR) k_lconv_inv(const float2* __restrict__ g
         v.x = fma((T)g.x, (T)scale, v.x);
         v.y = fma((T)g.y, (T)scale, v.y);
         w[o] = v;
-        dre = fma(pv.x, v.x, fma(pv.y, v.y, dre));
-        dim = fma(pv.x, v.y, fma(-pv.y, v.x, dim));
+        dot.add(pv, v);
     }
-    double2 d = make_double2((double)dre, (double)dim);
+    double2 d = dot.value();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         d.x += __shfl_down_sync(0xffffffffu, d.x, o);
