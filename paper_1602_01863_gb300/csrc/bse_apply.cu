@@ -17,6 +17,7 @@
 
 #include <cuda_fp16.h>
 
+#include "bse_cost.h"
 #include "bse_internal.cuh"
 
 namespace {
@@ -2350,6 +2351,13 @@ int bse_run_chains(bse_ctx* ctx, bse_interp* s, int npol, const double* pol_dirs
     return run_chains_typed<float>(ctx, s, npol, pol_dirs, nsteps, flags, a, b, pnorm2, steps_done);
 }
 
+static double step_us(const bse_interp* s, int npol) {
+    const int p = s->co->kc_prec;
+    return bse_step_us(StepWork{s->scheme == BSE_SCHEME_M2 ? s->N : s->co->Nc, s->N, npol,
+                                p == BSE_PREC_F64 ? 16 : (p == BSE_PREC_F32 ? 8 : 4), s->scheme == BSE_SCHEME_M3, s->common,
+                                s->n_near, (long long)s->nk * s->npairs * s->t});
+}
+
 // Many independent systems in one CUDA graph: every system's whole Haydock
 // loop is captured on one of up to 8 side streams forked from the context
 // stream (longest systems first, each onto the least-loaded stream) and
@@ -2405,8 +2413,7 @@ int bse_run_batch(bse_ctx* ctx, bse_interp* const* sys, int nsys, const int* npo
         for (int i = 0; i < nsys; ++i) {
             const bse_interp* s = sys[i];
             order[i] = i;
-            cost[i] = (double)s->co->Nc * s->co->Nc * npol[i] + (double)s->N * npol[i] * 64.0 +
-                      (s->scheme == BSE_SCHEME_M3 ? (double)s->nk * s->npairs * s->t * npol[i] * 8.0 : 0.0);
+            cost[i] = step_us(s, npol[i]);
         }
         std::sort(order.begin(), order.end(), [&](int x, int y) { return cost[x] > cost[y]; });
         cudaGraph_t g = nullptr;
