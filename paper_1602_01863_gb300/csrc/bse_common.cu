@@ -807,17 +807,7 @@ __global__ void __launch_bounds__(128, 3) k_common_near(const double* __restrict
 // of the two (zero weights beyond their own).  Coarse 8^3, n_div 4, 4x4 bands, 3 chains beside
 // the K_c apply: 130 us with weights stored twice, 122 us so, 110 us since the apply leaves it
 // registers (84 us alone); with 80 registers (six blocks per SM, all warps at once) 124 us.
-using F2 = unsigned long long;                                        // a register pair
-__device__ __forceinline__ F2 ffma2(F2 w, F2 v, F2 a) {
-    F2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(w), "l"(v), "l"(a));
-    return d;
-}
-__device__ __forceinline__ F2 twice(float x) {
-    F2 d;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
-    return d;
-}
+__device__ __forceinline__ F2 twice(float x) { return f2_pair(x, x); }
 // The TZ weight pairs of one offset (16-byte loads where each offset starts on 16 bytes).
 template <int TZ>
 __device__ __forceinline__ void near_pairs(F2 (&w)[TZ], const float* p) {
@@ -845,7 +835,7 @@ __device__ __forceinline__ void near_row32(F2 (&acc)[NT], const float* __restric
         F2 w[TZ];
         near_pairs<TZ>(w, wb + d * 2 * TZ);
 #pragma unroll
-        for (int i = 0; i < NT; ++i) acc[i] = ffma2(w[i % TZ], v[i + d + rm], acc[i]);
+        for (int i = 0; i < NT; ++i) acc[i] = f2_fma(w[i % TZ], v[i + d + rm], acc[i]);
     }
 }
 
@@ -896,7 +886,7 @@ __device__ __forceinline__ void near_body32(const float* __restrict__ phi, const
                 F2 w[TZ];
                 near_pairs<TZ>(w, wb + d * 2 * TZ);
 #pragma unroll
-                for (int z = 0; z < NT; ++z) acc[z] = ffma2(w[z % TZ], twice(__ldg(row + (z + d) * 32)), acc[z]);
+                for (int z = 0; z < NT; ++z) acc[z] = f2_fma(w[z % TZ], twice(__ldg(row + (z + d) * 32)), acc[z]);
             }
         }
         __syncwarp();

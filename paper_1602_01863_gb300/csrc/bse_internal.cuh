@@ -64,14 +64,43 @@ template <> __host__ __device__ inline float2 from_d2<float2>(double2 a) {
 __host__ __device__ inline double2 to_d2(double2 a) { return a; }
 __host__ __device__ inline double2 to_d2(float2 a) { return make_double2(a.x, a.y); }
 
+// --------------------------------------------- packed pairs of FP32 numbers
+using F2 = unsigned long long;                                        // a register pair
+__device__ __forceinline__ F2 f2_pair(float x, float y) {
+    F2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+__device__ __forceinline__ float2 f2_get(F2 v) { return make_float2(__uint_as_float((unsigned)v), __uint_as_float((unsigned)(v >> 32))); }
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+    F2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+    F2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+    F2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ F2 f2_sub(F2 a, F2 b) {
+    F2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // ------------------------------------------- a thread's share of <psi, w>
 // FP64 vectors: plain sums.  FP32 vectors: every product exactly (its rounded value and
 // the rest of an FMA) into a sum that keeps what its additions round off (Knuth's
 // two-sum), so a_i loses nothing to the number of products a thread has (up to 1024 per
-// cell at n_div 16 with 64 transitions); 40 FP32 operations per complex entry, where
+// cell at n_div 16 with 64 transitions); 20 packed operations per complex entry, where
 // FP64 would take 4 conversions and 4 multiply-adds at a 64th of the rate.  24 mixed
 // steps, coarse 8^3, n_div 4, 4x4 bands, 3 chains: 4.95 ms with single FP32 sums (a_1 off
-// by up to 1e-8 of itself), 4.99 ms so (1e-14).
+// by up to 1e-8 of itself), 4.99 ms with 40 scalar operations, 4.94 ms so (1e-14).
 template <typename T> struct DotSum;
 template <> struct DotSum<double> {
     double2 s = {0.0, 0.0};
@@ -85,17 +114,18 @@ template <> struct DotSum<double> {
 };
 template <> struct DotSum<float> {
     float2 s = {0.f, 0.f}, c = {0.f, 0.f};                      // sums and what they lack
-    static __device__ __forceinline__ void one(float& s, float& c, float a, float b) {
-        const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
-        const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
-        c = __fadd_rn(c, __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z))));
-        s = t;
+    // both parts at once, in packed operations: s += a b, c += what that rounded off
+    __device__ __forceinline__ void one(float a, float bx, float by) {
+        const F2 s0 = f2_pair(s.x, s.y), b = f2_pair(bx, by);
+        const F2 m = f2_mul(f2_pair(-a, -a), b), e = f2_fma(f2_pair(a, a), b, m);      // -(a b) rounded, and a b + m exactly
+        const F2 t = f2_sub(s0, m), z = f2_sub(t, s0);
+        const F2 r = f2_sub(f2_sub(s0, f2_sub(t, z)), f2_add(m, z));
+        c = f2_get(f2_add(f2_pair(c.x, c.y), f2_add(e, r)));
+        s = f2_get(t);
     }
     __device__ __forceinline__ void add(float2 p, float2 w) {
-        one(s.x, c.x, p.x, w.x);
-        one(s.x, c.x, p.y, w.y);
-        one(s.y, c.y, p.x, w.y);
-        one(s.y, c.y, -p.y, w.x);
+        one(p.x, w.x, w.y);
+        one(p.y, w.y, -w.x);
     }
     __device__ __forceinline__ double2 value() const { return make_double2((double)s.x + c.x, (double)s.y + c.y); }
     __device__ __forceinline__ void into(double2& d, DotSum& low) const {
