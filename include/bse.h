@@ -221,12 +221,13 @@ int bse_dipoles(bse_ctx* ctx, bse_interp* interp, int npol, const double* pol_di
 int bse_apply_h(bse_ctx* ctx, bse_interp* interp, int nvec, const void* x, void* y);
 
 /* Same result as bse_apply_h, but allocates no device memory: the per-call
- * Q, R, operands and partials come from one static device array of 32 MiB inside the library
+ * scratch comes from one static device array of 32 MiB inside the library
  * (held by a device from the time the library's device module is loaded on
  * it, at the latest the first bse_ctx_create on that device, until the
- * process exits); what set-up allocated for the handle's own intermediate
- * vectors is used as bse_apply_h uses it, so calls on one handle must not
- * overlap.  The paper has no counterpart; this
+ * process exits), not from the handle; where the overlaps are the model's, the
+ * intermediate vectors of these calls are a set of their own that
+ * bse_interp_setup allocates.  So one such call may run beside another call on
+ * the same handle (through a context of its own).  The paper has no counterpart; this
  * exists for callers that must not call cudaMalloc once their work has
  * started, such as a host framework that owns all device memory through its
  * own pool, or a loop where cudaMalloc's implicit device synchronisation is
@@ -236,8 +237,8 @@ int bse_apply_h(bse_ctx* ctx, bse_interp* interp, int nvec, const void* x, void*
  * All calls share the array and it keeps the
  * previous call's contents (what must start at zero is cleared each call):
  * calls that overlap on the GPU race.  Sizes whose scratch does not fit
- * (nvec vectors of Q and R, for M3 the per-corner pieces, for BF16 the
- * operand and tile partials) return BSE_ERR_UNSUPPORTED with the byte count
+ * (nvec vectors of Q and R, for M3 the per-corner pieces, which count whether
+ * the handle's path needs them or not, for BF16 the operand and tile partials) return BSE_ERR_UNSUPPORTED with the byte count
  * in bse_last_error.  Other errors as bse_apply_h. */
 int bse_apply_h_noalloc(bse_ctx* ctx, bse_interp* interp, int nvec, const void* x, void* y);
 

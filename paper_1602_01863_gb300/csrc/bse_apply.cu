@@ -1712,12 +1712,13 @@ __global__ void __launch_bounds__(256) k_chain_xscale(const double* __restrict__
     }
 }
 
-// The scales of nchains inputs into s->d_xscale_gen.  One block per chain read the
-// whole vector (346 us for 221184 entries of 3 chains); two blocks per SM take 4 us.
-void launch_xscale(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi) {
+// The scales of nchains inputs into `xscale`, through `part` [nchains][BSE_MAX_VEC_BLOCKS].
+// One block per chain read the whole vector (346 us for 221184 entries of 3 chains); two
+// blocks per SM take 4 us.
+void launch_xscale(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, double* part, float* xscale) {
     const int nb = std::min({(s->N + 255) / 256, 2 * std::max(ctx->sm_count, 1), BSE_MAX_VEC_BLOCKS});
-    k_chain_norm2<<<dim3(nb, nchains), 256, 0, ctx->stream>>>((const float2*)psi, s->N, s->d_part_nrm);
-    k_chain_xscale<<<nchains, 256, 0, ctx->stream>>>(s->d_part_nrm, nb, s->dbound, s->d_xscale_gen);
+    k_chain_norm2<<<dim3(nb, nchains), 256, 0, ctx->stream>>>((const float2*)psi, s->N, part);
+    k_chain_xscale<<<nchains, 256, 0, ctx->stream>>>(part, nb, s->dbound, xscale);
 }
 
 // Restrict: staged FP32 kernel for 3x3, 4x4 and 4x6 bands (N_div <= 64), generic otherwise.
@@ -1863,7 +1864,7 @@ int apply_h_common(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi, vo
     int rc;
     {
         Timer tm(ctx, prof, KC_RESTRICT);
-        if ((rc = bse_common_restrict(ctx, s, nchains, psi, s->d_Q, s->d_Bop, st)) != BSE_OK) return rc;
+        if ((rc = bse_common_restrict(ctx, s, s->cwork[0], nchains, psi, s->d_Q, s->d_Bop, st)) != BSE_OK) return rc;
     }
     cudaStream_t kst = beside ? ctx->aux[ln] : st;
     if (beside) {
@@ -1880,7 +1881,7 @@ int apply_h_common(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi, vo
     }
     if (m3) {
         Timer tm(ctx, prof, KC_NEAR);
-        if ((rc = bse_common_near(ctx, s, nchains, st)) != BSE_OK) return rc;
+        if ((rc = bse_common_near(ctx, s, s->cwork[0], nchains, st)) != BSE_OK) return rc;
     }
     if (beside) {
         BSE_CUDA_TRY(ctx, cudaEventRecord(ctx->aux_join[ln], kst));
@@ -1888,7 +1889,7 @@ int apply_h_common(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi, vo
     }
     {
         Timer tm(ctx, prof, KC_PROLONG);
-        if ((rc = bse_common_prolong(ctx, s, nchains, s->d_R, psi, W, s->d_part_dot, st)) != BSE_OK) return rc;
+        if ((rc = bse_common_prolong(ctx, s, s->cwork[0], nchains, s->d_R, psi, W, s->d_part_dot, st)) != BSE_OK) return rc;
     }
     if (s->learned) {
         Timer tm(ctx, prof, KC_NEAR);
@@ -1918,7 +1919,7 @@ int apply_h_typed(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi_v, v
     const bool xh = near_tc_active(s);
     void* X = m3 ? s->d_X : nullptr;
     const float* xscale = unit ? s->d_xscale : s->d_xscale_gen;
-    if (xh && !unit) launch_xscale(ctx, s, nchains, psi);
+    if (xh && !unit) launch_xscale(ctx, s, nchains, psi, s->d_part_nrm, s->d_xscale_gen);
     {
         Timer tm(ctx, prof, KC_RESTRICT);
         launch_restrict<T>(ctx, s, nchains, psi, s->d_Q, s->d_Bop, X, xh, xscale, s->d_U);
@@ -2530,29 +2531,32 @@ int apply_scratch_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const vo
         int rc;
         if (c->kc_prec == BSE_PREC_BF16) {
             BSE_CUDA_TRY(ctx, cudaMemsetAsync(sc.bop, 0, sizeof(__nv_bfloat16) * 16 * (size_t)c->ldk, st));
-            if ((rc = bse_common_restrict(ctx, s, nchains, psi, nullptr, sc.bop, st)) != BSE_OK) return rc;
+            if ((rc = bse_common_restrict(ctx, s, s->cwork[1], nchains, psi, nullptr, sc.bop, st)) != BSE_OK) return rc;
             if ((rc = bse_tc_apply_scratch(ctx, s, nchains, sc.bop, sc.part, sc.R)) != BSE_OK) return rc;
         } else {
-            if ((rc = bse_common_restrict(ctx, s, nchains, psi, sc.Q, nullptr, st)) != BSE_OK) return rc;
+            if ((rc = bse_common_restrict(ctx, s, s->cwork[1], nchains, psi, sc.Q, nullptr, st)) != BSE_OK) return rc;
             launch_kc_simt<T>(ctx, c, sc.Q, nchains, sc.R, st);
         }
-        if (m3 && (rc = bse_common_near(ctx, s, nchains, st)) != BSE_OK) return rc;
-        return bse_common_prolong(ctx, s, nchains, sc.R, psi, W, sc.dot, st);
+        if (m3 && (rc = bse_common_near(ctx, s, s->cwork[1], nchains, st)) != BSE_OK) return rc;
+        return bse_common_prolong(ctx, s, s->cwork[1], nchains, sc.R, psi, W, sc.dot, st);
     }
     const bool xh = near_tc_active(s);
     void* X = m3 ? sc.X : nullptr;
-    if (xh) launch_xscale(ctx, s, nchains, psi);
+    // the piece scales and their partials lie where prolong writes its own partials later
+    double* npart = (double*)sc.dot;
+    float* xscale = (float*)(npart + (size_t)nchains * BSE_MAX_VEC_BLOCKS);
+    if (xh) launch_xscale(ctx, s, nchains, psi, npart, xscale);
     if (c->kc_prec == BSE_PREC_BF16) {
         BSE_CUDA_TRY(ctx, cudaMemsetAsync(sc.bop, 0, sizeof(__nv_bfloat16) * 16 * (size_t)c->ldk, st));
-        launch_restrict<T>(ctx, s, nchains, psi, nullptr, sc.bop, X, xh, s->d_xscale_gen, sc.U);
+        launch_restrict<T>(ctx, s, nchains, psi, nullptr, sc.bop, X, xh, xscale, sc.U);
         int rc = bse_tc_apply_scratch(ctx, s, nchains, sc.bop, sc.part, sc.R);
         if (rc != BSE_OK) return rc;
     } else {
-        launch_restrict<T>(ctx, s, nchains, psi, sc.Q, nullptr, X, xh, s->d_xscale_gen, sc.U);
+        launch_restrict<T>(ctx, s, nchains, psi, sc.Q, nullptr, X, xh, xscale, sc.U);
         launch_kc_simt<T>(ctx, c, sc.Q, nchains, sc.R, st);
     }
     if (m3) {
-        int rc = bse_launch_near_field(ctx, s, nchains, X, s->d_xscale_gen, sc.U);
+        int rc = bse_launch_near_field(ctx, s, nchains, X, xscale, sc.U);
         if (rc != BSE_OK) return rc;
     }
     launch_prolong<T>(ctx, s, nchains, sc.R, m3 ? sc.U : nullptr, psi, W, sc.dot);

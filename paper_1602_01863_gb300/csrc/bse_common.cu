@@ -1033,7 +1033,7 @@ int near_wrow(int nd, int R) {
 }
 
 template <typename T, typename K>
-int launch_near_k(bse_ctx* ctx, const bse_interp* s, K kernel, int RM, NearStencil ns, cudaStream_t st) {
+int launch_near_k(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, K kernel, int RM, NearStencil ns, cudaStream_t st) {
     const int groups = (ns.cols + 31) / 32, n = s->n;
     auto tiles = [&](int cz) {
         int c = n / cz;
@@ -1059,19 +1059,19 @@ int launch_near_k(bse_ctx* ctx, const bse_interp* s, K kernel, int RM, NearStenc
     const int wpb = ns.split ? 4 : (warps >= 8LL * ctx->sm_count ? 4 : 2);
     const size_t smem = (size_t)ns.wbytes * wpb + (ns.split ? 3 * 32 * sizeof(double) * near_ty<T>(ns.nd) * near_tz(ns.nd) : 0);
     BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, 0));
-    kernel<<<(unsigned)(ns.split ? warps : (warps + wpb - 1) / wpb), 32 * wpb, smem, st>>>((const T*)s->d_cphi, (const T*)s->d_cw, s->d_csteps,
-                                                                       (T*)s->d_cV, ns);
+    kernel<<<(unsigned)(ns.split ? warps : (warps + wpb - 1) / wpb), 32 * wpb, smem, st>>>((const T*)work.phi, (const T*)s->d_cw, s->d_csteps,
+                                                                       (T*)work.V, ns);
     BSE_CUDA_TRY(ctx, cudaGetLastError());
     return BSE_OK;
 }
 template <typename T, int TY, int TZ, int RM>
-int launch_near_r(bse_ctx* ctx, const bse_interp* s, const NearStencil& ns, cudaStream_t st) {
-    if constexpr (sizeof(T) == 4) return launch_near_k<T>(ctx, s, k_common_near32<TZ, RM>, RM, ns, st);
-    else return launch_near_k<T>(ctx, s, k_common_near<TY, TZ, RM>, RM, ns, st);
+int launch_near_r(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, const NearStencil& ns, cudaStream_t st) {
+    if constexpr (sizeof(T) == 4) return launch_near_k<T>(ctx, s, work, k_common_near32<TZ, RM>, RM, ns, st);
+    else return launch_near_k<T>(ctx, s, work, k_common_near<TY, TZ, RM>, RM, ns, st);
 }
 
 template <typename T>
-int near_typed(bse_ctx* ctx, const bse_interp* s, int nchains, cudaStream_t st) {
+int near_typed(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, cudaStream_t st) {
     NearStencil ns{};
     const int nd = s->nd;
     ns.n = s->n; ns.nd = nd; ns.L = s->n * nd; ns.R = s->cphi_R; ns.Lp = s->cphi_Lp;
@@ -1083,19 +1083,19 @@ int near_typed(bse_ctx* ctx, const bse_interp* s, int nchains, cudaStream_t st) 
     ns.t2 = 2 * s->t; ns.cols = ns.t2 * nchains; ns.N2 = 2LL * s->N;
     const bool r4 = ns.R <= 4, r6 = ns.R <= 6;
     switch (nd) {
-        case 1: return r4 ? launch_near_r<T, 1, 1, 4>(ctx, s, ns, st) : launch_near_r<T, 1, 1, 0>(ctx, s, ns, st);
-        case 2: return r4 ? launch_near_r<T, 2, 2, 4>(ctx, s, ns, st) : launch_near_r<T, 2, 2, 0>(ctx, s, ns, st);
-        case 3: return r4 ? launch_near_r<T, 3, 3, 4>(ctx, s, ns, st) : launch_near_r<T, 3, 3, 0>(ctx, s, ns, st);
+        case 1: return r4 ? launch_near_r<T, 1, 1, 4>(ctx, s, work, ns, st) : launch_near_r<T, 1, 1, 0>(ctx, s, work, ns, st);
+        case 2: return r4 ? launch_near_r<T, 2, 2, 4>(ctx, s, work, ns, st) : launch_near_r<T, 2, 2, 0>(ctx, s, work, ns, st);
+        case 3: return r4 ? launch_near_r<T, 3, 3, 4>(ctx, s, work, ns, st) : launch_near_r<T, 3, 3, 0>(ctx, s, work, ns, st);
         default:
-            return r4   ? launch_near_r<T, 2, 4, 4>(ctx, s, ns, st)
-                   : r6 ? launch_near_r<T, 2, 4, 6>(ctx, s, ns, st)
-                        : launch_near_r<T, 2, 4, 0>(ctx, s, ns, st);
+            return r4   ? launch_near_r<T, 2, 4, 4>(ctx, s, work, ns, st)
+                   : r6 ? launch_near_r<T, 2, 4, 6>(ctx, s, work, ns, st)
+                        : launch_near_r<T, 2, 4, 0>(ctx, s, work, ns, st);
     }
 }
 
 template <typename T>
-int restrict_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, void* Q, __nv_bfloat16* bop,
-                   cudaStream_t st) {
+int restrict_typed(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, const void* psi, void* Q,
+                   __nv_bfloat16* bop, cudaStream_t st) {
     using V = typename Cx<T>::V;
     const bse_coarse* c = s->co;
     const int KP = rot_points<T>(s), CPB = rot_chains(ctx, s, nchains);
@@ -1107,7 +1107,7 @@ int restrict_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* p
         BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, 64));
         kernel<<<grid, 256, smem, st>>>((const V*)psi, (const V*)s->d_cUv, (const V*)s->d_cUc, (const V*)s->d_cUvc,
                                         (const V*)s->d_cUcc, s->n, s->nd, s->nv, s->nc, s->nb1, nchains, CPB, KP,
-                                        m3 ? (T*)s->d_cphi : nullptr, lay, (V*)s->d_cshare, s->d_cctr, (V*)Q, bop, c->ldk);
+                                        m3 ? (T*)work.phi : nullptr, lay, (V*)work.share, work.ctr, (V*)Q, bop, c->ldk);
         BSE_CUDA_TRY(ctx, cudaGetLastError());
         return BSE_OK;
     };
@@ -1116,8 +1116,8 @@ int restrict_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* p
 }
 
 template <typename T>
-int prolong_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* R, const void* psi, void* W, double2* dot,
-                  cudaStream_t st) {
+int prolong_typed(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, const void* R, const void* psi, void* W,
+                  double2* dot, cudaStream_t st) {
     using V = typename Cx<T>::V;
     const int KP = rot_points<T>(s), CPB = rot_chains(ctx, s, nchains);
     const size_t smem = (sizeof(V) * (sizeof(T) == 8 ? 2 : 1) * 8 * CPB * odd(s->t) + 15) / 16 * 16 +
@@ -1125,7 +1125,7 @@ int prolong_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void* R,
     const dim3 grid(bse_common_dot_blocks(s), (nchains + CPB - 1) / CPB);
     auto go = [&](auto kernel) -> int {
         BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, sizeof(DotSum<T>) * BSE_MAX_CHAINS * 256));
-        kernel<<<grid, 256, smem, st>>>((const V*)R, s->scheme == BSE_SCHEME_M3 ? (const V*)s->d_cV : nullptr,
+        kernel<<<grid, 256, smem, st>>>((const V*)R, s->scheme == BSE_SCHEME_M3 ? (const V*)work.V : nullptr,
                                         (const V*)s->d_cUv, (const V*)s->d_cUc, (const V*)s->d_cUvc, (const V*)s->d_cUcc,
                                         (const T*)s->d_dE, (const V*)psi, s->n, s->nd, s->nv, s->nc, s->nb1, nchains, CPB, KP,
                                         (V*)W, dot);
@@ -1154,9 +1154,18 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s) {
         if ((rc_ = bse_alloc(ctx, x.dst, sizeof(V) * x.n, "gauge tables")) != BSE_OK) return rc_;
         k_gauge_to<T><<<(unsigned)((x.n + 255) / 256), 256, 0, st>>>(x.src, (long long)x.n, (V*)*x.dst);
     }
-    if ((rc_ = bse_alloc(ctx, &s->d_cshare, sizeof(V) * BSE_MAX_CHAINS * 8 * (size_t)c->Nc, "corner shares")) != BSE_OK) return rc_;
-    if ((rc_ = bse_alloc(ctx, (void**)&s->d_cctr, sizeof(int) * BSE_MAX_CHAINS * (size_t)c->nkc, "corner counters")) != BSE_OK) return rc_;
-    BSE_CUDA_TRY(ctx, cudaMemsetAsync(s->d_cctr, 0, sizeof(int) * BSE_MAX_CHAINS * (size_t)c->nkc, st));
+    // both sets of intermediate vectors, each kind in one allocation that the first owns
+    auto both = [&](void** first, void** second, size_t bytes, bool clear, const char* what) -> int {
+        bytes = (bytes + 255) / 256 * 256;
+        const int rc = bse_alloc(ctx, first, 2 * bytes, what);
+        if (rc != BSE_OK) return rc;
+        *second = (unsigned char*)*first + bytes;
+        if (clear) BSE_CUDA_TRY(ctx, cudaMemsetAsync(*first, 0, 2 * bytes, st));
+        return BSE_OK;
+    };
+    CommonWork &w0 = s->cwork[0], &w1 = s->cwork[1];
+    if ((rc_ = both(&w0.share, &w1.share, sizeof(V) * BSE_MAX_CHAINS * 8 * (size_t)c->Nc, false, "corner shares")) != BSE_OK) return rc_;
+    if ((rc_ = both((void**)&w0.ctr, (void**)&w1.ctr, sizeof(int) * BSE_MAX_CHAINS * (size_t)c->nkc, true, "corner counters")) != BSE_OK) return rc_;
     if (s->scheme != BSE_SCHEME_M3) {
         BSE_CUDA_TRY(ctx, cudaStreamSynchronize(st));
         return BSE_OK;
@@ -1166,9 +1175,8 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s) {
     s->cphi_Lp = L + 2 * R + (nd > 4 ? 3 : 0);
     const size_t groups = (2 * (size_t)s->t * BSE_MAX_CHAINS + 31) / 32;
     const size_t nphi = groups * L * L * (size_t)s->cphi_Lp * 32;
-    if ((rc_ = bse_alloc(ctx, &s->d_cphi, sizeof(T) * nphi, "common-basis vectors")) != BSE_OK) return rc_;
-    BSE_CUDA_TRY(ctx, cudaMemsetAsync(s->d_cphi, 0, sizeof(T) * nphi, st));      // unused columns stay zero
-    if ((rc_ = bse_alloc(ctx, &s->d_cV, sizeof(V) * BSE_MAX_CHAINS * (size_t)s->N, "near stencil result")) != BSE_OK) return rc_;
+    if ((rc_ = both(&w0.phi, &w1.phi, sizeof(T) * nphi, true, "common-basis vectors")) != BSE_OK) return rc_;   // unused columns stay zero
+    if ((rc_ = both(&w0.V, &w1.V, sizeof(V) * BSE_MAX_CHAINS * (size_t)s->N, false, "near stencil result")) != BSE_OK) return rc_;
     // source rows of a warp's targets: (delta_1 + R, u), u - y the delta_2 + R of target row y,
     // with the reach along z of each row (a byte each, plus one; 0: outside the ball) and the largest
     std::vector<int2> steps;
@@ -1210,18 +1218,18 @@ int bse_common_prepare(bse_ctx* ctx, bse_interp* s) {
     return s->vec_prec == BSE_PREC_F64 ? prepare_typed<double>(ctx, s) : prepare_typed<float>(ctx, s);
 }
 
-int bse_common_restrict(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, void* Q, __nv_bfloat16* bop,
-                        cudaStream_t st) {
-    return s->vec_prec == BSE_PREC_F64 ? restrict_typed<double>(ctx, s, nchains, psi, Q, bop, st)
-                                       : restrict_typed<float>(ctx, s, nchains, psi, Q, bop, st);
+int bse_common_restrict(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, const void* psi, void* Q,
+                        __nv_bfloat16* bop, cudaStream_t st) {
+    return s->vec_prec == BSE_PREC_F64 ? restrict_typed<double>(ctx, s, work, nchains, psi, Q, bop, st)
+                                       : restrict_typed<float>(ctx, s, work, nchains, psi, Q, bop, st);
 }
 
-int bse_common_near(bse_ctx* ctx, const bse_interp* s, int nchains, cudaStream_t st) {
-    return s->vec_prec == BSE_PREC_F64 ? near_typed<double>(ctx, s, nchains, st) : near_typed<float>(ctx, s, nchains, st);
+int bse_common_near(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, cudaStream_t st) {
+    return s->vec_prec == BSE_PREC_F64 ? near_typed<double>(ctx, s, work, nchains, st) : near_typed<float>(ctx, s, work, nchains, st);
 }
 
-int bse_common_prolong(bse_ctx* ctx, const bse_interp* s, int nchains, const void* R, const void* psi, void* W,
-                       double2* dot, cudaStream_t st) {
-    return s->vec_prec == BSE_PREC_F64 ? prolong_typed<double>(ctx, s, nchains, R, psi, W, dot, st)
-                                       : prolong_typed<float>(ctx, s, nchains, R, psi, W, dot, st);
+int bse_common_prolong(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, const void* R, const void* psi,
+                       void* W, double2* dot, cudaStream_t st) {
+    return s->vec_prec == BSE_PREC_F64 ? prolong_typed<double>(ctx, s, work, nchains, R, psi, W, dot, st)
+                                       : prolong_typed<float>(ctx, s, work, nchains, R, psi, W, dot, st);
 }

@@ -232,6 +232,13 @@ struct bse_coarse {
 // g holding the columns 32 g .. 32 g + 31 of the (chain, transition, re|im)
 // components of a dense point; z starts R points before 0 (periodic halo; rows of Lp points).
 struct CommonPhi { int R, Lp; };
+// What one H application in the common basis writes on its way.
+struct CommonWork {
+    void* phi = nullptr;             // T, layout CommonPhi
+    void* V = nullptr;               // V [4][N] near stencil result
+    void* share = nullptr;           // V [4][nkc][8][t] the cells' shares of their corners
+    int* ctr = nullptr;              // [4][nkc] shares written (zero between launches)
+};
 
 struct NearEntry { int co; int js_src; int l_src; int near_idx; };   // co packed 3 x 4 bits (+8 bias)
 
@@ -252,15 +259,12 @@ struct bse_interp {
     int common = 0;
     void *d_cUv = nullptr, *d_cUc = nullptr;     // V [nk][nv*nv], [nk][nc*nc] dense gauge
     void *d_cUvc = nullptr, *d_cUcc = nullptr;   // V [nkc][nv*nv], [nkc][nc*nc] coarse gauge
-    void* d_cshare = nullptr;        // V [4][nkc][8][t] the cells' shares of their corners
-    int* d_cctr = nullptr;           // [4][nkc] shares written (zero between launches)
+    CommonWork cwork[2];             // the handle's own calls; bse_apply_h_noalloc (parts of the same allocations)
     int cphi_R = 0, near_R2 = 0;     // near offsets: |delta|^2 <= near_R2, components within cphi_R
     int cphi_Lp = 0;
     int n_csteps = 0;
     int2* d_csteps = nullptr;        // source rows of the near stencil
     double* d_chead = nullptr;       // [nkc] h_head over coarse differences (set-up only)
-    void* d_cphi = nullptr;          // T, layout CommonPhi
-    void* d_cV = nullptr;            // V [4][N] near stencil result
     void* d_cw = nullptr;            // T near stencil weights
     // M3 tables
     int n_near = 0, smin = 0, ns1 = 0, nslot = 0, rmin = 0, nr1 = 0, nrel = 0;
@@ -427,11 +431,11 @@ int bse_near_tc_launch(bse_ctx* ctx, const bse_interp* s, int nchains, const voi
 // common-basis path (bse_common.cu)
 int bse_common_prepare(bse_ctx* ctx, bse_interp* s);
 int bse_common_dot_blocks(const bse_interp* s);
-int bse_common_restrict(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, void* Q, __nv_bfloat16* bop,
-                        cudaStream_t st);
-int bse_common_near(bse_ctx* ctx, const bse_interp* s, int nchains, cudaStream_t st);
-int bse_common_prolong(bse_ctx* ctx, const bse_interp* s, int nchains, const void* R, const void* psi, void* W,
-                       double2* dot, cudaStream_t st);
+int bse_common_restrict(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, const void* psi, void* Q,
+                        __nv_bfloat16* bop, cudaStream_t st);
+int bse_common_near(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, cudaStream_t st);
+int bse_common_prolong(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, const void* R, const void* psi,
+                       void* W, double2* dot, cudaStream_t st);
 float bse_near_tc_xscale(const bse_interp* s, double norm);
 size_t bse_tc_part_bytes(const bse_interp* s);
 int bse_tc_apply_scratch(bse_ctx* ctx, const bse_interp* s, int nchains, __nv_bfloat16* bop, float* part, void* R);

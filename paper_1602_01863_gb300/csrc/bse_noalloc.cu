@@ -7,7 +7,9 @@
 // loop in which cudaMalloc's implicit device-wide synchronisation is not
 // allowed.  bse_apply_h takes its per-call scratch from the handle, which
 // bse_interp_setup allocated; this variant takes it from the file-scope
-// array below instead, so after set-up nothing is allocated on any path.
+// array below, and on the common-basis path its intermediate vectors from a
+// set of their own in the handle, so after set-up nothing is allocated on any
+// path and the call may run beside another one on the same handle.
 //
 // The array is a static __device__ object of the library's device module: a
 // device holds BSE_NOALLOC_SCRATCH_BYTES of it from the moment that module is
