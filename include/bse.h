@@ -62,8 +62,11 @@ extern "C" {
                               the nearest coarse corner) instead of trilinear 8NB   */
 #define BSE_NF_CUDA_CORES 32 /* OR-flag: apply the M3 near field on the CUDA cores
                               even where the tensor-core kernel applies (FP32
-                              vectors, t <= 16, n_div <= 4); same result to
-                              TF32 rounding of the head blocks and y1, z        */
+                              vectors, t <= 16, n_div <= 4, overlaps given by the
+                              caller); same result to TF32 rounding of the head
+                              blocks and y1, z.  No effect where the overlaps are
+                              the model's: their near field is a scalar stencil
+                              on the CUDA cores in the vector precision         */
 
 /* ------------------------------------------------------------ Haydock flags */
 #define BSE_REORTH_CGS2   1  /* full reorthogonalisation, classical Gram-Schmidt x2 */
