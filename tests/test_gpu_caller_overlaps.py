@@ -142,4 +142,7 @@ def test_stencil_weights_in_fp32(ctx, nv, nc, n, nd, width):
     other = np.where(m1 == m1.max(axis=1, keepdims=True), 0.0, m1).max()      # without the points' own energies
     bar = 2.0 ** -18 * (near + m1) + 2.0 ** -20 * other
     assert np.all(np.abs(out[1, 1] - out[0, 1]).max(axis=2) <= bar)
-    assert np.count_nonzero(near > 1e-12 * near.max()) >= 4 * 7     # seven offsets and more were reached
+    if nd == 1:
+        assert not np.any(near)                                    # every dense difference is a coarse one: the heads cancel
+    else:
+        assert np.count_nonzero(near > 1e-12 * near.max()) >= 4 * 7     # seven offsets and more were reached
