@@ -1708,7 +1708,7 @@ __global__ void __launch_bounds__(256) k_chain_xscale(const double* __restrict__
         const double b = fmax(dbound * fmax(sqrt(r.x), 1e-300), 1e-300);
         int e = 0;
         frexp(32768.0 / b, &e);
-        xscale[ch] = (float)ldexp(1.0, e - 1);
+        xscale[ch] = (float)ldexp(1.0, min(e - 1, 80));        // a zero vector has no largest one
     }
 }
 

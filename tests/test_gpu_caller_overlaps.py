@@ -146,3 +146,16 @@ def test_stencil_weights_in_fp32(ctx, nv, nc, n, nd, width):
         assert not np.any(near)                                    # every dense difference is a coarse one: the heads cancel
     else:
         assert np.count_nonzero(near > 1e-12 * near.max()) >= 4 * 7     # seven offsets and more were reached
+
+
+@pytest.mark.parametrize("nv,nc,n,nd", [(3, 3, 4, 2), (2, 3, 5, 3)])
+def test_zero_and_tiny_vectors(ctx, nv, nc, n, nd):
+    """H 0 = 0 beside another vector, and a vector of norm 1e-18 keeps its scale."""
+    m = synth.draw_model(46, nv, nc)
+    I = oi.Interp(m, n, nd, build_dense_kc=False)
+    co, it = _handles(ctx, m, I, n, nd, 1, 1)
+    x = synth.random_vectors(12, (1, it.N)).astype(np.complex64).astype(np.complex128)
+    y = _apply(ctx, it, np.concatenate([0 * x, x, 2.0 ** -66 * x]))
+    assert not np.any(y[0])
+    assert np.all(np.isfinite(y)) and np.array_equal(y[2], 2.0 ** -66 * y[1])
+    _free(it, co)
