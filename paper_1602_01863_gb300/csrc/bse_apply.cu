@@ -1642,15 +1642,9 @@ inline int vec_blocks(long long N) {
     return (int)std::min<long long>(std::max<long long>(b, 1), BSE_MAX_VEC_BLOCKS);
 }
 
-// Raise a kernel's dynamic shared-memory limit when a launch needs more than the
-// current one (by default 48 KB less the kernel's static shared memory); only
-// ever raised: handles of different sizes share the attribute.
+// The staged kernels' limit (below 8 KB of static shared memory); the launch reports a refusal.
 template <typename K>
-void ensure_smem(K kernel, size_t bytes) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kernel) == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < bytes)
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
+void ensure_smem(K kernel, size_t bytes) { bse_raise_smem(kernel, bytes, 8192); }
 
 // The staged FP32 restrict / prolong kernels serve 3x3, 4x4 and 4x6 bands with N_div <= 64.
 inline bool staged_bands(const bse_interp* s) {
@@ -2576,8 +2570,7 @@ template <typename T, int NVP>
 int launch_near_cell(bse_ctx* ctx, const bse_interp* s, int nchains, const void* X, void* U) {
     using V = typename Cx<T>::V;
     const int smem = (int)s->cell_smem;
-    if (smem > 48 * 1024)
-        BSE_CUDA_TRY(ctx, cudaFuncSetAttribute(k_near_cell<T, NVP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BSE_CUDA_TRY(ctx, bse_raise_smem((k_near_cell<T, NVP>), smem));
     dim3 grid(s->co->nkc, nchains);
     k_near_cell<T, NVP><<<grid, 512, smem, ctx->stream>>>(
         (const V*)X, s->d_clist, s->d_cstart, s->d_pairs, s->npairs, (const T*)s->d_hd, s->n_near, (const V*)s->d_Hv,
@@ -2591,8 +2584,7 @@ int launch_near_rb(bse_ctx* ctx, const bse_interp* s, int nchains, const void* X
     const size_t bytes = sizeof(float2) * ((size_t)s->npairs * tp + 2 * (size_t)s->Ndiv * tp + 8 * (NV * NV + NC * NC)) +
                          sizeof(float) * (8 + (size_t)s->n_near) + sizeof(int) * ((size_t)s->npairs + 8 * (size_t)s->nslot);
     const int smem = (int)bytes;
-    if (smem > 48 * 1024)
-        BSE_CUDA_TRY(ctx, cudaFuncSetAttribute(k_near_cell_rb<NV, NC, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    BSE_CUDA_TRY(ctx, bse_raise_smem((k_near_cell_rb<NV, NC, PF>), smem));
     // one thread per active (target, corner) pair; with at most 256 pairs and no
     // register prefetch, 256-thread CTAs let two CTAs share an SM (128 registers)
     dim3 grid(s->co->nkc, nchains);
@@ -2626,8 +2618,7 @@ int launch_near_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const void
         return launch_near_cell<T, 8>(ctx, s, nchains, X, U);
     }
     const size_t smem = sizeof(V) * 2 * s->nslot * s->t;
-    if (smem > 48 * 1024)
-        BSE_CUDA_TRY(ctx, cudaFuncSetAttribute(k_near_field<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    BSE_CUDA_TRY(ctx, bse_raise_smem(k_near_field<T>, smem));
     k_near_field<T><<<s->nk, 256, smem, ctx->stream>>>((const V*)X, s->d_list, s->d_list_start, (const T*)s->d_hd,
                                                       (const V*)s->d_Hv, (const V*)s->d_Hc, (const T*)s->d_hc, s->n,
                                                       s->nd, s->nv, s->nc, s->nb1, s->smin, s->ns1, s->rmin, s->nr1,

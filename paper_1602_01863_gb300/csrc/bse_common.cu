@@ -1003,18 +1003,6 @@ int rot_chains(const bse_ctx* ctx, const bse_interp* s, int nchains) {
     return s->co->nkc >= 2 * std::max(ctx->sm_count, 1) ? nchains : 1;
 }
 
-// `fixed`: at least the kernel's static shared memory.  Within the 48 KB that every
-// kernel has there is nothing to ask the driver for (2 to 4 us a launch).
-template <typename K>
-cudaError_t raise_smem(K kernel, size_t bytes, size_t fixed) {
-    if (bytes + fixed <= 48 * 1024) return cudaSuccess;
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-    if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < bytes)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    return e;
-}
-
 // Targets of a warp within a cell: TZ = n_div up to 4 (then blocks of 4), TY rows
 // (FP32: pairs of rows of the zone).
 inline int near_tz(int nd) { return std::min(nd, 4); }
@@ -1058,7 +1046,7 @@ int launch_near_k(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, K k
     ns.split = ns.cz == 1 && warps <= 4LL * ctx->sm_count && ns.nsteps >= 8;
     const int wpb = ns.split ? 4 : (warps >= 8LL * ctx->sm_count ? 4 : 2);
     const size_t smem = (size_t)ns.wbytes * wpb + (ns.split ? 3 * 32 * sizeof(double) * near_ty<T>(ns.nd) * near_tz(ns.nd) : 0);
-    BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, 0));
+    BSE_CUDA_TRY(ctx, bse_raise_smem(kernel, smem, 0));
     kernel<<<(unsigned)(ns.split ? warps : (warps + wpb - 1) / wpb), 32 * wpb, smem, st>>>((const T*)work.phi, (const T*)s->d_cw, s->d_csteps,
                                                                        (T*)work.V, ns);
     BSE_CUDA_TRY(ctx, cudaGetLastError());
@@ -1104,7 +1092,7 @@ int restrict_typed(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, in
     CommonPhi lay{s->cphi_R, s->cphi_Lp};
     const dim3 grid(c->nkc, (nchains + CPB - 1) / CPB);
     auto go = [&](auto kernel) -> int {
-        BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, 64));
+        BSE_CUDA_TRY(ctx, bse_raise_smem(kernel, smem, 64));
         kernel<<<grid, 256, smem, st>>>((const V*)psi, (const V*)s->d_cUv, (const V*)s->d_cUc, (const V*)s->d_cUvc,
                                         (const V*)s->d_cUcc, s->n, s->nd, s->nv, s->nc, s->nb1, nchains, CPB, KP,
                                         m3 ? (T*)work.phi : nullptr, lay, (V*)work.share, work.ctr, (V*)Q, bop, c->ldk);
@@ -1124,7 +1112,7 @@ int prolong_typed(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int
                         8 * WarpStage<T>::bytes(KP, s->nv, s->nc);
     const dim3 grid(bse_common_dot_blocks(s), (nchains + CPB - 1) / CPB);
     auto go = [&](auto kernel) -> int {
-        BSE_CUDA_TRY(ctx, raise_smem(kernel, smem, sizeof(DotSum<T>) * BSE_MAX_CHAINS * 256));
+        BSE_CUDA_TRY(ctx, bse_raise_smem(kernel, smem, sizeof(DotSum<T>) * BSE_MAX_CHAINS * 256));
         kernel<<<grid, 256, smem, st>>>((const V*)R, s->scheme == BSE_SCHEME_M3 ? (const V*)work.V : nullptr,
                                         (const V*)s->d_cUv, (const V*)s->d_cUc, (const V*)s->d_cUvc, (const V*)s->d_cUcc,
                                         (const T*)s->d_dE, (const V*)psi, s->n, s->nd, s->nv, s->nc, s->nb1, nchains, CPB, KP,

@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -378,6 +379,25 @@ inline cudaError_t bse_download(bse_ctx* ctx, void* dst, const void* src, size_t
 inline const char* bse_timeout_message(int status) {
     if (status & 2) return "a bounded device wait in the tensor-core near field gave up";
     return "a bounded device wait in the tensor-core K_c apply gave up";
+}
+
+// Raises a kernel's limit of dynamic shared memory to `bytes`, never lowers it: handles of
+// different sizes share the limit, and so do threads with contexts of their own, hence the
+// lock.  `fixed`: at least the kernel's static shared memory; within the 48 KB that every
+// kernel has there is nothing to ask the driver for (2 to 4 us a launch).
+inline std::mutex& bse_smem_mutex() {
+    static std::mutex m;
+    return m;
+}
+template <typename K>
+inline cudaError_t bse_raise_smem(K kernel, size_t bytes, size_t fixed = 0) {
+    if (bytes + fixed <= 48 * 1024) return cudaSuccess;
+    std::lock_guard<std::mutex> lock(bse_smem_mutex());
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+    if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < bytes)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return e;
 }
 
 // setup kernels (bse_setup.cu)

@@ -352,16 +352,8 @@ LShape shape(const bse_interp* s, int nch) {
 }
 
 size_t plane_smem(int L) { return sizeof(float2) * (64 + (size_t)EG * L * (L | 1)); }
+constexpr size_t kPlaneFixed = 1024;          // axis tables and warp sums, rounded up
 size_t mix_smem(int L, int t, int nch) { return sizeof(float2) * (64 + 2 * (size_t)L * nch * t); }
-
-template <typename K>
-int raise_smem(bse_ctx* ctx, K kernel, size_t bytes) {
-    cudaFuncAttributes fa;
-    BSE_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, kernel));
-    if ((size_t)fa.maxDynamicSharedSizeBytes < bytes)
-        BSE_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    return BSE_OK;
-}
 
 template <typename T>
 int apply_typed(bse_ctx* ctx, const bse_interp* s, int nch, const void* psi, void* w, double2* dot) {
@@ -370,16 +362,15 @@ int apply_typed(bse_ctx* ctx, const bse_interp* s, int nch, const void* psi, voi
     const int L = q.L, eb = (s->t + EG - 1) / EG;
     cudaStream_t st = ctx->stream;
     const size_t ps = plane_smem(L), ms = mix_smem(L, s->t, nch);
-    int rc;
-    if ((rc = raise_smem(ctx, k_lconv_fwd<T, false>, ps)) != BSE_OK || (rc = raise_smem(ctx, k_lconv_inv<T>, ps)) != BSE_OK) return rc;
+    BSE_CUDA_TRY(ctx, bse_raise_smem((k_lconv_fwd<T, false>), ps, kPlaneFixed));
+    BSE_CUDA_TRY(ctx, bse_raise_smem(k_lconv_inv<T>, ps, kPlaneFixed));
     k_lconv_fwd<T, false><<<dim3(L, eb, nch), LTHR, ps, st>>>((const V*)psi, q, s->t, s->d_tw_fwd, s->d_lgrid);
     auto mix = [&](auto kernel) -> int {
-        int r = raise_smem(ctx, kernel, ms);
-        if (r != BSE_OK) return r;
+        BSE_CUDA_TRY(ctx, bse_raise_smem(kernel, ms));
         kernel<<<L * L, LTHR, ms, st>>>(s->d_lgrid, s->d_lker, q, s->d_tw_fwd);
         return BSE_OK;
     };
-    rc = nch == 1 ? mix(k_lconv_mix<1>) : nch == 2 ? mix(k_lconv_mix<2>) : nch == 3 ? mix(k_lconv_mix<3>) : mix(k_lconv_mix<4>);
+    const int rc = nch == 1 ? mix(k_lconv_mix<1>) : nch == 2 ? mix(k_lconv_mix<2>) : nch == 3 ? mix(k_lconv_mix<3>) : mix(k_lconv_mix<4>);
     if (rc != BSE_OK) return rc;
     k_lconv_inv<T><<<dim3(L, eb, nch), LTHR, ps, st>>>(s->d_lgrid, q, s->d_tw_fwd, (const V*)psi, (V*)w,
                                                         1.f / ((float)L * L * L), dot);
@@ -407,8 +398,8 @@ int bse_lconv_kernel(bse_ctx* ctx, const bse_interp* s, const float2* ker, float
     const LShape q = shape(s, 1);
     const int L = q.L, chan = s->t * s->t, chunk = std::min(chan, 2048 / L);
     const size_t ps = plane_smem(L), xs = sizeof(float2) * (64 + (size_t)L * chunk);
-    int rc;
-    if ((rc = raise_smem(ctx, k_lconv_fwd<float, true>, ps)) != BSE_OK || (rc = raise_smem(ctx, k_lconv_x, xs)) != BSE_OK) return rc;
+    BSE_CUDA_TRY(ctx, bse_raise_smem((k_lconv_fwd<float, true>), ps, kPlaneFixed));
+    BSE_CUDA_TRY(ctx, bse_raise_smem(k_lconv_x, xs));
     k_lconv_fwd<float, true><<<dim3(L, (chan + EG - 1) / EG, 1), LTHR, ps, ctx->stream>>>(ker, q, chan, s->d_tw_fwd, out);
     k_lconv_x<<<dim3(L * L, (chan + chunk - 1) / chunk), LTHR, xs, ctx->stream>>>(out, q, chan, chunk, s->d_tw_fwd);
     BSE_CUDA_TRY(ctx, cudaGetLastError());

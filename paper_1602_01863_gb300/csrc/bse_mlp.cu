@@ -364,20 +364,10 @@ MlpOffs mlp_offs(int d_in) {
     return o;
 }
 
-template <typename Kern>
-int mlp_attr(bse_ctx* ctx, Kern k, size_t bytes) {
-    cudaFuncAttributes fa;
-    BSE_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, k));
-    if ((size_t)fa.maxDynamicSharedSizeBytes < bytes)
-        BSE_CUDA_TRY(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    return BSE_OK;
-}
-
 // Forward over a batch: out [B][2] (device).
 int mlp_forward(bse_ctx* ctx, bse_mlp* m, int B, const float* X, float* out) {
     const size_t sm = mlp_smem(false);
-    int rc = mlp_attr(ctx, k_mlp<false>, sm);
-    if (rc != BSE_OK) return rc;
+    BSE_CUDA_TRY(ctx, bse_raise_smem(k_mlp<false>, sm));
     k_mlp<false><<<std::min((B + RT - 1) / RT, 2 * std::max(ctx->sm_count, 1)), TPB, sm, ctx->stream>>>(
         X, nullptr, m->d_in, B, m->d_w, m->d_p, mlp_offs(m->d_in), 0.f, out, nullptr, m->nparams, nullptr);
     BSE_CUDA_TRY(ctx, cudaGetLastError());
@@ -388,8 +378,7 @@ int mlp_forward(bse_ctx* ctx, bse_mlp* m, int B, const float* X, float* out) {
 // error summed over Re, Im) into *loss.
 int mlp_grads(bse_ctx* ctx, bse_mlp* m, int B, const float* X, const float* Y, double* loss) {
     const size_t sm = mlp_smem(true);
-    int rc = mlp_attr(ctx, k_mlp<true>, sm);
-    if (rc != BSE_OK) return rc;
+    BSE_CUDA_TRY(ctx, bse_raise_smem(k_mlp<true>, sm));
     const int nblk = std::min((B + RT - 1) / RT, m->blocks);
     k_mlp<true><<<nblk, TPB, sm, ctx->stream>>>(X, Y, m->d_in, B, m->d_w, m->d_p, mlp_offs(m->d_in), 1.f / B, nullptr,
                                                 m->d_gpart, m->nparams, m->d_part);
@@ -897,11 +886,7 @@ int dft3(bse_ctx* ctx, float2* a, float2* tmp, int L, long long nchan, const flo
         const long long nlines = nchan * L * L;
         const int P = (L & 1) ? L + 2 : L + 1;
         const size_t smem = sizeof(float2) * (64 + 2 * 32 * (size_t)P);
-        static bool attr = false;
-        if (!attr) {
-            BSE_CUDA_TRY(ctx, cudaFuncSetAttribute(k_dft_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-            attr = true;
-        }
+        BSE_CUDA_TRY(ctx, bse_raise_smem(k_dft_tile, smem));
         const unsigned blocks = (unsigned)((nlines + 31) / 32);
         for (int axis = 0; axis < 3; ++axis) k_dft_tile<<<blocks, 256, smem, ctx->stream>>>(a, L, nlines, axis, tw);
         return BSE_OK;
@@ -1050,8 +1035,7 @@ int bse_pairs_generate(bse_ctx* ctx, const bse_interp* s, int nblocks, const int
     auto go = [&](auto tag) -> int {
         using T = decltype(tag);
         using V = typename Cx<T>::V;
-        int r = mlp_attr(ctx, k_pairs<T>, sm);
-        if (r != BSE_OK) return r;
+        BSE_CUDA_TRY(ctx, bse_raise_smem(k_pairs<T>, sm, 1024));
         k_pairs<T><<<nblocks, PTHR, sm, ctx->stream>>>(d1, d2, c->d_gen_v, c->d_gen_c, c->d_mu, c->d_Uv, c->d_Uc,
                                                        (const V*)c->d_kc, (const V*)s->d_Dv, (const V*)s->d_Dc, (const T*)s->d_dE,
                                                        s->n, s->nd, s->nv, s->nc, s->nb1, c->e_k, 1.0 / c->eps_inf, c->kappa,

@@ -640,11 +640,7 @@ int bse_near_tc_launch(bse_ctx* ctx, const bse_interp* s, int nchains, const voi
     for (int c0 = 0; c0 < nchains; c0 += 3) {
         const int nch = std::min(3, nchains - c0);
         const size_t smem = near_tc_smem(nch, s->nf_tc_nsl, s->nf_tc_nkg, s->nslot);
-        // handles of different sizes share the kernel's attribute: only ever raise it
-        cudaFuncAttributes fa;
-        BSE_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, k_near_tc));
-        if ((size_t)fa.maxDynamicSharedSizeBytes < smem)
-            BSE_CUDA_TRY(ctx, cudaFuncSetAttribute(k_near_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        BSE_CUDA_TRY(ctx, bse_raise_smem(k_near_tc, smem, 1024));
         const size_t xoff = (size_t)c0 * s->nk * 8 * s->nf_tc_tpad;
         const size_t uoff = (size_t)c0 * s->nk * 8 * s->t;
         // One CTA per coarse cell fills the SMs in waves; when the last wave

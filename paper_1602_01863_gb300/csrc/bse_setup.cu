@@ -501,18 +501,6 @@ __global__ void k_near_head(const int* __restrict__ offs, int n_near, int L, dou
     hd[i] = (T)(1.0 / (qa * qa + qb * qb + qc * qc + kappa * kappa));
 }
 
-// Within the 48 KB that every kernel has there is nothing to ask the driver for (these
-// kernels have no shared memory but the dynamic one).
-template <typename K>
-int raise_smem(bse_ctx* ctx, K kernel, size_t bytes) {
-    if (bytes <= 48 * 1024) return BSE_OK;
-    cudaFuncAttributes fa;
-    BSE_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, kernel));
-    if ((size_t)fa.maxDynamicSharedSizeBytes < bytes)
-        BSE_CUDA_TRY(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    return BSE_OK;
-}
-
 inline int blocks_for(long long n, int bs) { return (int)((n + bs - 1) / bs); }
 
 }  // namespace
@@ -543,7 +531,7 @@ int bse_setup_coarse_device(bse_ctx* ctx, bse_coarse* c, const void* user_kc) {
     TRY(bse_alloc(ctx, (void**)&c->d_Uv, sizeof(double2) * nkc * nv * nv, "coarse Uv"));
     TRY(bse_alloc(ctx, (void**)&c->d_Uc, sizeof(double2) * nkc * nc * nc, "coarse Uc"));
     const size_t gsm = sizeof(double2) * 4 * kGaugeMats * (nv * nv + nc * nc);
-    TRY(raise_smem(ctx, k_gauge, gsm));
+    BSE_CUDA_TRY(ctx, bse_raise_smem(k_gauge, gsm));
     k_gauge<<<blocks_for(nkc, 4), 128, gsm, st>>>(c->d_gen_v, c->d_gen_c, nv, nc, n, c->d_Uv, c->d_Uc);
     double2* d_M = nullptr;
     double* d_h = nullptr;
@@ -551,7 +539,7 @@ int bse_setup_coarse_device(bse_ctx* ctx, bse_coarse* c, const void* user_kc) {
         TRY(bse_alloc(ctx, (void**)&d_M, sizeof(double2) * nkc * 26 * nv * nc, "form factors"));
         TRY(bse_alloc(ctx, (void**)&d_h, sizeof(double) * nkc, "shape table"));
         const size_t fsm = sizeof(double2) * (52 * nv * nc + nv * nv + nc * nc);
-        TRY(raise_smem(ctx, k_form_factors, fsm));
+        BSE_CUDA_TRY(ctx, bse_raise_smem(k_form_factors, fsm));
         k_form_factors<<<nkc, 256, fsm, st>>>(c->d_Uv, c->d_Uc, c->d_mu, n, nv, nc, d_M);
         k_shape_table<<<blocks_for(nkc, 4), 128, 0, st>>>(n, c->kappa, c->direct_shells, c->h_const, c->h0, 0, d_h);
     }
@@ -573,8 +561,7 @@ int bse_setup_coarse_device(bse_ctx* ctx, bse_coarse* c, const void* user_kc) {
     const dim3 gs(kt, kt);
     const size_t ksm = kc_smem(nv, nc, P);
     auto build = [&](auto kernel, void* out, __nv_bfloat16* kr, __nv_bfloat16* ki) -> int {
-        int r = raise_smem(ctx, kernel, ksm);
-        if (r != BSE_OK) return r;
+        BSE_CUDA_TRY(ctx, bse_raise_smem(kernel, ksm));
         kernel<<<gs, 256, ksm, st>>>(d_M, c->d_Uv, c->d_Uc, d_h, n, nv, nc, P, pref, 1.0 / c->eps_inf, c->exchange_on, Nc, c->ldk,
                                      out, kr, ki);
         return BSE_OK;
@@ -759,7 +746,7 @@ int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dens
     auto tables = [&](auto lanes) -> int {
         constexpr int G = decltype(lanes)::value;
         const size_t dsm = dense_smem(nv, nc, n * nd);
-        TRY(raise_smem(ctx, k_dense_tables<T, G>, dsm));
+        BSE_CUDA_TRY(ctx, bse_raise_smem((k_dense_tables<T, G>), dsm));
         const int blocks = std::min(blocks_for(nk, kDenseWarps * (16 / G)), 16 * std::max(ctx->sm_count, 1));
         k_dense_tables<T, G><<<blocks, 32 * kDenseWarps, dsm, st>>>(
             c->d_gen_v, c->d_gen_c, c->d_Uv, c->d_Uc, c->d_offsets, c->d_dip, n, nd, nv, nc, c->e_gap, c->band_width,
