@@ -33,8 +33,7 @@ sys.path.insert(0, ROOT)
 
 N_OMEGA = 1000
 # DRAM bytes (read + write) of one near-stencil launch on this workload from the
-# committed ncu capture (profiles/k_common_single_system.md), or None when the
-# kernel changed since the capture.
+# committed ncu capture, or None when the kernel changed since the capture.
 NEAR_TRAFFIC = 15.9e6
 
 
@@ -127,14 +126,13 @@ class Clocks:
 def algorithmic(sysd, nchains, kc_bytes_per_entry, vec_bytes):
     """Algorithmic bytes / flops per launch of each kernel class (one Lanczos step)."""
     nv, nc = sysd["nv"], sysd["nc"]
-    t = nv * nc
-    Nc, N, Nk, nd = sysd["Nc"], sysd["N"], sysd["Nk"], sysd["n_div"]
-    nbar = ((nd + (nd - 1)) / nd) ** 3                      # non-zero-weight corners per dense k
-    dbytes = Nk * nbar * (nv * nv + nc * nc) * vec_bytes     # one pass over the d tables
+    Nc, N, Nk = sysd["Nc"], sysd["N"], sysd["Nk"]
+    gauge = Nk * (nv * nv + nc * nc) * vec_bytes             # one pass over U(k), both manifolds
     return {
         "kc_apply": {"bytes": Nc * Nc * kc_bytes_per_entry, "flops": 8.0 * nchains * Nc * Nc},
-        "restrict": {"bytes": dbytes + nchains * N * vec_bytes + nchains * Nk * nbar * t * vec_bytes},
-        "prolong": {"bytes": dbytes + nchains * (3 * N * vec_bytes + Nk * nbar * t * vec_bytes) + N * vec_bytes / 2},
+        # psi in, phi out, Q out; then R, V, psi and dE in, w out
+        "restrict": {"bytes": gauge + nchains * (2 * N + Nc) * vec_bytes},
+        "prolong": {"bytes": gauge + nchains * (3 * N + Nc) * vec_bytes + N * vec_bytes / 2},
     }
 
 
@@ -274,7 +272,9 @@ def run_ours(args):
         # the scalar stencil in the common basis: one FP32 multiply-add per target column and near offset
         flops = 2.0 * near_field_offsets(sysm.n_div, 1.0) * 2 * info["N"] * p
         achieved = flops / (kt[dom][0] * 1e-3) / 1e12
-        fp32_peak = 2 * 128 * 152 * 2.07e-3                 # nominal: 128 FP32 multiply-adds per SM and clock at 2070 MHz
+        # nominal: 128 FP32 multiply-adds per SM and clock, at the clock sampled during the timed runs
+        sms = torch.cuda.get_device_properties(local).multi_processor_count
+        fp32_peak = 2 * 128 * sms * (clk["sm_mhz"] or 2070.0) * 1e-6
         roof = {"bound": "fp32", "kernel": "k_common_near32 (M3 near pairs as a stencil in the common basis, packed FP32)",
                 "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s", "frac": achieved / fp32_peak,
                 "traffic": NEAR_TRAFFIC, "peak_source": "nominal FP32 rate (no measured one)",

@@ -176,9 +176,11 @@ typedef struct bse_dense_inputs {
  * |delta|^2 <= floor(width_w^2 n_div^2 + 1e-9).
  * `vec_prec` (F64 or F32) is the precision of the Lanczos vectors and of the
  * restrict / prolong / near-field arithmetic; the Lanczos reductions sum
- * across warps and blocks in FP64 in every mode (with F32 vectors each
- * thread first sums its few products in FP32, and the ||w||^2 of the Lanczos
- * update is also summed over a warp's 32 threads in FP32).  The coarse
+ * across warps and blocks in FP64 in every mode.  With F32 vectors a thread's
+ * share of <psi, w> keeps the roundings of its sum in a second FP32 word where
+ * the overlaps are the model's; with the caller's, rows of a few products are
+ * summed in FP32 for 3x3, 4x4 and 4x6 bands; the ||w||^2 of the Lanczos update
+ * is summed in FP32 over a thread's few products and a warp's 32 threads.  The coarse
  * handle must outlive the interp handle.
  * With BF16 K_c the set-up autotunes the tensor-core apply: it times its
  * pipeline depths (4, 5, 6 stages) and chunk lengths (8 to 64 k-blocks) on

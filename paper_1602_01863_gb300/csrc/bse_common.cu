@@ -129,37 +129,37 @@ __device__ __forceinline__ void rotate_warp(V* x, V* tmp, int tp, const V* Uv, i
             x[p * tp + e] = a;
         }
     } else {
-    for (int i = lane; i < np * nv; i += 32) {
-        const int p = quot(i, inv_v), v = i - p * nv;
-        V* r = x + p * tp + v * nc;
-        const V* U = Uc + p * rcp;
-        switch (nc) {
-            case 1: rot_row<TO, 1>(r, U); break;
-            case 2: rot_row<TO, 2>(r, U); break;
-            case 3: rot_row<TO, 3>(r, U); break;
-            case 4: rot_row<TO, 4>(r, U); break;
-            case 5: rot_row<TO, 5>(r, U); break;
-            case 6: rot_row<TO, 6>(r, U); break;
-            case 7: rot_row<TO, 7>(r, U); break;
-            default: rot_row<TO, 8>(r, U); break;
+        for (int i = lane; i < np * nv; i += 32) {
+            const int p = quot(i, inv_v), v = i - p * nv;
+            V* r = x + p * tp + v * nc;
+            const V* U = Uc + p * rcp;
+            switch (nc) {
+                case 1: rot_row<TO, 1>(r, U); break;
+                case 2: rot_row<TO, 2>(r, U); break;
+                case 3: rot_row<TO, 3>(r, U); break;
+                case 4: rot_row<TO, 4>(r, U); break;
+                case 5: rot_row<TO, 5>(r, U); break;
+                case 6: rot_row<TO, 6>(r, U); break;
+                case 7: rot_row<TO, 7>(r, U); break;
+                default: rot_row<TO, 8>(r, U); break;
+            }
         }
-    }
-    __syncwarp();
-    for (int i = lane; i < np * nc; i += 32) {
-        const int p = quot(i, inv_c), c = i - p * nc;
-        V* r = x + p * tp + c;
-        const V* U = Uv + p * rvp;
-        switch (nv) {
-            case 1: rot_col<TO, 1>(r, nc, U); break;
-            case 2: rot_col<TO, 2>(r, nc, U); break;
-            case 3: rot_col<TO, 3>(r, nc, U); break;
-            case 4: rot_col<TO, 4>(r, nc, U); break;
-            case 5: rot_col<TO, 5>(r, nc, U); break;
-            case 6: rot_col<TO, 6>(r, nc, U); break;
-            case 7: rot_col<TO, 7>(r, nc, U); break;
-            default: rot_col<TO, 8>(r, nc, U); break;
+        __syncwarp();
+        for (int i = lane; i < np * nc; i += 32) {
+            const int p = quot(i, inv_c), c = i - p * nc;
+            V* r = x + p * tp + c;
+            const V* U = Uv + p * rvp;
+            switch (nv) {
+                case 1: rot_col<TO, 1>(r, nc, U); break;
+                case 2: rot_col<TO, 2>(r, nc, U); break;
+                case 3: rot_col<TO, 3>(r, nc, U); break;
+                case 4: rot_col<TO, 4>(r, nc, U); break;
+                case 5: rot_col<TO, 5>(r, nc, U); break;
+                case 6: rot_col<TO, 6>(r, nc, U); break;
+                case 7: rot_col<TO, 7>(r, nc, U); break;
+                default: rot_col<TO, 8>(r, nc, U); break;
+            }
         }
-    }
     }
     __syncwarp();
 }

@@ -116,7 +116,7 @@ __device__ __forceinline__ int quot(int i, float inv) { return (int)(((float)i +
 // TW: multiply element j by tw[c j] (conjugated for INV) after (forward) or before
 // (inverse) the DFT.
 template <int N, bool INV, bool TW, typename At>
-__device__ __forceinline__ void stage_n(float2* s, int nlines, At at, int es, int cnt, int first, int step, int L, const float2* tw) {
+__device__ __forceinline__ void stage_n(float2* s, int nlines, At at, int es, int cnt, int first, int step, const float2* tw) {
     const float inv = 1.f / (float)nlines;
     for (int it = threadIdx.x; it < nlines * cnt; it += LTHR) {
         const int c = quot(it, inv), l = it - c * nlines;
@@ -138,29 +138,29 @@ __device__ __forceinline__ void stage_n(float2* s, int nlines, At at, int es, in
     }
 }
 template <bool INV, bool TW, typename At>
-__device__ __forceinline__ void stage(int N, float2* s, int nlines, At at, int es, int cnt, int first, int step, int L, const float2* tw) {
+__device__ __forceinline__ void stage(int N, float2* s, int nlines, At at, int es, int cnt, int first, int step, const float2* tw) {
     switch (N) {
-        case 1: stage_n<1, INV, TW>(s, nlines, at, es, cnt, first, step, L, tw); break;
-        case 2: stage_n<2, INV, TW>(s, nlines, at, es, cnt, first, step, L, tw); break;
-        case 3: stage_n<3, INV, TW>(s, nlines, at, es, cnt, first, step, L, tw); break;
-        case 4: stage_n<4, INV, TW>(s, nlines, at, es, cnt, first, step, L, tw); break;
-        case 5: stage_n<5, INV, TW>(s, nlines, at, es, cnt, first, step, L, tw); break;
-        case 6: stage_n<6, INV, TW>(s, nlines, at, es, cnt, first, step, L, tw); break;
-        case 7: stage_n<7, INV, TW>(s, nlines, at, es, cnt, first, step, L, tw); break;
-        default: stage_n<8, INV, TW>(s, nlines, at, es, cnt, first, step, L, tw); break;
+        case 1: stage_n<1, INV, TW>(s, nlines, at, es, cnt, first, step, tw); break;
+        case 2: stage_n<2, INV, TW>(s, nlines, at, es, cnt, first, step, tw); break;
+        case 3: stage_n<3, INV, TW>(s, nlines, at, es, cnt, first, step, tw); break;
+        case 4: stage_n<4, INV, TW>(s, nlines, at, es, cnt, first, step, tw); break;
+        case 5: stage_n<5, INV, TW>(s, nlines, at, es, cnt, first, step, tw); break;
+        case 6: stage_n<6, INV, TW>(s, nlines, at, es, cnt, first, step, tw); break;
+        case 7: stage_n<7, INV, TW>(s, nlines, at, es, cnt, first, step, tw); break;
+        default: stage_n<8, INV, TW>(s, nlines, at, es, cnt, first, step, tw); break;
     }
     __syncthreads();
 }
 // Line transforms, block-wide: n = B n1 + n2, k = k1 + A k2 left at place B k1 + k2.
 template <typename At>
-__device__ __forceinline__ void lines_fwd(float2* s, int nlines, At at, int es, int L, int A, int B, const float2* tw) {
-    stage<false, true>(A, s, nlines, at, es, B, 1, B, L, tw);      // over n1 for every n2, then w^{n2 k1}
-    stage<false, false>(B, s, nlines, at, es, A, B, 1, L, tw);     // over n2 for every k1
+__device__ __forceinline__ void lines_fwd(float2* s, int nlines, At at, int es, int A, int B, const float2* tw) {
+    stage<false, true>(A, s, nlines, at, es, B, 1, B, tw);      // over n1 for every n2, then w^{n2 k1}
+    stage<false, false>(B, s, nlines, at, es, A, B, 1, tw);     // over n2 for every k1
 }
 template <typename At>
-__device__ __forceinline__ void lines_inv(float2* s, int nlines, At at, int es, int L, int A, int B, const float2* tw) {
-    stage<true, false>(B, s, nlines, at, es, A, B, 1, L, tw);
-    stage<true, true>(A, s, nlines, at, es, B, 1, B, L, tw);
+__device__ __forceinline__ void lines_inv(float2* s, int nlines, At at, int es, int A, int B, const float2* tw) {
+    stage<true, false>(B, s, nlines, at, es, A, B, 1, tw);
+    stage<true, true>(A, s, nlines, at, es, B, 1, B, tw);
 }
 
 struct LShape { int L, A, B, n, nd, t, nch, P; };   // P: row pitch of a plane (odd)
@@ -212,8 +212,8 @@ __global__ void __launch_bounds__(LTHR) k_lconv_fwd(const typename Cx<T>::V* __r
     }
     __syncthreads();
     // z lines: one per (e, y); y lines: one per (e, z)
-    lines_fwd(s, ne * L, [&](int l) { return l * P; }, 1, L, q.A, q.B, tw);
-    lines_fwd(s, ne * L, [&](int l) { const int e = quot(l, inv_L); return e * (L - 1) * P + e * (P - L) + l; }, P, L, q.A, q.B, tw);
+    lines_fwd(s, ne * L, [&](int l) { return l * P; }, 1, q.A, q.B, tw);
+    lines_fwd(s, ne * L, [&](int l) { const int e = quot(l, inv_L); return e * (L - 1) * P + e * (P - L) + l; }, P, q.A, q.B, tw);
     float2* out = grid + (size_t)x * q.nch * chan + (size_t)ch * chan + e0;
     for (int i = tid; i < L2 * EG; i += LTHR) {
         const int e = i & (EG - 1), p = i / EG, y = quot(p, inv_L), z = p - y * L;
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(LTHR) k_lconv_x(float2* __restrict__ grid, con
     float2* g = grid + (size_t)blockIdx.x * L * chan + c0;
     for (int i = tid; i < L * nc; i += LTHR) s[i] = g[(size_t)(i / nc) * chan + i % nc];
     __syncthreads();
-    lines_fwd(s, nc, [](int l) { return l; }, nc, L, q.A, q.B, tw);
+    lines_fwd(s, nc, [](int l) { return l; }, nc, q.A, q.B, tw);
     for (int i = tid; i < L * nc; i += LTHR) g[(size_t)(i / nc) * chan + i % nc] = s[i];
 }
 
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(LTHR) k_lconv_mix(float2* __restrict__ grid, c
     float2* g = grid + (size_t)blockIdx.x * L * c;
     for (int i = tid; i < L * c; i += LTHR) a[i] = g[i];
     __syncthreads();
-    lines_fwd(a, c, [](int l) { return l; }, c, L, q.A, q.B, tw);
+    lines_fwd(a, c, [](int l) { return l; }, c, q.A, q.B, tw);
     const float2* Tq = That + (size_t)blockIdx.x * L * t * t;
     const float inv_t = 1.f / (float)t;
     for (int i = tid; i < L * t; i += LTHR) {
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(LTHR) k_lconv_mix(float2* __restrict__ grid, c
         for (int ch = 0; ch < NCH; ++ch) b[x * c + ch * t + e1] = acc[ch];
     }
     __syncthreads();
-    lines_inv(b, c, [](int l) { return l; }, c, L, q.A, q.B, tw);
+    lines_inv(b, c, [](int l) { return l; }, c, q.A, q.B, tw);
     for (int i = tid; i < L * c; i += LTHR) g[i] = b[i];
 }
 
@@ -301,8 +301,8 @@ __global__ void __launch_bounds__(LTHR) k_lconv_inv(const float2* __restrict__ g
         if (e < ne) s[(e * L + y) * P + z] = in[(size_t)p * L * q.nch * q.t + e];
     }
     __syncthreads();
-    lines_inv(s, ne * L, [&](int l) { const int e = quot(l, inv_L); return e * (L - 1) * P + e * (P - L) + l; }, P, L, q.A, q.B, tw);
-    lines_inv(s, ne * L, [&](int l) { return l * P; }, 1, L, q.A, q.B, tw);
+    lines_inv(s, ne * L, [&](int l) { const int e = quot(l, inv_L); return e * (L - 1) * P + e * (P - L) + l; }, P, q.A, q.B, tw);
+    lines_inv(s, ne * L, [&](int l) { return l * P; }, 1, q.A, q.B, tw);
     const size_t nk = (size_t)L2 * L;
     DotSum<T> dot;
 #pragma unroll 4

@@ -24,7 +24,7 @@
 // 64 registers a thread (five blocks' bound; the grid has one per SM): what it leaves of an SM's
 // registers the near stencil uses beside it.  With 190 registers one of that kernel's
 // blocks fitted, with 64 four do: the stencil beside the apply 123 -> 110 us, the apply 64 -> 70 us
-// there (N_c 8192) and 1.05 ms either way for 6.9 GB alone.
+// there (N_c 8192) and 1.05 ms either way for 6.9 GB alone.  32 bytes a thread spill.
 //
 // Warp roles (192 threads): warp 0 TMA producer, warp 1 MMA issuer and TMEM
 // owner, warps 2-5 epilogue (TMEM lanes 32 (w % 4) .. + 31).  Every mbarrier
