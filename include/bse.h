@@ -229,9 +229,9 @@ int bse_apply_h(bse_ctx* ctx, bse_interp* interp, int nvec, const void* x, void*
  * scratch comes from one static device array of 32 MiB inside the library
  * (held by a device from the time the library's device module is loaded on
  * it, at the latest the first bse_ctx_create on that device, until the
- * process exits), not from the handle; where the overlaps are the model's, the
- * intermediate vectors of these calls are a set of their own that
- * bse_interp_setup allocates.  So one such call may run beside another call on
+ * process exits), not from the buffers of the handle's other calls (for some
+ * sizes with up to three transitions bse_interp_setup allocates a set of
+ * intermediate vectors for it).  So one such call may run beside another call on
  * the same handle (through a context of its own).  The paper has no counterpart; this
  * exists for callers that must not call cudaMalloc once their work has
  * started, such as a host framework that owns all device memory through its

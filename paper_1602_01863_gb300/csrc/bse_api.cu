@@ -59,7 +59,7 @@ void free_interp(bse_interp* s) {
                     s->d_basis, s->d_cgs_part, s->d_cgs_h, s->d_cgs_ctr, s->d_pairs, s->d_clist, s->d_cstart,
                     s->d_lker, s->d_lgrid, s->d_tw_fwd, s->d_tc_rows, s->d_tc_slots,
                     s->d_tc_kinfo, s->d_tc_simg, s->d_tc_aimg, s->d_xscale, s->d_xscale_gen, s->d_H2,
-                    s->d_cUv, s->d_cUc, s->d_cUvc, s->d_cUcc, s->cwork[0].share, s->cwork[0].ctr, s->d_chead, s->cwork[0].phi, s->cwork[0].V,
+                    s->d_cUv, s->d_cUc, s->d_cUvc, s->d_cUcc, s->cwork.share, s->cwork.ctr, s->d_chead, s->cwork.phi, s->cwork.V, s->d_na,
                     s->d_cw, s->d_csteps};
     for (void* p : ptrs) cudaFree(p);
     bse_tc_release(s);

@@ -1858,7 +1858,7 @@ int apply_h_common(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi, vo
     int rc;
     {
         Timer tm(ctx, prof, KC_RESTRICT);
-        if ((rc = bse_common_restrict(ctx, s, s->cwork[0], nchains, psi, s->d_Q, s->d_Bop, st)) != BSE_OK) return rc;
+        if ((rc = bse_common_restrict(ctx, s, s->cwork, nchains, psi, s->d_Q, s->d_Bop, st)) != BSE_OK) return rc;
     }
     cudaStream_t kst = beside ? ctx->aux[ln] : st;
     if (beside) {
@@ -1875,7 +1875,7 @@ int apply_h_common(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi, vo
     }
     if (m3) {
         Timer tm(ctx, prof, KC_NEAR);
-        if ((rc = bse_common_near(ctx, s, s->cwork[0], nchains, st)) != BSE_OK) return rc;
+        if ((rc = bse_common_near(ctx, s, s->cwork, nchains, st)) != BSE_OK) return rc;
     }
     if (beside) {
         BSE_CUDA_TRY(ctx, cudaEventRecord(ctx->aux_join[ln], kst));
@@ -1883,7 +1883,7 @@ int apply_h_common(bse_ctx* ctx, bse_interp* s, int nchains, const void* psi, vo
     }
     {
         Timer tm(ctx, prof, KC_PROLONG);
-        if ((rc = bse_common_prolong(ctx, s, s->cwork[0], nchains, s->d_R, psi, W, s->d_part_dot, st)) != BSE_OK) return rc;
+        if ((rc = bse_common_prolong(ctx, s, s->cwork, nchains, s->d_R, psi, W, s->d_part_dot, st)) != BSE_OK) return rc;
     }
     if (s->learned) {
         Timer tm(ctx, prof, KC_NEAR);
@@ -2523,16 +2523,17 @@ int apply_scratch_typed(bse_ctx* ctx, const bse_interp* s, int nchains, const vo
     const bool m3 = s->scheme == BSE_SCHEME_M3;
     if (s->common) {
         int rc;
+        BSE_CUDA_TRY(ctx, cudaMemsetAsync(sc.work.ctr, 0, sizeof(int) * nchains * (size_t)c->nkc, st));
         if (c->kc_prec == BSE_PREC_BF16) {
             BSE_CUDA_TRY(ctx, cudaMemsetAsync(sc.bop, 0, sizeof(__nv_bfloat16) * 16 * (size_t)c->ldk, st));
-            if ((rc = bse_common_restrict(ctx, s, s->cwork[1], nchains, psi, nullptr, sc.bop, st)) != BSE_OK) return rc;
+            if ((rc = bse_common_restrict(ctx, s, sc.work, nchains, psi, nullptr, sc.bop, st)) != BSE_OK) return rc;
             if ((rc = bse_tc_apply_scratch(ctx, s, nchains, sc.bop, sc.part, sc.R)) != BSE_OK) return rc;
         } else {
-            if ((rc = bse_common_restrict(ctx, s, s->cwork[1], nchains, psi, sc.Q, nullptr, st)) != BSE_OK) return rc;
+            if ((rc = bse_common_restrict(ctx, s, sc.work, nchains, psi, sc.Q, nullptr, st)) != BSE_OK) return rc;
             launch_kc_simt<T>(ctx, c, sc.Q, nchains, sc.R, st);
         }
-        if (m3 && (rc = bse_common_near(ctx, s, s->cwork[1], nchains, st)) != BSE_OK) return rc;
-        return bse_common_prolong(ctx, s, s->cwork[1], nchains, sc.R, psi, W, sc.dot, st);
+        if (m3 && (rc = bse_common_near(ctx, s, sc.work, nchains, st)) != BSE_OK) return rc;
+        return bse_common_prolong(ctx, s, sc.work, nchains, sc.R, psi, W, sc.dot, st);
     }
     const bool xh = near_tc_active(s);
     void* X = m3 ? sc.X : nullptr;

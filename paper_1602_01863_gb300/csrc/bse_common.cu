@@ -1142,18 +1142,9 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s) {
         if ((rc_ = bse_alloc(ctx, x.dst, sizeof(V) * x.n, "gauge tables")) != BSE_OK) return rc_;
         k_gauge_to<T><<<(unsigned)((x.n + 255) / 256), 256, 0, st>>>(x.src, (long long)x.n, (V*)*x.dst);
     }
-    // both sets of intermediate vectors, each kind in one allocation that the first owns
-    auto both = [&](void** first, void** second, size_t bytes, bool clear, const char* what) -> int {
-        bytes = (bytes + 255) / 256 * 256;
-        const int rc = bse_alloc(ctx, first, 2 * bytes, what);
-        if (rc != BSE_OK) return rc;
-        *second = (unsigned char*)*first + bytes;
-        if (clear) BSE_CUDA_TRY(ctx, cudaMemsetAsync(*first, 0, 2 * bytes, st));
-        return BSE_OK;
-    };
-    CommonWork &w0 = s->cwork[0], &w1 = s->cwork[1];
-    if ((rc_ = both(&w0.share, &w1.share, sizeof(V) * BSE_MAX_CHAINS * 8 * (size_t)c->Nc, false, "corner shares")) != BSE_OK) return rc_;
-    if ((rc_ = both((void**)&w0.ctr, (void**)&w1.ctr, sizeof(int) * BSE_MAX_CHAINS * (size_t)c->nkc, true, "corner counters")) != BSE_OK) return rc_;
+    if ((rc_ = bse_alloc(ctx, &s->cwork.share, sizeof(V) * BSE_MAX_CHAINS * 8 * (size_t)c->Nc, "corner shares")) != BSE_OK) return rc_;
+    if ((rc_ = bse_alloc(ctx, (void**)&s->cwork.ctr, sizeof(int) * BSE_MAX_CHAINS * (size_t)c->nkc, "corner counters")) != BSE_OK) return rc_;
+    BSE_CUDA_TRY(ctx, cudaMemsetAsync(s->cwork.ctr, 0, sizeof(int) * BSE_MAX_CHAINS * (size_t)c->nkc, st));
     if (s->scheme != BSE_SCHEME_M3) {
         BSE_CUDA_TRY(ctx, cudaStreamSynchronize(st));
         return BSE_OK;
@@ -1163,8 +1154,10 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s) {
     s->cphi_Lp = L + 2 * R + (nd > 4 ? 3 : 0);
     const size_t groups = (2 * (size_t)s->t * BSE_MAX_CHAINS + 31) / 32;
     const size_t nphi = groups * L * L * (size_t)s->cphi_Lp * 32;
-    if ((rc_ = both(&w0.phi, &w1.phi, sizeof(T) * nphi, true, "common-basis vectors")) != BSE_OK) return rc_;   // unused columns stay zero
-    if ((rc_ = both(&w0.V, &w1.V, sizeof(V) * BSE_MAX_CHAINS * (size_t)s->N, false, "near stencil result")) != BSE_OK) return rc_;
+    // unused columns stay zero (they and what a padded target reads are summed up but never stored)
+    if ((rc_ = bse_alloc(ctx, &s->cwork.phi, sizeof(T) * nphi, "common-basis vectors")) != BSE_OK) return rc_;
+    BSE_CUDA_TRY(ctx, cudaMemsetAsync(s->cwork.phi, 0, sizeof(T) * nphi, st));
+    if ((rc_ = bse_alloc(ctx, &s->cwork.V, sizeof(V) * BSE_MAX_CHAINS * (size_t)s->N, "near stencil result")) != BSE_OK) return rc_;
     // source rows of a warp's targets: (delta_1 + R, u), u - y the delta_2 + R of target row y,
     // with the reach along z of each row (a byte each, plus one; 0: outside the ball) and the largest
     std::vector<int2> steps;
@@ -1201,6 +1194,25 @@ int prepare_typed(bse_ctx* ctx, bse_interp* s) {
 }  // namespace
 
 int bse_common_dot_blocks(const bse_interp* s) { return std::min(s->co->nkc, BSE_MAX_VEC_BLOCKS); }
+
+size_t bse_common_work(const bse_interp* s, int nvec, unsigned char* base, CommonWork* w) {
+    const size_t T = s->vec_prec == BSE_PREC_F64 ? sizeof(double) : sizeof(float), V = 2 * T, L = (size_t)s->n * s->nd;
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        unsigned char* p = base + off;
+        off += (bytes + 255) / 256 * 256;
+        return (void*)p;
+    };
+    CommonWork q;
+    if (s->scheme == BSE_SCHEME_M3) {
+        q.phi = take(T * ((2 * (size_t)s->t * nvec + 31) / 32) * 32 * L * L * s->cphi_Lp);
+        q.V = take(V * nvec * (size_t)s->N);
+    }
+    q.share = take(V * nvec * 8 * (size_t)s->co->Nc);
+    q.ctr = (int*)take(sizeof(int) * nvec * (size_t)s->co->nkc);
+    *w = q;
+    return off;
+}
 
 int bse_common_prepare(bse_ctx* ctx, bse_interp* s) {
     return s->vec_prec == BSE_PREC_F64 ? prepare_typed<double>(ctx, s) : prepare_typed<float>(ctx, s);

@@ -260,7 +260,9 @@ struct bse_interp {
     int common = 0;
     void *d_cUv = nullptr, *d_cUc = nullptr;     // V [nk][nv*nv], [nk][nc*nc] dense gauge
     void *d_cUvc = nullptr, *d_cUcc = nullptr;   // V [nkc][nv*nv], [nkc][nc*nc] coarse gauge
-    CommonWork cwork[2];             // the handle's own calls; bse_apply_h_noalloc (parts of the same allocations)
+    CommonWork cwork;                // of the handle's own calls
+    CommonWork cwork_na;             // of bse_apply_h_noalloc, where its static array has no room,
+    void* d_na = nullptr;            // in this allocation
     int cphi_R = 0, near_R2 = 0;     // near offsets: |delta|^2 <= near_R2, components within cphi_R
     int cphi_Lp = 0;
     int n_csteps = 0;
@@ -437,6 +439,7 @@ struct ApplyScratch {
     double2* dot;            // [nvec][BSE_MAX_VEC_BLOCKS]
     __nv_bfloat16* bop;      // [16][ldk]          (BF16 path only)
     float* part;             // tile partials      (BF16 path only)
+    CommonWork work;         // common-basis path
 };
 int bse_launch_near_field(bse_ctx* ctx, const bse_interp* s, int nchains, const void* X, const float* xscale, void* U);
 int bse_apply_learned(bse_ctx* ctx, const bse_interp* s, int nchains, const void* psi, void* w, double2* dot);
@@ -451,6 +454,9 @@ int bse_near_tc_launch(bse_ctx* ctx, const bse_interp* s, int nchains, const voi
 // common-basis path (bse_common.cu)
 int bse_common_prepare(bse_ctx* ctx, bse_interp* s);
 int bse_common_dot_blocks(const bse_interp* s);
+// Carves the intermediate vectors of an application to nvec vectors out of `base`; returns the bytes.
+size_t bse_common_work(const bse_interp* s, int nvec, unsigned char* base, CommonWork* w);
+int bse_noalloc_setup(bse_ctx* ctx, bse_interp* s);
 int bse_common_restrict(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, const void* psi, void* Q,
                         __nv_bfloat16* bop, cudaStream_t st);
 int bse_common_near(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, cudaStream_t st);

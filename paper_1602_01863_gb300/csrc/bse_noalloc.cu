@@ -7,9 +7,11 @@
 // loop in which cudaMalloc's implicit device-wide synchronisation is not
 // allowed.  bse_apply_h takes its per-call scratch from the handle, which
 // bse_interp_setup allocated; this variant takes it from the file-scope
-// array below, and on the common-basis path its intermediate vectors from a
-// set of their own in the handle, so after set-up nothing is allocated on any
-// path and the call may run beside another one on the same handle.
+// array below instead, so after set-up nothing is allocated on any path and the
+// call may run beside another one on the same handle.  On the common-basis path
+// the intermediate vectors lie where the general path has its pieces (reserved on
+// both), or behind the rest; with few transitions (up to three, in columns of 32)
+// and a size near the array's end they may fit in neither: set-up then allocates them.
 //
 // The array is a static __device__ object of the library's device module: a
 // device holds BSE_NOALLOC_SCRATCH_BYTES of it from the moment that module is
@@ -39,7 +41,59 @@ std::mutex g_scratch_mu;
 
 size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
+// Per-call buffers (each 256-byte aligned) of an application to nvec vectors.
+struct Layout {
+    size_t Q, R, X, U, D, B = 0, P = 0, total = 0;        // total: what counts towards the array's size
+    size_t work = 0;                                       // common-basis path: its intermediate vectors,
+    bool work_fits = true;                                 // where the array has room for them
+};
+Layout layout(const bse_interp* s, int nvec) {
+    const bse_coarse* c = s->co;
+    const size_t vsz = (s->vec_prec == BSE_PREC_F64) ? sizeof(double2) : sizeof(float2);
+    const bool m3 = s->scheme == BSE_SCHEME_M3, bf16 = c->kc_prec == BSE_PREC_BF16;
+    Layout l;
+    auto take = [&](size_t bytes) {
+        const size_t o = l.total;
+        l.total += align256(bytes);
+        return o;
+    };
+    l.Q = take(vsz * nvec * c->Nc);
+    l.R = take(vsz * nvec * c->Nc);
+    l.X = take(m3 ? vsz * nvec * (size_t)s->nk * 8 * s->t : 0);
+    l.U = take(m3 ? vsz * nvec * (size_t)s->nk * 8 * s->t : 0);
+    l.D = take(sizeof(double2) * nvec * BSE_MAX_VEC_BLOCKS);
+    if (bf16) {
+        l.B = take(sizeof(__nv_bfloat16) * 16 * (size_t)c->ldk);
+        l.P = take(bse_tc_part_bytes(s));
+    }
+    if (s->common) {
+        CommonWork w;
+        const size_t need = bse_common_work(s, nvec, nullptr, &w);
+        l.work = need <= l.D - l.X ? l.X : l.total;
+        l.work_fits = l.work + need <= (l.work == l.X ? l.D : (size_t)BSE_NOALLOC_SCRATCH_BYTES);
+    }
+    return l;
+}
+
 }  // namespace
+
+// A set of intermediate vectors for the sizes that bse_apply_h_noalloc takes and
+// the array has no room for; most handles need none.
+int bse_noalloc_setup(bse_ctx* ctx, bse_interp* s) {
+    size_t bytes = 0;
+    int most = 0;
+    for (int nvec = 1; nvec <= BSE_MAX_CHAINS; ++nvec) {
+        const Layout l = layout(s, nvec);
+        if (l.total > BSE_NOALLOC_SCRATCH_BYTES || l.work_fits) continue;
+        CommonWork w;
+        bytes = bse_common_work(s, nvec, nullptr, &w);
+        most = nvec;
+    }
+    if (!most) return BSE_OK;
+    const int rc = bse_alloc(ctx, &s->d_na, bytes, "intermediate vectors of bse_apply_h_noalloc");
+    if (rc == BSE_OK) bse_common_work(s, most, (unsigned char*)s->d_na, &s->cwork_na);
+    return rc;
+}
 
 int bse_noalloc_prepare(bse_ctx* ctx) {
     if (ctx->device < 0 || ctx->device >= BSE_NOALLOC_MAX_DEVICES) return BSE_OK;   // the entry point refuses it
@@ -79,38 +133,26 @@ extern "C" int bse_apply_h_noalloc(bse_ctx* ctx, bse_interp* s, int nvec, const 
         ctx->err = "the static scratch of this device was not set up (bse_ctx_create)";
         return BSE_ERR_CUDA;
     }
-    // Carve the per-call buffers (each 256-byte aligned) out of the array.
-    const bse_coarse* c = s->co;
-    const size_t vsz = (s->vec_prec == BSE_PREC_F64) ? sizeof(double2) : sizeof(float2);
-    const bool m3 = s->scheme == BSE_SCHEME_M3;
-    const bool bf16 = c->kc_prec == BSE_PREC_BF16;
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        const size_t o = off;
-        off += align256(bytes);
-        return o;
-    };
-    const size_t oQ = take(vsz * nvec * c->Nc);
-    const size_t oR = take(vsz * nvec * c->Nc);
-    const size_t oX = m3 ? take(vsz * nvec * (size_t)s->nk * 8 * s->t) : 0;
-    const size_t oU = m3 ? take(vsz * nvec * (size_t)s->nk * 8 * s->t) : 0;
-    const size_t oD = take(sizeof(double2) * nvec * BSE_MAX_VEC_BLOCKS);
-    const size_t oB = bf16 ? take(sizeof(__nv_bfloat16) * 16 * (size_t)c->ldk) : 0;
-    const size_t oP = bf16 ? take(bse_tc_part_bytes(s)) : 0;
-    if (off > BSE_NOALLOC_SCRATCH_BYTES) {
-        ctx->err = "bse_apply_h_noalloc needs " + std::to_string(off) + " bytes of scratch; the static array holds " +
+    const Layout l = layout(s, nvec);
+    if (l.total > BSE_NOALLOC_SCRATCH_BYTES) {
+        ctx->err = "bse_apply_h_noalloc needs " + std::to_string(l.total) + " bytes of scratch; the static array holds " +
                    std::to_string((size_t)BSE_NOALLOC_SCRATCH_BYTES) + " (use bse_apply_h)";
         return BSE_ERR_UNSUPPORTED;
     }
+    const bool m3 = s->scheme == BSE_SCHEME_M3, bf16 = s->co->kc_prec == BSE_PREC_BF16;
     unsigned char* b = static_cast<unsigned char*>(base);
     ApplyScratch sc;
-    sc.Q = b + oQ;
-    sc.R = b + oR;
-    sc.X = m3 ? b + oX : nullptr;
-    sc.U = m3 ? b + oU : nullptr;
-    sc.dot = reinterpret_cast<double2*>(b + oD);
-    sc.bop = bf16 ? reinterpret_cast<__nv_bfloat16*>(b + oB) : nullptr;
-    sc.part = bf16 ? reinterpret_cast<float*>(b + oP) : nullptr;
+    sc.Q = b + l.Q;
+    sc.R = b + l.R;
+    sc.X = m3 ? b + l.X : nullptr;
+    sc.U = m3 ? b + l.U : nullptr;
+    sc.dot = reinterpret_cast<double2*>(b + l.D);
+    sc.bop = bf16 ? reinterpret_cast<__nv_bfloat16*>(b + l.B) : nullptr;
+    sc.part = bf16 ? reinterpret_cast<float*>(b + l.P) : nullptr;
+    if (s->common) {
+        if (l.work_fits) bse_common_work(s, nvec, b + l.work, &sc.work);
+        else sc.work = s->cwork_na;
+    }
     int rc = bse_apply_scratch(ctx, s, nvec, x, y, sc);
     if (rc != BSE_OK) return rc;
     cudaError_t e = cudaStreamSynchronize(ctx->stream);

@@ -896,6 +896,7 @@ int setup_interp_typed(bse_ctx* ctx, bse_interp* s, const bse_dense_inputs* dens
         }
     }
     if (c->kc_prec == BSE_PREC_BF16) TRY(bse_tc_prepare(ctx, s));
+    if (s->common) TRY(bse_noalloc_setup(ctx, s));
     return BSE_OK;
 }
 

@@ -17,14 +17,19 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("name,kc,vec,scheme,caller", [
-    ("m3-f64", 0, 0, 1, False), ("m3-mixed", 2, 1, 1, False), ("m1-f32", 1, 1, 0, False),
-    ("caller-f32", 1, 1, 1, True), ("caller-mixed", 2, 1, 1, True)], ids=lambda v: v if isinstance(v, str) else "")
-def test_noalloc_beside_a_recursion(name, kc, vec, scheme, caller):
+@pytest.mark.parametrize("name,kc,vec,scheme,caller,shape", [
+    ("m3-f64", 0, 0, 1, False, (3, 3, 4, 2, 2)), ("m3-mixed", 2, 1, 1, False, (3, 3, 4, 2, 2)),
+    ("m1-f32", 1, 1, 0, False, (3, 3, 4, 2, 2)),
+    ("caller-f32", 1, 1, 1, True, (3, 3, 4, 2, 2)), ("caller-mixed", 2, 1, 1, True, (3, 3, 4, 2, 2)),
+    ("behind-the-rest", 1, 1, 1, False, (1, 1, 4, 2, 1)),     # columns of 32 take more than the pieces' place
+    ("set-of-its-own", 0, 0, 1, False, (1, 1, 11, 4, 1)),     # and more than the array: 21.9 MB count, 27 MB follow
+], ids=lambda v: v if isinstance(v, str) else "")
+def test_noalloc_beside_a_recursion(name, kc, vec, scheme, caller, shape):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_1602_01863_gb300 import bse
-    m, n, nd, nvec = synth.draw_model(95, 3, 3), 4, 2, 2
+    nv, nc, n, nd, nvec = shape
+    m = synth.draw_model(95, nv, nc)
     dense = None
     if caller:
         I = oi.Interp(m, n, nd, build_dense_kc=False)
@@ -40,7 +45,7 @@ def test_noalloc_beside_a_recursion(name, kc, vec, scheme, caller):
 
     dt = torch.complex128 if vec == 0 else torch.complex64
     # norms that differ by far, so that FP16 pieces need scales of their own
-    x = (torch.from_numpy(synth.random_vectors(11, (nvec, it.N))) * torch.tensor([[1e3], [1e-4]])).cuda().to(dt)
+    x = (torch.from_numpy(synth.random_vectors(11, (nvec, it.N))) * torch.tensor([[1e3], [1e-4]])[:nvec]).cuda().to(dt)
     y = torch.empty_like(x)
     torch.cuda.synchronize()
 
@@ -50,7 +55,11 @@ def test_noalloc_beside_a_recursion(name, kc, vec, scheme, caller):
             return y.clone()
 
     ref_run, ref_y = recursion(), apply()
+    own = torch.empty_like(x)
+    run.bse_apply_h(it, nvec, x.data_ptr(), own.data_ptr())
     torch.cuda.synchronize()
+    tol = 1e-12 if vec == 0 else 1e-5
+    assert all(bool((p - q).abs().max() <= tol * p.abs().max()) for p, q in zip(own, ref_y))
     assert all(np.all(np.isfinite(v)) for v in ref_run) and bool(torch.isfinite(torch.view_as_real(ref_y)).all())
     got, done = [], threading.Event()
 
