@@ -375,8 +375,9 @@ int mlp_forward(bse_ctx* ctx, bse_mlp* m, int B, const float* X, float* out) {
 }
 
 // Loss and gradients into m->d_g; the loss (mean over the batch of the squared
-// error summed over Re, Im) into *loss.
-int mlp_grads(bse_ctx* ctx, bse_mlp* m, int B, const float* X, const float* Y, double* loss) {
+// error summed over Re, Im) into *loss, the gradients also to the host where asked
+// for, with one wait for both.
+int mlp_grads(bse_ctx* ctx, bse_mlp* m, int B, const float* X, const float* Y, double* loss, float* grad_host) {
     const size_t sm = mlp_smem(true);
     BSE_CUDA_TRY(ctx, bse_raise_smem(k_mlp<true>, sm));
     const int nblk = std::min((B + RT - 1) / RT, m->blocks);
@@ -386,6 +387,8 @@ int mlp_grads(bse_ctx* ctx, bse_mlp* m, int B, const float* X, const float* Y, d
     BSE_CUDA_TRY(ctx, cudaGetLastError());
     std::vector<double> part(nblk);
     BSE_CUDA_TRY(ctx, cudaMemcpyAsync(part.data(), m->d_part, sizeof(double) * nblk, cudaMemcpyDeviceToHost, ctx->stream));
+    if (grad_host)
+        BSE_CUDA_TRY(ctx, cudaMemcpyAsync(grad_host, m->d_g, sizeof(float) * m->nparams, cudaMemcpyDeviceToHost, ctx->stream));
     BSE_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
     double s = 0.0;
     for (double v : part) s += v;
@@ -994,16 +997,13 @@ int bse_mlp_forward(bse_ctx* ctx, bse_mlp* m, int batch, const float* X, float* 
 int bse_mlp_gradients(bse_ctx* ctx, bse_mlp* m, int batch, const float* X, const float* Y, float* grad_host, double* loss) {
     if (!ctx || !m || !X || !Y || !grad_host) return BSE_ERR_ARG;
     if (batch < 1 || batch > m->max_batch) { ctx->err = "batch outside 1..max_batch"; return BSE_ERR_ARG; }
-    int rc = mlp_grads(ctx, m, batch, X, Y, loss);
-    if (rc != BSE_OK) return rc;
-    BSE_CUDA_TRY(ctx, bse_download(ctx, grad_host, m->d_g, sizeof(float) * m->nparams));
-    return BSE_OK;
+    return mlp_grads(ctx, m, batch, X, Y, loss, grad_host);
 }
 
 int bse_mlp_train_step(bse_ctx* ctx, bse_mlp* m, int batch, const float* X, const float* Y, float lr, double* loss) {
     if (!ctx || !m || !X || !Y) return BSE_ERR_ARG;
     if (batch < 1 || batch > m->max_batch || !(lr > 0.f)) { ctx->err = "bad batch or learning rate"; return BSE_ERR_ARG; }
-    int rc = mlp_grads(ctx, m, batch, X, Y, loss);
+    int rc = mlp_grads(ctx, m, batch, X, Y, loss, nullptr);
     if (rc != BSE_OK) return rc;
     m->step += 1;
     const float b1 = 0.9f, b2 = 0.999f;
