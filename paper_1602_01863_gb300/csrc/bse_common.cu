@@ -1058,6 +1058,11 @@ int launch_near_r(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, con
     else return launch_near_k<T>(ctx, s, work, k_common_near<TY, TZ, RM>, RM, ns, st);
 }
 
+// The bodies with the reach unrolled end at R = 4 (n_div up to 3) and 6; beyond, and with
+// n_div above 4 for the runs of cells, the offsets are looped over.  That form against
+// the general kernels, FP32, one application: coarse 8^3, n_div 4, 4x4 bands, 3 vectors, R = 8
+// 24.6 -> 1.17 ms, R = 12 72.5 -> 3.08 ms; coarse 12^3, n_div 2, 2x3 bands, 3 vectors, R = 6
+// 25.8 -> 0.57 ms; coarse 4^3, n_div 8, 2x2 bands, 1 vector, R = 8 39.0 -> 0.48 ms (FP64 58.7 -> 4.29).
 template <typename T>
 int near_typed(bse_ctx* ctx, const bse_interp* s, const CommonWork& work, int nchains, cudaStream_t st) {
     NearStencil ns{};

@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(256) k_form_factors(const double2* __restrict_
 // not four.  Its imaginary part is a difference of larger sums: over random form
 // factors the error of the 64-bit sums is 2.1e-14 against 1.5e-14 of four products
 // (real part 1.2e-14 against 1.5e-14; sums up to 330), far below the rounding of either
-// storage, but not of complex128, which keeps four.  N_c = 8192, BF16: 26.1 ms
+// storage, but not of complex128, which keeps four (N_c = 8192: 7.0 ms, three take
+// 6.0).  N_c = 8192, BF16: 26.1 ms
 // with one thread per entry of the whole matrix (a run of set-up, 24 steps and
 // spectrum: 58.7 ms; 17.3 ms with this set-up and the common-basis step loop).
 // Output in the storage precision of the handle.

@@ -92,7 +92,8 @@ def test_dense_tables_of_few_bands(ctx, nv, nc, n, nd, prec):
 
 
 def test_time_of_dense_tables_with_one_band_pair(ctx):
-    """A point of 1x1 bands is less work than one of 2x2 bands, so it takes no longer (a tenth for noise)."""
+    """A point of 1x1 bands is a quarter of the work of one of 2x2 bands and has a quarter of the lanes, so its
+    tables take well below the time of theirs (a warp to each point: 0.85 of it)."""
     from paper_1602_01863_gb300 import bse
     t = []
     for nb in (1, 2):
@@ -100,4 +101,4 @@ def test_time_of_dense_tables_with_one_band_pair(ctx):
         t.append(_median_ms(lambda: ctx.bse_interp_setup(co, 8, bse.SCHEME_M1, 1.0, 1)))
         co.free()
     print(f"set-up of 262144 points, 1x1 bands {t[0]:.2f} ms, 2x2 bands {t[1]:.2f} ms")
-    assert t[0] <= 1.1 * t[1] and t[0] <= 1.5
+    assert t[0] <= 0.7 * t[1]
