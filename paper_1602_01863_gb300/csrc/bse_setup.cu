@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(256) k_form_factors(const double2* __restrict_
 // spectrum: 58.7 ms; 17.3 ms with this set-up and the common-basis step loop).
 // Output in the storage precision of the handle.
 // A tile is filled with as many points as 64 entries hold, so that no multiply-add is
-// spent on padding; only the pairs' overlaps of 1x1 bands have to leave some (54 points
+// spent on padding; only the pairs' overlaps of 1x1 bands have to leave some (55 points
 // of 64).  Coarse 16^3, 1x1 bands, the whole of bse_build_coarse: 5.8 ms with a thread per
 // entry, 74 ms with at most eight points to a tile (64 of 4096 entries used), 2.8 ms so.
 constexpr int KC_T = 64;

@@ -1,7 +1,7 @@
 """Set-up of systems with few bands: tiles of K_c and warps of the dense tables hold as many points as fit.
 
 K_c against the oracle (1e-13 of max |K|, the bar of the other K_c tests) where tiles of
-54, 32, 21, 16, 12 and 9 points end, and the time of bse_build_coarse for 1x1 bands
+55, 32, 21, 16, 12 and 9 points end, and the time of bse_build_coarse for 1x1 bands
 against 2x2 bands of nearly the same dimension: the work per entry is the
 same but for the smaller tiles and the padding of the last ones, so three times
 as long is too long.
