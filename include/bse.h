@@ -230,7 +230,7 @@ int bse_apply_h(bse_ctx* ctx, bse_interp* interp, int nvec, const void* x, void*
  * (held by a device from the time the library's device module is loaded on
  * it, at the latest the first bse_ctx_create on that device, until the
  * process exits), not from the buffers of the handle's other calls (for some
- * sizes with up to three transitions bse_interp_setup allocates a set of
+ * sizes near the array's end bse_interp_setup allocates a set of
  * intermediate vectors for it).  So one such call may run beside another call on
  * the same handle (through a context of its own).  The paper has no counterpart; this
  * exists for callers that must not call cudaMalloc once their work has

@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
         __syncthreads();
         for (int c = 0; c < ncb; ++c) {
             const int ch = c0 + c;
-            DotSum<T> dsm;
+            DotSum<T> dsm = DotSum<T>::zero();
             V rr[EPL][8];
 #pragma unroll
             for (int a = 0; a < EPL; ++a) {
@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(256, EPL == 2 ? 1 : (sizeof(T) == 4 ? 3 : 2)) 
         }
         __syncthreads();
         if (warp < ncb) {
-            DotSum<T> low;
+            DotSum<T> low = DotSum<T>::zero();
 #pragma unroll
             for (int q = 0; q < 8; ++q) dsum[warp][lane + 32 * q].into(dot, low);
             dot = cadd(dot, low.value());

@@ -104,7 +104,8 @@ __device__ __forceinline__ F2 f2_sub(F2 a, F2 b) {
 // by up to 1e-8 of itself), 4.99 ms with 40 scalar operations, 4.94 ms so (1e-14).
 template <typename T> struct DotSum;
 template <> struct DotSum<double> {
-    double2 s = {0.0, 0.0};
+    double2 s;
+    static __device__ __forceinline__ DotSum zero() { return DotSum{make_double2(0.0, 0.0)}; }
     __device__ __forceinline__ void add(double2 p, double2 w) {
         s.x = fma(p.x, w.x, fma(p.y, w.y, s.x));
         s.y = fma(p.x, w.y, fma(-p.y, w.x, s.y));
@@ -114,7 +115,8 @@ template <> struct DotSum<double> {
     __device__ __forceinline__ void into(double2& d, DotSum&) const { d.x += s.x; d.y += s.y; }
 };
 template <> struct DotSum<float> {
-    float2 s = {0.f, 0.f}, c = {0.f, 0.f};                      // sums and what they lack
+    float2 s, c;                                                 // sums and what they lack
+    static __device__ __forceinline__ DotSum zero() { return DotSum{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
     // both parts at once, in packed operations: s += a b, c += what that rounded off
     __device__ __forceinline__ void one(float a, float bx, float by) {
         const F2 s0 = f2_pair(s.x, s.y), b = f2_pair(bx, by);

@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(LTHR) k_lconv_inv(const float2* __restrict__ g
     lines_inv(s, ne * L, [&](int l) { const int e = quot(l, inv_L); return e * (L - 1) * P + e * (P - L) + l; }, P, q.A, q.B, tw);
     lines_inv(s, ne * L, [&](int l) { return l * P; }, 1, q.A, q.B, tw);
     const size_t nk = (size_t)L2 * L;
-    DotSum<T> dot;
+    DotSum<T> dot = DotSum<T>::zero();
 #pragma unroll 4
     for (int i = tid; i < L2 * EG; i += LTHR) {
         const int e = i & (EG - 1), p = i / EG, y = quot(p, inv_L), z = p - y * L;

@@ -10,8 +10,9 @@
 // array below instead, so after set-up nothing is allocated on any path and the
 // call may run beside another one on the same handle.  On the common-basis path
 // the intermediate vectors lie where the general path has its pieces (reserved on
-// both), or behind the rest; with few transitions (up to three, in columns of 32)
-// and a size near the array's end they may fit in neither: set-up then allocates them.
+// both), or behind the rest.  Near the array's end they may fit in neither (Method 3
+// with up to three transitions, in columns of 32; Method 1 with a large coarse mesh):
+// set-up then allocates them.
 //
 // The array is a static __device__ object of the library's device module: a
 // device holds BSE_NOALLOC_SCRATCH_BYTES of it from the moment that module is
